@@ -132,7 +132,9 @@ int launch_small_rr(const typename cplx_t<R>::type* GA, const typename cplx_t<R>
 // flops is given, the algorithmic flops of every problem solved are added to it (device counter).
 int launch_small_rr32(const float2* GA, const float2* GO, int n, int m, int nk, float drop_tol, const int* kdone,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
-                      cudaStream_t s);
+                      float4* rotlog, long long log_stride, cudaStream_t s);
+// float4 elements of global scratch a problem of size n needs for its rotations (log_stride at least this).
+long long small_rr32_log(int n);
 // Cholesky-QR transform of the Gram G (m x m per k).  When Gref is given (rows_ref x m per
 // k, scale -1, its last m rows holding -Y^H Omega Y before projection), a column whose
 // Omega-norm^2 after projection is below rel_tol times the one before is dropped.

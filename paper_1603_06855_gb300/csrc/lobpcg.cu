@@ -562,16 +562,17 @@ int launch_small_rr(const typename cplx_t<R>::type* GA, const typename cplx_t<R>
 template int launch_small_rr<double>(const double2*, const double2*, int, int, int, double, const int*, double*, double2*, int*, cudaStream_t);
 
 // Cholesky-QR transform: T = D Li^H with zero columns for dropped coordinates.
+// One warp factors (warp_chol_inverse); the others only load, scale and store.
 template <typename R>
-__global__ __launch_bounds__(256) void k_small_chol(const typename cplx_t<R>::type* __restrict__ G, int m, R drop_tol,
+__global__ __launch_bounds__(128) void k_small_chol(const typename cplx_t<R>::type* __restrict__ G, int m, R drop_tol,
                                                     const typename cplx_t<R>::type* __restrict__ Gref, int rows_ref,
                                                     R rel_tol, typename cplx_t<R>::type* __restrict__ T) {
   typedef typename cplx_t<R>::type C2;
   __shared__ C2 B[24 * 25];
-  __shared__ C2 tmp[24];
+  __shared__ C2 X[24 * 25];
   __shared__ R D[24];
   __shared__ int drop[24];
-  const int ld = m + ((m & 1) ? 0 : 1);
+  const int ld = m | 1;
   const int k = blockIdx.x;
   const C2* g = G + (long long)k * m * m;
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
@@ -592,13 +593,13 @@ __global__ __launch_bounds__(256) void k_small_chol(const typename cplx_t<R>::ty
     B[i * ld + c] = mk<R>((b1.x + b2.x) * s, (b1.y - b2.y) * s);
   }
   __syncthreads();
-  chol_drop<R>(B, m, ld, drop_tol, drop);
-  tri_inv_lower<R>(B, m, ld, tmp);
+  if (threadIdx.x < 32) warp_chol_inverse<R>(B, X, m, ld, drop_tol, drop);
+  __syncthreads();
   C2* tk = T + (long long)k * m * m;
   for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
     int i = t / m, c = t % m;
     // T[i][c] = D_i conj(Li[c][i]); dropped columns vanish
-    C2 v = (c >= i && !drop[c]) ? cscale(cconj(B[c * ld + i]), D[i]) : mk<R>(0, 0);
+    C2 v = (c >= i && !drop[c]) ? cscale(cconj(X[c * ld + i]), D[i]) : mk<R>(0, 0);
     tk[t] = v;
   }
 }
@@ -607,7 +608,7 @@ int launch_small_chol(const typename cplx_t<R>::type* G, int m, int nk, R drop_t
                       const typename cplx_t<R>::type* Gref, int rows_ref, R rel_tol, typename cplx_t<R>::type* T,
                       cudaStream_t s) {
   if (m > 24) return PC_EINVAL;
-  k_small_chol<R><<<nk, 256, 0, s>>>(G, m, drop_tol, Gref, rows_ref, rel_tol, T);
+  k_small_chol<R><<<nk, 128, 0, s>>>(G, m, drop_tol, Gref, rows_ref, rel_tol, T);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }

@@ -74,6 +74,8 @@ struct pc_ctx {
   void *E = nullptr, *S = nullptr;  // strain / stress stacks (R precision)
   void *gpart = nullptr, *GA = nullptr, *GO = nullptr, *Cc = nullptr, *Ct = nullptr;
   void* lam = nullptr;           // nk*m (R)
+  float4* rotlog = nullptr;      // per k: rotations of the FP32 projected problem (small_rr.cu)
+  long long log_stride = 0;
   double *rnorm = nullptr;
   int *active = nullptr, *d_unconv = nullptr, *kdone = nullptr, *kdone_f = nullptr;
   double* stall_best = nullptr;  // per k: best worst-wanted residual so far (stagnation test)
@@ -235,7 +237,7 @@ static void free_kset(pc_ctx* c) {
   if (c->S) cudaFree(c->S); c->S = nullptr;
   void** vs[] = {&c->gpart, &c->GA, &c->GO, &c->Cc, &c->Ct, &c->lam};
   for (auto v : vs) { if (*v) cudaFree(*v); *v = nullptr; }
-  dfree(c->rnorm); dfree(c->active); dfree(c->d_unconv); dfree(c->kdone); dfree(c->kdone_f);
+  dfree(c->rotlog); dfree(c->rnorm); dfree(c->active); dfree(c->d_unconv); dfree(c->kdone); dfree(c->kdone_f);
   dfree(c->stall_best); dfree(c->stall_since);
   dfree(c->Xd); dfree(c->AXd); dfree(c->OXd); dfree(c->Ed); dfree(c->Sd); dfree(c->Th); dfree(c->St);
   dfree(c->gpartd); dfree(c->GAd); dfree(c->GOd); dfree(c->Cd);
@@ -455,6 +457,10 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   if (cudaMalloc(&c->Cc, g * esz) != cudaSuccess) { c->Cc = nullptr; rc = PC_ENOMEM; }
   if (cudaMalloc(&c->Ct, g * esz) != cudaSuccess) { c->Ct = nullptr; rc = PC_ENOMEM; }
   if (cudaMalloc(&c->lam, nvec * rsz) != cudaSuccess) { c->lam = nullptr; rc = PC_ENOMEM; }
+  if (c->prm.precision == PC_MIXED) {
+    c->log_stride = small_rr32_log(3 * m);
+    rc |= dalloc(&c->rotlog, (size_t)nk * c->log_stride);
+  }
   rc |= dalloc(&c->rnorm, nvec);
   rc |= dalloc(&c->active, nvec);
   rc |= dalloc(&c->d_unconv, (size_t)kMaxGroups);
@@ -716,12 +722,13 @@ template <> struct SmallTol<double> { static constexpr double pdir_abs = 1e-26; 
 template <> struct SmallTol<float> { static constexpr float pdir_abs = 1e-12f; };
 
 template <typename R>
-static int small_rr_any(pc_ctx* c, int nk, const typename Ops<R>::C2* GA, const typename Ops<R>::C2* GO, int n, int m,
+static int small_rr_any(pc_ctx* c, int k0, int nk, const typename Ops<R>::C2* GA, const typename Ops<R>::C2* GO, int n, int m,
                         const int* kdone, R* lam, typename Ops<R>::C2* cX, typename Ops<R>::C2* cP, cudaStream_t s) {
   int rc;
   if constexpr (std::is_same<R, float>::value) {  // the conjugate directions from the same CTAs
     rc = launch_small_rr32(GA, GO, n, m, nk, Ops<R>::drop_small, kdone, lam, cX, cP, SmallTol<R>::pdir_abs,
-                           c->status, c->profiling ? c->small_flops : nullptr, s);
+                           c->status, c->profiling ? c->small_flops : nullptr, c->rotlog + k0 * c->log_stride,
+                           c->log_stride, s);
   } else {
     rc = launch_small_rr<R>(GA, GO, n, m, nk, Ops<R>::drop_small, kdone, lam, cX, c->status, s);
     if (!rc && cP) rc = launch_small_pdir<R>(GO, cX, n, m, nk, kdone, SmallTol<R>::pdir_abs, cP, s);
@@ -808,7 +815,7 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
     BlockList<R> A1 = {{X, nullptr, nullptr}}, B1 = {{AX, nullptr, nullptr}}, B2 = {{OX, nullptr, nullptr}};
     TRY(gram_ph<R>(c, A1, 1, B1, 1, nk, m, n3, (R)1, part, GA, s));
     TRY(gram_ph<R>(c, A1, 1, B2, 1, nk, m, n3, (R)1, part, GO, s));
-    TRY(small_rr_any<R>(c, nk, GA, GO, m, m, kdone, lam, Cc, nullptr, s));
+    TRY(small_rr_any<R>(c, k0, nk, GA, GO, m, m, kdone, lam, Cc, nullptr, s));
     UpdateArgs<R> u = upd<R>(c, nk, 1, 0, Cc, (long long)m * m, m, m);
     u.in[0][0] = X; u.in[1][0] = AX; u.in[2][0] = OX;
     u.out[0] = Xn; u.out[1] = AXn; u.out[2] = OXn;
@@ -900,7 +907,7 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
     TRY(gram_ph<R>(c, S1, ns, SO, ns, nk, m, n3, (R)1, part, GO, s));
     {
       int sl = ph_begin(c, PH_SMALL, 0.0, s);
-      TRY(small_rr_any<R>(c, nk, GA, GO, n, m, kdone, lam, Cc, Ct, s));
+      TRY(small_rr_any<R>(c, k0, nk, GA, GO, n, m, kdone, lam, Cc, Ct, s));
       ph_end(c, sl, s);
     }
     {

@@ -4,28 +4,35 @@
 //
 // Steps (per k):
 //  1. unit-diagonal scaling D = diag(GO)^-1/2 and Hermitian symmetrisation of both matrices;
-//  2. Cholesky GO = L L^H, blocked: 8-column panels factored by one warp, then the trailing
-//     update by all threads.  A pivot at or below drop_tol drops its coordinate (its row and
-//     column of L become e_j);
-//  3. T = L^-1 GA and L^-1, then C = L^-1 T^H = L^-1 GA L^-H, by blocked forward substitution
-//     (8-row blocks: the update from the solved rows by all threads, then the 8 x 8 diagonal
-//     solve one thread per column); V = L^-H is kept transposed (V^T = conj(L^-1));
+//  2. Cholesky GO = L L^H, blocked: the 8 x 8 diagonal block is factored in registers by the warps
+//     that then solve the panel rows below it (one row per lane, shuffles instead of barriers);
+//     the trailing update is shared by all warps.  A pivot at or below drop_tol drops its
+//     coordinate (its row and column of L become e_j);
+//  3. T = L^-1 GA and L^-1, then the upper triangle of C = L^-1 T^H = L^-1 GA L^-H, by right-looking
+//     blocked forward substitution (8 x 8 diagonal solve, one thread per column, then the rank-8
+//     update of the rows below, four rows per thread);
 //  4. the kept coordinates are packed into a position-ordered upper-triangular copy of C and
 //     diagonalised by cyclic two-sided Jacobi, the n_k/2 disjoint planes of a round ordered
 //     by the circle method.  Positions are pair-ordered: the planes of every round are the
-//     position pairs (2t, 2t+1), and the rotated matrix is written to the other buffer at
-//     the positions the next round gives its indices, so every 2 x 2 block is read from
-//     adjacent rows and columns (16-byte loads).  The planes of the next round are computed
-//     in the same pass from the entries they need (recomputed with the same arithmetic as
-//     the block updates), so a round costs one barrier; blocks, planes and the updates of
-//     V^T (two rows of two elements per unit, on the original coordinates) form one work list
-//     shared by all threads.  A plane rotates when |a_uv| > eps sqrt(|a_uu a_vv|) +
-//     eps max_{i < m} |a_ii| (the absolute floor is the rounding level of the current Ritz
-//     block); after each sweep one pass over all pairs ends the iteration when none would
-//     rotate.
-//  5. the lowest m eigenvalues of the kept coordinates and their coefficients D V;
+//     position pairs (2t, 2t+1), and the rotated matrix is written to the other buffer at the
+//     positions the next round gives its indices.  So a thread reads and writes the same places in
+//     every round (a full sweep is the identity permutation): its addresses and signs are computed
+//     once, in registers, and a round is loads, rotations, stores and one barrier.  Warps have fixed
+//     roles: 2 x 2 blocks of the matrix (one per thread) and the planes of the next round (three lanes
+//     per plane, from the entries they need, recomputed with the same arithmetic as the block
+//     updates).  The planes of every round are logged to global memory (L2).
+//     A plane rotates when |a_uv| > eps sqrt(|a_uu a_vv|) + eps max_{i < m} |a_ii| (the absolute
+//     floor is the rounding level of the current Ritz block); after each sweep one pass over the
+//     pairs ends the iteration when none that concerns the m lowest would rotate.
+//  5. the lowest m eigenvalues of the kept coordinates, their eigenvectors Y from the logged
+//     rotations applied to m unit vectors, last round first, and the coefficients D L^-H Y;
 //  6. when asked, the conjugate-direction coefficients of the next iteration from the same
 //     CTA (pdir32: Cholesky-QR of the part of the old Ritz block outside the new one).
+// Bound: the chain of a Jacobi round (barrier, plane loads, rotated entry, new plane: 740 of 970
+// cycles at n = 57) for small n, issue and shared-memory bandwidth of one SM for n near 72.  50
+// problems of the design workloads: n = 45 400 -> 177 us, n = 57 583 -> 279 us, n = 69 885 -> 389-437 us
+// against positions that moved by index tables, V accumulated beside the rotations (its traffic was
+// 60 % of the rounds' shared-memory bytes) and CTA-wide barriers in every column of the reductions.
 // This is the mixed form's version (FP32, four 72 x 74 complex matrices in shared memory);
 // the FP64 form keeps the kernel in lobpcg.cu.
 #include "kernels.h"
@@ -37,8 +44,7 @@ constexpr int SR_THREADS = 1024;
 constexpr int SR_NMAX = 72;
 constexpr int SR_LD = 74;                       // even row stride: 16-byte aligned element pairs
 constexpr int SR_MAT = SR_NMAX * SR_LD;         // complex elements per matrix
-constexpr int SR_MAX_SWEEPS = 30;
-constexpr int SR_BLK = 36 * 37 / 2;             // upper 2 x 2 blocks of 36 planes
+constexpr int SR_MAX_SWEEPS = 16;               // 5 to 7 are taken
 constexpr int SR_PB = 8;                        // panel / row-block width of the reductions
 
 // Complex arithmetic with explicit roundings, so that every call site computes bitwise the
@@ -54,20 +60,22 @@ __device__ __forceinline__ float2 zaxpy(float c, float2 x, float2 z) {
 }
 __device__ __forceinline__ float2 zneg(float2 a) { return make_float2(-a.x, -a.y); }
 
+// Rotation of a plane: col_u <- c col_u - conj(s) col_v, col_v <- s col_u + c col_v; on: s != 0.
 struct __align__(16) Plane {
-  float2 s;  // rotation: col_u <- c col_u - conj(s) col_v, col_v <- s col_u + c col_v
+  float2 s;
   float c;
-  int on;    // rotates (s != 0)
+  int on;
 };
 
-// Column part of the two-sided rotation of a 2 x 2 block M (rows: plane 1, columns: plane 2):
-// y_a = (J2 applied to row a of M)[col].
-__device__ __forceinline__ float2 col_rot(float2 ma0, float2 ma1, const Plane& p2, int col) {
-  return col == 0 ? zaxpy(p2.c, ma0, zneg(zmul(zconj(p2.s), ma1))) : zaxpy(p2.c, ma1, zmul(p2.s, ma0));
-}
-// Row part: entry (row, col) of J1^H Y from the column-rotated pair (y0, y1) of that column.
-__device__ __forceinline__ float2 row_rot(float2 y0, float2 y1, const Plane& p1, int row) {
-  return row == 0 ? zaxpy(p1.c, y0, zneg(zmul(p1.s, y1))) : zaxpy(p1.c, y1, zmul(zconj(p1.s), y0));
+// Entry (r, col) of J1^H M J2 for a 2 x 2 block M (rows: plane 1, columns: plane 2) from the entries
+// named relative to it: ms[a] = M[a == 0 ? r : 1 - r][col], mo[a] the same rows' other column.
+// sg2 = -1 for col = 0, +1 for col = 1; sg1 the same of r.
+__device__ __forceinline__ float2 rotated(float2 ms0, float2 mo0, float2 ms1, float2 mo1, const Plane& p1, float sg1,
+                                          const Plane& p2, float sg2) {
+  const float2 s2 = make_float2(sg2 * p2.s.x, p2.s.y);    // -conj(s) or s
+  const float2 y0 = zaxpy(p2.c, ms0, zmul(s2, mo0)), y1 = zaxpy(p2.c, ms1, zmul(s2, mo1));
+  const float2 s1 = make_float2(sg1 * p1.s.x, -p1.s.y);   // -s or conj(s)
+  return zaxpy(p1.c, y0, zmul(s1, y1));
 }
 
 // Next position of the circle method in pair-ordered positions (top[t] = 2t, bottom[t] = 2t+1):
@@ -84,79 +92,173 @@ __device__ __forceinline__ int prev_pos(int pos, int np) {
   return pos == 2 ? 1 : pos - 2;
 }
 
-// Upper-stored element (i, j) of a position-ordered Hermitian matrix.
-__device__ __forceinline__ float2 uget(const float2* S, int i, int j) {
-  return i <= j ? S[i * SR_LD + j] : zconj(S[j * SR_LD + i]);
-}
+// Element (i, j) of the rotated matrix in its buffer: the even (top) columns of a row, then the odd
+// ones, so that neighbouring planes' entries are neighbours both where they are read and, shifted
+// by one plane, where they are written: no bank conflicts on either side.
+__device__ __forceinline__ int spos(int i, int j) { return i * SR_LD + (j & 1) * (SR_LD / 2) + (j >> 1); }
 
-// Entry (u, v) (positions, any order) of J^H A J for the planes pl of the current round.
-__device__ __forceinline__ float2 rotated_entry(const float2* S, const Plane* pl, int u, int v) {
-  int tu = u >> 1, tv = v >> 1, r = u & 1, c = v & 1;
-  bool tr = false;
-  if (tu > tv) { int t = tu; tu = tv; tv = t; t = r; r = c; c = t; tr = true; }
-  const Plane p1 = pl[tu], p2 = pl[tv];
-  if (tu == tv && p1.on && r != c) return make_float2(0.f, 0.f);  // annihilated by its own plane
-  const int a0 = 2 * tu, b0 = 2 * tv;
-  const float2 m00 = uget(S, a0, b0), m01 = uget(S, a0, b0 + 1), m10 = uget(S, a0 + 1, b0),
-               m11 = uget(S, a0 + 1, b0 + 1);
-  const float2 y0 = col_rot(m00, m01, p2, c), y1 = col_rot(m10, m11, p2, c);
-  float2 e = row_rot(y0, y1, p1, r);
-  if (tu == tv && r == c) e.y = 0.f;
-  return tr ? zconj(e) : e;
+__device__ __forceinline__ float sqrt_approx(float x) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Whether the plane of entries a_uu, a_vv (real) and a_uv rotates.  (A plane of the padding
+// coordinate, whose row and column are zero and stay zero, never does.)
+__device__ __forceinline__ bool plane_rotates(float app, float aqq, float b2, float floor_abs) {
+  return sqrt_approx(b2) > 1.1920929e-07f * sqrt_approx(fabsf(app * aqq)) + floor_abs;
 }
 
 // Rotation of the plane of positions (u, v) from a_uu, a_vv (real) and a_uv:
 // with d = a_vv - a_uu and b = |a_uv|, t = 2 b sgn(d) / (|d| + sqrt(d^2 + 4 b^2)) is the tangent
-// of the smaller rotation angle, c = 1 / sqrt(1 + t^2) and s = c t a_uv / b.
-__device__ __forceinline__ Plane make_plane(float app, float aqq, float2 apq, float floor_abs, bool valid) {
+// of the smaller rotation angle, c = 1 / sqrt(1 + t^2) and s = c t a_uv / b.  The chain of a round
+// runs through here, so it has no branch, and the root and reciprocal are the hardware
+// approximations: their error (a few units in the last place) turns the angle by as little, which
+// only leaves that share of a_uv, below its rounding.  c comes from the tangent that is used, as
+// 1 - t^2 r(t^2) with r(x) = 1 / (1 + x + sqrt(1 + x)) on [0, 1] (its Chebyshev interpolant of degree 9,
+// 5e-8 relative): an error of r counts by t^2 only, so c^2 + |s|^2 = 1 holds to rounding also for the
+// many small rotations of the last sweeps (with the approximate reciprocal root and a Newton step
+// the columns' norms drifted by 1e-5 over a solve).
+__device__ __forceinline__ Plane make_plane(float app, float aqq, float2 apq, float floor_abs) {
+  const float b2 = __fmaf_rn(apq.x, apq.x, apq.y * apq.y);
+  const bool on = plane_rotates(app, aqq, b2, floor_abs);
+  const float d = aqq - app;
+  const float inv = rcp_approx(fabsf(d) + sqrt_approx(__fmaf_rn(d, d, 4.f * b2)));
+  const float g = 2.f * inv;                     // |tangent| / b
+  const float x = g * g * b2, x2 = x * x, x4 = x2 * x2;
+  const float r01 = __fmaf_rn(-0.37499827f, x, 0.5f), r23 = __fmaf_rn(-0.2726586f, x, 0.31244183f);
+  const float r45 = __fmaf_rn(-0.20286512f, x, 0.24065118f), r67 = __fmaf_rn(-0.08192697f, x, 0.14801665f);
+  const float r89 = __fmaf_rn(-0.00477741f, x, 0.02900993f);
+  const float r0 = __fmaf_rn(r23, x2, r01), r4 = __fmaf_rn(r67, x2, r45);
+  const float c = 1.f - x * __fmaf_rn(__fmaf_rn(r89, x4, r4), x4, r0);
+  const float f = (d >= 0.f ? g : -g) * c;       // c t / b
   Plane w;
-  w.c = 1.f;
-  w.s = make_float2(0.f, 0.f);
-  w.on = 0;
-  const float eps = 1.1920929e-07f;
-  const float b2 = apq.x * apq.x + apq.y * apq.y;
-  const float b = __fsqrt_rn(b2);
-  if (valid && b > eps * __fsqrt_rn(fabsf(app) * fabsf(aqq)) + floor_abs) {
-    const float d = aqq - app;
-    const float sg = d >= 0.f ? 1.f : -1.f;
-    const float inv = __frcp_rn(fabsf(d) + __fsqrt_rn(d * d + 4.f * b2));
-    const float t = 2.f * b * inv;                  // |tangent|
-    const float c = __frsqrt_rn(1.f + t * t);
-    const float f = 2.f * sg * inv * c;             // c t / b
-    w.c = c;
-    w.s = make_float2(f * apq.x, f * apq.y);
-    w.on = 1;
-  }
+  w.c = on ? c : 1.f;
+  w.s = make_float2(on ? f * apq.x : 0.f, on ? f * apq.y : 0.f);
+  w.on = on ? 1 : 0;
   return w;
 }
 
-// Forward substitution L X = R in place for ncol columns (column c of R is column c of P[0] for
-// c < n0, else column c - n0 of P[1]); L lower with row stride SR_LD, drops already turned into
-// e_j.  8-row blocks: the update of the block's rows from the rows solved before it (all
-// threads, one output each), then the 8 x 8 diagonal solve (one thread per column).
-__device__ __forceinline__ void block_forward(const float2* L, float2* const P[2], int n0, int n, int ncol) {
+// Barrier over the first `threads` threads of the CTA (a multiple of 32), and the same with an OR.
+__device__ __forceinline__ void bar_first(int threads) {
+  asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+__device__ __forceinline__ bool bar_first_or(int threads, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred q, w;\n\tsetp.ne.s32 q, %2, 0;\n\tbar.red.or.pred w, 1, %1, q;\n\tselp.s32 %0, 1, 0, w;\n\t}"
+      : "=r"(r)
+      : "r"(threads), "r"((int)p)
+      : "memory");
+  return r != 0;
+}
+
+// Cholesky of the Hermitian B (lower, row stride SR_LD) with dropped pivots; invd: the reciprocal
+// diagonal.  On return dropped rows and columns are e_j.
+__device__ __forceinline__ void block_cholesky(float2* B, int n, float drop_tol, int* drop, float* invd) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int j0 = 0; j0 < n; j0 += SR_PB) {
+    const int jb = min(SR_PB, n - j0), j1 = j0 + jb;
+    float2 a[SR_PB];
+    if (warp == 0 || j1 + 32 * warp < n) {
+      // every warp with panel rows factors the diagonal block (row lane % 8) for itself
+      const int r = lane & 7;
+      float inv[SR_PB];
+#pragma unroll
+      for (int c = 0; c < SR_PB; ++c) a[c] = (r < jb && c < jb) ? B[(j0 + r) * SR_LD + j0 + c] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < SR_PB; ++j) {
+        const float d = __shfl_sync(0xffffffffu, a[j].x, j);
+        const bool keep = d > drop_tol;
+        const float sq = sqrtf(d);
+        inv[j] = keep ? 1.f / sq : 0.f;
+        if (r == j) a[j] = make_float2(keep ? sq : 1.f, 0.f);
+        else a[j] = make_float2(a[j].x * inv[j], a[j].y * inv[j]);
+#pragma unroll
+        for (int c = j + 1; c < SR_PB; ++c) {
+          const float2 lc = make_float2(__shfl_sync(0xffffffffu, a[j].x, c), __shfl_sync(0xffffffffu, a[j].y, c));
+          if (r >= c) {  // a_rc -= l_rj conj(l_cj)
+            a[c].x -= a[j].x * lc.x + a[j].y * lc.y;
+            a[c].y -= a[j].y * lc.x - a[j].x * lc.y;
+          }
+        }
+      }
+      const int i = j1 + 32 * warp + lane;
+      float2 b[SR_PB];
+#pragma unroll
+      for (int c = 0; c < SR_PB; ++c) b[c] = i < n && c < jb ? B[i * SR_LD + j0 + c] : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int j = 0; j < SR_PB; ++j) {
+#pragma unroll
+        for (int k = 0; k < j; ++k) {
+          const float2 l = make_float2(__shfl_sync(0xffffffffu, a[k].x, j), __shfl_sync(0xffffffffu, a[k].y, j));
+          b[j].x -= b[k].x * l.x + b[k].y * l.y;
+          b[j].y -= b[k].y * l.x - b[k].x * l.y;
+        }
+        b[j].x *= inv[j];
+        b[j].y *= inv[j];
+      }
+      if (i < n)
+#pragma unroll
+        for (int c = 0; c < SR_PB; ++c)
+          if (c < jb) B[i * SR_LD + j0 + c] = b[c];
+      if (warp == 0)
+#pragma unroll
+        for (int c = 0; c < SR_PB; ++c)
+          if (lane == c && c < jb) {
+            drop[j0 + c] = inv[c] == 0.f ? 1 : 0;
+            invd[j0 + c] = inv[c] == 0.f ? 1.f : inv[c];
+          }
+    }
+    __syncthreads();
+    if (warp == 0 && lane < jb)  // every warp has read the diagonal block
+#pragma unroll
+      for (int c = 0; c < SR_PB; ++c)
+        if (c <= lane) B[(j0 + lane) * SR_LD + j0 + c] = a[c];
+    // trailing update of the rows and columns from j1 on by the panel (dropped columns are zero)
+    const int nt = n - j1;
+    for (int rr = warp; rr < nt; rr += 32) {
+      const int i = j1 + rr;
+      const float4* Li = reinterpret_cast<const float4*>(B + i * SR_LD + j0);
+      for (int q = lane; q <= rr; q += 32) {
+        const int c = j1 + q;
+        const float4* Lc = reinterpret_cast<const float4*>(B + c * SR_LD + j0);
+        float2 v = B[i * SR_LD + c];
+#pragma unroll
+        for (int h = 0; h < SR_PB / 2; ++h) {  // jb = SR_PB wherever rows remain below the panel
+          const float4 x = Li[h], y = Lc[h];
+          v.x -= x.x * y.x + x.y * y.y;
+          v.y -= x.y * y.x - x.x * y.y;
+          v.x -= x.z * y.z + x.w * y.w;
+          v.y -= x.w * y.z - x.z * y.w;
+        }
+        B[i * SR_LD + c] = v;
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = warp; i < n; i += 32)
+    for (int c = lane; c <= i; c += 32)
+      if (drop[i] || drop[c]) B[i * SR_LD + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
+  __syncthreads();
+}
+
+// Forward substitution L X = R in place, right-looking in blocks of 8 rows.  Columns c < n0 of R are
+// columns of P0, the others columns c - n0 of P1.  tri = 1: P1 starts as the identity, whose
+// column j is zero above row j; tri = 2 (n0 = ncol): only rows i <= c of column c are wanted.
+__device__ __forceinline__ void block_forward(const float2* L, const float* invd, float2* P0, float2* P1, int n0, int n,
+                                              int ncol, int tri) {
   const int tid = threadIdx.x;
   for (int i0 = 0; i0 < n; i0 += SR_PB) {
-    const int ib = min(SR_PB, n - i0);
-    if (i0 > 0) {
-      for (int e = tid; e < ib * ncol; e += SR_THREADS) {
-        const int ii = e / ncol, c = e - ii * ncol;
-        float2* R = c < n0 ? P[0] + c : P[1] + (c - n0);
-        const float2* Li = L + (i0 + ii) * SR_LD;
-        float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-        int k = 0;
-        for (; k + 1 < i0; k += 2) {
-          cfma(a0, Li[k], R[k * SR_LD]);
-          cfma(a1, Li[k + 1], R[(k + 1) * SR_LD]);
-        }
-        if (k < i0) cfma(a0, Li[k], R[k * SR_LD]);
-        const float2 r = R[(i0 + ii) * SR_LD];
-        R[(i0 + ii) * SR_LD] = make_float2(r.x - a0.x - a1.x, r.y - a0.y - a1.y);
-      }
-      __syncthreads();
-    }
-    for (int c = tid; c < ncol; c += SR_THREADS) {
-      float2* R = c < n0 ? P[0] + c : P[1] + (c - n0);
+    const int ib = min(SR_PB, n - i0), i1 = i0 + ib;
+    const int c_lo = tri == 2 ? i0 : 0;
+    const int c_hi = tri == 1 ? n0 + min(n, i1) : ncol;
+    for (int c = c_lo + tid; c < c_hi; c += SR_THREADS) {
+      float2* R = c < n0 ? P0 + c : P1 + (c - n0);
       float2 x[SR_PB];
 #pragma unroll
       for (int ii = 0; ii < SR_PB; ++ii) {
@@ -169,14 +271,136 @@ __device__ __forceinline__ void block_forward(const float2* L, float2* const P[2
             acc.x -= l.x * x[kk].x - l.y * x[kk].y;
             acc.y -= l.x * x[kk].y + l.y * x[kk].x;
           }
-          const float il = 1.f / L[i * SR_LD + i].x;
-          x[ii] = make_float2(acc.x * il, acc.y * il);
+          x[ii] = make_float2(acc.x * invd[i], acc.y * invd[i]);
           R[i * SR_LD] = x[ii];
         }
       }
     }
     __syncthreads();
+    if (i1 >= n) break;
+    // rows below: four rows of one column per thread (i1 is a multiple of 8 here)
+    const int nc = c_hi - c_lo, ng = (n - i1 + 3) / 4;
+    for (int e = tid; e < nc * ng; e += SR_THREADS) {
+      const int g = e / nc, c = c_lo + e - g * nc;
+      const int r0 = i1 + 4 * g;
+      if (tri == 2 && c < r0) continue;
+      float2* R = c < n0 ? P0 + c : P1 + (c - n0);
+      float2 acc[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < SR_PB; ++k) {
+        const float2 x = R[(i0 + k) * SR_LD];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cfma(acc[q], L[(r0 + q) * SR_LD + i0 + k], x);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (r0 + q < n) R[(r0 + q) * SR_LD] = csub(R[(r0 + q) * SR_LD], acc[q]);
+    }
+    __syncthreads();
   }
+}
+
+__device__ __forceinline__ float4 as_float4(const Plane& w) {
+  return make_float4(w.s.x, w.s.y, w.c, __int_as_float(w.on));
+}
+
+// Eigenvectors of the packed matrix from the logged rotations (np planes per round, K rounds):
+// column j of Y (nk_ x m) = J_1 P_1 J_2 P_2 ... J_K P_K e, e the unit vector of position perm[j],
+// P the circle method's moves.  Applied to the m wanted columns only, from the last round back, which
+// is a third of the work of accumulating all of V beside the rotations and leaves the shared-memory
+// bandwidth of the rounds to the matrix (it was their bound: 147 KB a round at n = 69, of which
+// V took 87).  Half a warp holds a column, PPL planes (2 PPL positions) per lane in registers; a move
+// is one complex value from each neighbouring lane.  The other warps bring the log from L2 in chunks
+// of SR_CHUNK rounds, one ahead.
+constexpr int SR_CHUNK = 64;  // rounds x 36 planes x 16 bytes = 36 KB per buffer
+template <int PPL>
+__device__ __forceinline__ void replay(const float4* __restrict__ logk, int K, int np, int nk_, int m, const int* perm,
+                                       float4* buf0, float4* buf1, float2* Y) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int cw = (m + 1) / 2;  // warps that hold columns
+  const int hl = lane & 15, j = 2 * warp + (lane >> 4);
+  const bool col = warp < cw;
+  float2 top[PPL], bot[PPL];
+  int tp[PPL];       // plane read (those past the last hold nothing: their values reach no column)
+  bool last[PPL];
+  const bool first = hl == 0;
+#pragma unroll
+  for (int b = 0; b < PPL; ++b) {
+    tp[b] = min(hl * PPL + b, np - 1);
+    last[b] = hl * PPL + b == np - 1;
+  }
+  if (col) {
+    const int p = j < m ? perm[j] : -1;
+#pragma unroll
+    for (int b = 0; b < PPL; ++b) {
+      const int t = hl * PPL + b;
+      top[b] = make_float2(2 * t == p ? 1.f : 0.f, 0.f);
+      bot[b] = make_float2(2 * t + 1 == p ? 1.f : 0.f, 0.f);
+    }
+  }
+  const int nchunk = (K + SR_CHUNK - 1) / SR_CHUNK;
+  auto bring = [&](int c, int first, int step) {  // rounds c SR_CHUNK .. of the log
+    float4* dst = (c & 1) ? buf1 : buf0;
+    const int cnt = min(SR_CHUNK, K - c * SR_CHUNK) * np;
+    const float4* src = logk + (long long)c * SR_CHUNK * np;
+    for (int e = first; e < cnt; e += step) dst[e] = __ldcg(src + e);
+  };
+  __syncthreads();  // the buffers are free
+  bring(nchunk - 1, tid, SR_THREADS);
+  __syncthreads();
+  for (int c = nchunk - 1; c >= 0; --c) {
+    if (!col) {
+      if (c > 0) bring(c - 1, tid - 32 * cw, SR_THREADS - 32 * cw);
+    } else {
+      const float4* pl = ((c & 1) ? buf1 : buf0);
+      const int cnt = min(SR_CHUNK, K - c * SR_CHUNK);
+      float4 w[PPL];
+#pragma unroll
+      for (int b = 0; b < PPL; ++b) w[b] = pl[(cnt - 1) * np + tp[b]];
+#pragma unroll 2
+      for (int r = cnt - 1; r >= 0; --r) {
+        // value that position p of this round has: the one at its next position
+        const float2 below = make_float2(__shfl_down_sync(0xffffffffu, top[0].x, 1, 16),
+                                         __shfl_down_sync(0xffffffffu, top[0].y, 1, 16));
+        const float2 above = make_float2(__shfl_up_sync(0xffffffffu, bot[PPL - 1].x, 1, 16),
+                                         __shfl_up_sync(0xffffffffu, bot[PPL - 1].y, 1, 16));
+        float4 nw[PPL];  // the planes of the round before it, in flight meanwhile
+        const float4* pn = pl + max(r - 1, 0) * np;
+#pragma unroll
+        for (int b = 0; b < PPL; ++b) nw[b] = pn[tp[b]];
+        float2 u[PPL], v[PPL];
+#pragma unroll
+        for (int b = 0; b < PPL; ++b) {
+          u[b] = b + 1 < PPL ? top[b + 1 < PPL ? b + 1 : 0] : below;
+          v[b] = b > 0 ? bot[b > 0 ? b - 1 : 0] : above;
+          if (last[b]) u[b] = bot[b];
+        }
+        if (first) {
+          v[0] = np == 1 ? bot[0] : u[0];
+          u[0] = top[0];
+        }
+#pragma unroll
+        for (int b = 0; b < PPL; ++b) {
+          const float2 s = make_float2(w[b].x, w[b].y);
+          top[b] = zaxpy(w[b].z, u[b], zmul(s, v[b]));                           // c u + s v
+          bot[b] = zaxpy(w[b].z, v[b], zmul(make_float2(-s.x, s.y), u[b]));      // c v - conj(s) u
+          w[b] = nw[b];
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (col && j < m) {
+#pragma unroll
+    for (int b = 0; b < PPL; ++b) {
+      const int p = 2 * (hl * PPL + b);
+      if (p < nk_) Y[p * m + j] = top[b];
+      if (p + 1 < nk_) Y[(p + 1) * m + j] = bot[b];
+    }
+  }
+  __syncthreads();
 }
 
 // Conjugate-direction coefficients, inside the CTA that solved the projected problem.  With the
@@ -186,70 +410,120 @@ __device__ __forceinline__ void block_forward(const float2* L, float2* const P[2
 // unit-diagonal scaled, Cholesky-QR; columns with H_jj at or below abs_drop carry only rounding
 // and are dropped), cP = Z T.  go: the projected Gram matrix (global); G (stride SR_LD), cx, z, gz
 // (n x m compact), Mm (m x m), tmp (m), Dd (m), drp (m): shared workspaces; cp: output (n x m).
+// go: the projected Gram matrix (global); G (stride SR_LD), cx, z, gz (n x m compact), Mm, Mi (m x m,
+// stride m | 1), Dd (m), drp (m): shared workspaces; cp: output (n x m).  The products give each
+// thread four rows of one column (the row operands are shared by the warp's lanes).
 __device__ void pdir32(const float2* __restrict__ go, int n, int m, float abs_drop, float2* G, const float2* cx,
-                       float2* z, float2* gz, float2* Mm, float2* tmp, float* Dd, int* drp, float2* __restrict__ cp) {
-  const int tid = threadIdx.x;
-  for (int t = tid; t < n * n; t += SR_THREADS) {  // GO, symmetrised
-    const int r = t / n, q = t - (t / n) * n;
-    const float2 g1 = go[r * n + q], g2 = go[q * n + r];
-    G[r * SR_LD + q] = make_float2(0.5f * (g1.x + g2.x), 0.5f * (g1.y - g2.y));
-  }
-  __syncthreads();
-  for (int t = tid; t < m * m; t += SR_THREADS) {  // M = cX^H GO E
-    const int i = t / m, j = t - (t / m) * m;
-    float2 s = make_float2(0.f, 0.f);
-    for (int r = 0; r < n; ++r) cfmac(s, cx[r * m + i], G[r * SR_LD + j]);
-    Mm[t] = s;
-  }
-  __syncthreads();
-  for (int t = tid; t < n * m; t += SR_THREADS) {  // Z = E - cX M
-    const int r = t / m, j = t - (t / m) * m;
-    float2 s = make_float2(r == j ? 1.f : 0.f, 0.f);
-    for (int i = 0; i < m; ++i) {
-      const float2 v = cmul(cx[r * m + i], Mm[i * m + j]);
-      s.x -= v.x;
-      s.y -= v.y;
+                       float2* z, float2* gz, float2* Mm, float2* Mi, float* Dd, int* drp, float2* __restrict__ cp) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ldm = m | 1;
+  for (int r = warp; r < n; r += 32)  // GO, symmetrised
+    for (int q = lane; q < n; q += 32) {
+      const float2 g1 = go[r * n + q], g2 = go[q * n + r];
+      G[r * SR_LD + q] = make_float2(0.5f * (g1.x + g2.x), 0.5f * (g1.y - g2.y));
     }
-    z[t] = s;
-  }
   __syncthreads();
-  for (int t = tid; t < n * m; t += SR_THREADS) {  // GZ = GO Z
-    const int r = t / m, j = t - (t / m) * m;
-    float2 s = make_float2(0.f, 0.f);
-    for (int q = 0; q < n; ++q) cfma(s, G[r * SR_LD + q], z[q * m + j]);
-    gz[t] = s;
-  }
-  __syncthreads();
-  for (int i = tid; i < m; i += SR_THREADS) {  // column scales of H = Z^H GZ
-    float2 s = make_float2(0.f, 0.f);
-    for (int r = 0; r < n; ++r) cfmac(s, z[r * m + i], gz[r * m + i]);
-    Dd[i] = (s.x > abs_drop && s.x == s.x) ? 1.f / sqrtf(s.x) : 0.f;
-    drp[i] = 0;
-  }
-  __syncthreads();
-  for (int t = tid; t < m * m; t += SR_THREADS) {  // H, unit-diagonal scaled and symmetrised
-    const int i = t / m, j = t - (t / m) * m;
-    float2 s1 = make_float2(0.f, 0.f), s2 = make_float2(0.f, 0.f);
+  const int mg = (m + 1) / 2, n4 = (n + 3) / 4;
+  for (int t = tid; t < mg * m; t += SR_THREADS) {  // M = cX^H GO E, two rows per thread
+    const int g = t / m, j = t - g * m, i0 = 2 * g, i1 = min(2 * g + 1, m - 1);
+    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll 4
     for (int r = 0; r < n; ++r) {
-      cfmac(s1, z[r * m + i], gz[r * m + j]);
-      cfmac(s2, z[r * m + j], gz[r * m + i]);
+      const float2 v = G[r * SR_LD + j];
+      cfmac(s0, cx[r * m + i0], v);
+      cfmac(s1, cx[r * m + i1], v);
     }
-    const float sc = Dd[i] * Dd[j] * 0.5f;
-    Mm[t] = make_float2((s1.x + s2.x) * sc, (s1.y - s2.y) * sc);
+    Mm[i0 * ldm + j] = s0;
+    if (2 * g + 1 < m) Mm[i1 * ldm + j] = s1;
   }
   __syncthreads();
-  chol_drop<float>(Mm, m, m, 1e-10f, drp);
-  tri_inv_lower<float>(Mm, m, m, tmp);
-  for (int t = tid; t < n * m; t += SR_THREADS) {  // cP = Z T, T[i][c] = D_i conj(Li[c][i]) for c >= i
-    const int r = t / m, c = t - (t / m) * m;
-    float2 s = make_float2(0.f, 0.f);
+  for (int t = tid; t < n4 * m; t += SR_THREADS) {  // Z = E - cX M
+    const int g = t / m, j = t - g * m;
+    float2 s[4];
+    int rr[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      rr[q] = min(4 * g + q, n - 1);
+      s[q] = make_float2(4 * g + q == j ? 1.f : 0.f, 0.f);
+    }
+    for (int i = 0; i < m; ++i) {
+      const float2 v = Mm[i * ldm + j];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cfma(s[q], zneg(cx[rr[q] * m + i]), v);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (4 * g + q < n) z[(4 * g + q) * m + j] = s[q];
+  }
+  __syncthreads();
+  for (int t = tid; t < n4 * m; t += SR_THREADS) {  // GZ = GO Z
+    const int g = t / m, j = t - g * m;
+    float2 s[4];
+    int rr[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      rr[q] = min(4 * g + q, n - 1) * SR_LD;
+      s[q] = make_float2(0.f, 0.f);
+    }
+#pragma unroll 2
+    for (int k = 0; k < n; ++k) {
+      const float2 v = z[k * m + j];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cfma(s[q], G[rr[q] + k], v);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (4 * g + q < n) gz[(4 * g + q) * m + j] = s[q];
+  }
+  __syncthreads();
+  for (int t = tid; t < mg * m; t += SR_THREADS) {  // H = Z^H GZ, two rows per thread
+    const int g = t / m, j = t - g * m, i0 = 2 * g, i1 = min(2 * g + 1, m - 1);
+    float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll 4
+    for (int r = 0; r < n; ++r) {
+      const float2 v = gz[r * m + j];
+      cfmac(s0, z[r * m + i0], v);
+      cfmac(s1, z[r * m + i1], v);
+    }
+    Mi[i0 * ldm + j] = s0;
+    if (2 * g + 1 < m) Mi[i1 * ldm + j] = s1;
+  }
+  __syncthreads();
+  if (tid < m) {  // column scales
+    const float d = Mi[tid * ldm + tid].x;
+    Dd[tid] = (d > abs_drop && d == d) ? 1.f / sqrtf(d) : 0.f;
+    drp[tid] = 0;
+  }
+  __syncthreads();
+  for (int t = tid; t < m * m; t += SR_THREADS) {  // unit-diagonal scaled and symmetrised
+    const int i = t / m, j = t - i * m;
+    const float2 s1 = Mi[i * ldm + j], s2 = Mi[j * ldm + i];
+    const float sc = Dd[i] * Dd[j] * 0.5f;
+    Mm[i * ldm + j] = make_float2((s1.x + s2.x) * sc, (s1.y - s2.y) * sc);
+  }
+  __syncthreads();
+  if (warp == 0) warp_chol_inverse<float>(Mm, Mi, m, ldm, 1e-10f, drp);
+  __syncthreads();
+  for (int t = tid; t < n4 * m; t += SR_THREADS) {  // cP = Z T, T[i][c] = D_i conj(Li[c][i]) for c >= i
+    const int g = t / m, c = t - g * m;
+    float2 s[4];
+    int rr[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      rr[q] = min(4 * g + q, n - 1) * m;
+      s[q] = make_float2(0.f, 0.f);
+    }
     if (!drp[c] && Dd[c] != 0.f) {
       for (int i = 0; i <= c; ++i) {
-        const float2 li = Mm[c * m + i];
-        cfma(s, z[r * m + i], make_float2(li.x * Dd[i], -li.y * Dd[i]));
+        const float2 li = Mi[c * ldm + i];
+        const float2 v = make_float2(li.x * Dd[i], -li.y * Dd[i]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cfma(s[q], z[rr[q] + i], v);
       }
     }
-    cp[t] = s;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (4 * g + q < n) cp[(4 * g + q) * m + c] = s[q];
   }
 }
 
@@ -259,27 +533,26 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
                                                          int n, int m, float drop_tol, const int* __restrict__ kdone,
                                                          float* __restrict__ lam_out, float2* __restrict__ coef,
                                                          float2* __restrict__ cpo, float pdir_abs, int* status,
-                                                         double* flops) {
+                                                         double* flops, float4* __restrict__ rotlog, long long log_stride) {
   extern __shared__ __align__(16) unsigned char smem[];
   float2* B0 = (float2*)smem;          // GO -> L -> Jacobi buffer 1
   float2* B1 = B0 + SR_MAT;            // GA -> T = L^-1 GA -> Jacobi buffer 0
-  float2* Vt = B1 + SR_MAT;            // V^T = conj(L^-1), then rotated (rows: coordinates)
-  float2* Cm = Vt + SR_MAT;            // C = L^-1 GA L^-H (original order)
+  float2* Vt = B1 + SR_MAT;            // L^-1
+  float2* Cm = Vt + SR_MAT;            // C = L^-1 GA L^-H (original order) -> Y
   Plane* pl = (Plane*)(Cm + SR_MAT);   // 2 x 36 planes (by round parity)
   float* D = (float*)(pl + 2 * 36);    // SR_NMAX
-  float* ev = D + SR_NMAX;             // SR_NMAX
+  float* ev = D + SR_NMAX;             // SR_NMAX: reciprocal diagonal of L, then eigenvalues
   int* drop = (int*)(ev + SR_NMAX);    // SR_NMAX
-  int* idx = drop + SR_NMAX;           // 2 x SR_NMAX: position -> coordinate (-1: padding)
-  int* perm = idx + 2 * SR_NMAX;       // SR_NMAX
-  int* npos = perm + SR_NMAX;          // SR_NMAX: position in the next round
-  int* ppos = npos + SR_NMAX;          // SR_NMAX: position in the previous round
-  int* blk = ppos + SR_NMAX;           // SR_BLK: upper blocks t1 | t2 << 8, row-major
-  int* misc = blk + SR_BLK;            // [0] kept count, [2] floor bits
+  int* idx = drop + SR_NMAX;           // SR_NMAX: position -> coordinate (-1: padding)
+  int* perm = idx + SR_NMAX;           // SR_NMAX
+  int* low = perm + SR_NMAX;           // SR_NMAX: among the m smallest diagonal entries
+  int* misc = low + SR_NMAX;           // [0] kept count, [2] floor bits, [3] sweeps
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
   const int k = blockIdx.x;
   const float2* ga = GA + (long long)k * n * n;
   const float2* go = GO + (long long)k * n * n;
+  float4* logk = rotlog + k * log_stride;  // rotations of this problem, np planes per round
   float2* ck = coef + (long long)k * n * m;
   float2* cpk = cpo ? cpo + (long long)k * n * m : nullptr;  // conjugate-direction coefficients (or none)
   if (kdone && kdone[k]) {  // locked k-point: keep its block, leave lambda untouched, no conjugate block
@@ -297,89 +570,24 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
     drop[i] = 0;
   }
   __syncthreads();
-  for (int t = tid; t < n * n; t += blockDim.x) {
-    const int i = t / n, c = t % n;
-    const float2 a1 = ga[i * n + c], a2 = ga[c * n + i];
-    const float2 b1 = go[i * n + c], b2 = go[c * n + i];
-    const float s = D[i] * D[c] * 0.5f;
-    B1[i * SR_LD + c] = make_float2((a1.x + a2.x) * s, (a1.y - a2.y) * s);
-    B0[i * SR_LD + c] = make_float2((b1.x + b2.x) * s, (b1.y - b2.y) * s);
-    Vt[i * SR_LD + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
-  }
-  for (int t = tid; t < n * (SR_NMAX - n); t += blockDim.x)  // padding columns n .. 71
-    Vt[(t / (SR_NMAX - n)) * SR_LD + n + t % (SR_NMAX - n)] = make_float2(0.f, 0.f);
-  __syncthreads();
-  // 2. blocked Cholesky of B0 (lower)
-  for (int j0 = 0; j0 < n; j0 += SR_PB) {
-    const int j1 = min(j0 + SR_PB, n);
-    if (warp == 0) {
-      for (int j = j0; j < j1; ++j) {
-        const float d = B0[j * SR_LD + j].x;
-        if (!(d > drop_tol)) {  // dropped: no update; its row and column are reset below
-          if (lane == 0) drop[j] = 1;
-          __syncwarp();
-          continue;
-        }
-        const float sq = sqrtf(d), inv = 1.f / sq;
-        for (int i = j + 1 + lane; i < n; i += 32) {
-          const float2 v = B0[i * SR_LD + j];
-          B0[i * SR_LD + j] = make_float2(v.x * inv, v.y * inv);
-        }
-        if (lane == 0) B0[j * SR_LD + j] = make_float2(sq, 0.f);
-        __syncwarp();
-        for (int c = j + 1; c < j1; ++c) {
-          const float2 lc = B0[c * SR_LD + j];
-          for (int i = c + lane; i < n; i += 32) {
-            const float2 li = B0[i * SR_LD + j];
-            float2 v = B0[i * SR_LD + c];
-            v.x -= li.x * lc.x + li.y * lc.y;  // v -= li conj(lc)
-            v.y -= li.y * lc.x - li.x * lc.y;
-            B0[i * SR_LD + c] = v;
-          }
-        }
-        __syncwarp();
-      }
+  for (int i = warp; i < n; i += 32)
+    for (int c = lane; c < n; c += 32) {
+      const float2 a1 = ga[i * n + c], a2 = ga[c * n + i];
+      const float2 b1 = go[i * n + c], b2 = go[c * n + i];
+      const float s = D[i] * D[c] * 0.5f;
+      B1[i * SR_LD + c] = make_float2((a1.x + a2.x) * s, (a1.y - a2.y) * s);
+      B0[i * SR_LD + c] = make_float2((b1.x + b2.x) * s, (b1.y - b2.y) * s);
+      Vt[i * SR_LD + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
     }
-    __syncthreads();
-    // trailing update of rows and columns >= j1 by the panel's kept columns
-    const int nt = n - j1;
-    for (int r = warp; r < nt; r += 32) {
-      const int i = j1 + r;
-      for (int q = lane; q <= r; q += 32) {
-        const int c = j1 + q;
-        float2 v = B0[i * SR_LD + c];
-        for (int jj = j0; jj < j1; ++jj) {
-          if (drop[jj]) continue;
-          const float2 li = B0[i * SR_LD + jj], lc = B0[c * SR_LD + jj];
-          v.x -= li.x * lc.x + li.y * lc.y;
-          v.y -= li.y * lc.x - li.x * lc.y;
-        }
-        B0[i * SR_LD + c] = v;
-      }
-    }
-    __syncthreads();
-  }
-  // dropped coordinates: row and column of L become e_j
-  for (int t = tid; t < n * n; t += blockDim.x) {
-    const int i = t / n, c = t % n;
-    if (c <= i && (drop[i] || drop[c])) B0[i * SR_LD + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
-  }
   __syncthreads();
-  // 3. T = L^-1 GA (in place in B1) and L^-1 (in place in Vt), then C = L^-1 T^H in Cm
-  {
-    float2* const P[2] = {B1, Vt};
-    block_forward(B0, P, n, n, 2 * n);
-  }
-  for (int t = tid; t < n * n; t += blockDim.x) {
-    const int i = t / n, j = t % n;
-    Cm[i * SR_LD + j] = zconj(B1[j * SR_LD + i]);
-    Vt[i * SR_LD + j] = zconj(Vt[i * SR_LD + j]);  // V^T = conj(L^-1)
-  }
+  // 2. Cholesky of B0 (lower)
+  block_cholesky(B0, n, drop_tol, drop, ev);
+  // 3. T = L^-1 GA (in place in B1) and L^-1 (in place in Vt), then C = L^-1 T^H in Cm (upper)
+  block_forward(B0, ev, B1, Vt, n, n, 2 * n, 1);
+  for (int i = warp; i < n; i += 32)
+    for (int j = lane; j < n; j += 32) Cm[i * SR_LD + j] = zconj(B1[j * SR_LD + i]);
   __syncthreads();
-  {
-    float2* const P[2] = {Cm, Cm};
-    block_forward(B0, P, n, n, n);
-  }
+  block_forward(B0, ev, Cm, nullptr, n, n, n, 2);
   if (tid == 0) {
     int kept = 0;
     for (int i = 0; i < n; ++i)
@@ -403,36 +611,26 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
         B1[t] = make_float2(i == j ? 1.f : 0.f, 0.f);
       }
       __syncthreads();
-      pdir32(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * m, ev, drop, cpk);
+      pdir32(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * (m | 1), ev, drop, cpk);
     }
     return;
   }
   const int npad = nk_ + (nk_ & 1), np = npad / 2, nrounds = npad - 1;
   const int nblk = np * (np + 1) / 2;
-  // 4. packed position-ordered upper copy in B1 (T is no longer needed) and the round tables
-  for (int t = tid; t < npad * npad; t += blockDim.x) {
-    const int i = t / npad, j = t % npad;
-    if (i <= j) {
+  // 4. packed position-ordered upper copy in B1 (T is no longer needed)
+  for (int i = warp; i < npad; i += 32)
+    for (int j = i + lane; j < npad; j += 32) {
       const int a = idx[i], b = idx[j];
       float2 v = (a < 0 || b < 0) ? make_float2(0.f, 0.f) : Cm[a * SR_LD + b];
       if (i == j) v.y = 0.f;
-      B1[i * SR_LD + j] = v;
+      B1[spos(i, j)] = v;
     }
-  }
-  for (int p = tid; p < npad; p += blockDim.x) {
-    npos[p] = next_pos(p, np);
-    ppos[p] = prev_pos(p, np);
-  }
-  for (int t1 = tid; t1 < np; t1 += blockDim.x) {
-    const int base = t1 * np - t1 * (t1 - 1) / 2;  // first block of row t1
-    for (int t2 = t1; t2 < np; ++t2) blk[base + t2 - t1] = t1 | (t2 << 8);
-  }
   __syncthreads();
   // rounding floor: eps * max |a_ii| over the kept coordinates of the current Ritz block
   if (warp == 0) {
     float mx = 0.f;
     for (int p = lane; p < nk_; p += 32)
-      if (idx[p] < m) mx = fmaxf(mx, fabsf(B1[p * SR_LD + p].x));
+      if (idx[p] < m) mx = fmaxf(mx, fabsf(B1[spos(p, p)].x));
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0) misc[2] = __float_as_int(1.1920929e-07f * mx);
   }
@@ -440,158 +638,194 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
   const float floor_abs = __int_as_float(misc[2]);
   if (tid < np) {  // planes of the first round
     const int u = 2 * tid, v = u + 1;
-    const bool valid = idx[u] >= 0 && idx[v] >= 0;
-    pl[tid] = make_plane(B1[u * SR_LD + u].x, B1[v * SR_LD + v].x, B1[u * SR_LD + v], floor_abs, valid);
+    const Plane w = make_plane(B1[spos(u, u)].x, B1[spos(v, v)].x, B1[spos(u, v)], floor_abs);
+    pl[tid] = w;
+    logk[tid] = as_float4(w);
   }
   __syncthreads();
-  // Jacobi sweeps.  Every round, the last pw warps compute the planes of the next round, three
-  // lanes per plane (a_uu, a_vv, a_uv of the rotated matrix, combined by shuffles), ten planes per
-  // warp; the other threads take the remaining work list: the upper 2 x 2 blocks of the matrix and
-  // (plane, six-column group) updates of V^T, units tid, tid + nthr_o, ...  V^T units:
-  // v = plane * nq + group, decoded with a multiply-shift (exact for v < 2^11 and nq <= 12: the
-  // rounding error of 2^20 / nq times v stays below 1 / nq).
-  const int nq = (n + 5) / 6;
-  const int pw = (np + 9) / 10;
-  const int nthr_o = SR_THREADS - 32 * pw;
-  const int nunits = nblk + np * nq;
-  const unsigned vinv = (1u << 20) / (unsigned)nq + 1u;
-  const bool plane_warp = warp >= SR_THREADS / 32 - pw;
-  const int pt = (warp - (SR_THREADS / 32 - pw)) * 10 + lane / 3;  // plane of this lane
-  const int pe = lane % 3;                                          // 0: a_uu, 1: a_vv, 2: a_uv
-  const int pbase = lane - pe;
-  float2* Scur = B1;
-  float2* Snxt = B0;
-  int par = 0;
-  int sweeps = 0;
-  for (int sweep = 0; sweep < SR_MAX_SWEEPS; ++sweep) {
-    for (int round = 0; round < nrounds; ++round) {
-      const Plane* cur = pl + par * 36;
-      Plane* nxt = pl + (par ^ 1) * 36;
-      const int* icur = idx + par * SR_NMAX;
-      int* inxt = idx + (par ^ 1) * SR_NMAX;
-      if (plane_warp) {
-        // plane pt of the next round: its positions come from u0, v0 of this round
-        const bool mine = lane < 30 && pt < np;
-        float2 e = make_float2(0.f, 0.f);
-        int u0 = 0, v0 = 0;
-        if (mine) {
-          u0 = ppos[2 * pt];
-          v0 = ppos[2 * pt + 1];
-          e = pe == 0 ? rotated_entry(Scur, cur, u0, u0)
-                      : (pe == 1 ? rotated_entry(Scur, cur, v0, v0) : rotated_entry(Scur, cur, u0, v0));
-        }
+  // Jacobi sweeps.  Roles by warp, in this order: pw plane warps (ten planes of three lanes each) and
+  // bw block warps (one 2 x 2 block of the upper triangle per thread).  Only these take part in the
+  // rounds' barriers; the rest wait at the end.  S is in B1 in even rounds and B0 in odd ones.
+  const int pw = (np + 9) / 10, bw = (nblk + 31) / 32;
+  const int nact = 32 * (pw + bw);
+  int sweeps = 0, par = 0;
+  // After a sweep every index is back at its own position.  Only the m lowest eigenpairs are wanted:
+  // converged when no pair with one of the m smallest diagonal entries would rotate and the other
+  // pairs are below 1e-3 of sqrt(a_ii a_jj), which keeps the eigenvalues among them away from the
+  // lowest (each within 7 % of a diagonal entry for n <= 72).  Saves the last sweep of about half the
+  // problems against asking it of all pairs.  ev: the diagonal, perm: positions by ascending entry.
+  auto more = [&]() {
+    ++sweeps;
+    const float2* S = par ? B0 : B1;
+    for (int p = tid; p < nk_; p += nact) ev[p] = S[spos(p, p)].x;
+    bar_first(nact);
+    for (int p = tid; p < nk_; p += nact) {
+      int r = 0;
+      const float vi = ev[p];
+      for (int q = 0; q < nk_; ++q) r += (ev[q] < vi || (ev[q] == vi && q < p)) ? 1 : 0;
+      perm[r] = p;
+      low[p] = r < m ? 1 : 0;
+    }
+    bar_first(nact);
+    bool any = false;
+    for (int i = warp; i < nk_; i += nact / 32) {
+      const float aii = ev[i];
+      const int li = low[i];
+      for (int j = i + 1 + lane; j < nk_; j += 32) {
+        const float2 a = S[spos(i, j)];
+        const float b2 = __fmaf_rn(a.x, a.x, a.y * a.y);
+        any |= (li | low[j]) ? plane_rotates(aii, ev[j], b2, floor_abs) : b2 > 1e-6f * fabsf(aii * ev[j]) + floor_abs * floor_abs;
+      }
+    }
+    return bar_first_or(nact, any) && sweeps < SR_MAX_SWEEPS;
+  };
+  auto flip = [](float2 a, unsigned f) { return make_float2(a.x, __uint_as_float(__float_as_uint(a.y) ^ f)); };
+  if (warp < pw) {
+    // plane pt of the next round from the entries at its positions u0, v0 of this one:
+    // pe = 0: a_uu, 1: a_vv, 2: a_uv
+    const int pt = warp * 10 + lane / 3, pe = lane % 3, pbase = lane - pe;
+    const bool mine = lane < 30 && pt < np;
+    int l0 = 0, l1 = 0, l2 = 0, l3 = 0, t1 = 0, t2 = 0;
+    unsigned g0 = 0, g1 = 0, g2 = 0, g3 = 0, ge = 0;
+    float sg1 = 0.f, sg2 = 0.f;
+    if (mine) {
+      const int u0 = prev_pos(2 * pt, np), v0 = prev_pos(2 * pt + 1, np);
+      int u = pe == 1 ? v0 : u0, v = pe == 0 ? u0 : v0;
+      if ((u >> 1) > (v >> 1)) {  // the stored block is the transposed one: conjugate the result
+        const int x = u;
+        u = v;
+        v = x;
+        ge = 0x80000000u;
+      }
+      t1 = u >> 1;
+      t2 = v >> 1;
+      const int r = u & 1, c = v & 1;
+      sg1 = r ? 1.f : -1.f;
+      sg2 = c ? 1.f : -1.f;
+      // entries M[r][c], M[r][1-c], M[1-r][c], M[1-r][1-c]; below the diagonal the conjugate above it
+      auto at = [&](int rr, int cc, unsigned& f) {
+        const int i = 2 * t1 + rr, j = 2 * t2 + cc;
+        if (i > j) f = 0x80000000u;
+        return i <= j ? spos(i, j) : spos(j, i);
+      };
+      l0 = at(r, c, g0);
+      l1 = at(r, 1 - c, g1);
+      l2 = at(1 - r, c, g2);
+      l3 = at(1 - r, 1 - c, g3);
+    }
+    float4* log_next = logk + np;
+    do {
+      for (int round = 0; round < nrounds; ++round) {
+        const float2* S = par ? B0 : B1;
+        const Plane* cur = pl + par * 36;
+        const Plane p1 = cur[t1], p2 = cur[t2];
+        float2 e = rotated(flip(S[l0], g0), flip(S[l1], g1), flip(S[l2], g2), flip(S[l3], g3), p1, sg1, p2, sg2);
+        if (np == 1 && p1.on) e = make_float2(pe == 2 ? 0.f : e.x, 0.f);  // its own plane annihilated it
+        e = flip(e, ge);
         const float auu = __shfl_sync(0xffffffffu, e.x, pbase & 31);
         const float avv = __shfl_sync(0xffffffffu, e.x, (pbase + 1) & 31);
         const float2 auv = make_float2(__shfl_sync(0xffffffffu, e.x, (pbase + 2) & 31),
                                        __shfl_sync(0xffffffffu, e.y, (pbase + 2) & 31));
         if (mine && pe == 0) {
-          const bool valid = icur[u0] >= 0 && icur[v0] >= 0;
-          nxt[pt] = make_plane(auu, avv, auv, floor_abs, valid);
+          const Plane w = make_plane(auu, avv, auv, floor_abs);
+          pl[(par ^ 1) * 36 + pt] = w;
+          log_next[pt] = as_float4(w);
         }
-      } else {
-        if (tid < npad) inxt[npos[tid]] = icur[tid];
-        for (int u = tid; u < nunits; u += nthr_o) {
-          if (u < nblk) {
-            const int bt = blk[u];
-            const int t1 = bt & 255, t2 = bt >> 8;
-            const Plane p1 = cur[t1], p2 = cur[t2];
-            const int a0 = 2 * t1, b0 = 2 * t2;
-            const int ra = npos[a0], rb = npos[a0 + 1];
-            const float4 r0 = *reinterpret_cast<const float4*>(Scur + a0 * SR_LD + b0);
-            const float4 r1 = *reinterpret_cast<const float4*>(Scur + (a0 + 1) * SR_LD + b0);
-            if (t1 == t2) {
-              const float2 m00 = make_float2(r0.x, r0.y), m01 = make_float2(r0.z, r0.w);
-              const float2 m10 = zconj(m01), m11 = make_float2(r1.z, r1.w);
-              const float2 y00 = col_rot(m00, m01, p2, 0), y10 = col_rot(m10, m11, p2, 0);
-              const float2 y01 = col_rot(m00, m01, p2, 1), y11 = col_rot(m10, m11, p2, 1);
-              const float2 e00 = row_rot(y00, y10, p1, 0), e11 = row_rot(y01, y11, p1, 1);
-              const float2 e01 = p1.on ? make_float2(0.f, 0.f) : row_rot(y01, y11, p1, 0);
-              Snxt[ra * SR_LD + ra] = make_float2(e00.x, 0.f);
-              Snxt[rb * SR_LD + rb] = make_float2(e11.x, 0.f);
-              const bool sw = ra > rb;
-              Snxt[(sw ? rb : ra) * SR_LD + (sw ? ra : rb)] = sw ? zconj(e01) : e01;
-            } else {
-              const int ca = npos[b0], cb = npos[b0 + 1];
-              const float2 m00 = make_float2(r0.x, r0.y), m01 = make_float2(r0.z, r0.w);
-              const float2 m10 = make_float2(r1.x, r1.y), m11 = make_float2(r1.z, r1.w);
-              const float2 y00 = col_rot(m00, m01, p2, 0), y10 = col_rot(m10, m11, p2, 0);
-              const float2 y01 = col_rot(m00, m01, p2, 1), y11 = col_rot(m10, m11, p2, 1);
-              const float2 e00 = row_rot(y00, y10, p1, 0), e01 = row_rot(y01, y11, p1, 0);
-              const float2 e10 = row_rot(y00, y10, p1, 1), e11 = row_rot(y01, y11, p1, 1);
-              bool sw;
-              sw = ra > ca; Snxt[(sw ? ca : ra) * SR_LD + (sw ? ra : ca)] = sw ? zconj(e00) : e00;
-              sw = ra > cb; Snxt[(sw ? cb : ra) * SR_LD + (sw ? ra : cb)] = sw ? zconj(e01) : e01;
-              sw = rb > ca; Snxt[(sw ? ca : rb) * SR_LD + (sw ? rb : ca)] = sw ? zconj(e10) : e10;
-              sw = rb > cb; Snxt[(sw ? cb : rb) * SR_LD + (sw ? rb : cb)] = sw ? zconj(e11) : e11;
-            }
+        log_next += np;
+        bar_first(nact);
+        par ^= 1;
+      }
+    } while (more());
+    if (tid == 0) misc[3] = sweeps;
+  } else if (warp < pw + bw) {
+    const int u = tid - 32 * pw;
+    const bool mine = u < nblk;
+    int t1 = 0, t2 = 0, l0 = 0, w0 = 0, w1 = 0, w2 = 0, w3 = 0;
+    unsigned f0 = 0, f1 = 0, f2 = 0, f3 = 0;
+    if (mine) {
+      int rem = u;
+      while (rem >= np - t1) { rem -= np - t1; ++t1; }
+      t2 = t1 + rem;
+      l0 = spos(2 * t1, 2 * t2);
+      const int ra = next_pos(2 * t1, np), rb = next_pos(2 * t1 + 1, np);
+      const int ca = next_pos(2 * t2, np), cb = next_pos(2 * t2 + 1, np);
+      auto to = [&](int i, int j, unsigned& f) {
+        if (i > j) f = 0x80000000u;
+        return i <= j ? spos(i, j) : spos(j, i);
+      };
+      w0 = to(ra, ca, f0);
+      w1 = to(ra, cb, f1);
+      w2 = to(rb, ca, f2);
+      w3 = to(rb, cb, f3);
+    }
+    const bool dg = t1 == t2;
+    do {
+      for (int round = 0; round < nrounds; ++round) {
+        if (mine) {
+          const float2* S = par ? B0 : B1;
+          float2* T = par ? B1 : B0;
+          const Plane* cur = pl + par * 36;
+          const Plane p1 = cur[t1], p2 = cur[t2];
+          const float2 m00 = S[l0], m01 = S[l0 + SR_LD / 2], m11 = S[l0 + SR_LD + SR_LD / 2];
+          float2 m10 = S[l0 + SR_LD];
+          if (dg) m10 = zconj(m01);
+          float2 e00 = rotated(m00, m01, m10, m11, p1, -1.f, p2, -1.f);
+          float2 e01 = rotated(m01, m00, m11, m10, p1, -1.f, p2, 1.f);
+          const float2 e10 = rotated(m10, m11, m00, m01, p1, 1.f, p2, -1.f);
+          float2 e11 = rotated(m11, m10, m01, m00, p1, 1.f, p2, 1.f);
+          if (dg) {
+            e00.y = 0.f;
+            e11.y = 0.f;
+            if (p1.on) e01 = make_float2(0.f, 0.f);
           } else {
-            const unsigned v = (unsigned)(u - nblk);
-            const int t = (int)((v * vinv) >> 20);
-            const int h = (int)v - t * nq;
-            const Plane w = cur[t];
-            if (w.on) {
-              // rows p, q of V^T, elements 6h .. 6h + 5 (columns n .. 71 are zero padding)
-              float4* vp4 = reinterpret_cast<float4*>(Vt + icur[2 * t] * SR_LD + 6 * h);
-              float4* vq4 = reinterpret_cast<float4*>(Vt + icur[2 * t + 1] * SR_LD + 6 * h);
-              const float2 sc = zconj(w.s);
-#pragma unroll
-              for (int g = 0; g < 3; ++g) {
-                const float4 a = vp4[g], b = vq4[g];
-                const float2 p0 = zaxpy(w.c, make_float2(a.x, a.y), zneg(zmul(sc, make_float2(b.x, b.y))));
-                const float2 p1_ = zaxpy(w.c, make_float2(a.z, a.w), zneg(zmul(sc, make_float2(b.z, b.w))));
-                const float2 q0 = zaxpy(w.c, make_float2(b.x, b.y), zmul(w.s, make_float2(a.x, a.y)));
-                const float2 q1 = zaxpy(w.c, make_float2(b.z, b.w), zmul(w.s, make_float2(a.z, a.w)));
-                vp4[g] = make_float4(p0.x, p0.y, p1_.x, p1_.y);
-                vq4[g] = make_float4(q0.x, q0.y, q1.x, q1.y);
-              }
-            }
+            T[w2] = flip(e10, f2);
           }
+          T[w0] = flip(e00, f0);
+          T[w1] = flip(e01, f1);
+          T[w3] = flip(e11, f3);
         }
+        bar_first(nact);
+        par ^= 1;
       }
-      __syncthreads();
-      float2* t_ = Scur; Scur = Snxt; Snxt = t_;
-      par ^= 1;
-    }
-    sweeps = sweep + 1;
-    // converged when no pair of the current matrix would rotate
-    bool any = false;
-    const int* icur = idx + par * SR_NMAX;
-    for (int t = tid; t < npad * npad; t += blockDim.x) {
-      const int i = t / npad, j = t % npad;
-      if (i < j && icur[i] >= 0 && icur[j] >= 0) {
-        const float2 a = Scur[i * SR_LD + j];
-        const float beta = sqrtf(a.x * a.x + a.y * a.y);
-        any |= beta > 1.1920929e-07f * sqrtf(fabsf(Scur[i * SR_LD + i].x) * fabsf(Scur[j * SR_LD + j].x)) + floor_abs;
-      }
-    }
-    if (!__syncthreads_or(any)) break;
+    } while (more());
   }
+  __syncthreads();
   // 5. lowest m eigenpairs of the kept coordinates
-  const int* icur = idx + par * SR_NMAX;
-  for (int p = tid; p < npad; p += blockDim.x) ev[p] = Scur[p * SR_LD + p].x;
-  __syncthreads();
-  for (int p = tid; p < npad; p += blockDim.x) {
-    if (icur[p] < 0) continue;
-    int r = 0;
-    const float vi = ev[p];
-    for (int q = 0; q < npad; ++q) {
-      if (icur[q] < 0) continue;
-      r += (ev[q] < vi || (ev[q] == vi && icur[q] < icur[p])) ? 1 : 0;
+  sweeps = misc[3];
+  // eigenvectors of the packed matrix for these m: the logged rotations, last round first
+  float2* Y = Cm;  // nk_ x m
+  const int K = sweeps * nrounds;
+  if (np <= 16) replay<1>(logk, K, np, nk_, m, perm, (float4*)B1, (float4*)B0, Y);
+  else if (np <= 32) replay<2>(logk, K, np, nk_, m, perm, (float4*)B1, (float4*)B0, Y);
+  else replay<3>(logk, K, np, nk_, m, perm, (float4*)B1, (float4*)B0, Y);
+  // coefficients D L^-H Y
+  const int n4 = (n + 3) / 4;
+  for (int t = tid; t < n4 * m; t += SR_THREADS) {
+    const int g = t / m, j = t - g * m;
+    float2 a[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int p = 0; p < nk_; ++p) {
+      const float2 y = Y[p * m + j];
+      const float2* li = Vt + idx[p] * SR_LD + 4 * g;  // columns past n: unused sums
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cfmac(a[q], li[q], y);
     }
-    perm[r] = p;
-  }
-  __syncthreads();
-  for (int t = tid; t < n * m; t += blockDim.x) {
-    const int i = t / m, j = t % m;
-    const float2 v = Vt[icur[perm[j]] * SR_LD + i];  // V[i][col] = V^T[col][i]
-    const float2 c = make_float2(v.x * D[i], v.y * D[i]);
-    ck[t] = c;
-    B1[t] = c;  // the Jacobi buffers are free: cX for the conjugate directions
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = 4 * g + q;
+      if (i < n) {
+        const float2 c = make_float2(a[q].x * D[i], a[q].y * D[i]);
+        ck[i * m + j] = c;
+        B1[i * m + j] = c;  // cX for the conjugate directions
+      }
+    }
   }
   for (int j = tid; j < m; j += blockDim.x) lam_out[(long long)k * m + j] = ev[perm[j]];
   if (cpk) {
     __syncthreads();
-    pdir32(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * m, ev, drop, cpk);
+    pdir32(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * (m | 1), ev, drop, cpk);
   }
   if (flops && tid == 0) {
     // algorithmic work: Cholesky n^3/6, L^-1 GA n^3/2, L^-1 T^H n^3/2 and L^-1 n^3/6 complex
@@ -602,16 +836,20 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
   }
 }
 
+// Rotations of the most sweeps, and the planes of the round after them.
+long long small_rr32_log(int n) { return ((long long)SR_MAX_SWEEPS * n + 1) * ((n + 1) / 2); }
+
 int launch_small_rr32(const float2* GA, const float2* GO, int n, int m, int nk, float drop_tol, const int* kdone,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
-                      cudaStream_t s) {
-  if (n > SR_NMAX || m > n || n < 1) return PC_EINVAL;
+                      float4* rotlog, long long log_stride, cudaStream_t s) {
+  if (n > SR_NMAX || m > n || n < 1 || log_stride < small_rr32_log(n)) return PC_EINVAL;
   const size_t sm = sizeof(float2) * 4 * (size_t)SR_MAT + sizeof(Plane) * 72 + sizeof(float) * 2 * SR_NMAX +
-                    sizeof(int) * (7 * SR_NMAX + SR_BLK + 8);
+                    sizeof(int) * (4 * SR_NMAX + 8);
   static const cudaError_t attr =  // once, thread-safe (k groups launch from several host threads)
       cudaFuncSetAttribute(k_small_rr32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   (void)attr;
-  k_small_rr32<<<nk, SR_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, kdone, lam_out, coef, cp, pdir_abs, status, flops);
+  k_small_rr32<<<nk, SR_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, kdone, lam_out, coef, cp, pdir_abs, status, flops, rotlog,
+                                             log_stride);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
