@@ -122,19 +122,21 @@ int launch_gram_tc(const float2* const A[3], int na, const float2* const B[3], i
                    float scale, float2* part, int max_split, float2* G, int* status, cudaStream_t s);
 int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s);
 
-template <typename R>
-int launch_small_rr(const typename cplx_t<R>::type* GA, const typename cplx_t<R>::type* GO, int n, int m,
-                    int nk, R drop_tol, const int* kdone, R* lam_out, typename cplx_t<R>::type* coef, int* status,
-                    cudaStream_t s);
-// The FP32 projected problems of the mixed form (small_rr.cu): same contract as
-// launch_small_rr<float>; when cp is given, the conjugate-direction coefficients of
-// launch_small_pdir<float> (absolute drop level pdir_abs) are computed by the same CTAs; when
-// flops is given, the algorithmic flops of every problem solved are added to it (device counter).
+// Projected problems, one CTA per k: the pencil (GA, GO) of n <= 72 basis columns, unit-diagonal
+// scaling, Cholesky of GO that drops dependent columns (pivots at or below drop_tol), reduction to
+// standard form, cyclic Jacobi; the lowest m eigenvalues and their coefficients (n x m).  Locked
+// k-points (kdone) keep their block.  When cp is given, the conjugate-direction coefficients of the next
+// iteration come from the same CTA (directions at or below pdir_abs dropped); when flops is given, the
+// algorithmic flops of every problem solved are added to it (device counter).  scratch: global scratch of
+// `stride` bytes per problem, at least small_rr32_scratch(n) / small_rr64_scratch(n), a multiple of 16.
 int launch_small_rr32(const float2* GA, const float2* GO, int n, int m, int nk, float drop_tol, const int* kdone,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
-                      float4* rotlog, long long log_stride, cudaStream_t s);
-// float4 elements of global scratch a problem of size n needs for its rotations (log_stride at least this).
-long long small_rr32_log(int n);
+                      void* scratch, long long stride, cudaStream_t s);
+int launch_small_rr64(const double2* GA, const double2* GO, int n, int m, int nk, double drop_tol, const int* kdone,
+                      double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
+                      long long stride, cudaStream_t s);
+long long small_rr32_scratch(int n);
+long long small_rr64_scratch(int n);
 // Cholesky-QR transform of the Gram G (m x m per k).  When Gref is given (rows_ref x m per
 // k, scale -1, its last m rows holding -Y^H Omega Y before projection), a column whose
 // Omega-norm^2 after projection is below rel_tol times the one before is dropped.
@@ -142,11 +144,6 @@ template <typename R>
 int launch_small_chol(const typename cplx_t<R>::type* G, int m, int nk, R drop_tol,
                       const typename cplx_t<R>::type* Gref, int rows_ref, R rel_tol,
                       typename cplx_t<R>::type* T, cudaStream_t s);
-
-// Conjugate-direction coefficients from the Ritz coefficients (see lobpcg.cu).
-template <typename R>
-int launch_small_pdir(const typename cplx_t<R>::type* GO, const typename cplx_t<R>::type* CX, int n, int m, int nk,
-                      const int* kdone, R abs_drop, typename cplx_t<R>::type* CP, cudaStream_t s);
 
 int launch_convert_f2d(const float2* src, double2* dst, long long n, cudaStream_t s);
 

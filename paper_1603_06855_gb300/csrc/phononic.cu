@@ -74,8 +74,8 @@ struct pc_ctx {
   void *E = nullptr, *S = nullptr;  // strain / stress stacks (R precision)
   void *gpart = nullptr, *GA = nullptr, *GO = nullptr, *Cc = nullptr, *Ct = nullptr;
   void* lam = nullptr;           // nk*m (R)
-  float4* rotlog = nullptr;      // per k: rotations of the FP32 projected problem (small_rr.cu)
-  long long log_stride = 0;
+  unsigned char* sr_scratch = nullptr;  // per k: scratch of the projected problems (small_rr.cu, small_rr64.cu)
+  long long sr_stride = 0;
   double *rnorm = nullptr;
   int *active = nullptr, *d_unconv = nullptr, *kdone = nullptr, *kdone_f = nullptr;
   double* stall_best = nullptr;  // per k: best worst-wanted residual so far (stagnation test)
@@ -237,7 +237,7 @@ static void free_kset(pc_ctx* c) {
   if (c->S) cudaFree(c->S); c->S = nullptr;
   void** vs[] = {&c->gpart, &c->GA, &c->GO, &c->Cc, &c->Ct, &c->lam};
   for (auto v : vs) { if (*v) cudaFree(*v); *v = nullptr; }
-  dfree(c->rotlog); dfree(c->rnorm); dfree(c->active); dfree(c->d_unconv); dfree(c->kdone); dfree(c->kdone_f);
+  dfree(c->sr_scratch); dfree(c->rnorm); dfree(c->active); dfree(c->d_unconv); dfree(c->kdone); dfree(c->kdone_f);
   dfree(c->stall_best); dfree(c->stall_since);
   dfree(c->Xd); dfree(c->AXd); dfree(c->OXd); dfree(c->Ed); dfree(c->Sd); dfree(c->Th); dfree(c->St);
   dfree(c->gpartd); dfree(c->GAd); dfree(c->GOd); dfree(c->Cd);
@@ -457,10 +457,10 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   if (cudaMalloc(&c->Cc, g * esz) != cudaSuccess) { c->Cc = nullptr; rc = PC_ENOMEM; }
   if (cudaMalloc(&c->Ct, g * esz) != cudaSuccess) { c->Ct = nullptr; rc = PC_ENOMEM; }
   if (cudaMalloc(&c->lam, nvec * rsz) != cudaSuccess) { c->lam = nullptr; rc = PC_ENOMEM; }
-  if (c->prm.precision == PC_MIXED) {
-    c->log_stride = small_rr32_log(3 * m);
-    rc |= dalloc(&c->rotlog, (size_t)nk * c->log_stride);
-  }
+  // FP32 problems of up to 3m columns and the FP64 ones of m of the final step, or FP64 ones of up to 3m
+  c->sr_stride = c->prm.precision == PC_MIXED ? std::max(small_rr32_scratch(3 * m), small_rr64_scratch(m))
+                                              : small_rr64_scratch(3 * m);
+  rc |= dalloc(&c->sr_scratch, (size_t)nk * c->sr_stride);
   rc |= dalloc(&c->rnorm, nvec);
   rc |= dalloc(&c->active, nvec);
   rc |= dalloc(&c->d_unconv, (size_t)kMaxGroups);
@@ -719,21 +719,21 @@ static UpdateArgs<R> upd(pc_ctx* c, int nk, int nblk, int identity_last, const v
 // in FP64 on FP64 Grams.
 template <typename R> struct SmallTol;
 template <> struct SmallTol<double> { static constexpr double pdir_abs = 1e-26; };
-template <> struct SmallTol<float> { static constexpr float pdir_abs = 1e-12f; };
+// FP32: directions of norm 1e-7 still lead somewhere after the second projection (one or two iterations
+// fewer than with 1e-12 on the design workloads).
+template <> struct SmallTol<float> { static constexpr float pdir_abs = 1e-14f; };
 
 template <typename R>
 static int small_rr_any(pc_ctx* c, int k0, int nk, const typename Ops<R>::C2* GA, const typename Ops<R>::C2* GO, int n, int m,
                         const int* kdone, R* lam, typename Ops<R>::C2* cX, typename Ops<R>::C2* cP, cudaStream_t s) {
-  int rc;
-  if constexpr (std::is_same<R, float>::value) {  // the conjugate directions from the same CTAs
-    rc = launch_small_rr32(GA, GO, n, m, nk, Ops<R>::drop_small, kdone, lam, cX, cP, SmallTol<R>::pdir_abs,
-                           c->status, c->profiling ? c->small_flops : nullptr, c->rotlog + k0 * c->log_stride,
-                           c->log_stride, s);
-  } else {
-    rc = launch_small_rr<R>(GA, GO, n, m, nk, Ops<R>::drop_small, kdone, lam, cX, c->status, s);
-    if (!rc && cP) rc = launch_small_pdir<R>(GO, cX, n, m, nk, kdone, SmallTol<R>::pdir_abs, cP, s);
-  }
-  return rc;
+  // the conjugate directions come from the same CTAs
+  unsigned char* scratch = c->sr_scratch + k0 * c->sr_stride;
+  if constexpr (std::is_same<R, float>::value)
+    return launch_small_rr32(GA, GO, n, m, nk, Ops<R>::drop_small, kdone, lam, cX, cP, SmallTol<R>::pdir_abs,
+                             c->status, c->profiling ? c->small_flops : nullptr, scratch, c->sr_stride, s);
+  else
+    return launch_small_rr64(GA, GO, n, m, nk, Ops<R>::drop_small, kdone, lam, cX, cP, SmallTol<R>::pdir_abs,
+                             c->status, scratch, c->sr_stride, s);
 }
 template <typename R>
 static int small_chol_any(pc_ctx* c, int nk, const typename Ops<R>::C2* G, int m, typename Ops<R>::C2* T,
@@ -1022,7 +1022,8 @@ static int fp64_rayleigh_ritz(pc_ctx* c, const KSet& ks) {
   if (rc) return rc;
   rc = launch_gram<double>(A1, 1, B2, 1, nk, m, n3, 1.0, gpartd, GOd, s);
   if (rc) return rc;
-  rc = launch_small_rr<double>(GAd, GOd, m, m, nk, 1e-12, nullptr, lamd, Cd, c->status, s);
+  rc = launch_small_rr64(GAd, GOd, m, m, nk, 1e-12, nullptr, lamd, Cd, nullptr, 0.0, c->status,
+                         c->sr_scratch + k0 * c->sr_stride, c->sr_stride, s);
   if (rc) return rc;
   // theta = X C; A theta and Omega theta for the residual report
   UpdateArgs<double> u = upd<double>(c, nk, 1, 0, Cd, (long long)m * m, m, m);
