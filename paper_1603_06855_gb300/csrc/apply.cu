@@ -61,80 +61,113 @@ __device__ __forceinline__ void kvec_r(const Geom& g, const double* Q, const flo
 }
 
 // ---------------------------------------------------------------------------
-// Complex GEMM on CUDA cores: C[col][p] = alpha * sum_q A[p][q] * B[col][q].
-// 64 x 64 output tile, 16-deep K slices staged in shared memory, 4 x 4 outputs per thread.
-template <typename R>
-__global__ __launch_bounds__(256) void k_gemm(int Mrows, int ncols, int K, const typename cplx_t<R>::type* __restrict__ A,
-                                              int lda, const typename cplx_t<R>::type* __restrict__ B, long long ldb,
-                                              typename cplx_t<R>::type* __restrict__ C, long long ldc, R alpha) {
+// Complex GEMMs on CUDA cores, up to three products of the same row count and depth in one launch:
+// C[col][p] = alpha * sum_q A[p][q] * B[col][q].  16 U x 16 U output tile, 16-deep K slices staged in
+// shared memory, U x U outputs per thread, each accumulated over q in order.
+//
+// Bound (FP64): the two multiply-adds a clock of an SM's FP64 pipe; staging costs nothing beside it at
+// any U.  So the tile is the one whose busiest SM has the least work, ceil(tiles / SMs) x tile area: the
+// operator of a reference solve (N = 125, 64 vectors) is 18 tiles of 64 x 64 in three launches on 152 SMs
+// (1.55 ms an application) but 288 of 16 x 16 in one (0.067 ms); N = 343 with 48 vectors 4.2 -> 0.36 ms.
+template <typename R> struct GemmSegs {
+  GemmSeg<R> s[3];
+  int tile0[4];  // first column tile of each product, and their total
+};
+template <typename R, int U>
+__global__ __launch_bounds__(256) void k_gemm(int Mrows, int K, int lda, long long ldb, long long ldc, GemmSegs<R> segs) {
   typedef typename cplx_t<R>::type C2;
-  __shared__ C2 As[16][65];
-  __shared__ C2 Bs[16][65];
+  constexpr int T = 16 * U;
+  __shared__ C2 As[16][T + 1];
+  __shared__ C2 Bs[16][T + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int p0 = blockIdx.x * 64;
-  const long long c0 = (long long)blockIdx.y * 64;
-  C2 acc[4][4];
+  const int g = ((int)blockIdx.x >= segs.tile0[1]) + ((int)blockIdx.x >= segs.tile0[2]);
+  const GemmSeg<R> sg = segs.s[g];
+  const int p0 = blockIdx.y * T;
+  const long long c0 = (long long)((int)blockIdx.x - segs.tile0[g]) * T;
+  C2 acc[U][U];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < U; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = mk<R>(0, 0);
+    for (int j = 0; j < U; ++j) acc[i][j] = mk<R>(0, 0);
   for (int k0 = 0; k0 < K; k0 += 16) {
 #pragma unroll
-    for (int t = threadIdx.x; t < 1024; t += 256) {
+    for (int t = threadIdx.x; t < 16 * T; t += 256) {
       int r = t >> 4, kk = t & 15;
       int p = p0 + r, q = k0 + kk;
-      As[kk][r] = (p < Mrows && q < K) ? A[(long long)p * lda + q] : mk<R>(0, 0);
+      As[kk][r] = (p < Mrows && q < K) ? sg.A[(long long)p * lda + q] : mk<R>(0, 0);
       long long col = c0 + r;
-      Bs[kk][r] = (col < ncols && q < K) ? B[col * ldb + q] : mk<R>(0, 0);
+      Bs[kk][r] = (col < sg.ncols && q < K) ? sg.B[col * ldb + q] : mk<R>(0, 0);
     }
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < 16; ++kk) {
-      C2 a[4], b[4];
+      C2 a[U], b[U];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][tx + 16 * i];
+      for (int i = 0; i < U; ++i) a[i] = As[kk][tx + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][ty + 16 * j];
+      for (int j = 0; j < U; ++j) b[j] = Bs[kk][ty + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < U; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], b[j]);
+        for (int j = 0; j < U; ++j) cfma(acc[i][j], a[i], b[j]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < U; ++j) {
     long long col = c0 + ty + 16 * j;
-    if (col >= ncols) continue;
+    if (col >= sg.ncols) continue;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < U; ++i) {
       int p = p0 + tx + 16 * i;
-      if (p < Mrows) C[col * ldc + p] = cscale(acc[i][j], alpha);
+      if (p < Mrows) sg.C[col * ldc + p] = cscale(acc[i][j], sg.alpha);
     }
   }
 }
 
+static int sm_count_apply() {
+  static const int n = [] {  // queried once; thread-safe static initialisation
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 152;
+    cudaGetLastError();
+    return v;
+  }();
+  return n;
+}
+
 template <typename R>
-int launch_gemm(int Mrows, int ncols, int K, const typename cplx_t<R>::type* A, int lda,
-                const typename cplx_t<R>::type* B, long long ldb, typename cplx_t<R>::type* C,
-                long long ldc, R alpha, cudaStream_t s) {
-  if (ncols <= 0) return PC_OK;
-  long long gy = (ncols + 63) / 64;
-  while (gy > 0) {  // grid.y is limited to 65535
-    int chunk = (int)(gy > 65535 ? 65535 : gy);
-    dim3 grid(cdiv(Mrows, 64), chunk);
-    int cols_here = (int)((long long)chunk * 64 < ncols ? (long long)chunk * 64 : ncols);
-    k_gemm<R><<<grid, 256, 0, s>>>(Mrows, cols_here, K, A, lda, B, ldb, C, ldc, alpha);
-    PC_LAUNCH_CHECK();
-    B += (long long)chunk * 64 * ldb;
-    C += (long long)chunk * 64 * ldc;
-    ncols -= cols_here;
-    gy -= chunk;
+int launch_gemms(int Mrows, int K, int lda, long long ldb, long long ldc, const GemmSeg<R>* seg, int nseg, cudaStream_t s) {
+  if (nseg < 1 || nseg > 3 || Mrows < 1) return PC_EINVAL;
+  int best = 4;
+  long long best_t = -1;
+  for (int u = 4; u >= 1; u >>= 1) {
+    const long long T = 16 * u;
+    long long tiles = 0;
+    for (int g = 0; g < nseg; ++g) tiles += (seg[g].ncols + T - 1) / T;
+    tiles *= cdiv(Mrows, T);
+    const long long t = (tiles + sm_count_apply() - 1) / sm_count_apply() * T * T;
+    if (best_t < 0 || t < best_t) { best_t = t; best = u; }
   }
+  GemmSegs<R> a;
+  int tiles = 0;
+  for (int g = 0; g < 3; ++g) {
+    a.s[g] = seg[g < nseg ? g : nseg - 1];
+    a.tile0[g] = tiles;
+    if (g < nseg) tiles += cdiv(seg[g].ncols, 16 * best);
+    else a.tile0[g] = 0x7fffffff;
+  }
+  a.tile0[3] = tiles;
+  if (tiles == 0) return PC_OK;
+  const dim3 grid(tiles, cdiv(Mrows, 16 * best));
+  if (best == 4) k_gemm<R, 4><<<grid, 256, 0, s>>>(Mrows, K, lda, ldb, ldc, a);
+  else if (best == 2) k_gemm<R, 2><<<grid, 256, 0, s>>>(Mrows, K, lda, ldb, ldc, a);
+  else k_gemm<R, 1><<<grid, 256, 0, s>>>(Mrows, K, lda, ldb, ldc, a);
+  PC_LAUNCH_CHECK();
   return PC_OK;
 }
-template int launch_gemm<double>(int, int, int, const double2*, int, const double2*, long long, double2*, long long, double, cudaStream_t);
-template int launch_gemm<float>(int, int, int, const float2*, int, const float2*, long long, float2*, long long, float, cudaStream_t);
+template int launch_gemms<double>(int, int, int, long long, long long, const GemmSeg<double>*, int, cudaStream_t);
+template int launch_gemms<float>(int, int, int, long long, long long, const GemmSeg<float>*, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // Strain stacks: E[s][vec][q] = sum_c B_s(K_q)[c] U[vec][c][q].

@@ -47,11 +47,17 @@ struct Geom {
   int N;
 };
 
-// Complex GEMM C[col][p] = alpha * sum_q A[p][q] B[col][q]   (both operands K-contiguous)
+// Complex GEMMs C[col][p] = alpha * sum_q A[p][q] B[col][q] (both operands K-contiguous) of the same
+// shape but for their columns, nseg <= 3 in one launch.
+template <typename R> struct GemmSeg {
+  const typename cplx_t<R>::type* A;
+  const typename cplx_t<R>::type* B;
+  typename cplx_t<R>::type* C;
+  int ncols;
+  R alpha;
+};
 template <typename R>
-int launch_gemm(int Mrows, int ncols, int K, const typename cplx_t<R>::type* A, int lda,
-                const typename cplx_t<R>::type* B, long long ldb, typename cplx_t<R>::type* C,
-                long long ldc, R alpha, cudaStream_t s);
+int launch_gemms(int Mrows, int K, int lda, long long ldb, long long ldc, const GemmSeg<R>* seg, int nseg, cudaStream_t s);
 
 // Operator pieces.  Vector blocks are [vec][3][N] complex, vec = k*m + j.
 template <typename R>

@@ -533,7 +533,8 @@ int oz_self_check(int N, int ncols, double* rel_err) {
   if (!rc) rc = oz_prepare_operators(p, W, W, 1.0, 1.0, 0);  // W1 = T = the first block, W2 the second
   if (!rc) rc = oz_slice_columns(p, X, ncols, 0, 0);
   if (!rc) rc = oz_gemm(p, 0, 0, ncols, Co, 0);
-  if (!rc) rc = launch_gemm<double>(N, ncols, N, W, N, X, N, Cr, N, 1.0, 0);
+  const GemmSeg<double> ref = {W, X, Cr, ncols, 1.0};
+  if (!rc) rc = launch_gemms<double>(N, N, N, N, N, &ref, 1, 0);
   if (!rc) {
     k_oz_maxdiff<<<64, 256>>>(Co, Cr, nx, red);
     double h[128];

@@ -596,20 +596,14 @@ static int apply_fp64(pc_ctx* c, const double2* X, double2* AX, double2* OX, int
   const double f = 8.0 * (double)N * (double)N;  // algorithmic flops per complex column
   int rc = launch_strain<double>(X, nvec, m, c->geom, Q, E, s);
   if (rc) return rc;
-  int slot = phase >= 0 ? ph_begin(c, phase, f * nvec, s) : -1;
-  rc = launch_gemm<double>(N, nvec, N, c->W, N, E, N, S, N, 1.0, s);
+  const long long o = (long long)nvec * N;
+  const GemmSeg<double> seg[3] = {
+      {c->W, E, S, nvec, 1.0}, {c->W + NN, E + o, S + o, 5 * nvec, 1.0}, {c->T, X, OX, 3 * nvec, alpha_omega}};
+  const int slot = phase >= 0 ? ph_begin(c, phase, f * 9.0 * nvec, s) : -1;
+  rc = launch_gemms<double>(N, N, N, N, N, seg, 3, s);
   ph_end(c, slot, s);
   if (rc) return rc;
-  slot = phase >= 0 ? ph_begin(c, phase, f * 5.0 * nvec, s) : -1;
-  rc = launch_gemm<double>(N, 5 * nvec, N, c->W + NN, N, E + (long long)nvec * N, N, S + (long long)nvec * N, N, 1.0, s);
-  ph_end(c, slot, s);
-  if (rc) return rc;
-  rc = launch_epilogue<double>(S, nvec, m, c->geom, Q, epi, epi, AX, s);
-  if (rc) return rc;
-  slot = phase >= 0 ? ph_begin(c, phase, f * 3.0 * nvec, s) : -1;
-  rc = launch_gemm<double>(N, 3 * nvec, N, c->T, N, X, N, OX, N, alpha_omega, s);
-  ph_end(c, slot, s);
-  return rc;
+  return launch_epilogue<double>(S, nvec, m, c->geom, Q, epi, epi, AX, s);
 }
 
 // The same products as apply_fp64 (operators prepared with Omega scaled by 1/sO) from the
@@ -657,13 +651,12 @@ static int apply_fp32(pc_ctx* c, const float2* X, float2* AX, float2* OX, int nv
   float2* S = (float2*)c->S;
   int rc = launch_strain<float>(X, nvec, m, c->geom, Q, E, s, Kf);
   if (rc) return rc;
-  rc = launch_gemm<float>(N, nvec, N, c->Wf, N, E, N, S, N, 1.0f, s);
+  const long long o = (long long)nvec * N;
+  const GemmSeg<float> seg[3] = {
+      {c->Wf, E, S, nvec, 1.f}, {c->Wf + NN, E + o, S + o, 5 * nvec, 1.f}, {c->Tf, X, OX, 3 * nvec, 1.f}};
+  rc = launch_gemms<float>(N, N, N, N, N, seg, 3, s);
   if (rc) return rc;
-  rc = launch_gemm<float>(N, 5 * nvec, N, c->Wf + NN, N, E + (long long)nvec * N, N, S + (long long)nvec * N, N, 1.0f, s);
-  if (rc) return rc;
-  rc = launch_epilogue<float>(S, nvec, m, c->geom, Q, 1.0f, 1.0f, AX, s, Kf);
-  if (rc) return rc;
-  return launch_gemm<float>(N, 3 * nvec, N, c->Tf, N, X, N, OX, N, 1.0f, s);
+  return launch_epilogue<float>(S, nvec, m, c->geom, Q, 1.0f, 1.0f, AX, s, Kf);
 }
 
 // A subset of the k-points run by one host thread on one stream: k in [k0, k0 + nk).
