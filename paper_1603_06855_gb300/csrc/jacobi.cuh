@@ -116,11 +116,6 @@ __device__ __forceinline__ Plane<float> make_plane(float app, float aqq, float2 
 // Newton step each gives the angle to about 1e-12, and what that leaves of a_uv goes to the next
 // sweep (the entry is not set to zero).  c = (1 + t^2)^-1/2 is exact to rounding for the tangent used: its
 // binomial series for small t^2 (all but a few rotations here), else the correctly rounded root.
-__device__ __forceinline__ double rcp_approx(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
 __device__ __forceinline__ bool plane_rotates(double app, double aqq, double b2, double floor_abs) {
   const double x = fabs(app * aqq);
   const double t = x > 0.0 ? fma(2.220446049250313e-16 * x, rsqrt_approx(x), floor_abs) : floor_abs;

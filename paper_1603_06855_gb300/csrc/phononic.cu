@@ -63,7 +63,7 @@ struct pc_ctx {
   int* h_unconv = nullptr;  // pinned
   // per-design (FP64)
   double *fields = nullptr, *dchi = nullptr, *chi = nullptr, *chi_mean = nullptr, *dfc = nullptr;
-  double2 *t1 = nullptr, *t2s = nullptr, *sfac = nullptr, *T = nullptr, *W = nullptr, *gj_row = nullptr, *gj_col = nullptr;
+  double2 *t1 = nullptr, *t2s = nullptr, *sfac = nullptr, *T = nullptr, *W = nullptr, *gj = nullptr;
   float2 *Wf = nullptr, *Tf = nullptr;  // scaled FP32 copies (mixed path)
   int* status = nullptr;
   double* small_flops = nullptr;  // device: algorithmic flops of the FP32 projected problems while profiling
@@ -97,8 +97,6 @@ struct pc_ctx {
   bool oz_ready = false;         // oz holds the slices of the current design
   cudaStream_t sk[kMaxGroups] = {};  // non-blocking streams of the k groups
   cudaEvent_t ev_fork = nullptr, ev_join[kMaxGroups] = {};
-  cudaEvent_t ev_gj_rows = nullptr, ev_gj_pivot = nullptr;  // look-ahead of the Gauss-Jordan pivot blocks
-  cudaStream_t s_gj = nullptr;  // their stream, at the highest priority: dispatched ahead of the bulk update
   int split = 1;                // PC_SPLIT=0: the block iteration of the mixed form on one stream
   int groups = 2;               // k groups run concurrently (PC_KGROUPS, 2..kMaxGroups)
   std::mutex ph_mu;             // profiling records from the two k-half threads
@@ -261,7 +259,7 @@ extern "C" void pc_destroy(pc_ctx* c) {
   if (!c) return;
   free_kset(c);
   dfree(c->fields); dfree(c->dchi); dfree(c->chi); dfree(c->chi_mean); dfree(c->dfc);
-  dfree(c->t1); dfree(c->t2s); dfree(c->sfac); dfree(c->T); dfree(c->W); dfree(c->gj_row); dfree(c->gj_col);
+  dfree(c->t1); dfree(c->t2s); dfree(c->sfac); dfree(c->T); dfree(c->W); dfree(c->gj);
   dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
@@ -275,9 +273,6 @@ extern "C" void pc_destroy(pc_ctx* c) {
     if (c->ev_join[i]) cudaEventDestroy(c->ev_join[i]);
   }
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_gj_rows) cudaEventDestroy(c->ev_gj_rows);
-  if (c->ev_gj_pivot) cudaEventDestroy(c->ev_gj_pivot);
-  if (c->s_gj) cudaStreamDestroy(c->s_gj);
   delete c;
 }
 
@@ -398,8 +393,7 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
   rc |= dalloc(&c->sfac, 3 * L * L * L);
   rc |= dalloc(&c->T, 3 * NN);
   rc |= dalloc(&c->W, 2 * NN);
-  rc |= dalloc(&c->gj_row, 4 * 32 * (size_t)N);              // blocked Gauss-Jordan: old pivot rows (2 panels)
-  rc |= dalloc(&c->gj_col, 4 * 32 * ((size_t)N + 32));       // pivot-block inverses, column panels (2 panels)
+  rc |= dalloc(&c->gj, (size_t)setup_gj_scratch(N));
   rc |= dalloc(&c->status, 1);
   rc |= dalloc(&c->small_flops, 1);
   if (p->precision == PC_MIXED) {
@@ -412,15 +406,7 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
       cudaEventCreate(&c->ev_s0) != cudaSuccess || cudaEventCreate(&c->ev_s1) != cudaSuccess ||
       cudaEventCreate(&c->ev_g0) != cudaSuccess || cudaEventCreate(&c->ev_g1) != cudaSuccess ||
       cudaMallocHost((void**)&c->h_unconv, kMaxGroups * sizeof(int)) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->ev_gj_rows, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->ev_gj_pivot, cudaEventDisableTiming) != cudaSuccess) {
-    pc_destroy(c);
-    return PC_ECUDA;
-  }
-  int prio_low = 0, prio_high = 0;
-  if (cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high) != cudaSuccess ||
-      cudaStreamCreateWithPriority(&c->s_gj, cudaStreamNonBlocking, prio_high) != cudaSuccess) {
+      cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess) {
     pc_destroy(c);
     return PC_ECUDA;
   }
@@ -540,8 +526,7 @@ extern "C" int pc_set_design(pc_ctx* c, const double* rho, void* stream) {
   a.mc = c->mc;
   a.fields = c->fields; a.dchi = c->dchi; a.chi = c->chi; a.chi_mean = c->chi_mean; a.dfc = c->dfc;
   a.t1 = c->t1; a.t2 = c->t2s; a.sfac = c->sfac; a.T = c->T; a.W = c->W;
-  a.gj_row = c->gj_row; a.gj_col = c->gj_col;
-  a.side = c->s_gj; a.ev_rows = c->ev_gj_rows; a.ev_pivot = c->ev_gj_pivot;
+  a.gj = c->gj;
   a.status = c->status;
   int rc = launch_setup(a, s);
   if (rc) return rc;

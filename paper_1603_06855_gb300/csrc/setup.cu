@@ -8,6 +8,7 @@
 //                                   isotropic, so Phi^-1 only needs the inverses of the bulk
 //                                   (f1 = (1-2nu)/E) and shear (f2 = (1+nu)/E) Toeplitz blocks.
 #include "kernels.h"
+#include "small_dense.cuh"
 
 // ---------------------------------------------------------------------------
 // SIMP interpolation: fields[0] = density, fields[1] = f1, fields[2] = f2 per element, and
@@ -67,28 +68,43 @@ __global__ void k_mean(const double* __restrict__ x, int n, double* out) {
   if (threadIdx.x == 0) *out = red[0] / (double)n;
 }
 
-// Structure factors by three separable sums, one grid axis at a time.
+// Structure factors by three separable sums, one grid axis at a time.  The phases of an axis of n
+// voxels, exp(i pi D (2j+1)/n), take only 2n values: a CTA tabulates them in shared memory (8 KB at
+// most) and steps through the table, two or four FP64 multiply-adds a term instead of a sine and a cosine
+// (32^3 voxels, M = 4: 460 -> 37 us for the three stages, the same bits).
+#define SFAC_NMAX 256
+__device__ __forceinline__ void phase_table(double2* tab, int n) {
+  for (int t = threadIdx.x; t < 2 * n; t += blockDim.x) tab[t] = phase_pi_over(t, n);
+  __syncthreads();
+}
 // Stage 1 (axis 2): t1[f][i][j][d3] = sum_l c_f[i][j][l] exp(i pi D3 (2l+1)/n2), D3 = d3 - 2M.
 __global__ void k_sfac1(const double* __restrict__ fields, int n0, int n1, int n2, int M,
                         double2* __restrict__ t1) {
+  __shared__ double2 tab[2 * SFAC_NMAX];
+  phase_table(tab, n2);
   int L = 4 * M + 1;
   long long total = 3LL * n0 * n1 * L;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= total) return;
   int d3 = (int)(t % L);
   long long r = t / L;           // (f, i, j)
-  int D = d3 - 2 * M;
+  const int D = (((d3 - 2 * M) % (2 * n2)) + 2 * n2) % (2 * n2);  // phase index of l = 0, its step is 2 D
+  const int step = (2 * D) % (2 * n2);
   const double* src = fields + r * n2;
   double2 acc = make_double2(0.0, 0.0);
-  for (int l = 0; l < n2; ++l) {
-    double2 ph = phase_pi_over((long long)D * (2 * l + 1), n2);
+  for (int l = 0, q = D; l < n2; ++l) {
+    const double2 ph = tab[q];
     acc.x = fma(src[l], ph.x, acc.x);
     acc.y = fma(src[l], ph.y, acc.y);
+    q += step;
+    q -= q >= 2 * n2 ? 2 * n2 : 0;
   }
   t1[t] = acc;
 }
 // Stage 2 (axis 1): t2[f][i][d2][d3] = sum_j t1[f][i][j][d3] exp(i pi D2 (2j+1)/n1).
 __global__ void k_sfac2(const double2* __restrict__ t1, int n0, int n1, int M, double2* __restrict__ t2) {
+  __shared__ double2 tab[2 * SFAC_NMAX];
+  phase_table(tab, n1);
   int L = 4 * M + 1;
   long long total = 3LL * n0 * L * L;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -96,16 +112,19 @@ __global__ void k_sfac2(const double2* __restrict__ t1, int n0, int n1, int M, d
   int d3 = (int)(t % L);
   int d2 = (int)((t / L) % L);
   long long fi = t / ((long long)L * L);
-  int D = d2 - 2 * M;
+  const int D = (((d2 - 2 * M) % (2 * n1)) + 2 * n1) % (2 * n1), step = (2 * D) % (2 * n1);
   double2 acc = make_double2(0.0, 0.0);
-  for (int j = 0; j < n1; ++j) {
-    double2 ph = phase_pi_over((long long)D * (2 * j + 1), n1);
-    cfma(acc, t1[(fi * n1 + j) * L + d3], ph);
+  for (int j = 0, q = D; j < n1; ++j) {
+    cfma(acc, t1[(fi * n1 + j) * L + d3], tab[q]);
+    q += step;
+    q -= q >= 2 * n1 ? 2 * n1 : 0;
   }
   t2[t] = acc;
 }
 // Stage 3 (axis 0): sfac[f][d1][d2][d3] = (1/ne) sum_i t2[f][i][d2][d3] exp(i pi D1 (2i+1)/n0).
 __global__ void k_sfac3(const double2* __restrict__ t2, int n0, int M, double inv_ne, double2* __restrict__ sf) {
+  __shared__ double2 tab[2 * SFAC_NMAX];
+  phase_table(tab, n0);
   int L = 4 * M + 1;
   long long L2 = (long long)L * L;
   long long total = 3LL * L * L2;
@@ -114,11 +133,12 @@ __global__ void k_sfac3(const double2* __restrict__ t2, int n0, int M, double in
   long long d23 = t % L2;
   int d1 = (int)((t / L2) % L);
   int f = (int)(t / (L2 * L));
-  int D = d1 - 2 * M;
+  const int D = (((d1 - 2 * M) % (2 * n0)) + 2 * n0) % (2 * n0), step = (2 * D) % (2 * n0);
   double2 acc = make_double2(0.0, 0.0);
-  for (int i = 0; i < n0; ++i) {
-    double2 ph = phase_pi_over((long long)D * (2 * i + 1), n0);
-    cfma(acc, t2[((long long)f * n0 + i) * L2 + d23], ph);
+  for (int i = 0, q = D; i < n0; ++i) {
+    cfma(acc, t2[((long long)f * n0 + i) * L2 + d23], tab[q]);
+    q += step;
+    q -= q >= 2 * n0 ? 2 * n0 : 0;
   }
   sf[t] = cscale(acc, inv_ne);
 }
@@ -139,110 +159,162 @@ __global__ void k_toeplitz(const double2* __restrict__ sf, int M, double V, doub
   T[t] = cscale(v, V);
 }
 
-// In-place blocked Gauss-Jordan inversion of Hermitian positive definite matrices (no
-// pivoting is needed for HPD).  For the pivot block [k0, k0 + bb) with P = A11^-1, one panel
-// step maps
-//   A11 <- P,   A1j <- P A1j,   Ai1 <- -Ai1 P,   Aij <- Aij - Ai1 P A1j   (i, j outside the block),
-// which is bb scalar Gauss-Jordan steps at once.  Three launches per panel: the pivot block
-// inverse (with a copy of the old pivot rows), the column panel Ai1 P, and the update of the
-// whole matrix.  blockIdx.z selects the matrix.
-#define GJ_B 32
-__global__ void k_gj_pivot(const double2* __restrict__ A, int N, long long mstride, int k0, int bb,
-                           double2* __restrict__ Pbuf, double2* __restrict__ Ar) {
-  __shared__ double2 P[GJ_B * (GJ_B + 1)];
-  __shared__ double2 prow[GJ_B], pcol[GJ_B], qrow[GJ_B];
-  __shared__ double2 sip;
-  const int z = blockIdx.z;
-  const double2* Az = A + z * mstride;
-  const int ld = GJ_B + 1;
-  for (int t = threadIdx.x; t < bb * bb; t += blockDim.x) {
-    int r = t / bb, c = t % bb;
-    P[r * ld + c] = Az[(long long)(k0 + r) * N + k0 + c];
-  }
-  // old pivot rows for the update of the rest of the matrix
-  double2* arz = Ar + (long long)z * GJ_B * N;
-  for (long long t = threadIdx.x; t < (long long)bb * N; t += blockDim.x) {
-    int r = (int)(t / N), c = (int)(t % N);
-    arz[(long long)r * N + c] = Az[(long long)(k0 + r) * N + c];
-  }
-  __syncthreads();
-  // One scalar step per pivot k.  The reciprocal of the pivot and the scaled pivot row
-  // q_c = prow_c / piv are formed once (FP64 division and complex products are scarce on one SM's
-  // FP64 pipe), then every element takes its update.
-  for (int k = 0; k < bb; ++k) {
-    if ((int)threadIdx.x < bb) {
-      prow[threadIdx.x] = P[k * ld + threadIdx.x];
-      pcol[threadIdx.x] = P[threadIdx.x * ld + k];
-    }
-    if (threadIdx.x == 0) {
-      const double2 piv = P[k * ld + k];
-      const double den = piv.x * piv.x + piv.y * piv.y;
-      sip = make_double2(piv.x / den, -piv.y / den);
-    }
+// In-place blocked Gauss-Jordan inversion of Hermitian positive definite matrices (no pivoting is
+// needed), on the upper triangle.  With the pivot block 1, P = A11^-1 and R = A1: (its rows), one panel step
+// is
+//   A11 <- P,   A1j <- (P R)_j,   Ai1 <- -Ai1 P,   Aij <- Aij - Ai1 (P R)_j   (i, j outside the block).
+// Rows already swept (i before the block) and those to come keep A_ij = -A_ji^H between them and
+// A_ij = A_ji^H among themselves, so the upper triangle of 16 x 16 tiles is enough: R_j = -A_j1^H for a
+// swept j, Ai1 = s_i R_i^H with s_i = -1 for a swept i and +1 else, and Ai1 <- ((P R)_i)^H above the block.
+// Two launches a panel: P R, and the update of the tiles, in which one more CTA per matrix inverts the
+// next pivot block.  That block is ready early: the update before stored it as of then, and the CTA
+// applies this panel's term itself.  The tiles of the next panel's rows store R for the next step.
+// blockIdx.z or .y selects the matrix.
+//
+// Bound: FP64 multiply-adds, 4 N^3 per matrix for the half (N = 729, two matrices: 2.5 ms); 16 columns a
+// panel keep the next pivot's chain (16 dependent steps on one SM, some 20 us) beside the update (30 us a
+// panel at N = 343, 72 at 729, 200 at 1331).  Both matrices, against the whole matrix with 32 columns a panel,
+// three to four launches and two events between streams: N = 343 2.7 -> 0.8 ms, 729 7.6 -> 3.6, 1331 33 -> 18.
+constexpr int GJ_B = 16;
+struct GjBufs {
+  double2* A;   // 2 x N x N
+  double2* R;   // 2 parities x 2 x GJ_B x N: rows of the pivot block
+  double2* PR;  // 2 x GJ_B x N
+  double2* P;   // 2 parities x 2 x GJ_B x GJ_B: inverse pivot blocks
+  double2* D;   // 2 parities x 2 x GJ_B x GJ_B: diagonal blocks two panels ahead
+};
+
+// Inverse of the Hermitian positive definite block held by 256 threads, one entry each (rows and columns
+// past N: the identity), scalar Gauss-Jordan steps.  Every warp forms the pivot's reciprocal for itself (a
+// broadcast would cost a barrier), so it is kept to a few FP64 instructions.
+__device__ __forceinline__ double2 gj_block_inverse(double2 v, double2 (*S)[GJ_B + 1]) {
+  const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  for (int k = 0; k < GJ_B; ++k) {
+    S[r][c] = v;
     __syncthreads();
-    const double2 ip = sip;
-    if ((int)threadIdx.x < bb) qrow[threadIdx.x] = cmul(prow[threadIdx.x], ip);
-    __syncthreads();
-    for (int t = threadIdx.x; t < bb * bb; t += blockDim.x) {
-      int r = t / bb, c = t % bb;
-      double2 v;
-      if (r == k && c == k) v = ip;
-      else if (r == k) v = qrow[c];
-      else if (c == k) v = cmul(make_double2(-pcol[r].x, -pcol[r].y), ip);
-      else v = csub(P[r * ld + c], cmul(pcol[r], qrow[c]));
-      P[r * ld + c] = v;
-    }
+    const double ip = inv_newton(S[k][k].x);  // real for a Hermitian block
+    const double2 row = S[k][c], col = cscale(S[r][k], -ip);
+    if (r == k) v = c == k ? make_double2(ip, 0.0) : cscale(row, ip);
+    else if (c == k) v = col;
+    else cfma(v, col, row);
     __syncthreads();
   }
-  double2* pz = Pbuf + (long long)z * GJ_B * GJ_B;
-  for (int t = threadIdx.x; t < bb * bb; t += blockDim.x) pz[t] = P[(t / bb) * ld + t % bb];
+  return v;
 }
 
-// Cp[i][l] = sum_m A[i][k0 + m] P[m][l]: the old column panel times the pivot-block inverse.
-__global__ void k_gj_colpanel(const double2* __restrict__ A, int N, long long mstride, int k0, int bb,
-                              const double2* __restrict__ Pbuf, double2* __restrict__ Cp) {
-  const int z = blockIdx.z;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)N * bb) return;
-  const int i = (int)(t / bb), l = (int)(t % bb);
-  const double2* arow = A + z * mstride + (long long)i * N + k0;
-  const double2* pz = Pbuf + (long long)z * GJ_B * GJ_B;
+// Start: R of panel 0, the inverse of pivot block 0 and the diagonal block of panel 1.
+__global__ __launch_bounds__(256) void k_gj_start(GjBufs g, int N) {
+  __shared__ double2 S[GJ_B][GJ_B + 1];
+  const int z = blockIdx.y;
+  const double2* A = g.A + (long long)z * N * N;
+  const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  if (blockIdx.x == 0) {
+    double2 v = make_double2(r == c ? 1.0 : 0.0, 0.0);
+    if (r < N && c < N) v = A[(long long)r * N + c];
+    g.P[z * GJ_B * GJ_B + threadIdx.x] = gj_block_inverse(v, S);
+    const int r1 = GJ_B + r, c1 = GJ_B + c;
+    g.D[2 * GJ_B * GJ_B + z * GJ_B * GJ_B + threadIdx.x] =
+        (r1 < N && c1 < N) ? A[(long long)r1 * N + c1] : make_double2(r == c ? 1.0 : 0.0, 0.0);
+  }
+  const int j = blockIdx.x * GJ_B + c;
+  if (j < N) g.R[((long long)z * GJ_B + r) * N + j] = r < N ? A[(long long)r * N + j] : make_double2(0.0, 0.0);
+}
+
+// P R of one panel.
+__global__ __launch_bounds__(256) void k_gj_panel(GjBufs g, int N, int par) {
+  __shared__ double2 Ps[GJ_B][GJ_B + 1], Rs[GJ_B][GJ_B + 1];
+  const int z = blockIdx.y, r = threadIdx.x >> 4, c = threadIdx.x & 15, j = blockIdx.x * GJ_B + c;
+  const long long o = ((long long)z * GJ_B + r) * N + j;
+  Ps[r][c] = g.P[(2 * par + z) * GJ_B * GJ_B + threadIdx.x];
+  Rs[r][c] = j < N ? g.R[(long long)par * 2 * GJ_B * N + o] : make_double2(0.0, 0.0);
+  __syncthreads();
   double2 acc = make_double2(0.0, 0.0);
-  for (int m = 0; m < bb; ++m) cfma(acc, arow[m], pz[m * bb + l]);
-  Cp[(long long)z * GJ_B * N + (long long)i * GJ_B + l] = acc;
+#pragma unroll
+  for (int l = 0; l < GJ_B; ++l) cfma(acc, Ps[r][l], Rs[l][c]);
+  if (j < N) g.PR[o] = acc;
 }
 
-// Update of one panel step for a set of rows, one row per blockIdx.y: rows r0 + y, except that
-// the nskip rows from skip0 on are stepped over (y >= skip0 - r0 maps to y + nskip).
-__global__ void k_gj_update(double2* __restrict__ A, int N, long long mstride, int k0, int bb,
-                            const double2* __restrict__ Pbuf, const double2* __restrict__ Ar,
-                            const double2* __restrict__ Cp, int r0, int skip0, int nskip) {
-  __shared__ double2 crow[GJ_B];
-  const int z = blockIdx.z;
-  int i = r0 + (int)blockIdx.y;
-  if (i >= skip0) i += nskip;
-  const double2* arz = Ar + (long long)z * GJ_B * N;
-  const double2* pz = Pbuf + (long long)z * GJ_B * GJ_B;
-  const bool iblk = i >= k0 && i < k0 + bb;
-  if ((int)threadIdx.x < bb)
-    crow[threadIdx.x] = iblk ? pz[(i - k0) * bb + threadIdx.x] : Cp[(long long)z * GJ_B * N + (long long)i * GJ_B + threadIdx.x];
-  __syncthreads();
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
-  double2* a = A + z * mstride + (long long)i * N + j;
-  const bool jblk = j >= k0 && j < k0 + bb;
-  double2 v;
-  if (iblk && jblk) {
-    v = crow[j - k0];                        // P
-  } else if (jblk) {
-    const double2 c = crow[j - k0];          // -Ai1 P
-    v = make_double2(-c.x, -c.y);
-  } else {
-    double2 acc = make_double2(0.0, 0.0);    // (P or Ai1 P) times the old pivot rows
-    for (int l = 0; l < bb; ++l) cfma(acc, crow[l], arz[(long long)l * N + j]);
-    v = iblk ? acc : csub(*a, acc);
+// One panel step: the upper tiles (blockIdx.x - 1 numbers them by rows), and in blockIdx.x = 0 the next
+// pivot block's inverse.
+__global__ __launch_bounds__(256) void k_gj_update(GjBufs g, int N, int p, int nt) {
+  __shared__ double2 X[GJ_B][GJ_B + 1], Y[GJ_B][GJ_B + 1];
+  const int z = blockIdx.y, par = p & 1, r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  double2* A = g.A + (long long)z * N * N;
+  const double2* R = g.R + (long long)(2 * par + z) * GJ_B * N;
+  double2* Rn = g.R + (long long)(2 * (par ^ 1) + z) * GJ_B * N;
+  const double2* PR = g.PR + (long long)z * GJ_B * N;
+  const double2 zero = make_double2(0.0, 0.0);
+  if (blockIdx.x == 0) {
+    if (p + 1 >= nt) return;
+    const int j = (p + 1) * GJ_B + c;
+    X[r][c] = j < N ? R[(long long)r * N + j] : zero;
+    Y[r][c] = j < N ? PR[(long long)r * N + j] : zero;
+    double2 v = g.D[(2 * (par ^ 1) + z) * GJ_B * GJ_B + threadIdx.x];
+    __syncthreads();
+    double2 acc = zero;
+#pragma unroll
+    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Y[l][c]);
+    v = csub(v, acc);
+    __syncthreads();
+    g.P[(2 * (par ^ 1) + z) * GJ_B * GJ_B + threadIdx.x] = gj_block_inverse(v, X);
+    return;
   }
-  *a = v;
+  // tile (I, J), I <= J, number t = I nt - I (I - 1) / 2 + J - I
+  const int t = blockIdx.x - 1;
+  int I = (int)((2 * nt + 1 - sqrtf((float)(2 * nt + 1) * (2 * nt + 1) - 8.f * t)) * 0.5f);
+  I = max(0, min(I, nt - 1));
+  while (I > 0 && t < I * nt - I * (I - 1) / 2) --I;
+  while (I + 1 < nt && t >= (I + 1) * nt - (I + 1) * I / 2) ++I;
+  const int J = I + t - (I * nt - I * (I - 1) / 2);
+  const int i = I * GJ_B + r, j = J * GJ_B + c;
+  const bool in = i < N && j < N;
+  double2 v = zero;
+  if (I == p) {
+    if (J == p) v = g.P[(2 * par + z) * GJ_B * GJ_B + threadIdx.x];
+    else if (j < N) v = PR[(long long)r * N + j];
+  } else if (J == p) {  // above the block: transposed through shared memory
+    const int ii = I * GJ_B + c;
+    X[r][c] = ii < N ? PR[(long long)r * N + ii] : zero;
+    __syncthreads();
+    v = cconj(X[c][r]);
+  } else {
+    const int ii = I * GJ_B + c;
+    X[r][c] = ii < N ? R[(long long)r * N + ii] : zero;
+    Y[r][c] = j < N ? PR[(long long)r * N + j] : zero;
+    if (in) v = A[(long long)i * N + j];
+    __syncthreads();
+    double2 acc = zero;
+#pragma unroll
+    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Y[l][c]);
+    v = I < p ? cadd(v, acc) : csub(v, acc);
+  }
+  if (in) A[(long long)i * N + j] = v;
+  const int n1 = p + 1;
+  if (I == n1) {
+    if (j < N) Rn[(long long)r * N + j] = i < N ? v : zero;
+  } else if (J == n1) {  // R of the swept columns: -A_i1^H, written by rows
+    __syncthreads();
+    X[r][c] = in ? v : zero;
+    __syncthreads();
+    const int ii = I * GJ_B + c;  // c: row of the tile, r: column within the panel
+    if (ii < N) Rn[(long long)r * N + ii] = make_double2(-X[c][r].x, X[c][r].y);
+  }
+  if (I == p + 2 && J == I)
+    g.D[(2 * par + z) * GJ_B * GJ_B + threadIdx.x] = in ? v : make_double2(r == c ? 1.0 : 0.0, 0.0);
+}
+
+// Lower triangle from the upper one, tile by tile through shared memory.
+__global__ __launch_bounds__(256) void k_gj_mirror(double2* __restrict__ A0, int N, int nt) {
+  __shared__ double2 X[GJ_B][GJ_B + 1];
+  const int I = blockIdx.x, J = blockIdx.y;
+  if (I > J) return;
+  double2* A = A0 + (long long)blockIdx.z * N * N;
+  const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  const int i = I * GJ_B + r, j = J * GJ_B + c;
+  if (i < N && j < N) X[r][c] = A[(long long)i * N + j];
+  __syncthreads();
+  const int ti = J * GJ_B + r, tj = I * GJ_B + c;
+  if (ti < N && tj < N && ti > tj) A[(long long)ti * N + tj] = cconj(X[c][r]);
 }
 
 // Copies the f1 and f2 Toeplitz operators into the workspace that is inverted in place.
@@ -275,34 +347,25 @@ int launch_setup(const SetupArgs& a, cudaStream_t s) {
   // W1 = T_f1^-1, W2 = T_f2^-1
   k_copy2<<<cdiv(2 * NN, 256), 256, 0, s>>>(a.T + NN, a.W, 2 * NN);
   PC_LAUNCH_CHECK();
-  // Scratch of two panels (parity p): pivot-block inverses, column panels, old pivot rows.
-  const long long colsz = 2LL * GJ_B * (N + GJ_B), rowsz = 2LL * GJ_B * N;
-  double2* Pbuf[2] = {a.gj_col, a.gj_col + colsz};                                   // 2 x GJ_B x GJ_B each
-  double2* Cp[2] = {a.gj_col + 2LL * GJ_B * GJ_B, a.gj_col + colsz + 2LL * GJ_B * GJ_B};  // 2 x N x GJ_B
-  double2* Ar[2] = {a.gj_row, a.gj_row + rowsz};                                     // 2 x GJ_B x N
-  // Look-ahead: the pivot block of panel k + 1 needs only panel k's update of its own rows, so
-  // those rows are updated first and the next pivot block (one CTA per matrix) runs on the side
-  // stream while the main stream updates the other rows.
-  const bool ahead = a.side && a.ev_rows && a.ev_pivot;
-  k_gj_pivot<<<dim3(1, 1, 2), 512, 0, s>>>(a.W, N, NN, 0, min(GJ_B, N), Pbuf[0], Ar[0]);
-  for (int k0 = 0, pi = 0; k0 < N; k0 += GJ_B, ++pi) {
-    const int bb = min(GJ_B, N - k0), p = pi & 1;
-    const int kn = k0 + bb, bbn = min(GJ_B, N - kn);
-    k_gj_colpanel<<<dim3(cdiv((long long)N * bb, 256), 1, 2), 256, 0, s>>>(a.W, N, NN, k0, bb, Pbuf[p], Cp[p]);
-    const dim3 gx(cdiv(N, 256), 1, 2);
-    if (bbn > 0 && ahead) {
-      k_gj_update<<<dim3(gx.x, bbn, 2), 256, 0, s>>>(a.W, N, NN, k0, bb, Pbuf[p], Ar[p], Cp[p], kn, N, 0);
-      PC_CUDA_TRY(cudaEventRecord(a.ev_rows, s));
-      PC_CUDA_TRY(cudaStreamWaitEvent(a.side, a.ev_rows, 0));
-      k_gj_pivot<<<dim3(1, 1, 2), 512, 0, a.side>>>(a.W, N, NN, kn, bbn, Pbuf[p ^ 1], Ar[p ^ 1]);
-      PC_CUDA_TRY(cudaEventRecord(a.ev_pivot, a.side));
-      k_gj_update<<<dim3(gx.x, N - bbn, 2), 256, 0, s>>>(a.W, N, NN, k0, bb, Pbuf[p], Ar[p], Cp[p], 0, kn, bbn);
-      PC_CUDA_TRY(cudaStreamWaitEvent(s, a.ev_pivot, 0));
-    } else {
-      k_gj_update<<<dim3(gx.x, N, 2), 256, 0, s>>>(a.W, N, NN, k0, bb, Pbuf[p], Ar[p], Cp[p], 0, N, 0);
-      if (bbn > 0) k_gj_pivot<<<dim3(1, 1, 2), 512, 0, s>>>(a.W, N, NN, kn, bbn, Pbuf[p ^ 1], Ar[p ^ 1]);
-    }
+  const int nt = cdiv(N, GJ_B);
+  GjBufs g;
+  g.A = a.W;
+  g.R = a.gj;
+  g.PR = g.R + 4LL * GJ_B * N;
+  g.P = g.PR + 2LL * GJ_B * N;
+  g.D = g.P + 4LL * GJ_B * GJ_B;
+  k_gj_start<<<dim3(nt, 2), 256, 0, s>>>(g, N);
+  PC_LAUNCH_CHECK();
+  for (int p = 0; p < nt; ++p) {
+    k_gj_panel<<<dim3(nt, 2), 256, 0, s>>>(g, N, p & 1);
+    PC_LAUNCH_CHECK();
+    k_gj_update<<<dim3(1 + nt * (nt + 1) / 2, 2), 256, 0, s>>>(g, N, p, nt);
+    PC_LAUNCH_CHECK();
   }
+  k_gj_mirror<<<dim3(nt, nt, 2), 256, 0, s>>>(a.W, N, nt);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
+
+// double2 elements of SetupArgs::gj for N plane waves.
+long long setup_gj_scratch(int N) { return 6LL * GJ_B * N + 8LL * GJ_B * GJ_B; }
