@@ -137,8 +137,8 @@ typedef struct {
   double ms_host_idle;     /* stream idle time while the host reads the convergence count of each block
                               iteration and enqueues the next one (profiling; summed over the k groups) */
   int rr_sliced;           /* 1 when the Rayleigh-Ritz operator products run as exact 6-bit slice products on
-                              the tensor cores (36 bf16 products per FP64-accurate one; mixed form,
-                              N <= 1008), 0 when they run as the FP64 CUDA-core GEMM */
+                              the tensor cores (36 bf16 products per FP64-accurate one, 55 for N > 1008;
+                              mixed form), 0 when they run as the FP64 CUDA-core GEMM */
   long long small_calls;   /* calls timed in ms_small (profiling): the projected eigenproblem kernel and the
                               small Cholesky factorisations of the orthonormalisation */
 } pc_stats;

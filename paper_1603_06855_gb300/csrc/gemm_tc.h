@@ -18,9 +18,8 @@ int tc_apply(TcPlan* p, const float2* X, float2* AX, float2* OX, int nvec, int m
              const float4* Kf = nullptr);
 
 // FP64-accurate operator products by exact 6-bit slicing on the tensor cores (oz_gemm.cu), for
-// the mixed form's final Rayleigh-Ritz step.  Eligible for 2N (padded to 32) below 2048.
+// the mixed form's final Rayleigh-Ritz step.
 struct OzPlan;
-bool oz_eligible(int N);
 // ncap: right-hand-side columns the plan holds; share: a plan whose operator slices to use.
 OzPlan* oz_plan_create(int N, int ncap, int* status, const OzPlan* share);
 void oz_plan_destroy(OzPlan* p);

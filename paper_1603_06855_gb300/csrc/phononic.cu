@@ -485,7 +485,7 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
       c->tcg[g] = tc_plan_create_sharing(c->tc, gk * m, c->status);
     }
     // the final Rayleigh-Ritz step's products: 6 strain stacks and 3 displacement columns per vector
-    if (c->tc && oz_eligible(N)) {
+    if (c->tc) {
       c->oz = oz_plan_create(N, 9 * (int)nvec, c->status, nullptr);
       for (int g = 1; g < ng && oz_available(c->oz); ++g) {
         const int gk = (int)(((long long)nk * (g + 1)) / ng - ((long long)nk * g) / ng);
