@@ -209,12 +209,12 @@ template int launch_strain<float>(const float2*, int, int, Geom, const double*, 
 template <typename R>
 __global__ void k_epilogue(const typename cplx_t<R>::type* __restrict__ S, int nvec, int m, Geom g,
                            const double* __restrict__ Q, const float4* __restrict__ Kf, R c0, R c1,
-                           typename cplx_t<R>::type* __restrict__ AX) {
+                           typename cplx_t<R>::type* __restrict__ AX, VecSel sel) {
   typedef typename cplx_t<R>::type C2;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int N = g.N;
   if (t >= (long long)nvec * N) return;
-  int vec = (int)(t / N), p = (int)(t % N);
+  const int vec = sel((int)(t / N)), p = (int)(t % N);
   R k0, k1, k2;
   kvec_r<R>(g, Q, Kf, vec / m, p, k0, k1, k2);
   const long long st = (long long)nvec * N;
@@ -232,15 +232,16 @@ __global__ void k_epilogue(const typename cplx_t<R>::type* __restrict__ S, int n
 }
 template <typename R>
 int launch_epilogue(const typename cplx_t<R>::type* Sig, int nvec, int m, Geom g, const double* Q,
-                    R c0, R c1, typename cplx_t<R>::type* AX, cudaStream_t s, const float4* Kf) {
+                    R c0, R c1, typename cplx_t<R>::type* AX, cudaStream_t s, const float4* Kf, VecSel sel) {
   long long n = (long long)nvec * g.N;
   if (sizeof(R) != sizeof(float)) Kf = nullptr;  // the table is FP32
-  k_epilogue<R><<<cdiv(n, 256), 256, 0, s>>>(Sig, nvec, m, g, Q, Kf, c0, c1, AX);
+  if (n == 0) return PC_OK;
+  k_epilogue<R><<<cdiv(n, 256), 256, 0, s>>>(Sig, nvec, m, g, Q, Kf, c0, c1, AX, sel);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
-template int launch_epilogue<double>(const double2*, int, int, Geom, const double*, double, double, double2*, cudaStream_t, const float4*);
-template int launch_epilogue<float>(const float2*, int, int, Geom, const double*, float, float, float2*, cudaStream_t, const float4*);
+template int launch_epilogue<double>(const double2*, int, int, Geom, const double*, double, double, double2*, cudaStream_t, const float4*, VecSel);
+template int launch_epilogue<float>(const float2*, int, int, Geom, const double*, float, float, float2*, cudaStream_t, const float4*, VecSel);
 
 // ---------------------------------------------------------------------------
 // Relative residuals ||A x - lambda Omega x|| / (max(|lambda|, floor) ||Omega x||), one block per vector.
@@ -248,11 +249,11 @@ template int launch_epilogue<float>(const float2*, int, int, Geom, const double*
 template <typename R>
 __global__ void k_resnorm(const typename cplx_t<R>::type* __restrict__ AX, const typename cplx_t<R>::type* __restrict__ OX,
                           const R* __restrict__ lam, int m, int nb, int n3, double tol, double* __restrict__ rnorm,
-                          int* __restrict__ active) {
+                          int* __restrict__ active, const int* __restrict__ klist) {
   typedef typename cplx_t<R>::type C2;
   __shared__ double ra[256], rb[256];
-  int vec = blockIdx.x;
-  int k = vec / m;
+  const int k = klist ? klist[blockIdx.x / m] : (int)blockIdx.x / m;
+  const int vec = k * m + (int)blockIdx.x % m;
   R l = lam[vec];
   const C2* ax = AX + (long long)vec * n3;
   const C2* ox = OX + (long long)vec * n3;
@@ -279,68 +280,119 @@ __global__ void k_resnorm(const typename cplx_t<R>::type* __restrict__ AX, const
     active[vec] = rn > tol ? 1 : 0;
   }
 }
-// Number of k-points with a wanted band above tolerance.  A k-point whose wanted bands
-// are all below tolerance is locked for good (kdone = 1): its block is no longer updated.
+// The convergence test of the open k-points (in klist order, `nopen` of them, or all nk without a list),
+// by one CTA.  A k-point whose wanted bands are all below tolerance is locked for good (kdone = 1): its
+// block is no longer updated.
 // Stagnation: the carried FP32 products A X and Omega X drift by rounding, so a k-point's
 // residual can settle at an attainable floor a little above the tolerance.  A k-point whose
 // worst wanted residual has not dropped below 0.95 of its best for STALL_ITERS iterations and
 // lies within STALL_FACTOR times the tolerance is accepted at that floor.
+// The lists of the next iteration come out compacted and in order; klist is read before it is rewritten
+// (a chunk's outputs never pass the inputs already read).
 #define STALL_ITERS 20
 #define STALL_FACTOR 10.0
-__global__ void k_count_unconv(const int* __restrict__ active, const double* __restrict__ rnorm, double tol, int nk,
-                               int m, int nb, int* __restrict__ kdone, double* __restrict__ best,
-                               int* __restrict__ since, int* out) {
-  __shared__ int red[256];
-  int c = 0;
-  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-    int a = 0;
-    double worst = 0.0;
-    for (int j = 0; j < nb; ++j) {
-      a |= active[k * m + j];
-      worst = fmax(worst, rnorm[k * m + j]);
-    }
-    if (!a) kdone[k] = 1;
-    if (best && !kdone[k]) {
-      if (best[k] == 0.0 || worst < 0.95 * best[k]) {
-        best[k] = worst;
-        since[k] = 0;
-      } else if (++since[k] >= STALL_ITERS && worst <= STALL_FACTOR * tol) {
-        kdone[k] = 1;
-      }
-    }
-    c += kdone[k] ? 0 : 1;
-  }
-  red[threadIdx.x] = c;
+__global__ __launch_bounds__(256) void k_open(const int* __restrict__ active, const double* __restrict__ rnorm, double tol,
+                                              int nopen, int m, int nb, int* __restrict__ kdone, double* __restrict__ best,
+                                              int* __restrict__ since, OpenSet o, int lists) {
+  __shared__ int sums[3][8], base[3];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid < 3) base[tid] = 0;
   __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+  for (int p0 = 0; p0 < nopen; p0 += 256) {
+    const int p = p0 + tid;
+    int k = -1, open = 0, fresh = 0, cols = 0;
+    if (p < nopen) {
+      k = lists ? o.klist[p] : p;
+      int a = 0;
+      double worst = 0.0;
+      for (int j = 0; j < m; ++j) {
+        const int aj = active[k * m + j];
+        cols += aj;
+        if (j < nb) {
+          a |= aj;
+          worst = fmax(worst, rnorm[k * m + j]);
+        }
+      }
+      bool done = !a;
+      if (best && !done) {
+        if (best[k] == 0.0 || worst < 0.95 * best[k]) {
+          best[k] = worst;
+          since[k] = 0;
+        } else if (++since[k] >= STALL_ITERS && worst <= STALL_FACTOR * tol) {
+          done = true;
+        }
+      }
+      kdone[k] = done ? 1 : 0;
+      open = done ? 0 : 1;
+      fresh = done ? 1 : 0;
+      if (done) cols = 0;
+    }
+    int v[3] = {open, cols, fresh}, x[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      x[i] = v[i];
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x[i], d);
+        if (lane >= d) x[i] += y;
+      }
+      if (lane == 31) sums[i][warp] = x[i];
+    }
+    __syncthreads();  // also: every k of this chunk has been read
+    int off[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      off[i] = base[i] + x[i] - v[i];
+      for (int w = 0; w < warp; ++w) off[i] += sums[i][w];
+    }
+    if (lists && k >= 0) {
+      if (open) o.klist[off[0]] = k;
+      if (fresh) o.fresh[off[2]] = k;
+      if (open)
+        for (int j = 0; j < m; ++j)
+          if (active[k * m + j]) o.vlist[off[1]++] = k * m + j;
+    }
+    __syncthreads();
+    if (tid < 3)
+      for (int w = 0; w < 8; ++w) base[tid] += sums[tid][w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *out = red[0];
+  if (tid < 3) o.count[tid] = base[tid];
 }
-template <typename R>
-int launch_resnorm(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX, const R* lam,
-                   int nk, int m, int nb, int n3, double tol, double* rnorm, int* active, int* kdone, int* unconv,
-                   cudaStream_t s, double* best, int* since) {
-  k_resnorm<R><<<nk * m, 256, 0, s>>>(AX, OX, lam, m, nb, n3, tol, rnorm, active);
-  PC_LAUNCH_CHECK();
-  k_count_unconv<<<1, 256, 0, s>>>(active, rnorm, tol, nk, m, nb, kdone, best, since, unconv);
+__global__ void k_open_all(int* klist, int nk) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < nk) klist[k] = k;
+}
+int launch_open_all(OpenSet o, int nk, cudaStream_t s) {
+  k_open_all<<<cdiv(nk, 256), 256, 0, s>>>(o.klist, nk);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
-template int launch_resnorm<double>(const double2*, const double2*, const double*, int, int, int, int, double, double*, int*, int*, int*, cudaStream_t, double*, int*);
-template int launch_resnorm<float>(const float2*, const float2*, const float*, int, int, int, int, double, double*, int*, int*, int*, cudaStream_t, double*, int*);
+template <typename R>
+int launch_resnorm(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX, const R* lam,
+                   int nk, int m, int nb, int n3, double tol, double* rnorm, int* active, int* kdone, OpenSet o, int nopen,
+                   cudaStream_t s, double* best, int* since) {
+  const int lists = o.klist != nullptr;
+  const int n = lists ? nopen : nk;
+  k_resnorm<R><<<n * m, 256, 0, s>>>(AX, OX, lam, m, nb, n3, tol, rnorm, active, o.klist);
+  PC_LAUNCH_CHECK();
+  k_open<<<1, 256, 0, s>>>(active, rnorm, tol, n, m, nb, kdone, best, since, o, lists);
+  PC_LAUNCH_CHECK();
+  return PC_OK;
+}
+template int launch_resnorm<double>(const double2*, const double2*, const double*, int, int, int, int, double, double*, int*, int*, OpenSet, int, cudaStream_t, double*, int*);
+template int launch_resnorm<float>(const float2*, const float2*, const float*, int, int, int, int, double, double*, int*, int*, OpenSet, int, cudaStream_t, double*, int*);
 
 // Preconditioned residual W = P_q (A x - lambda Omega x) with P_q the inverse of a shifted
 // homogeneous Christoffel operator a I + b K K^T of a reference medium (mean chi):
 // (a I + b K K^T)^-1 = (I - b/(a + b|K|^2) K K^T) / a, a = mu |K|^2 + s rho sigma, b = lambda + mu,
 // sigma the largest wanted Ritz value at the k-point and s the weight of the mass term.
-// Converged columns get W = 0.
+// Converged columns get W = 0, and A W = Omega W = 0 with it (the operator is applied to the others only).
 template <typename R>
 __global__ void k_precond(const typename cplx_t<R>::type* __restrict__ AX, const typename cplx_t<R>::type* __restrict__ OX,
-                          const R* __restrict__ lam, const int* __restrict__ active, const int* __restrict__ kdone,
+                          const R* __restrict__ lam, const int* __restrict__ active, const int* __restrict__ klist,
                           int nvec, int m, int nb, Geom g, const double* __restrict__ Q, const float4* __restrict__ Kf,
-                          PrecRef pr, const double* __restrict__ chi_mean, typename cplx_t<R>::type* __restrict__ W) {
+                          PrecRef pr, const double* __restrict__ chi_mean, typename cplx_t<R>::type* __restrict__ W,
+                          typename cplx_t<R>::type* __restrict__ AW, typename cplx_t<R>::type* __restrict__ OW) {
   typedef typename cplx_t<R>::type C2;
   // the reference medium (Lame constants and density at the mean chi), once per block in FP64
   __shared__ R ref[3];
@@ -363,11 +415,11 @@ __global__ void k_precond(const typename cplx_t<R>::type* __restrict__ AX, const
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int N = g.N;
   if (t >= (long long)nvec * N) return;
-  int vec = (int)(t / N), q = (int)(t % N);
-  int k = vec / m;
+  const int q = (int)(t % N), k = klist[(int)(t / N) / m], vec = k * m + (int)(t / N) % m;
   C2* w = W + (long long)vec * 3 * N + q;
-  if (!active[vec] || kdone[k]) {
-    w[0] = mk<R>(0, 0); w[N] = mk<R>(0, 0); w[2 * N] = mk<R>(0, 0);
+  if (!active[vec]) {
+    C2 *aw = AW + (long long)vec * 3 * N + q, *ow = OW + (long long)vec * 3 * N + q;
+    for (int c = 0; c < 3; ++c) w[c * N] = aw[c * N] = ow[c * N] = mk<R>(0, 0);
     return;
   }
   const R lam_r = ref[0];
@@ -399,16 +451,33 @@ __global__ void k_precond(const typename cplx_t<R>::type* __restrict__ AX, const
 }
 template <typename R>
 int launch_precond(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX, const R* lam,
-                   const int* active, const int* kdone, int nk, int m, int nb, Geom g, const double* Q, PrecRef pr,
-                   const double* chi_mean, typename cplx_t<R>::type* W, cudaStream_t s, const float4* Kf) {
-  long long n = (long long)nk * m * g.N;
+                   const int* active, const int* klist, int nopen, int m, int nb, Geom g, const double* Q, PrecRef pr,
+                   const double* chi_mean, typename cplx_t<R>::type* W, typename cplx_t<R>::type* AW,
+                   typename cplx_t<R>::type* OW, cudaStream_t s, const float4* Kf) {
+  long long n = (long long)nopen * m * g.N;
   if (sizeof(R) != sizeof(float)) Kf = nullptr;  // the table is FP32
-  k_precond<R><<<cdiv(n, 256), 256, 0, s>>>(AX, OX, lam, active, kdone, nk * m, m, nb, g, Q, Kf, pr, chi_mean, W);
+  k_precond<R><<<cdiv(n, 256), 256, 0, s>>>(AX, OX, lam, active, klist, nopen * m, m, nb, g, Q, Kf, pr, chi_mean, W, AW, OW);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
-template int launch_precond<double>(const double2*, const double2*, const double*, const int*, const int*, int, int, int, Geom, const double*, PrecRef, const double*, double2*, cudaStream_t, const float4*);
-template int launch_precond<float>(const float2*, const float2*, const float*, const int*, const int*, int, int, int, Geom, const double*, PrecRef, const double*, float2*, cudaStream_t, const float4*);
+template int launch_precond<double>(const double2*, const double2*, const double*, const int*, const int*, int, int, int, Geom, const double*, PrecRef, const double*, double2*, double2*, double2*, cudaStream_t, const float4*);
+template int launch_precond<float>(const float2*, const float2*, const float*, const int*, const int*, int, int, int, Geom, const double*, PrecRef, const double*, float2*, float2*, float2*, cudaStream_t, const float4*);
+
+template <typename R>
+__global__ void k_store(const typename cplx_t<R>::type* __restrict__ src, double2* __restrict__ dst,
+                        const int* __restrict__ list, long long per) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < per) dst[list[blockIdx.y] * per + t] = to_d2(src[list[blockIdx.y] * per + t]);
+}
+template <typename R>
+int launch_store(const typename cplx_t<R>::type* src, double2* dst, const int* list, int nsel, long long per, cudaStream_t s) {
+  if (nsel <= 0) return PC_OK;
+  k_store<R><<<dim3(cdiv(per, 256), nsel), 256, 0, s>>>(src, dst, list, per);
+  PC_LAUNCH_CHECK();
+  return PC_OK;
+}
+template int launch_store<double>(const double2*, double2*, const int*, int, long long, cudaStream_t);
+template int launch_store<float>(const float2*, double2*, const int*, int, long long, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // Initial block: the m lowest homogeneous plane waves (ranked by |K_q|, ties by index),

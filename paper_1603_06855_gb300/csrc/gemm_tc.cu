@@ -55,6 +55,8 @@ struct TcSeg {
   int col_base, ncols;     // columns of the right-hand sides (and of the output)
   int tile0, ntiles;       // first tile of the segment, column tiles
   float* C;                // output, column col_base + j at C + (col_base + j) * ldc
+  VecSel sel;              // (T_rho segment) selected vectors: column j belongs to vector sel(j / 3)
+  int mapped;              // its output columns are mapped through sel
 };
 struct TcGemmParams {
   CUtensorMap A[3][3];     // [operator][slice hi, mid, lo]
@@ -207,6 +209,7 @@ __global__ __launch_bounds__(192, 1) void k_tc_gemm(const __grid_constant__ TcGe
       const int n0 = (lt / mtiles) * TC_BN;
       const int col_base = sg.col_base, ncols = sg.ncols;
       float* const C = sg.C;
+      const int mapped = sg.mapped;
 #pragma unroll 1
       for (int c = 0; c < TC_BN / 16; ++c) {
         float v[16];
@@ -214,8 +217,11 @@ __global__ __launch_bounds__(192, 1) void k_tc_gemm(const __grid_constant__ TcGe
         if (!ok || row >= m_valid) continue;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const int col = n0 + c * 16 + j;
-          if (col < ncols) C[(long long)(col_base + col) * ldc + row] = v[j];
+          int col = n0 + c * 16 + j;
+          if (col < ncols) {
+            if (mapped) col = 3 * sg.sel(col / 3) + col % 3;
+            C[(long long)(col_base + col) * ldc + row] = v[j];
+          }
         }
       }
       tc_fence_before();
@@ -283,7 +289,7 @@ __device__ __forceinline__ void split3_store2(float2 v, __nv_bfloat16* p, long l
 
 __global__ void k_tc_split_strain(const float2* __restrict__ X, int nvec, int m, Geom g, const double* __restrict__ Q,
                                   const float4* __restrict__ Kf, int Kp, __nv_bfloat16* __restrict__ E, long long es,
-                                  __nv_bfloat16* __restrict__ Xs, long long xs) {
+                                  __nv_bfloat16* __restrict__ Xs, long long xs, VecSel sel) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int N = g.N;
   const int Kh = Kp / 2;  // complex slots per column (>= N)
@@ -292,9 +298,10 @@ __global__ void k_tc_split_strain(const float2* __restrict__ X, int nvec, int m,
   float2 u0 = make_float2(0.f, 0.f), u1 = u0, u2 = u0;
   float k0 = 0.f, k1 = 0.f, k2 = 0.f;
   if (q < N) {
-    const float2* x = X + (long long)vec * 3 * N;
+    const int src = sel(vec);
+    const float2* x = X + (long long)src * 3 * N;
     u0 = x[q]; u1 = x[N + q]; u2 = x[2 * N + q];
-    const int k = vec / m;
+    const int k = src / m;
     if (Kf) {  // the k-set's FP32 wavevectors
       const float4 kk = Kf[(long long)k * N + q];
       k0 = kk.x; k1 = kk.y; k2 = kk.z;
@@ -481,6 +488,8 @@ int tc_prepare_operators(TcPlan* p, const double2* W, const double2* T, double w
 struct TcSegSpec {
   int which, bset, col_base, ncols;
   float* C;
+  VecSel sel;
+  int mapped;
 };
 static int launch_tc_gemm(TcPlan* p, const TcSegSpec* sp, int nseg, cudaStream_t s) {
   static const int sms = [] {  // queried once; thread-safe static initialisation
@@ -505,10 +514,10 @@ static int launch_tc_gemm(TcPlan* p, const TcSegSpec* sp, int nseg, cudaStream_t
   int tiles = 0;
   for (int g = 0; g < nseg; ++g) {
     const int nt = (sp[g].ncols + TC_BN - 1) / TC_BN;
-    P.seg[g] = TcSeg{sp[g].which, sp[g].bset, sp[g].col_base, sp[g].ncols, tiles, nt, sp[g].C};
+    P.seg[g] = TcSeg{sp[g].which, sp[g].bset, sp[g].col_base, sp[g].ncols, tiles, nt, sp[g].C, sp[g].sel, sp[g].mapped};
     tiles += mtiles * nt;
   }
-  for (int g = nseg; g < 3; ++g) P.seg[g] = TcSeg{0, 0, 0, 0, tiles, 0, nullptr};
+  for (int g = nseg; g < 3; ++g) P.seg[g] = TcSeg{0, 0, 0, 0, tiles, 0, nullptr, {}, 0};
   P.nseg = nseg;
   P.num_kb = p->Kp / TC_BK;
   P.m_valid = 2 * p->N;
@@ -524,18 +533,19 @@ static int launch_tc_gemm(TcPlan* p, const TcSegSpec* sp, int nseg, cudaStream_t
 }
 
 int tc_apply(TcPlan* p, const float2* X, float2* AX, float2* OX, int nvec, int m, Geom g, const double* Q,
-             cudaStream_t s, const float4* Kf) {
+             cudaStream_t s, const float4* Kf, VecSel sel) {
   if (!tc_available(p) || nvec > p->nvec_max) return PC_EINVAL;
+  if (nvec == 0) return PC_OK;
   const long long n = (long long)nvec * (p->Kp / 2);
   const long long es = (long long)6 * p->nvec_max * p->Kp, xs = (long long)3 * p->nvec_max * p->Kp;
-  k_tc_split_strain<<<cdiv(n, 256), 256, 0, s>>>(X, nvec, m, g, Q, Kf, p->Kp, p->E, es, p->X, xs);
+  k_tc_split_strain<<<cdiv(n, 256), 256, 0, s>>>(X, nvec, m, g, Q, Kf, p->Kp, p->E, es, p->X, xs, sel);
   PC_LAUNCH_CHECK();
-  // E column s * nvec + v holds stack s of vector v (the maps span the plan's capacity).  One
-  // launch: W1 on the dilatation stack, W2 on the five deviatoric stacks (both into S), T_rho on
-  // the displacements (into OX).
-  const TcSegSpec seg[3] = {{0, 0, 0, nvec, (float*)p->S}, {1, 0, nvec, 5 * nvec, (float*)p->S},
-                            {2, 1, 0, 3 * nvec, (float*)OX}};
+  // E column s * nvec + v holds stack s of the v-th selected vector (the maps span the plan's
+  // capacity).  One launch: W1 on the dilatation stack, W2 on the five deviatoric stacks (both into
+  // S), T_rho on the displacements (into the vectors' columns of OX).
+  const TcSegSpec seg[3] = {{0, 0, 0, nvec, (float*)p->S, {}, 0}, {1, 0, nvec, 5 * nvec, (float*)p->S, {}, 0},
+                            {2, 1, 0, 3 * nvec, (float*)OX, sel, sel.list != nullptr}};
   int rc = launch_tc_gemm(p, seg, 3, s);
   if (rc) return rc;
-  return launch_epilogue<float>(p->S, nvec, m, g, Q, 1.0f, 1.0f, AX, s, Kf);
+  return launch_epilogue<float>(p->S, nvec, m, g, Q, 1.0f, 1.0f, AX, s, Kf, sel);
 }

@@ -684,19 +684,24 @@ __device__ __forceinline__ void replay(const Plane<R>* __restrict__ logk, int K,
 // of nearly equal vectors whose rounding lies in the Ritz block, and normalising it put noise at cosines
 // of 0.5 to X into P, which broke single k-points of high-contrast cells late in the iteration (4 of 16
 // start blocks on the SC 16^3 cell under the Young's-modulus law; none since).
-// go: the projected Gram matrix (global); G (stride SR_LD), cx, z, gz (n x m compact), Mm, Mi (m x m,
+// GO: the projected Gram matrix (global), of problem prob; G (stride SR_LD), cx, z, gz (n x m compact), Mm, Mi (m x m,
 // stride m | 1), Dd (m), drp (m): shared workspaces; cp: output (n x m).  The products give each
 // thread four rows of one column (the row operands are shared by the warp's lanes).
 template <typename R, int THREADS, typename C2 = typename cplx_t<R>::type>
-__device__ void pdir(const C2* __restrict__ go, int n, int m, R abs_drop, C2* G, const C2* cx, C2* z, C2* gz, C2* Mm, C2* Mi,
+__device__ void pdir(const MatRef<R>& GO, int prob, int n, int m, R abs_drop, C2* G, const C2* cx, C2* z, C2* gz, C2* Mm, C2* Mi,
                      R* Dd, int* drp, C2* __restrict__ cp) {
   constexpr int W = THREADS / 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int ldm = m | 1;
   for (int r = warp; r < n; r += W)  // GO, symmetrised
-    for (int q = lane; q < n; q += 32) {
-      const C2 g1 = go[r * n + q], g2 = go[q * n + r];
-      G[r * SR_LD + q] = mk<R>((R)0.5 * (g1.x + g2.x), (R)0.5 * (g1.y - g2.y));
+    for (int q = lane; q < n; q += 32) G[r * SR_LD + q] = GO.at(prob, r * n + q);
+  __syncthreads();
+  for (int r = warp; r < n; r += W)
+    for (int q = r + lane; q < n; q += 32) {
+      const C2 g1 = G[r * SR_LD + q], g2 = G[q * SR_LD + r];
+      const C2 g = mk<R>((R)0.5 * (g1.x + g2.x), (R)0.5 * (g1.y - g2.y));
+      G[r * SR_LD + q] = g;
+      if (q > r) G[q * SR_LD + r] = cconj(g);
     }
   __syncthreads();
   const int mg = (m + 1) / 2, n4 = (n + 3) / 4;

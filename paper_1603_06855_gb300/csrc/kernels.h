@@ -57,12 +57,22 @@ template <typename R>
 int launch_gemms(int Mrows, int K, int lda, long long ldb, long long ldc, const GemmSeg<R>* seg, int nseg, cudaStream_t s);
 
 // Operator pieces.  Vector blocks are [vec][3][N] complex, vec = k*m + j.
+// A selection of the vectors of a block: entry v of nvec stands for vector list[v] (per = 1) or
+// list[v / per] * per + v % per (whole k-points, per = m), or for v itself without a list.
+struct VecSel {
+  const int* list = nullptr;
+  int per = 1;
+  __device__ __forceinline__ int operator()(int v) const {
+    return !list ? v : (per == 1 ? list[v] : list[v / per] * per + v % per);
+  }
+};
 template <typename R>
 int launch_strain(const typename cplx_t<R>::type* X, int nvec, int m, Geom g, const double* Q,
                   typename cplx_t<R>::type* E, cudaStream_t s, const float4* Kf = nullptr);
+// Stresses of nvec selected vectors (compact in Sig) into their columns of AX.
 template <typename R>
 int launch_epilogue(const typename cplx_t<R>::type* Sig, int nvec, int m, Geom g, const double* Q,
-                    R c0, R c1, typename cplx_t<R>::type* AX, cudaStream_t s, const float4* Kf = nullptr);
+                    R c0, R c1, typename cplx_t<R>::type* AX, cudaStream_t s, const float4* Kf = nullptr, VecSel sel = {});
 // Kf[k N + q] = FP32 wavevector (K_0, K_1, K_2, 0) of plane wave q at the k-th point of Q (nk points);
 // the FP32 kernels above and below read it when given (it is ignored for FP64 data).
 int launch_kvec_table(Geom g, const double* Q, int nk, float4* Kf, cudaStream_t s);
@@ -80,16 +90,29 @@ struct PrecRef {  // reference medium from the mean of chi (device scalar)
   int ref_mode;       // 0: Lame constants linear in chi; 1: compliance linear in chi (the material law)
   double shift_scale; // weight of the mass term rho sigma
 };
+// k-points still iterated, kept on the device and counted on the host: klist the open k-points in
+// order, vlist their unconverged vectors (k m + j), fresh the k-points that the last test locked, count
+// {open, unconverged vectors, fresh}.
+struct OpenSet {
+  int *klist, *vlist, *fresh, *count;
+};
+int launch_open_all(OpenSet o, int nk, cudaStream_t s);  // klist = all
+// Residuals of the nopen k-points of o.klist, then the convergence test: kdone, and the new lists.
 template <typename R>
 int launch_resnorm(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX,
                    const R* lam, int nk, int m, int nb, int n3, double tol, double* rnorm,
-                   int* active, int* kdone, int* unconv, cudaStream_t s, double* best = nullptr,
+                   int* active, int* kdone, OpenSet o, int nopen, cudaStream_t s, double* best = nullptr,
                    int* since = nullptr);
+// W = P(R) on the unconverged vectors of the open k-points; W, A W and Omega W = 0 on their others.
 template <typename R>
 int launch_precond(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX,
-                   const R* lam, const int* active, const int* kdone, int nk, int m, int nb, Geom g,
-                   const double* Q, PrecRef pr, const double* chi_mean, typename cplx_t<R>::type* W, cudaStream_t s,
+                   const R* lam, const int* active, const int* klist, int nopen, int m, int nb, Geom g,
+                   const double* Q, PrecRef pr, const double* chi_mean, typename cplx_t<R>::type* W,
+                   typename cplx_t<R>::type* AW, typename cplx_t<R>::type* OW, cudaStream_t s,
                    const float4* Kf = nullptr);
+// dst[k] = src[k] in FP64 for the nsel k-points of list, `per` values each.
+template <typename R>
+int launch_store(const typename cplx_t<R>::type* src, double2* dst, const int* list, int nsel, long long per, cudaStream_t s);
 template <typename R>
 int launch_init_guess(typename cplx_t<R>::type* X, int nk, int m, Geom g, const double* Q, unsigned long long seed,
                       cudaStream_t s);
@@ -99,21 +122,41 @@ int launch_init_guess(typename cplx_t<R>::type* X, int nk, int m, Geom g, const 
 template <typename R> struct BlockList {
   const typename cplx_t<R>::type* p[3];
 };
+// A batch of small matrices of nel entries as its consumers read it: entry e of problem i is
+// scale * sum_{t < nsplit} p[(i nsplit + t) nel + e], so that the row-split partial sums of a Gram
+// product need no reduction launch of their own.
+template <typename R> struct MatRef {
+  typedef typename cplx_t<R>::type C2;
+  const C2* p = nullptr;
+  long long nel = 0;
+  int nsplit = 1;
+  R scale = 1;
+  __device__ __forceinline__ C2 at(long long i, int e) const {
+    const C2* q = p + i * nsplit * nel + e;
+    C2 s = q[0];
+    for (int t = 1; t < nsplit; ++t) s = cadd(s, q[t * nel]);
+    return cscale(s, scale);
+  }
+};
+// Gram products of nk k-points (of klist, or all); problem i of the result is the i-th of them.  part:
+// workspace of at most max_split partial results per problem; G: the reduced result, where the kernel
+// reduces (FP64 and the CUDA-core FP32 kernel).
 template <typename R>
 int launch_gram(BlockList<R> A, int na, BlockList<R> B, int nb_, int nk, int m, int n3, R scale,
-                typename cplx_t<R>::type* part, typename cplx_t<R>::type* G, cudaStream_t s, int* status = nullptr);
+                typename cplx_t<R>::type* part, typename cplx_t<R>::type* G, MatRef<R>* out, cudaStream_t s,
+                int* status = nullptr, const int* klist = nullptr, int max_split = 8);
 template <typename R> struct UpdateArgs {
   const typename cplx_t<R>::type* in[3][3];  // [triplet][block]
   typename cplx_t<R>::type* out[3];
   int ntrip, nblk;
   int identity_last;   // out = in[last] + sum_{b<last} in[b] C_b
-  const typename cplx_t<R>::type* C;  // per k: rows (nblk or nblk-1)*m, cols mout
-  long long cstride;   // elements per k in C
+  MatRef<R> C;         // per problem: rows (nblk or nblk-1)*m, cols mout
   int cld;             // leading dimension (columns) of C
+  const int* klist = nullptr;  // k-point of problem i (or i itself)
   int m, mout, n3, nk;
   long long in_kstride, out_kstride;  // elements per k (normally m*n3 / mout*n3)
   // optional second coefficient set over the same inputs: out2[t] = sum_b in[t][b] C2nd_b
-  const typename cplx_t<R>::type* C2nd = nullptr;
+  MatRef<R> C2nd;  // p = nullptr: none
   typename cplx_t<R>::type* out2[3] = {nullptr, nullptr, nullptr};
   int* status = nullptr;  // device status word (tensor-core kernels record a timeout there)
 };
@@ -122,31 +165,28 @@ template <typename R> int launch_update(const UpdateArgs<R>& a, cudaStream_t s);
 // Process-wide switches read by every launch, from any k-group thread.
 extern std::atomic<int> g_tc_tall;
 int launch_gram_tc(const float2* const A[3], int na, const float2* const B[3], int nbk, int nk, int m, int n3,
-                   float scale, float2* part, int max_split, float2* G, int* status, cudaStream_t s);
+                   float scale, float2* part, int max_split, MatRef<float>* out, int* status, const int* klist,
+                   cudaStream_t s);
 int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s);
 
 // Projected problems, one CTA per k: the pencil (GA, GO) of n <= 72 basis columns, unit-diagonal
 // scaling, Cholesky of GO that drops dependent columns (pivots at or below drop_tol), reduction to
-// standard form, cyclic Jacobi; the lowest m eigenvalues and their coefficients (n x m).  Locked
-// k-points (kdone) keep their block.  When cp is given, the conjugate-direction coefficients of the next
+// standard form, cyclic Jacobi; the lowest m eigenvalues (at the k-point of klist, or the problem's own
+// index) and their coefficients (n x m).  When cp is given, the conjugate-direction coefficients of the next
 // iteration come from the same CTA (directions at or below pdir_abs dropped); when flops is given, the
 // algorithmic flops of every problem solved are added to it (device counter).  scratch: global scratch of
 // `stride` bytes per problem, at least small_rr32_scratch(n) / small_rr64_scratch(n), a multiple of 16.
-int launch_small_rr32(const float2* GA, const float2* GO, int n, int m, int nk, float drop_tol, const int* kdone,
+int launch_small_rr32(const MatRef<float>& GA, const MatRef<float>& GO, int n, int m, int nk, float drop_tol, const int* klist,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
                       void* scratch, long long stride, cudaStream_t s);
-int launch_small_rr64(const double2* GA, const double2* GO, int n, int m, int nk, double drop_tol, const int* kdone,
+int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n, int m, int nk, double drop_tol, const int* klist,
                       double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
                       long long stride, cudaStream_t s);
 long long small_rr32_scratch(int n);
 long long small_rr64_scratch(int n);
-// Cholesky-QR transform of the Gram G (m x m per k).  When Gref is given (rows_ref x m per
-// k, scale -1, its last m rows holding -Y^H Omega Y before projection), a column whose
-// Omega-norm^2 after projection is below rel_tol times the one before is dropped.
+// Cholesky-QR transform of the Gram matrices G (m x m).
 template <typename R>
-int launch_small_chol(const typename cplx_t<R>::type* G, int m, int nk, R drop_tol,
-                      const typename cplx_t<R>::type* Gref, int rows_ref, R rel_tol,
-                      typename cplx_t<R>::type* T, cudaStream_t s);
+int launch_small_chol(const MatRef<R>& G, int m, int nk, R drop_tol, typename cplx_t<R>::type* T, cudaStream_t s);
 
 int launch_convert_f2d(const float2* src, double2* dst, long long n, cudaStream_t s);
 

@@ -18,15 +18,15 @@
 // multiplied.
 template <int TILE>
 __global__ __launch_bounds__(256) void k_gram(BlockList<float> A, int na, BlockList<float> B, int nbk, int m, int n3,
-                                              float2* __restrict__ part) {
+                                              const int* __restrict__ klist, float2* __restrict__ part) {
   typedef float2 C2;
   constexpr int GRAM_ROWS = 16;
   __shared__ C2 sA[2][GRAM_ROWS * GRAM_LD];
   __shared__ C2 sB[2][GRAM_ROWS * GRAM_LD];
   const int k = blockIdx.x, split = blockIdx.y;
   const int ca = na * m, cb = nbk * m;
-  const long long kofs = (long long)k * m * n3;
-  const int chunk = (n3 + GRAM_SPLIT - 1) / GRAM_SPLIT;
+  const long long kofs = (long long)(klist ? klist[k] : k) * m * n3;
+  const int chunk = (n3 + (int)gridDim.y - 1) / (int)gridDim.y;
   const int r_begin = split * chunk, r_end = min(n3, r_begin + chunk);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   // each thread stages elements t = threadIdx.x + 256 u of the (rows x cols) tiles
@@ -88,7 +88,7 @@ __global__ __launch_bounds__(256) void k_gram(BlockList<float> A, int na, BlockL
     __syncthreads();
     buf ^= 1;
   }
-  C2* out = part + ((long long)k * GRAM_SPLIT + split) * ca * cb;
+  C2* out = part + ((long long)k * gridDim.y + split) * ca * cb;
 #pragma unroll
   for (int i = 0; i < TILE; ++i)
 #pragma unroll
@@ -125,14 +125,14 @@ int launch_gram_reduce_f(const float2* part, int nsplit, int nel, int nk, float 
 // 48 x 48 columns, 375 rows, 4 k): 174 -> 28 us a launch on average.
 constexpr int GRAM64_ROWS = 16;
 __global__ __launch_bounds__(608) void k_gram64(BlockList<double> A, int na, BlockList<double> B, int nbk, int m, int n3,
-                                                int chunk, double2* __restrict__ part) {
+                                                int chunk, const int* __restrict__ klist, double2* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char gram_smem[];
   const int ca = na * m, cb = nbk * m;
   const int lda = ca | 1, ldb = cb | 1;
   double2* sA = (double2*)gram_smem;       // GRAM64_ROWS x lda
   double2* sB = sA + GRAM64_ROWS * lda;    // GRAM64_ROWS x ldb
   const int split = blockIdx.y, nsplit = gridDim.y, k = blockIdx.z;
-  const long long kofs = (long long)k * m * n3;
+  const long long kofs = (long long)(klist ? klist[k] : k) * m * n3;
   const int r_begin = split * chunk, r_end = min(n3, r_begin + chunk);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const bool mine = e < ca * cb;
@@ -157,15 +157,15 @@ __global__ __launch_bounds__(608) void k_gram64(BlockList<double> A, int na, Blo
 }
 
 static int launch_gram64(const BlockList<double>& A, int na, const BlockList<double>& B, int nbk, int nk, int m, int n3,
-                         double scale, double2* part, double2* G, cudaStream_t s) {
+                         double scale, double2* part, int max_split, double2* G, const int* klist, cudaStream_t s) {
   const int nel = na * m * nbk * m;
   const int nx = cdiv(nel, 608);
   const int threads = cdiv(cdiv(nel, nx), 32) * 32;
   int split = 1;
-  while (split < GRAM_SPLIT && (long long)nx * split * nk < 4 * 152) ++split;
+  while (split < max_split && (long long)nx * split * nk < 4 * 152) ++split;
   const int chunk = cdiv(cdiv(n3, split), GRAM64_ROWS) * GRAM64_ROWS;
   const size_t sm = sizeof(double2) * GRAM64_ROWS * ((size_t)((na * m) | 1) + ((nbk * m) | 1));
-  k_gram64<<<dim3(nx, split, nk), threads, sm, s>>>(A, na, B, nbk, m, n3, chunk, part);
+  k_gram64<<<dim3(nx, split, nk), threads, sm, s>>>(A, na, B, nbk, m, n3, chunk, klist, part);
   PC_LAUNCH_CHECK();
   dim3 g2(cdiv(nel, 256), nk);
   k_gram_reduce<double><<<g2, 256, 0, s>>>(part, split, nel, scale, G);
@@ -175,25 +175,31 @@ static int launch_gram64(const BlockList<double>& A, int na, const BlockList<dou
 
 template <typename R>
 int launch_gram(BlockList<R> A, int na, BlockList<R> B, int nbk, int nk, int m, int n3, R scale,
-                typename cplx_t<R>::type* part, typename cplx_t<R>::type* G, cudaStream_t s, int* status) {
-  if (na * m > 72 || nbk * m > 72 || na * m > 80) return PC_EINVAL;
+                typename cplx_t<R>::type* part, typename cplx_t<R>::type* G, MatRef<R>* out, cudaStream_t s, int* status,
+                const int* klist, int max_split) {
+  if (na * m > 72 || nbk * m > 72 || max_split < 1 || max_split > GRAM_SPLIT) return PC_EINVAL;
+  const int nel = na * m * nbk * m;
   if constexpr (std::is_same<R, float>::value) {
-    if (g_tc_tall && status) return launch_gram_tc(A.p, na, B.p, nbk, nk, m, n3, scale, part, GRAM_SPLIT, G, status, s);
+    if (g_tc_tall && status)
+      return launch_gram_tc(A.p, na, B.p, nbk, nk, m, n3, scale, part, max_split, out, status, klist, s);
   }
+  *out = MatRef<R>();
+  out->p = G;
+  out->nel = nel;
   if constexpr (std::is_same<R, double>::value) {
-    return launch_gram64(A, na, B, nbk, nk, m, n3, scale, part, G, s);
+    return launch_gram64(A, na, B, nbk, nk, m, n3, scale, part, max_split, G, klist, s);
   } else {
-    dim3 grid(nk, GRAM_SPLIT);
+    dim3 grid(nk, max_split);
     // 16 x 16 threads, TILE x TILE outputs each: 2 x 2 covers up to 32 columns per side
     const bool small = na * m <= 32 && nbk * m <= 32;
-    if (small) k_gram<2><<<grid, 256, 0, s>>>(A, na, B, nbk, m, n3, part);
-    else k_gram<5><<<grid, 256, 0, s>>>(A, na, B, nbk, m, n3, part);
+    if (small) k_gram<2><<<grid, 256, 0, s>>>(A, na, B, nbk, m, n3, klist, part);
+    else k_gram<5><<<grid, 256, 0, s>>>(A, na, B, nbk, m, n3, klist, part);
     PC_LAUNCH_CHECK();
-    return launch_gram_reduce_f(part, GRAM_SPLIT, na * m * nbk * m, nk, scale, G, s);
+    return launch_gram_reduce_f(part, max_split, nel, nk, scale, G, s);
   }
 }
-template int launch_gram<double>(BlockList<double>, int, BlockList<double>, int, int, int, int, double, double2*, double2*, cudaStream_t, int*);
-template int launch_gram<float>(BlockList<float>, int, BlockList<float>, int, int, int, int, float, float2*, float2*, cudaStream_t, int*);
+template int launch_gram<double>(BlockList<double>, int, BlockList<double>, int, int, int, int, double, double2*, double2*, MatRef<double>*, cudaStream_t, int*, const int*, int);
+template int launch_gram<float>(BlockList<float>, int, BlockList<float>, int, int, int, int, float, float2*, float2*, MatRef<float>*, cudaStream_t, int*, const int*, int);
 
 // ---------------------------------------------------------------------------
 // out[t][k][j][r] = (identity_last ? in[t][last][k][j][r] : 0) + sum_b sum_i in[t][b][k][i][r] C[k][b*m+i][j]
@@ -203,13 +209,12 @@ template <int MOUT>
 __global__ __launch_bounds__(128) void k_update(UpdateArgs<float> a) {
   typedef float2 C2;
   __shared__ C2 sC[72 * 24];
-  const int k = blockIdx.y, t = blockIdx.z;
+  const int k = a.klist ? a.klist[blockIdx.y] : (int)blockIdx.y, t = blockIdx.z;
   const int nsum = a.identity_last ? a.nblk - 1 : a.nblk;
   const int rows = nsum * a.m;
-  const C2* Ck = a.C + (long long)k * a.cstride;
   for (int e = threadIdx.x; e < rows * a.mout; e += blockDim.x) {
     int i = e / a.mout, j = e % a.mout;
-    sC[e] = Ck[(long long)i * a.cld + j];
+    sC[e] = a.C.at(blockIdx.y, i * a.cld + j);
   }
   __syncthreads();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -247,13 +252,12 @@ __global__ __launch_bounds__(128) void k_update(UpdateArgs<float> a) {
 template <int JT>
 __global__ __launch_bounds__(256) void k_update64(UpdateArgs<double> a) {
   __shared__ double2 sC[72 * 24];
-  const int k = blockIdx.y, t = blockIdx.z;
+  const int k = a.klist ? a.klist[blockIdx.y] : (int)blockIdx.y, t = blockIdx.z;
   const int nsum = a.identity_last ? a.nblk - 1 : a.nblk;
   const int rows = nsum * a.m;
-  const double2* Ck = a.C + (long long)k * a.cstride;
   for (int e = threadIdx.x; e < rows * 24; e += blockDim.x) {
     const int i = e / 24, j = e % 24;
-    sC[e] = j < a.mout ? Ck[(long long)i * a.cld + j] : make_double2(0.0, 0.0);
+    sC[e] = j < a.mout ? a.C.at(blockIdx.y, i * a.cld + j) : make_double2(0.0, 0.0);
   }
   __syncthreads();
   const int r = blockIdx.x * 32 + (threadIdx.x & 31);
@@ -312,11 +316,11 @@ template <typename R> int launch_update(const UpdateArgs<R>& a, cudaStream_t s) 
     if (g_tc_tall && a.status) return launch_update_tc(a, a.status, s);
   }
   int rc = launch_update_cuda<R>(a, s);
-  if (rc || !a.C2nd) return rc;
+  if (rc || !a.C2nd.p) return rc;
   UpdateArgs<R> b = a;
   b.C = a.C2nd;
   for (int t = 0; t < 3; ++t) b.out[t] = a.out2[t];
-  b.C2nd = nullptr;
+  b.C2nd.p = nullptr;
   return launch_update_cuda<R>(b, s);
 }
 template int launch_update<double>(const UpdateArgs<double>&, cudaStream_t);
@@ -326,9 +330,7 @@ template int launch_update<float>(const UpdateArgs<float>&, cudaStream_t);
 // Cholesky-QR transform: T = D Li^H with zero columns for dropped coordinates.
 // One warp factors (warp_chol_inverse); the others only load, scale and store.
 template <typename R>
-__global__ __launch_bounds__(128) void k_small_chol(const typename cplx_t<R>::type* __restrict__ G, int m, R drop_tol,
-                                                    const typename cplx_t<R>::type* __restrict__ Gref, int rows_ref,
-                                                    R rel_tol, typename cplx_t<R>::type* __restrict__ T) {
+__global__ __launch_bounds__(128) void k_small_chol(MatRef<R> G, int m, R drop_tol, typename cplx_t<R>::type* __restrict__ T) {
   typedef typename cplx_t<R>::type C2;
   __shared__ C2 B[24 * 25];
   __shared__ C2 X[24 * 25];
@@ -336,21 +338,17 @@ __global__ __launch_bounds__(128) void k_small_chol(const typename cplx_t<R>::ty
   __shared__ int drop[24];
   const int ld = m | 1;
   const int k = blockIdx.x;
-  const C2* g = G + (long long)k * m * m;
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) X[(t / m) * ld + t % m] = G.at(k, t);
+  __syncthreads();
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    R d = g[i * m + i].x;
-    bool keep = (d > (R)0 && d == d);
-    if (keep && Gref) {
-      R before = -Gref[(long long)k * rows_ref * m + (long long)(rows_ref - m + i) * m + i].x;
-      keep = d > rel_tol * before;
-    }
-    D[i] = keep ? (R)1 / sqrt(d) : (R)0;
+    const R d = X[i * ld + i].x;
+    D[i] = (d > (R)0 && d == d) ? (R)1 / sqrt(d) : (R)0;
     drop[i] = 0;
   }
   __syncthreads();
   for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
     int i = t / m, c = t % m;
-    C2 b1 = g[i * m + c], b2 = g[c * m + i];
+    const C2 b1 = X[i * ld + c], b2 = X[c * ld + i];
     R s = D[i] * D[c] * (R)0.5;
     B[i * ld + c] = mk<R>((b1.x + b2.x) * s, (b1.y - b2.y) * s);
   }
@@ -366,13 +364,11 @@ __global__ __launch_bounds__(128) void k_small_chol(const typename cplx_t<R>::ty
   }
 }
 template <typename R>
-int launch_small_chol(const typename cplx_t<R>::type* G, int m, int nk, R drop_tol,
-                      const typename cplx_t<R>::type* Gref, int rows_ref, R rel_tol, typename cplx_t<R>::type* T,
-                      cudaStream_t s) {
+int launch_small_chol(const MatRef<R>& G, int m, int nk, R drop_tol, typename cplx_t<R>::type* T, cudaStream_t s) {
   if (m > 24) return PC_EINVAL;
-  k_small_chol<R><<<nk, 128, 0, s>>>(G, m, drop_tol, Gref, rows_ref, rel_tol, T);
+  k_small_chol<R><<<nk, 128, 0, s>>>(G, m, drop_tol, T);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
-template int launch_small_chol<double>(const double2*, int, int, double, const double2*, int, double, double2*, cudaStream_t);
-template int launch_small_chol<float>(const float2*, int, int, float, const float2*, int, float, float2*, cudaStream_t);
+template int launch_small_chol<double>(const MatRef<double>&, int, int, double, double2*, cudaStream_t);
+template int launch_small_chol<float>(const MatRef<float>&, int, int, float, float2*, cudaStream_t);

@@ -42,8 +42,8 @@ constexpr int SR_THREADS = 1024;
 constexpr int SR_PB = 8;  // panel / row-block width of the reductions
 }  // namespace
 
-__global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restrict__ GA, const float2* __restrict__ GO,
-                                                         int n, int m, float drop_tol, const int* __restrict__ kdone,
+__global__ __launch_bounds__(SR_THREADS) void k_small_rr32(MatRef<float> GA, MatRef<float> GO, int n, int m,
+                                                          float drop_tol, const int* __restrict__ klist,
                                                          float* __restrict__ lam_out, float2* __restrict__ coef,
                                                          float2* __restrict__ cpo, float pdir_abs, int* status,
                                                          double* flops, unsigned char* scratch, long long stride) {
@@ -62,35 +62,37 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
   int* misc = low + SR_NMAX;           // [0] kept count, [2] floor bits, [3] sweeps
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-  const int k = blockIdx.x;
-  const float2* ga = GA + (long long)k * n * n;
-  const float2* go = GO + (long long)k * n * n;
+  const int k = blockIdx.x;                        // problem
+  const int kp = klist ? klist[k] : k;             // its k-point
   Plane<float>* logk = (Plane<float>*)(scratch + k * stride);  // rotations of this problem, np planes per round
   float2* ck = coef + (long long)k * n * m;
   float2* cpk = cpo ? cpo + (long long)k * n * m : nullptr;  // conjugate-direction coefficients (or none)
-  if (kdone && kdone[k]) {  // locked k-point: keep its block, leave lambda untouched, no conjugate block
-    for (int t = tid; t < n * m; t += blockDim.x) {
-      const int i = t / m, j = t % m;
-      ck[t] = make_float2(i == j ? 1.f : 0.f, 0.f);
-      if (cpk) cpk[t] = make_float2(0.f, 0.f);
-    }
-    return;
-  }
   // 1. scaling, symmetrised copies, identity right-hand side of L^-1 (in Vt)
+  for (int i = warp; i < n; i += 32)
+    for (int c = lane; c < n; c += 32) {
+      B1[i * SR_LD + c] = GA.at(k, i * n + c);
+      B0[i * SR_LD + c] = GO.at(k, i * n + c);
+      Vt[i * SR_LD + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
+    }
+  __syncthreads();
   for (int i = tid; i < n; i += blockDim.x) {
-    const float d = go[i * n + i].x;
+    const float d = B0[i * SR_LD + i].x;
     D[i] = (d > 0.f && d == d) ? 1.f / sqrtf(d) : 0.f;
     drop[i] = 0;
   }
   __syncthreads();
   for (int i = warp; i < n; i += 32)
-    for (int c = lane; c < n; c += 32) {
-      const float2 a1 = ga[i * n + c], a2 = ga[c * n + i];
-      const float2 b1 = go[i * n + c], b2 = go[c * n + i];
+    for (int c = i + lane; c < n; c += 32) {  // this thread alone reads and writes (i, c) and (c, i)
+      const float2 a1 = B1[i * SR_LD + c], a2 = B1[c * SR_LD + i];
+      const float2 b1 = B0[i * SR_LD + c], b2 = B0[c * SR_LD + i];
       const float s = D[i] * D[c] * 0.5f;
-      B1[i * SR_LD + c] = make_float2((a1.x + a2.x) * s, (a1.y - a2.y) * s);
-      B0[i * SR_LD + c] = make_float2((b1.x + b2.x) * s, (b1.y - b2.y) * s);
-      Vt[i * SR_LD + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
+      const float2 a = make_float2((a1.x + a2.x) * s, (a1.y - a2.y) * s), b = make_float2((b1.x + b2.x) * s, (b1.y - b2.y) * s);
+      B1[i * SR_LD + c] = a;
+      B0[i * SR_LD + c] = b;
+      if (c > i) {
+        B1[c * SR_LD + i] = cconj(a);
+        B0[c * SR_LD + i] = cconj(b);
+      }
     }
   __syncthreads();
   // 2. Cholesky of B0 (lower)
@@ -116,7 +118,7 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
       const int i = t / m, j = t % m;
       ck[t] = make_float2(i == j ? 1.f : 0.f, 0.f);
     }
-    for (int j = tid; j < m; j += blockDim.x) lam_out[(long long)k * m + j] = ga[j * n + j].x / go[j * n + j].x;
+    for (int j = tid; j < m; j += blockDim.x) lam_out[(long long)kp * m + j] = GA.at(k, j * n + j).x / GO.at(k, j * n + j).x;
     if (tid == 0) set_status(status, PC_ENOCONV);
     if (cpk) {
       for (int t = tid; t < n * m; t += blockDim.x) {
@@ -124,7 +126,7 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
         B1[t] = make_float2(i == j ? 1.f : 0.f, 0.f);
       }
       __syncthreads();
-      pdir<float, SR_THREADS>(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * (m | 1), ev, drop, cpk);
+      pdir<float, SR_THREADS>(GO, k, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * (m | 1), ev, drop, cpk);
     }
     return;
   }
@@ -182,10 +184,10 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
       }
     }
   }
-  for (int j = tid; j < m; j += blockDim.x) lam_out[(long long)k * m + j] = ev[perm[j]];
+  for (int j = tid; j < m; j += blockDim.x) lam_out[(long long)kp * m + j] = ev[perm[j]];
   if (cpk) {
     __syncthreads();
-    pdir<float, SR_THREADS>(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * (m | 1), ev, drop, cpk);
+    pdir<float, SR_THREADS>(GO, k, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, Cm, Cm + m * (m | 1), ev, drop, cpk);
   }
   if (flops && tid == 0) {
     // algorithmic work: Cholesky n^3/6, L^-1 GA n^3/2, L^-1 T^H n^3/2 and L^-1 n^3/6 complex
@@ -199,7 +201,7 @@ __global__ __launch_bounds__(SR_THREADS) void k_small_rr32(const float2* __restr
 // Planes (16 bytes) of the rotations of the most sweeps and of the round after them.
 long long small_rr32_scratch(int n) { return 16LL * ((long long)SR_MAX_SWEEPS * n + 1) * ((n + 1) / 2); }
 
-int launch_small_rr32(const float2* GA, const float2* GO, int n, int m, int nk, float drop_tol, const int* kdone,
+int launch_small_rr32(const MatRef<float>& GA, const MatRef<float>& GO, int n, int m, int nk, float drop_tol, const int* klist,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
                       void* scratch, long long stride, cudaStream_t s) {
   if (n > SR_NMAX || m > n || m > 24 || n < 1 || stride < small_rr32_scratch(n) || stride % 16) return PC_EINVAL;
@@ -208,7 +210,7 @@ int launch_small_rr32(const float2* GA, const float2* GO, int n, int m, int nk, 
   static const cudaError_t attr =  // once, thread-safe (k groups launch from several host threads)
       cudaFuncSetAttribute(k_small_rr32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   (void)attr;
-  k_small_rr32<<<nk, SR_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, kdone, lam_out, coef, cp, pdir_abs, status, flops,
+  k_small_rr32<<<nk, SR_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status, flops,
                                              (unsigned char*)scratch, stride);
   PC_LAUNCH_CHECK();
   return PC_OK;

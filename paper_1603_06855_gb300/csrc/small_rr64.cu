@@ -77,8 +77,8 @@ __device__ __forceinline__ void tiles(int n, const double2* A, int lda, bool her
 
 }  // namespace
 
-__global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(const double2* __restrict__ GA, const double2* __restrict__ GO,
-                                                            int n, int m, double drop_tol, const int* __restrict__ kdone,
+__global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA, MatRef<double> GO, int n, int m,
+                                                          double drop_tol, const int* __restrict__ klist,
                                                             double* __restrict__ lam_out, double2* __restrict__ coef,
                                                             double2* __restrict__ cpo, double pdir_abs, int* status,
                                                             unsigned char* scratch, long long stride) {
@@ -96,37 +96,39 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(const double2* __r
   int* low = perm + SR_NMAX;                 // SR_NMAX
   int* misc = low + SR_NMAX;                 // 8
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int k = blockIdx.x;
-  const double2* ga = GA + (long long)k * n * n;
-  const double2* go = GO + (long long)k * n * n;
+  const int k = blockIdx.x;                        // problem
+  const int kp = klist ? klist[k] : k;             // its k-point
   double2* Lg = (double2*)(scratch + k * stride);  // n x n: L
   double2* Qg = Lg + n * n;                        // n x n: Q
   double2* Eg = Qg + n * n;                        // n x n: E, then I - E/2 + 3/8 E^2
   void* logk = Eg + n * n;                         // rotations
   double2* ck = coef + (long long)k * n * m;
   double2* cpk = cpo ? cpo + (long long)k * n * m : nullptr;
-  if (kdone && kdone[k]) {  // locked k-point: keep its block, leave lambda untouched, no conjugate block
-    for (int t = tid; t < n * m; t += S6_THREADS) {
-      const int i = t / m, j = t % m;
-      ck[t] = make_double2(i == j ? 1.0 : 0.0, 0.0);
-      if (cpk) cpk[t] = make_double2(0.0, 0.0);
-    }
-    return;
-  }
   // scaling, symmetrised copies
+  for (int i = warp; i < n; i += W)
+    for (int c = lane; c < n; c += 32) {
+      B1[i * SR_LD + c] = GA.at(k, i * n + c);
+      B0[i * SR_LD + c] = GO.at(k, i * n + c);
+    }
+  __syncthreads();
   for (int i = tid; i < n; i += S6_THREADS) {
-    const double d = go[i * n + i].x;
+    const double d = B0[i * SR_LD + i].x;
     D[i] = (d > 0.0 && d == d) ? 1.0 / sqrt(d) : 0.0;
     drop[i] = 0;
   }
   __syncthreads();
   for (int i = warp; i < n; i += W)
-    for (int c = lane; c < n; c += 32) {
-      const double2 a1 = ga[i * n + c], a2 = ga[c * n + i];
-      const double2 b1 = go[i * n + c], b2 = go[c * n + i];
+    for (int c = i + lane; c < n; c += 32) {  // this thread alone reads and writes (i, c) and (c, i)
+      const double2 a1 = B1[i * SR_LD + c], a2 = B1[c * SR_LD + i];
+      const double2 b1 = B0[i * SR_LD + c], b2 = B0[c * SR_LD + i];
       const double s = D[i] * D[c] * 0.5;
-      B1[i * SR_LD + c] = make_double2((a1.x + a2.x) * s, (a1.y - a2.y) * s);
-      B0[i * SR_LD + c] = make_double2((b1.x + b2.x) * s, (b1.y - b2.y) * s);
+      const double2 a = make_double2((a1.x + a2.x) * s, (a1.y - a2.y) * s), b = make_double2((b1.x + b2.x) * s, (b1.y - b2.y) * s);
+      B1[i * SR_LD + c] = a;
+      B0[i * SR_LD + c] = b;
+      if (c > i) {
+        B1[c * SR_LD + i] = cconj(a);
+        B0[c * SR_LD + i] = cconj(b);
+      }
     }
   __syncthreads();
   // L, T = L^-1 GA, C = L^-1 T^H (upper triangle), all in place
@@ -161,7 +163,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(const double2* __r
       ck[t] = v;
       B1[t] = v;
     }
-    for (int j = tid; j < m; j += S6_THREADS) lam_out[(long long)k * m + j] = ga[j * n + j].x / go[j * n + j].x;
+    for (int j = tid; j < m; j += S6_THREADS) lam_out[(long long)kp * m + j] = GA.at(k, j * n + j).x / GO.at(k, j * n + j).x;
     if (tid == 0) set_status(status, PC_ENOCONV);
   } else {
     const int npad = nk_ + (nk_ & 1), np = npad / 2;
@@ -245,7 +247,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(const double2* __r
     __syncthreads();
     const int sw = jacobi_sweeps<double, S6_THREADS>(B1, B0, pl, (Plane<double>*)logk, nk_, m,
                                                      2.220446049250313e-16 * amax, true, ev, perm, low, misc);
-    for (int j = tid; j < m; j += S6_THREADS) lam_out[(long long)k * m + j] = ev[perm[j]];
+    for (int j = tid; j < m; j += S6_THREADS) lam_out[(long long)kp * m + j] = ev[perm[j]];
     const int K = sw * (npad - 1);
     Plane<double>*c0 = (Plane<double>*)B1, *c1 = (Plane<double>*)B0;
     const double2* Sf = (K & 1) ? B0 : B1;
@@ -276,7 +278,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(const double2* __r
   }
   if (cpk) {
     __syncthreads();
-    pdir<double, S6_THREADS>(go, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, (double2*)F, (double2*)F + m * (m | 1),
+    pdir<double, S6_THREADS>(GO, k, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, (double2*)F, (double2*)F + m * (m | 1),
                              ev, drop, cpk);
   }
 }
@@ -286,7 +288,7 @@ long long small_rr64_scratch(int n) {
   return 16LL * 3 * n * n + 32LL * ((long long)SR_MAX_SWEEPS * n + 1) * ((n + 1) / 2);
 }
 
-int launch_small_rr64(const double2* GA, const double2* GO, int n, int m, int nk, double drop_tol, const int* kdone,
+int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n, int m, int nk, double drop_tol, const int* klist,
                       double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
                       long long stride, cudaStream_t s) {
   if (n > SR_NMAX || m > n || m > 24 || n < 1 || stride < small_rr64_scratch(n) || stride % 16) return PC_EINVAL;
@@ -295,7 +297,7 @@ int launch_small_rr64(const double2* GA, const double2* GO, int n, int m, int nk
   static const cudaError_t attr =  // once, thread-safe (k groups launch from several host threads)
       cudaFuncSetAttribute(k_small_rr64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   (void)attr;
-  k_small_rr64<<<nk, S6_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, kdone, lam_out, coef, cp, pdir_abs, status,
+  k_small_rr64<<<nk, S6_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
                                           (unsigned char*)scratch, stride);
   PC_LAUNCH_CHECK();
   return PC_OK;

@@ -78,6 +78,7 @@ struct TcGramArgs {
   int na, nbk, m, n3;
   int nsplit, rows_per_split;  // rows_per_split: a multiple of 32
   float2* part;
+  const int* klist;            // k-point of problem i (or i itself)
   int* status;
 };
 
@@ -89,10 +90,10 @@ __global__ __launch_bounds__(G_THREADS, 1) void k_tc_gram(TcGramArgs a) {
   const uint32_t bars = base + 2 * G_STAGE;  // full[s] +8s, empty[s] +16+8s, accumulator +32
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + 2 * G_STAGE + 64);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k = blockIdx.x, split = blockIdx.y;
+  const int k = blockIdx.x, split = blockIdx.y;  // k: problem
   const int ca = a.na * a.m, cb = a.nbk * a.m;
   const int NP = ((2 * cb + 15) / 16) * 16;
-  const long long kofs = (long long)k * a.m * a.n3;
+  const long long kofs = (long long)(a.klist ? a.klist[k] : k) * a.m * a.n3;
   const int r_begin = split * a.rows_per_split;
   const int r_end = min(a.n3, r_begin + a.rows_per_split);
   const int nst = r_end > r_begin ? (r_end - r_begin + 31) / 32 : 0;
@@ -258,8 +259,8 @@ constexpr int U_MAXI = 128 * 16 / U_PRODUCERS;  // staged items per thread and s
 struct TcUpdateArgs {
   const float2* in[3][3];
   float2* out[2][3];           // [coefficient set][triplet]
-  const float2* C[2];
-  long long cstride;
+  MatRef<float> C[2];
+  const int* klist;            // k-point of problem i (or i itself)
   int cld, nblk, identity_last, m, mout, n3;
   long long in_kstride, out_kstride;
   int tiles, tiles_per_cta;
@@ -280,7 +281,7 @@ __global__ __launch_bounds__(U_THREADS, 1) void k_tc_update(TcUpdateArgs a) {
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + U_BOP + 2 * U_STAGE + 128);
   const float2** colp = reinterpret_cast<const float2**>(gbase + U_BOP + 2 * U_STAGE + 256);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int k = blockIdx.x, t = blockIdx.y;
+  const int k = a.klist ? a.klist[blockIdx.x] : (int)blockIdx.x, t = blockIdx.y;
   const int ncols = a.nblk * a.m;           // complex input columns
   const int Kt = 2 * ncols;                 // real K
   const int nat = (Kt + 63) / 64;           // K atoms
@@ -317,7 +318,7 @@ __global__ __launch_bounds__(U_THREADS, 1) void k_tc_update(TcUpdateArgs a) {
       cv[u] = make_float2(0.f, 0.f);
       if (e < ncel) {
         const int h = e / (crows * MOUT), rem = e % (crows * MOUT), i = rem / MOUT, j = rem % MOUT;
-        if (j < a.mout) cv[u] = (h == 0 ? a.C[0] : a.C[1])[(long long)k * a.cstride + (long long)i * a.cld + j];
+        if (j < a.mout) cv[u] = (h == 0 ? a.C[0] : a.C[1]).at(blockIdx.x, i * a.cld + j);
       }
     }
 #pragma unroll
@@ -517,11 +518,9 @@ void set_update_smem() {
 
 }  // namespace
 
-// Split-reduction of the partial Gram matrices (defined with the CUDA-core kernels).
-int launch_gram_reduce_f(const float2* part, int nsplit, int nel, int nk, float scale, float2* G, cudaStream_t s);
-
 int launch_gram_tc(const float2* const A[3], int na, const float2* const B[3], int nbk, int nk, int m, int n3,
-                   float scale, float2* part, int max_split, float2* G, int* status, cudaStream_t s) {
+                   float scale, float2* part, int max_split, MatRef<float>* out, int* status, const int* klist,
+                   cudaStream_t s) {
   if (na * m > 72 || nbk * m > 72 || nk < 1) return PC_EINVAL;
   static const cudaError_t attr =  // once, thread-safe static initialisation
       cudaFuncSetAttribute(k_tc_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM);
@@ -539,14 +538,19 @@ int launch_gram_tc(const float2* const A[3], int na, const float2* const B[3], i
   a.nsplit = ns;
   a.rows_per_split = 32 * per;
   a.part = part;
+  a.klist = klist;
   a.status = status;
   k_tc_gram<<<dim3(nk, ns), G_THREADS, G_SMEM, s>>>(a);
   PC_LAUNCH_CHECK();
-  return launch_gram_reduce_f(part, ns, na * m * nbk * m, nk, scale, G, s);
+  out->p = part;
+  out->nel = (long long)na * m * nbk * m;
+  out->nsplit = ns;
+  out->scale = scale;
+  return PC_OK;
 }
 
 int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s) {
-  const int nc = u.C2nd ? 2 : 1;
+  const int nc = u.C2nd.p ? 2 : 1;
   if (u.nblk * u.m > 72 || u.mout > 24 || u.mout < 1 || u.ntrip < 1 || u.ntrip > 3) return PC_EINVAL;
   TcUpdateArgs a;
   for (int t = 0; t < 3; ++t) {
@@ -556,7 +560,7 @@ int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s) {
   }
   a.C[0] = u.C;
   a.C[1] = u.C2nd;
-  a.cstride = u.cstride;
+  a.klist = u.klist;
   a.cld = u.cld;
   a.nblk = u.nblk;
   a.identity_last = u.identity_last;
@@ -589,6 +593,8 @@ int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------
 // Self-check of the tensor-core kernels against the CUDA-core kernels on seeded data.
+// Sum of the partial Gram matrices (defined with the CUDA-core kernels).
+int launch_gram_reduce_f(const float2* part, int nsplit, int nel, int nk, float scale, float2* G, cudaStream_t s);
 namespace {
 // A wait that cannot complete: no thread arrives on the barrier, so the bounded wait used by
 // every tensor-core kernel must give up after `limit` polls, record PC_ETIMEOUT and return.
@@ -675,15 +681,16 @@ extern "C" int pc_check_tensor_kernels(int what, int nk, int m, int nblk, int n3
       // G = [in_0 .. in_{nblk-1}]^H [in_3 .. in_{3+nblk-1}], scale 1
       BlockList<float> A = {{in, in + blk, in + 2 * blk}}, B = {{in + 3 * blk, in + 4 * blk, in + 5 * blk}};
       g_tc_tall = 1;
-      rc = launch_gram<float>(A, nblk, B, nblk, nk, m, n3, 1.f, part, out_tc, 0, status);
+      MatRef<float> g;
+      rc = launch_gram<float>(A, nblk, B, nblk, nk, m, n3, 1.f, part, nullptr, &g, 0, status);
+      if (!rc) rc = launch_gram_reduce_f(g.p, g.nsplit, (int)g.nel, nk, g.scale, out_tc, 0);
       g_tc_tall = 0;
-      if (!rc) rc = launch_gram<float>(A, nblk, B, nblk, nk, m, n3, 1.f, part, out_ref, 0, nullptr);
+      if (!rc) rc = launch_gram<float>(A, nblk, B, nblk, nk, m, n3, 1.f, part, out_ref, &g, 0, nullptr);
       cudaDeviceSynchronize();
       if (!rc) d = max_abs_diff(out_tc, out_ref, (long long)nk * nblk * m * nblk * m, &r);
     } else {
       // three triplets, two coefficient sets, last block identity when nblk > 1
-      UpdateArgs<float> u;
-      memset(&u, 0, sizeof(u));
+      UpdateArgs<float> u = {};
       for (int t = 0; t < 3; ++t) {
         for (int b = 0; b < nblk; ++b) u.in[t][b] = in + (3 * t + b) * blk;
         u.out[t] = out_tc + t * blk;
@@ -692,9 +699,9 @@ extern "C" int pc_check_tensor_kernels(int what, int nk, int m, int nblk, int n3
       u.ntrip = 3;
       u.nblk = nblk;
       u.identity_last = nblk > 1 ? 1 : 0;
-      u.C = C;
-      u.C2nd = C + cel;
-      u.cstride = 72 * 72;
+      u.C.p = C;
+      u.C2nd.p = C + cel;
+      u.C.nel = u.C2nd.nel = 72 * 72;
       u.cld = 72;
       u.m = m;
       u.mout = m;
