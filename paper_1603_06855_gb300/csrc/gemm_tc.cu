@@ -23,6 +23,7 @@
 #include <cuda_bf16.h>
 #include "gemm_tc.h"
 #include "tc_ptx.cuh"
+#include "waves.cuh"
 
 namespace {
 using namespace tcx;
@@ -47,6 +48,8 @@ __host__ __device__ constexpr uint32_t idesc_bf16() { return idesc_bf16_n(TC_BN)
 // next launch on the same stream.  The stage ring runs on across tiles, and the accumulator
 // alternates between two 128-column halves of tensor memory, so the epilogue warps drain tile i
 // while the MMAs of tile i + 1 run.
+constexpr int TC_OPS = 5;  // W1, W2, T_rho, T_f1, T_f2
+
 // The GEMMs of one launch: up to three segments, each an operator (A maps) times a range of
 // right-hand-side columns (B maps) into its own output; the tiles of segment g are tile0[g] ..
 // tile0[g] + mtiles * ntiles[g] - 1, M-fastest.
@@ -59,7 +62,7 @@ struct TcSeg {
   int mapped;              // its output columns are mapped through sel
 };
 struct TcGemmParams {
-  CUtensorMap A[3][3];     // [operator][slice hi, mid, lo]
+  CUtensorMap A[TC_OPS][3];  // [operator][slice hi, mid, lo]
   CUtensorMap B[2][3];     // [right-hand-side set][slice]
   TcSeg seg[3];
   int nseg, num_kb, m_valid, mtiles, tiles;
@@ -247,32 +250,31 @@ __global__ __launch_bounds__(192, 1) void k_tc_gemm(const __grid_constant__ TcGe
 
 // ---------------------------------------------------------------------------
 // Operand preparation.
-// Real embedding of a complex N x N operator (SI, times scale) into [Mp][Kp] hi / mid / lo.
-__global__ void k_tc_embed(const double2* __restrict__ W, int N, double scale, int Mp, int Kp,
-                           __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ mid,
-                           __nv_bfloat16* __restrict__ lo) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)Mp * Kp) return;
+// Real embedding of the complex N x N operators (SI, times scale) into [Mp][Kp] hi / mid / lo slices.
+struct TcEmbed {
+  const double2* op[TC_OPS];
+  double scale[TC_OPS];
+};
+__global__ void k_tc_embed(TcEmbed e, int N, int Mp, int Kp, __nv_bfloat16* __restrict__ out) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, sz = (long long)Mp * Kp;
+  if (t >= sz) return;
   int row = (int)(t / Kp), col = (int)(t % Kp);
   double v = 0.0;
   if (row < 2 * N && col < 2 * N) {
     int p = row >> 1, r = row & 1, q = col >> 1, rp = col & 1;
-    double2 w = W[(long long)p * N + q];
+    double2 w = e.op[blockIdx.y][(long long)p * N + q];
     double x = (r == rp) ? w.x : (r == 0 ? -w.y : w.y);
-    v = x * scale;
+    v = x * e.scale[blockIdx.y];
   }
   __nv_bfloat16 h = __double2bfloat16(v);
   double r1 = v - (double)__bfloat162float(h);
   __nv_bfloat16 mm = __double2bfloat16(r1);
   double r2 = r1 - (double)__bfloat162float(mm);
-  hi[t] = h;
-  mid[t] = mm;
-  lo[t] = __double2bfloat16(r2);
+  __nv_bfloat16* o = out + 3 * blockIdx.y * sz + t;
+  o[0] = h;
+  o[sz] = mm;
+  o[2 * sz] = __double2bfloat16(r2);
 }
-
-#define RS2 0.70710678118654752440f
-#define RS3 0.57735026918962576451f
-#define RS6 0.40824829046386301637f
 
 // Strain stacks of X (six per vector) and the three displacement components, written as
 // split bf16 K-major columns: E col = s * nvec + vec, X col = vec * 3 + c; K index 2q + {re, im}.
@@ -301,31 +303,34 @@ __global__ void k_tc_split_strain(const float2* __restrict__ X, int nvec, int m,
     const int src = sel(vec);
     const float2* x = X + (long long)src * 3 * N;
     u0 = x[q]; u1 = x[N + q]; u2 = x[2 * N + q];
-    const int k = src / m;
-    if (Kf) {  // the k-set's FP32 wavevectors
-      const float4 kk = Kf[(long long)k * N + q];
-      k0 = kk.x; k1 = kk.y; k2 = kk.z;
-    } else {
-      int M2 = 2 * g.M + 1;
-      double a0 = Q[3 * k] + (double)(q / (M2 * M2) - g.M);
-      double a1 = Q[3 * k + 1] + (double)((q / M2) % M2 - g.M);
-      double a2 = Q[3 * k + 2] + (double)(q % M2 - g.M);
-      k0 = (float)(g.T[0] * a0 + g.T[1] * a1 + g.T[2] * a2);
-      k1 = (float)(g.T[3] * a0 + g.T[4] * a1 + g.T[5] * a2);
-      k2 = (float)(g.T[6] * a0 + g.T[7] * a1 + g.T[8] * a2);
-    }
+    kvec_r<float>(g, Q, Kf, src / m, q, k0, k1, k2);
   }
   float2 e[6];
-  e[0] = make_float2((k0 * u0.x + k1 * u1.x + k2 * u2.x) * RS3, (k0 * u0.y + k1 * u1.y + k2 * u2.y) * RS3);
-  e[1] = make_float2((k0 * u0.x - k1 * u1.x) * RS2, (k0 * u0.y - k1 * u1.y) * RS2);
-  e[2] = make_float2((k0 * u0.x + k1 * u1.x - 2.f * k2 * u2.x) * RS6, (k0 * u0.y + k1 * u1.y - 2.f * k2 * u2.y) * RS6);
-  e[3] = make_float2((k1 * u2.x + k2 * u1.x) * RS2, (k1 * u2.y + k2 * u1.y) * RS2);
-  e[4] = make_float2((k0 * u2.x + k2 * u0.x) * RS2, (k0 * u2.y + k2 * u0.y) * RS2);
-  e[5] = make_float2((k0 * u1.x + k1 * u0.x) * RS2, (k0 * u1.y + k1 * u0.y) * RS2);
+  strain6<float>(k0, k1, k2, u0, u1, u2, e);
   // (re, im) slices side by side: one 4-byte store per slice (Kp and the slice strides are even)
   for (int s = 0; s < 6; ++s) split3_store2(e[s], E + ((long long)s * nvec + vec) * Kp + 2 * q, es);
   const float2 uu[3] = {u0, u1, u2};
   for (int c = 0; c < 3; ++c) split3_store2(uu[c], Xs + ((long long)vec * 3 + c) * Kp + 2 * q, xs);
+}
+
+// First half of the preconditioner on the vectors of vlist (as k_prec_in, the strain stacks as split columns).
+__global__ void k_tc_prec_in(const float2* __restrict__ AX, const float2* __restrict__ OX, const float* __restrict__ lam,
+                             const int* __restrict__ vlist, int nvec, int m, int nb, Geom g, const double* __restrict__ Q,
+                             const float4* __restrict__ Kf, const double* __restrict__ ref, float2* __restrict__ W, int Kp,
+                             __nv_bfloat16* __restrict__ E, long long es) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int Kh = Kp / 2;
+  if (t >= (long long)nvec * Kh) return;
+  const int v = (int)(t / Kh), q = (int)(t % Kh);
+  float2 u[3], e[6];
+  if (q < g.N) {
+    const int vec = vlist[v], k = vec / m;
+    prec_residual<float>(PrecTerm<float>(ref, lam + k * m, nb), AX, OX, W, lam[vec], vec, g, Q, Kf, k, q, u, e);
+  } else {
+#pragma unroll
+    for (int s = 0; s < 6; ++s) e[s] = make_float2(0.f, 0.f);
+  }
+  for (int s = 0; s < 6; ++s) split3_store2(e[s], E + ((long long)s * nvec + v) * Kp + 2 * q, es);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -363,12 +368,10 @@ bool make_map(CUtensorMap* m, void* ptr, long long rows, int Kp, int box_rows) {
 
 struct TcPlan {
   int N, nvec_max, Mp, Kp;
-  __nv_bfloat16* Ahi[3];  // W1, W2, T_rho (embedded, scaled)
-  __nv_bfloat16* Amid[3];
-  __nv_bfloat16* Alo[3];
+  __nv_bfloat16* ops;     // [operator][slice hi, mid, lo] of W1, W2, T_rho, T_f1, T_f2 (embedded, scaled), Mp x Kp each
   __nv_bfloat16 *E, *X;   // three slices each: slice t at + t * (rows * Kp)
   float2* S;              // FP32 stress stacks [6][nvec][N]
-  CUtensorMap mA_hi[3], mA_mid[3], mA_lo[3], mE[3], mX[3];
+  CUtensorMap mA[TC_OPS][3], mE[3], mX[3];
   int* status;
   int* tile_ctr;          // tile counter of k_tc_gemm and its finished-CTA count (zero between launches)
   bool ok;
@@ -385,12 +388,7 @@ TcPlan* tc_plan_create(int N, int nvec, int* status) {
   p->ok = false;
   p->owns_ops = true;
   size_t asz = (size_t)p->Mp * p->Kp;
-  bool good = true;
-  for (int i = 0; i < 3; ++i) {
-    good &= cudaMalloc(&p->Ahi[i], asz * 2) == cudaSuccess;
-    good &= cudaMalloc(&p->Amid[i], asz * 2) == cudaSuccess;
-    good &= cudaMalloc(&p->Alo[i], asz * 2) == cudaSuccess;
-  }
+  bool good = cudaMalloc(&p->ops, 3 * TC_OPS * asz * 2) == cudaSuccess;
   size_t esz = (size_t)6 * nvec * p->Kp, xsz = (size_t)3 * nvec * p->Kp;
   good &= cudaMalloc(&p->E, 3 * esz * 2) == cudaSuccess;
   good &= cudaMalloc(&p->X, 3 * xsz * 2) == cudaSuccess;
@@ -402,11 +400,7 @@ TcPlan* tc_plan_create(int N, int nvec, int* status) {
     return nullptr;
   }
   good = true;
-  for (int i = 0; i < 3; ++i) {
-    good &= make_map(&p->mA_hi[i], p->Ahi[i], p->Mp, p->Kp, TC_BM);
-    good &= make_map(&p->mA_mid[i], p->Amid[i], p->Mp, p->Kp, TC_BM);
-    good &= make_map(&p->mA_lo[i], p->Alo[i], p->Mp, p->Kp, TC_BM);
-  }
+  for (int i = 0; i < 3 * TC_OPS; ++i) good &= make_map(&p->mA[i / 3][i % 3], p->ops + i * asz, p->Mp, p->Kp, TC_BM);
   for (int t = 0; t < 3; ++t) {
     good &= make_map(&p->mE[t], p->E + t * esz, (long long)6 * nvec, p->Kp, TC_BN);
     good &= make_map(&p->mX[t], p->X + t * xsz, (long long)3 * nvec, p->Kp, TC_BN);
@@ -421,11 +415,7 @@ TcPlan* tc_plan_create(int N, int nvec, int* status) {
 
 void tc_plan_destroy(TcPlan* p) {
   if (!p) return;
-  for (int i = 0; i < 3 && p->owns_ops; ++i) {
-    if (p->Ahi[i]) cudaFree(p->Ahi[i]);
-    if (p->Amid[i]) cudaFree(p->Amid[i]);
-    if (p->Alo[i]) cudaFree(p->Alo[i]);
-  }
+  if (p->ops && p->owns_ops) cudaFree(p->ops);
   if (p->E) cudaFree(p->E);
   if (p->X) cudaFree(p->X);
   if (p->S) cudaFree(p->S);
@@ -445,14 +435,8 @@ TcPlan* tc_plan_create_sharing(const TcPlan* ops, int nvec, int* status) {
   p->status = status;
   p->ok = false;
   p->owns_ops = false;
-  for (int i = 0; i < 3; ++i) {
-    p->Ahi[i] = ops->Ahi[i];
-    p->Amid[i] = ops->Amid[i];
-    p->Alo[i] = ops->Alo[i];
-    p->mA_hi[i] = ops->mA_hi[i];
-    p->mA_mid[i] = ops->mA_mid[i];
-    p->mA_lo[i] = ops->mA_lo[i];
-  }
+  p->ops = ops->ops;
+  std::copy(&ops->mA[0][0], &ops->mA[0][0] + 3 * TC_OPS, &p->mA[0][0]);
   size_t esz = (size_t)6 * nvec * p->Kp, xsz = (size_t)3 * nvec * p->Kp;
   bool good = cudaMalloc(&p->E, 3 * esz * 2) == cudaSuccess;
   good &= cudaMalloc(&p->X, 3 * xsz * 2) == cudaSuccess;
@@ -475,12 +459,9 @@ TcPlan* tc_plan_create_sharing(const TcPlan* ops, int nvec, int* status) {
 int tc_prepare_operators(TcPlan* p, const double2* W, const double2* T, double w_scale, double t_scale, cudaStream_t s) {
   if (!p) return PC_OK;
   const long long NN = (long long)p->N * p->N, n = (long long)p->Mp * p->Kp;
-  const double2* src[3] = {W, W + NN, T};
-  const double sc[3] = {w_scale, w_scale, t_scale};
-  for (int i = 0; i < 3; ++i) {
-    k_tc_embed<<<cdiv(n, 256), 256, 0, s>>>(src[i], p->N, sc[i], p->Mp, p->Kp, p->Ahi[i], p->Amid[i], p->Alo[i]);
-    PC_LAUNCH_CHECK();
-  }
+  const TcEmbed e = {{W, W + NN, T, T + NN, T + 2 * NN}, {w_scale, w_scale, t_scale, 1.0 / w_scale, 1.0 / w_scale}};
+  k_tc_embed<<<dim3(cdiv(n, 256), TC_OPS), 256, 0, s>>>(e, p->N, p->Mp, p->Kp, p->ops);
+  PC_LAUNCH_CHECK();
   return PC_OK;
 }
 
@@ -501,11 +482,7 @@ static int launch_tc_gemm(TcPlan* p, const TcSegSpec* sp, int nseg, cudaStream_t
   }();
   if (nseg < 1 || nseg > 3) return PC_EINVAL;
   TcGemmParams P;
-  for (int w = 0; w < 3; ++w) {
-    P.A[w][0] = p->mA_hi[w];
-    P.A[w][1] = p->mA_mid[w];
-    P.A[w][2] = p->mA_lo[w];
-  }
+  std::copy(&p->mA[0][0], &p->mA[0][0] + 3 * TC_OPS, &P.A[0][0]);
   for (int t = 0; t < 3; ++t) {
     P.B[0][t] = p->mE[t];
     P.B[1][t] = p->mX[t];
@@ -548,4 +525,15 @@ int tc_apply(TcPlan* p, const float2* X, float2* AX, float2* OX, int nvec, int m
   int rc = launch_tc_gemm(p, seg, 3, s);
   if (rc) return rc;
   return launch_epilogue<float>(p->S, nvec, m, g, Q, 1.0f, 1.0f, AX, s, Kf, sel);
+}
+
+int tc_precond(TcPlan* p, const float2* AX, const float2* OX, const float* lam, const int* vlist, int ncol, int m, int nb,
+               Geom g, const double* Q, const double* ref, float2* W, const float2** S, cudaStream_t s, const float4* Kf) {
+  if (!tc_available(p) || ncol < 1 || ncol > p->nvec_max) return PC_EINVAL;
+  const long long n = (long long)ncol * (p->Kp / 2), es = (long long)6 * p->nvec_max * p->Kp;
+  k_tc_prec_in<<<cdiv(n, 256), 256, 0, s>>>(AX, OX, lam, vlist, ncol, m, nb, g, Q, Kf, ref, W, p->Kp, p->E, es);
+  PC_LAUNCH_CHECK();
+  *S = p->S;
+  const TcSegSpec seg[2] = {{3, 0, 0, ncol, (float*)p->S, {}, 0}, {4, 0, ncol, 5 * ncol, (float*)p->S, {}, 0}};
+  return launch_tc_gemm(p, seg, 2, s);
 }

@@ -10,12 +10,16 @@ TcPlan* tc_plan_create(int N, int nvec, int* status);
 TcPlan* tc_plan_create_sharing(const TcPlan* ops, int nvec, int* status);
 void tc_plan_destroy(TcPlan* p);
 bool tc_available(const TcPlan* p);
-// Converts the FP64 operators (W1, W2 in SI; T_rho in SI) into the scaled split-BF16
-// tensor-core operands: W * w_scale and T_rho * t_scale.
+// Converts the FP64 operators (W: W1, W2; T: T_rho, T_f1, T_f2; SI) into the scaled split-BF16
+// tensor-core operands: W * w_scale, T_rho * t_scale, T_f / w_scale.
 int tc_prepare_operators(TcPlan* p, const double2* W, const double2* T, double w_scale, double t_scale, cudaStream_t s);
 // AX, OX for nvec selected FP32 vectors (vector v at k = v / m).
 int tc_apply(TcPlan* p, const float2* X, float2* AX, float2* OX, int nvec, int m, Geom g, const double* Q, cudaStream_t s,
              const float4* Kf = nullptr, VecSel sel = {});
+
+// First half of the preconditioner on the ncol vectors of vlist: Y into W, and *S = T E (stacks [6][ncol][N]).
+int tc_precond(TcPlan* p, const float2* AX, const float2* OX, const float* lam, const int* vlist, int ncol, int m, int nb,
+               Geom g, const double* Q, const double* ref, float2* W, const float2** S, cudaStream_t s, const float4* Kf);
 
 // FP64-accurate operator products by exact 6-bit slicing on the tensor cores (oz_gemm.cu), for
 // the mixed form's final Rayleigh-Ritz step.

@@ -44,19 +44,6 @@ struct Geom {
   int N;
 };
 
-// Complex GEMMs C[col][p] = alpha * sum_q A[p][q] B[col][q] (both operands K-contiguous) of the same
-// shape but for their columns, nseg <= 3 in one launch.
-template <typename R> struct GemmSeg {
-  const typename cplx_t<R>::type* A;
-  const typename cplx_t<R>::type* B;
-  typename cplx_t<R>::type* C;
-  int ncols;
-  R alpha;
-};
-template <typename R>
-int launch_gemms(int Mrows, int K, int lda, long long ldb, long long ldc, const GemmSeg<R>* seg, int nseg, cudaStream_t s);
-
-// Operator pieces.  Vector blocks are [vec][3][N] complex, vec = k*m + j.
 // A selection of the vectors of a block: entry v of nvec stands for vector list[v] (per = 1) or
 // list[v / per] * per + v % per (whole k-points, per = m), or for v itself without a list.
 struct VecSel {
@@ -66,9 +53,27 @@ struct VecSel {
     return !list ? v : (per == 1 ? list[v] : list[v / per] * per + v % per);
   }
 };
+
+// Complex GEMMs C[col][p] = alpha * sum_q A[p][q] B[col][q] (both operands K-contiguous) of the same
+// shape but for their columns, nseg <= 3 in one launch.
+template <typename R> struct GemmSeg {
+  const typename cplx_t<R>::type* A;
+  const typename cplx_t<R>::type* B;
+  typename cplx_t<R>::type* C;
+  int ncols;
+  R alpha;
+  VecSel sel = {};  // selected vectors of three columns each: column j of B and C is that of vector sel(j / 3)
+  __device__ __forceinline__ long long column(long long j) const {
+    return sel.list ? 3LL * sel((int)(j / 3)) + j % 3 : j;
+  }
+};
+template <typename R>
+int launch_gemms(int Mrows, int K, int lda, long long ldb, long long ldc, const GemmSeg<R>* seg, int nseg, cudaStream_t s);
+
+// Operator pieces.  Vector blocks are [vec][3][N] complex, vec = k*m + j.
 template <typename R>
 int launch_strain(const typename cplx_t<R>::type* X, int nvec, int m, Geom g, const double* Q,
-                  typename cplx_t<R>::type* E, cudaStream_t s, const float4* Kf = nullptr);
+                  typename cplx_t<R>::type* E, cudaStream_t s, const float4* Kf = nullptr, VecSel sel = {});
 // Stresses of nvec selected vectors (compact in Sig) into their columns of AX.
 template <typename R>
 int launch_epilogue(const typename cplx_t<R>::type* Sig, int nvec, int m, Geom g, const double* Q,
@@ -77,17 +82,12 @@ int launch_epilogue(const typename cplx_t<R>::type* Sig, int nvec, int m, Geom g
 // the FP32 kernels above and below read it when given (it is ignored for FP64 data).
 int launch_kvec_table(Geom g, const double* Q, int nk, float4* Kf, cudaStream_t s);
 
-struct PrecConsts {
-  double c_mu;    // (2pi)^2 V mu_ref / sA ... multiplied by |K|^2
-  double c_lm;    // (2pi)^2 V (lambda_ref + mu_ref) / sA
-  double c_rho;   // 0.5 * lambda_scale * V rho_ref / sA
-};
 struct PrecRef {  // reference medium from the mean of chi (device scalar)
   double lam0, lam1, mu0, mu1, rho0, rho1;
   double f1_0, f1_1, f2_0, f2_1;  // compliance moduli (1-2nu)/E, (1+nu)/E of the phases
   double two_pi_sq_V_over_sA;
   double half_lref_V_over_sA;
-  int ref_mode;       // 0: Lame constants linear in chi; 1: compliance linear in chi (the material law)
+  int ref_mode;       // 0: Lame constants linear in chi; 1: compliance linear in chi (the material law); 2: between
   double shift_scale; // weight of the mass term rho sigma
 };
 // k-points still iterated, kept on the device and counted on the host: klist the open k-points in
@@ -95,21 +95,28 @@ struct PrecRef {  // reference medium from the mean of chi (device scalar)
 // {open, unconverged vectors, fresh}.
 struct OpenSet {
   int *klist, *vlist, *fresh, *count;
+  int* vpos;  // position of an open k-point's vector in vlist, or -1
 };
-int launch_open_all(OpenSet o, int nk, cudaStream_t s);  // klist = all
+// klist = all; ref (3 doubles) = 3 kappa and 2 mu of the preconditioner's reference medium and the factor of
+// its shift, nondimensional.
+int launch_open_all(OpenSet o, int nk, PrecRef pr, const double* chi_mean, double* ref, cudaStream_t s);
 // Residuals of the nopen k-points of o.klist, then the convergence test: kdone, and the new lists.
 template <typename R>
 int launch_resnorm(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX,
                    const R* lam, int nk, int m, int nb, int n3, double tol, double* rnorm,
                    int* active, int* kdone, OpenSet o, int nopen, cudaStream_t s, double* best = nullptr,
                    int* since = nullptr);
-// W = P(R) on the unconverged vectors of the open k-points; W, A W and Omega W = 0 on their others.
+// The preconditioner W = P(R) on the ncol vectors of vlist, in two halves around the products S = T E of the
+// compliance operators (T_f1 on stack 0, T_f2 on the others) with the strain stacks E; W, A W and Omega W = 0
+// on the other vectors of the open k-points.
 template <typename R>
-int launch_precond(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX,
-                   const R* lam, const int* active, const int* klist, int nopen, int m, int nb, Geom g,
-                   const double* Q, PrecRef pr, const double* chi_mean, typename cplx_t<R>::type* W,
-                   typename cplx_t<R>::type* AW, typename cplx_t<R>::type* OW, cudaStream_t s,
-                   const float4* Kf = nullptr);
+int launch_prec_in(const typename cplx_t<R>::type* AX, const typename cplx_t<R>::type* OX, const R* lam, const int* vlist,
+                   int ncol, int m, int nb, Geom g, const double* Q, const double* ref, typename cplx_t<R>::type* W,
+                   typename cplx_t<R>::type* E, cudaStream_t s, const float4* Kf = nullptr);
+template <typename R>
+int launch_prec_out(const typename cplx_t<R>::type* S, const R* lam, const int* klist, const int* vpos, int nopen, int ncol,
+                    int m, int nb, Geom g, const double* Q, const double* ref, typename cplx_t<R>::type* W,
+                    typename cplx_t<R>::type* AW, typename cplx_t<R>::type* OW, cudaStream_t s, const float4* Kf = nullptr);
 // dst[k] = src[k] in FP64 for the nsel k-points of list, `per` values each.
 template <typename R>
 int launch_store(const typename cplx_t<R>::type* src, double2* dst, const int* list, int nsel, long long per, cudaStream_t s);

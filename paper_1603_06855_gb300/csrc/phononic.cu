@@ -64,7 +64,9 @@ struct pc_ctx {
   // per-design (FP64)
   double *fields = nullptr, *dchi = nullptr, *chi = nullptr, *chi_mean = nullptr, *dfc = nullptr;
   double2 *t1 = nullptr, *t2s = nullptr, *sfac = nullptr, *T = nullptr, *W = nullptr, *gj = nullptr;
-  float2 *Wf = nullptr, *Tf = nullptr;  // scaled FP32 copies (mixed path)
+  float2 *Wf = nullptr, *Tf = nullptr;  // scaled FP32 W1, W2 and T_rho, T_f1, T_f2 (mixed form without a tensor-core plan)
+  bool f32_ready = false;               // they are of the current design
+  double* prec_ref = nullptr;           // preconditioner reference medium, 3 values per k group
   int* status = nullptr;
   double* small_flops = nullptr;  // device: algorithmic flops of the FP32 projected problems while profiling
   double grad_flops_per_pair = 0;  // algorithmic flops of the adjoint per weighted (k, band)
@@ -78,7 +80,7 @@ struct pc_ctx {
   long long sr_stride = 0;
   double *rnorm = nullptr;
   int *active = nullptr, *kdone = nullptr, *kdone_f = nullptr;
-  int *open_k = nullptr, *open_v = nullptr, *fresh_k = nullptr, *d_count = nullptr;  // OpenSet, per k group at its k0
+  int *open_k = nullptr, *open_v = nullptr, *open_pos = nullptr, *fresh_k = nullptr, *d_count = nullptr;  // OpenSet, per k group at its k0
   double* stall_best = nullptr;  // per k: best worst-wanted residual so far (stagnation test)
   int* stall_since = nullptr;     // per k: iterations since that best
   // FP64 Rayleigh-Ritz and adjoint
@@ -236,7 +238,7 @@ static void free_kset(pc_ctx* c) {
   if (c->S) cudaFree(c->S); c->S = nullptr;
   void** vs[] = {&c->gpart, &c->GA, &c->GO, &c->Cc, &c->Ct, &c->lam};
   for (auto v : vs) { if (*v) cudaFree(*v); *v = nullptr; }
-  dfree(c->sr_scratch); dfree(c->rnorm); dfree(c->active); dfree(c->open_k); dfree(c->open_v); dfree(c->fresh_k); dfree(c->d_count); dfree(c->kdone); dfree(c->kdone_f);
+  dfree(c->sr_scratch); dfree(c->rnorm); dfree(c->active); dfree(c->open_k); dfree(c->open_v); dfree(c->open_pos); dfree(c->fresh_k); dfree(c->d_count); dfree(c->kdone); dfree(c->kdone_f);
   dfree(c->stall_best); dfree(c->stall_since);
   dfree(c->Xd); dfree(c->AXd); dfree(c->OXd); dfree(c->Ed); dfree(c->Sd); dfree(c->Th); dfree(c->St);
   dfree(c->gpartd); dfree(c->GAd); dfree(c->GOd); dfree(c->Cd);
@@ -261,7 +263,7 @@ extern "C" void pc_destroy(pc_ctx* c) {
   free_kset(c);
   dfree(c->fields); dfree(c->dchi); dfree(c->chi); dfree(c->chi_mean); dfree(c->dfc);
   dfree(c->t1); dfree(c->t2s); dfree(c->sfac); dfree(c->T); dfree(c->W); dfree(c->gj);
-  dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops);
+  dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops); dfree(c->prec_ref);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   for (cudaEvent_t e : {c->ev_s0, c->ev_s1, c->ev_g0, c->ev_g1})
@@ -363,14 +365,14 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
   c->pr.f2_0 = (1.0 + p->phase0.nu) / p->phase0.E;
   c->pr.f2_1 = (1.0 + p->phase1.nu) / p->phase1.E;
   {
-    // Reference medium of the preconditioner: the homogeneous material at the mean chi, with
-    // compliance linear in chi as in the material law (PC_PREC_REF=0: Lame constants linear in
-    // chi, a stiffer medium); its mass term rho sigma weighted by 0.25 (PC_PREC_SHIFT).  On the
-    // FCC N = 729 designs this pair took 12 % fewer block iterations than (0, 1).
+    // Reference medium of the preconditioner at the mean chi: moduli between the material's with the mean
+    // compliance (PC_PREC_REF=1) and with the mean Lame constants (0), their geometric mean; its shift is
+    // PC_PREC_SHIFT times half the mass term rho sigma.  The iterations depend little on either: for shifts
+    // of 0.04 to 0.5 and the three media within 10 % on level sets and 25 % on spheres (M = 2, 3).
     const char* rm = getenv("PC_PREC_REF");
-    c->pr.ref_mode = (rm && rm[0] == '0') ? 0 : 1;
+    c->pr.ref_mode = (rm && rm[0] == '0') ? 0 : ((rm && rm[0] == '1') ? 1 : 2);
     const char* sh = getenv("PC_PREC_SHIFT");
-    c->pr.shift_scale = (sh && atof(sh) > 0) ? atof(sh) : 0.25;
+    c->pr.shift_scale = (sh && atof(sh) > 0) ? atof(sh) : 0.1;
   }
   {
     // adjoint per weighted (k, band): 9 fields synthesised along axis 2 (M2^3 n2 complex
@@ -397,9 +399,10 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
   rc |= dalloc(&c->gj, (size_t)setup_gj_scratch(N));
   rc |= dalloc(&c->status, 1);
   rc |= dalloc(&c->small_flops, 1);
+  rc |= dalloc(&c->prec_ref, 3 * (size_t)kMaxGroups);
   if (p->precision == PC_MIXED) {
     rc |= dalloc(&c->Wf, 2 * NN);
-    rc |= dalloc(&c->Tf, NN);
+    rc |= dalloc(&c->Tf, 3 * NN);
   }
   if (rc != PC_OK) { pc_destroy(c); return PC_ENOMEM; }
   if (cudaMemset(c->status, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->small_flops, 0, sizeof(double)) != cudaSuccess ||
@@ -454,6 +457,7 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   rc |= dalloc(&c->open_k, (size_t)nk);
   rc |= dalloc(&c->fresh_k, (size_t)nk);
   rc |= dalloc(&c->open_v, nvec);
+  rc |= dalloc(&c->open_pos, nvec);
   rc |= dalloc(&c->kdone, (size_t)nk);
   rc |= dalloc(&c->kdone_f, (size_t)nk);
   rc |= dalloc(&c->stall_best, (size_t)nk);
@@ -535,12 +539,7 @@ extern "C" int pc_set_design(pc_ctx* c, const double* rho, void* stream) {
   int rc = launch_setup(a, s);
   if (rc) return rc;
   if (c->prm.precision == PC_MIXED) {
-    const long long NN = (long long)c->N * c->N;
-    // scaled FP32 operators: W * (2 pi)^2 V^2 / sA and T_rho / sO are O(1)
-    rc = launch_d2f(c->W, c->Wf, 2 * NN, c->cA, s);
-    if (rc) return rc;
-    rc = launch_d2f(c->T, c->Tf, NN, 1.0 / c->sO, s);
-    if (rc) return rc;
+    c->f32_ready = false;
     c->tc_ready = false;
     if (c->tc) {
       rc = tc_prepare_operators(c->tc, c->W, c->T, c->cA, 1.0 / c->sO, s);
@@ -577,22 +576,22 @@ template <> struct Ops<float> {
   static constexpr float rel_drop = 1e-4f;
 };
 
-// A x and Omega x for nvec vectors with the per-k geometry Q (vector v belongs to k = v / m).
+// A x and Omega x for nvec (selected) vectors with the per-k geometry Q (vector v belongs to k = v / m).
 static int apply_fp64(pc_ctx* c, const double2* X, double2* AX, double2* OX, int nvec, int m, const double* Q,
-                      double epi, double alpha_omega, double2* E, double2* S, cudaStream_t s, int phase = -1) {
+                      double epi, double alpha_omega, double2* E, double2* S, cudaStream_t s, int phase = -1, VecSel sel = {}) {
   const int N = c->N;
   const long long NN = (long long)N * N;
   const double f = 8.0 * (double)N * (double)N;  // algorithmic flops per complex column
-  int rc = launch_strain<double>(X, nvec, m, c->geom, Q, E, s);
+  int rc = launch_strain<double>(X, nvec, m, c->geom, Q, E, s, nullptr, sel);
   if (rc) return rc;
   const long long o = (long long)nvec * N;
   const GemmSeg<double> seg[3] = {
-      {c->W, E, S, nvec, 1.0}, {c->W + NN, E + o, S + o, 5 * nvec, 1.0}, {c->T, X, OX, 3 * nvec, alpha_omega}};
+      {c->W, E, S, nvec, 1.0}, {c->W + NN, E + o, S + o, 5 * nvec, 1.0}, {c->T, X, OX, 3 * nvec, alpha_omega, sel}};
   const int slot = phase >= 0 ? ph_begin(c, phase, f * 9.0 * nvec, s) : -1;
   rc = launch_gemms<double>(N, N, N, N, N, seg, 3, s);
   ph_end(c, slot, s);
   if (rc) return rc;
-  return launch_epilogue<double>(S, nvec, m, c->geom, Q, epi, epi, AX, s);
+  return launch_epilogue<double>(S, nvec, m, c->geom, Q, epi, epi, AX, s, nullptr, sel);
 }
 
 // The same products as apply_fp64 (operators prepared with Omega scaled by 1/sO) from the
@@ -619,34 +618,52 @@ static int apply_sliced(pc_ctx* c, OzPlan* oz, const double2* X, double2* AX, do
   return launch_epilogue<double>(S, nvec, m, c->geom, Q, epi, epi, AX, s);
 }
 
-// Nondimensional A' X and Omega' X for FP32 vectors (vector v at k-point k0 + v / m): the split-BF16
-// tensor-core path; the FP32 CUDA-core GEMM only where the tensor-core plan could not be set up.
-// sel: the nsel vectors that are needed (the CUDA-core GEMM takes all nvec).
+// The FP32 operators of the CUDA-core products: W * (2 pi)^2 V^2 / sA, T_rho / sO and T_f over the former's
+// scale are O(1).  Only where the tensor-core plan could not be set up.
+static int prepare_f32(pc_ctx* c, cudaStream_t s) {
+  if (c->f32_ready) return PC_OK;
+  const long long NN = (long long)c->N * c->N;
+  int rc = launch_d2f(c->W, c->Wf, 2 * NN, c->cA, s);
+  if (!rc) rc = launch_d2f(c->T, c->Tf, NN, 1.0 / c->sO, s);
+  if (!rc) rc = launch_d2f(c->T + NN, c->Tf + NN, 2 * NN, 1.0 / c->cA, s);
+  c->f32_ready = rc == PC_OK;
+  return rc;
+}
+// The tensor-core plan to use, its operators prepared, or none (and the FP32 operators prepared).
+static int ready_f32(pc_ctx* c, TcPlan* plan, bool* tensor, cudaStream_t s) {
+  *tensor = plan && tc_available(plan);
+  if (!*tensor) return prepare_f32(c, s);
+  if (!c->tc_ready) {
+    int rc = tc_prepare_operators(c->tc, c->W, c->T, c->cA, 1.0 / c->sO, s);
+    if (rc) return rc;
+    c->tc_ready = true;
+  }
+  return PC_OK;
+}
+
+// Nondimensional A' X and Omega' X for nvec (selected) FP32 vectors (vector v at k-point k0 + v / m): the
+// split-BF16 tensor-core path; the FP32 CUDA-core GEMM only without a tensor-core plan.
 static int apply_fp32(pc_ctx* c, const float2* X, float2* AX, float2* OX, int nvec, int m, int k0,
-                      cudaStream_t s, TcPlan* plan = nullptr, int nsel = -1, VecSel sel = {}) {
+                      cudaStream_t s, TcPlan* plan = nullptr, VecSel sel = {}) {
   const double* Q = c->Q + 3LL * k0;
   const float4* Kf = c->Kf ? c->Kf + (long long)k0 * c->N : nullptr;
   if (!plan) plan = c->tc;
-  if (plan && tc_available(plan)) {
-    if (!c->tc_ready) {
-      int rc = tc_prepare_operators(c->tc, c->W, c->T, c->cA, 1.0 / c->sO, s);
-      if (rc) return rc;
-      c->tc_ready = true;
-    }
-    return tc_apply(plan, X, AX, OX, nsel < 0 ? nvec : nsel, m, c->geom, Q, s, Kf, sel);
-  }
+  bool tensor;
+  int rc = ready_f32(c, plan, &tensor, s);
+  if (rc) return rc;
+  if (tensor) return tc_apply(plan, X, AX, OX, nvec, m, c->geom, Q, s, Kf, sel);
   const int N = c->N;
   const long long NN = (long long)N * N;
   float2* E = (float2*)c->E;
   float2* S = (float2*)c->S;
-  int rc = launch_strain<float>(X, nvec, m, c->geom, Q, E, s, Kf);
+  rc = launch_strain<float>(X, nvec, m, c->geom, Q, E, s, Kf, sel);
   if (rc) return rc;
   const long long o = (long long)nvec * N;
   const GemmSeg<float> seg[3] = {
-      {c->Wf, E, S, nvec, 1.f}, {c->Wf + NN, E + o, S + o, 5 * nvec, 1.f}, {c->Tf, X, OX, 3 * nvec, 1.f}};
+      {c->Wf, E, S, nvec, 1.f}, {c->Wf + NN, E + o, S + o, 5 * nvec, 1.f}, {c->Tf, X, OX, 3 * nvec, 1.f, sel}};
   rc = launch_gemms<float>(N, N, N, N, N, seg, 3, s);
   if (rc) return rc;
-  return launch_epilogue<float>(S, nvec, m, c->geom, Q, 1.0f, 1.0f, AX, s, Kf);
+  return launch_epilogue<float>(S, nvec, m, c->geom, Q, 1.0f, 1.0f, AX, s, Kf, sel);
 }
 
 // A subset of the k-points run by one host thread on one stream: k in [k0, k0 + nk).
@@ -655,29 +672,56 @@ struct KSet {
   cudaStream_t s = nullptr;
   OpenSet open;             // its k-points still iterated (indices from k0), on the device
   int* h_count = nullptr;   // pinned host copy of open.count
-  int unconv = 0, iterations = 0;
+  int unconv = 0, iterations = 0, group = 0;
   TcPlan* tc = nullptr;     // tensor-core workspaces of this subset
   OzPlan* oz = nullptr;     // sliced products of this subset's final Rayleigh-Ritz step (or NULL)
 };
 
 static OpenSet open_set(const pc_ctx* c, int k0, int group) {
-  return OpenSet{c->open_k + k0, c->open_v + (long long)k0 * c->m, c->fresh_k + k0, c->d_count + 3 * group};
+  return OpenSet{c->open_k + k0, c->open_v + (long long)k0 * c->m, c->fresh_k + k0, c->d_count + 3 * group,
+                 c->open_pos + (long long)k0 * c->m};
 }
 
-// A X and Omega X of the nsel selected vectors of the subset.  The CUDA-core products (FP64, and FP32
-// without a tensor-core plan) take all its vectors: those not selected are zero or belong to locked
-// k-points, whose products nothing reads.
+// A X and Omega X of the nsel selected vectors of the subset.
 template <typename R>
 static int apply_R(pc_ctx* c, const KSet& ks, const typename Ops<R>::C2* X, typename Ops<R>::C2* AX,
-                   typename Ops<R>::C2* OX, int nsel, VecSel sel);
-template <>
-int apply_R<double>(pc_ctx* c, const KSet& ks, const double2* X, double2* AX, double2* OX, int, VecSel) {
-  return apply_fp64(c, X, AX, OX, ks.nk * c->m, c->m, c->Q + 3 * ks.k0, c->cA, 1.0 / c->sO, (double2*)c->E,
-                    (double2*)c->S, ks.s);
+                   typename Ops<R>::C2* OX, int nsel, VecSel sel) {
+  if constexpr (std::is_same<R, double>::value)
+    return apply_fp64(c, X, AX, OX, nsel, c->m, c->Q + 3 * ks.k0, c->cA, 1.0 / c->sO, (double2*)c->E, (double2*)c->S,
+                      ks.s, -1, sel);
+  else
+    return apply_fp32(c, X, AX, OX, nsel, c->m, ks.k0, ks.s, ks.tc, sel);
 }
-template <>
-int apply_R<float>(pc_ctx* c, const KSet& ks, const float2* X, float2* AX, float2* OX, int nsel, VecSel sel) {
-  return apply_fp32(c, X, AX, OX, ks.nk * c->m, c->m, ks.k0, ks.s, ks.tc, nsel, sel);
+// The preconditioner (waves.cuh) on the ncol unconverged columns of the nopen open k-points.
+template <typename R>
+static int precond_R(pc_ctx* c, const KSet& ks, const typename Ops<R>::C2* AX, const typename Ops<R>::C2* OX, const R* lam,
+                     int nopen, int ncol, double* ref, typename Ops<R>::C2* W, typename Ops<R>::C2* AW,
+                     typename Ops<R>::C2* OW) {
+  typedef typename Ops<R>::C2 C2;
+  const int N = c->N, m = c->m, nb = c->nb;
+  const double* Q = c->Q + 3 * ks.k0;
+  const float4* Kf = c->Kf ? c->Kf + (long long)ks.k0 * N : nullptr;
+  const C2* S = (const C2*)c->S;
+  bool tensor = false;
+  int rc = PC_OK;
+  if constexpr (std::is_same<R, float>::value) {
+    TcPlan* plan = ks.tc ? ks.tc : c->tc;
+    rc = ready_f32(c, plan, &tensor, ks.s);
+    if (!rc && tensor) rc = tc_precond(plan, AX, OX, lam, ks.open.vlist, ncol, m, nb, c->geom, Q, ref, W, &S, ks.s, Kf);
+    if (rc) return rc;
+  }
+  if (!tensor) {
+    C2 *E = (C2*)c->E, *So = (C2*)c->S;
+    const long long NN = (long long)N * N, o = (long long)ncol * N;
+    rc = launch_prec_in<R>(AX, OX, lam, ks.open.vlist, ncol, m, nb, c->geom, Q, ref, W, E, ks.s, Kf);
+    if (rc) return rc;
+    const C2* T = std::is_same<R, double>::value ? (const C2*)c->T : (const C2*)c->Tf;
+    const R al = std::is_same<R, double>::value ? (R)(1.0 / c->cA) : (R)1;
+    const GemmSeg<R> seg[2] = {{T + NN, E, So, ncol, al}, {T + 2 * NN, E + o, So + o, 5 * ncol, al}};
+    rc = launch_gemms<R>(N, N, N, N, N, seg, 2, ks.s);
+    if (rc) return rc;
+  }
+  return launch_prec_out<R>(S, lam, ks.open.klist, ks.open.vpos, nopen, ncol, m, nb, c->geom, Q, ref, W, AW, OW, ks.s, Kf);
 }
 
 template <typename R>
@@ -732,7 +776,7 @@ static int small_rr_any(pc_ctx* c, int k0, int nk, const MatRef<R>& GA, const Ma
                              c->status, scratch, c->sr_stride, s);
 }
 // The batched block iteration (all k at once).  Per iteration and k:
-//   R = A X - Omega X Lambda,  W = P(R) on the unconverged columns;
+//   R = A X - Omega X Lambda,  W = P R on the unconverged columns (P: waves.cuh);
 //   W <- W - X (OX^H W) - P (OP^H W); AW, OW = A W, Omega W (explicit products);
 //   W <- W T (Cholesky-QR in the Omega metric, dependent directions dropped);
 //   Rayleigh-Ritz on S = [X W P]: X <- S cX, P <- S cP (cP from the small space).
@@ -813,7 +857,8 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
   } else {
     TRY(launch_init_guess<R>(X, nk, m, c->geom, Qk, c->seed, s));
   }
-  TRY(launch_open_all(o, nk, s));
+  double* ref = c->prec_ref + 3 * ks.group;
+  TRY(launch_open_all(o, nk, c->pr, c->chi_mean, ref, s));
   TRY(apply_R<R>(c, ks, X, AX, OX, nk * m, VecSel{}));
   {
     BlockList<R> A1 = {{X, nullptr, nullptr}}, B1 = {{AX, nullptr, nullptr}}, B2 = {{OX, nullptr, nullptr}};
@@ -874,8 +919,11 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
     ph_end(c, idle_slot, s);
     TRY(launch_store<R>(X, Xd, o.fresh, nfresh, (long long)m * n3, s));
     if (nopen == 0) break;
-    TRY(launch_precond<R>(AX, OX, lam, active, klist, nopen, m, nb, c->geom, Qk, c->pr, c->chi_mean, Wb, AW, OW, s,
-                          c->Kf ? c->Kf + (long long)k0 * c->N : nullptr));
+    {
+      int sl = ph_begin(c, PH_ITER_APPLY, 8.0 * c->N * (double)c->N * 6.0 * ncol, s);
+      TRY(precond_R<R>(c, ks, AX, OX, lam, nopen, ncol, ref, Wb, AW, OW));
+      ph_end(c, sl, s);
+    }
     // W <- W - X (OX^H W) - P (OP^H W), before the operator is applied
     {
       const int nproj = hasP ? 2 : 1;
@@ -958,6 +1006,7 @@ static int run_split_iteration(pc_ctx* c, cudaStream_t s) {
     ks[g].k0 = (int)(((long long)c->nk * g) / ng);
     ks[g].nk = (int)(((long long)c->nk * (g + 1)) / ng) - ks[g].k0;
     ks[g].s = c->sk[g];
+    ks[g].group = g;
     ks[g].open = open_set(c, ks[g].k0, g);
     ks[g].h_count = c->h_count + 3 * g;
     ks[g].tc = g ? c->tcg[g] : c->tc;
@@ -1038,7 +1087,7 @@ static int fp64_rayleigh_ritz(pc_ctx* c, const KSet& ks) {
   if (rc) return rc;
   PC_CUDA_TRY(cudaMemsetAsync(c->kdone_f + k0, 0, sizeof(int) * nk, s));
   rc = launch_resnorm<double>(Ath, Oth, lamd, nk, m, c->nb, n3, c->prm.tol, c->rnormd + vo, c->actived + vo,
-                              c->kdone_f + k0, OpenSet{nullptr, nullptr, nullptr, ks.open.count}, nk, s);
+                              c->kdone_f + k0, OpenSet{nullptr, nullptr, nullptr, ks.open.count, nullptr}, nk, s);
   if (rc) return rc;
   // stresses of theta in the global layout [6][nk m][N]: St[s] = Sd[s] C
   for (int half = 0; half < 2; ++half) {
