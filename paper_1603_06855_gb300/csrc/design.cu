@@ -28,82 +28,131 @@ struct pc_design {
   int n[3], nd[3], spacing, octant;
   long long ne, nnodes, nvars;
   int nclass;
-  DesignEntry* table = nullptr;  // device: entries of class 0, then class 1, ...
-  int* class_start = nullptr;    // device: nclass + 1 offsets into table
-  double* phi = nullptr;         // device: nnodes, the expanded design field (octant maps)
-  double* gphi = nullptr;        // device: nnodes, dG/dphi before folding
-  double* dmu = nullptr;         // device: ne, d rho / d mu of the last projection
+  // one device allocation
+  double* exp2t = nullptr;       // 2^(j / 64), j < 64
+  DesignEntry* table = nullptr;  // entries of class 0, then class 1, ...
+  int* class_start = nullptr;    // nclass + 1 offsets into table
+  double* dmu = nullptr;         // ne, d rho / d mu of the last projection
+  double* gmu = nullptr;         // ne, dG/dmu (large maps)
 };
 
 namespace {
 
-__global__ void k_octant_expand(const double* __restrict__ x, int nd0, int nd1, int nd2, double* __restrict__ phi) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long nn = (long long)nd0 * nd1 * nd2;
-  if (t >= nn) return;
-  const int l = (int)(t % nd2), j = (int)((t / nd2) % nd1), i = (int)(t / ((long long)nd1 * nd2));
-  const int h1 = nd1 / 2, h2 = nd2 / 2;
-  const int a = min(i, nd0 - 1 - i), b = min(j, nd1 - 1 - j), c = min(l, nd2 - 1 - l);
-  phi[t] = x[((long long)a * h1 + b) * h2 + c];
-}
-
-// Adjoint of the expansion: each octant variable sums the gradient of its 8 images.
-__global__ void k_octant_fold(const double* __restrict__ g, int nd0, int nd1, int nd2, double* __restrict__ gx) {
-  const int h0 = nd0 / 2, h1 = nd1 / 2, h2 = nd2 / 2;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)h0 * h1 * h2) return;
-  const int c = (int)(t % h2), b = (int)((t / h2) % h1), a = (int)(t / ((long long)h1 * h2));
-  double s = 0.0;
-  for (int m = 0; m < 8; ++m) {
-    const int i = (m & 1) ? nd0 - 1 - a : a, j = (m & 2) ? nd1 - 1 - b : b, l = (m & 4) ? nd2 - 1 - c : c;
-    s += g[((long long)i * nd1 + j) * nd2 + l];
-  }
-  gx[t] = s;
-}
-
 __device__ __forceinline__ int wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
 
-__global__ void k_project(const double* __restrict__ phi, const DesignEntry* __restrict__ tab,
-                          const int* __restrict__ cstart, int n0, int n1, int n2, int nd0, int nd1, int nd2, int sp,
-                          double beta, double* __restrict__ rho, double* __restrict__ dmu) {
+// fmin(fmax(v, 0), 1), NaN to 0, on the integer units (the FP64 unit is the bound here).
+__device__ __forceinline__ double clamp01(double v) {
+  const long long b = __double_as_longlong(v);
+  if (b < 0 || b > 0x7ff0000000000000LL) return 0.0;
+  return b > 0x3ff0000000000000LL ? 1.0 : v;
+}
+
+// exp(x) for -690 < x <= 0 by table and polynomial (Tang, ACM Trans. Math. Softw. 15, 1989):
+// x = (64 k + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^k 2^(j/64) (1 + r + r^2/2 + ... + r^5/120).
+// The remainder r^6/720 is below 4e-17.  10 FP64 instructions.
+__device__ __forceinline__ double exp_tab(double x, const double* __restrict__ tab) {
+  constexpr double ln2_hi = 6.93147180369123816490e-01;  // ln 2 to 33 bits, and the rest
+  constexpr double ln2_lo = 1.90821492927058770002e-10;
+  constexpr double shift = 6755399441055744.0;  // 1.5 2^52: rounds to an integer in the low word
+  const double t = fma(x, 64.0 / 0.69314718055994530942, shift);
+  const int n = __double2loint(t);
+  const double nd = t - shift;
+  double r = fma(nd, -ln2_hi / 64.0, x);
+  r = fma(nd, -ln2_lo / 64.0, r);
+  double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+  p = fma(p, r, 1.0 / 6.0);
+  p = fma(p, r, 0.5);
+  p = fma(r * r, p, r);
+  const double s = tab[n & 63];
+  const double v = fma(s, p, s);
+  return __hiloint2double(__double2hiint(v) + ((n >> 6) << 20), __double2loint(v));
+}
+
+// The variable behind node (a0, a1, a2): the node itself, or its mirror image in the first octant.
+__device__ __forceinline__ int variable(int a0, int a1, int a2, int nd0, int nd1, int nd2, int octant) {
+  if (!octant) return (a0 * nd1 + a1) * nd2 + a2;
+  return (min(a0, nd0 - 1 - a0) * (nd1 / 2) + min(a1, nd1 - 1 - a1)) * (nd2 / 2) + min(a2, nd2 - 1 - a2);
+}
+
+// Average and projection.  Bound: the FP64 unit (one instruction of all elements of a 96^3 cell is 1.5 us):
+// one multiply-add per node within the radius (13 in FCC at the default), 10 for the exponential and 6 more.
+// Two library exponentials and FP64 clamps took 88 us on that cell, this 46 us.
+// eb: exp(-beta).  small: beta < 690.
+__global__ void k_project(const double* __restrict__ x, const DesignEntry* __restrict__ tab,
+                          const int* __restrict__ cstart, int n0, int n1, int n2, int nd0, int nd1, int nd2, int sp, int octant,
+                          double beta, double eb, int small, const double* __restrict__ exp2t, double* __restrict__ rho,
+                          double* __restrict__ dmu) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)n0 * n1 * n2) return;
   const int l = (int)(e % n2), j = (int)((e / n2) % n1), i = (int)(e / ((long long)n1 * n2));
   const int b0 = i / sp, b1 = j / sp, b2 = l / sp;
   const int p = ((i - b0 * sp) * sp + (j - b1 * sp)) * sp + (l - b2 * sp);
   double mu = 0.0;
+#pragma unroll 4
   for (int q = cstart[p]; q < cstart[p + 1]; ++q) {
     const DesignEntry t = tab[q];
     const int a0 = wrap(b0 + t.d0, nd0), a1 = wrap(b1 + t.d1, nd1), a2 = wrap(b2 + t.d2, nd2);
-    mu += t.w * phi[((long long)a0 * nd1 + a1) * nd2 + a2];
+    mu = fma(t.w, x[variable(a0, a1, a2, nd0, nd1, nd2, octant)], mu);
   }
   // mu is a convex combination of values in [0, 1]: the clamps only remove rounding excursions
   // (a density 1 ulp above 1 would be flagged PC_EDOMAIN by pc_set_design)
-  mu = fmin(fmax(mu, 0.0), 1.0);
-  const double em = exp(-beta * mu), eb = exp(-beta);
-  rho[e] = fmin(fmax(1.0 - em + mu * eb, 0.0), 1.0);
+  mu = clamp01(mu);
+  const double em = small ? exp_tab(-beta * mu, exp2t) : exp(-beta * mu);
+  rho[e] = clamp01(1.0 - em + mu * eb);
   dmu[e] = beta * em + eb;
 }
 
-// dG/dphi_a = sum over the elements e that average node a of w_ea dG/drho_e drho_e/dmu_e.
-__global__ void k_project_grad(const double* __restrict__ g_rho, const double* __restrict__ dmu,
+__global__ void k_grad_mu(const double* __restrict__ g_rho, const double* __restrict__ dmu, long long ne,
+                          double* __restrict__ gmu) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < ne) gmu[e] = g_rho[e] * dmu[e];
+}
+
+// dG/dphi_a = sum over the elements e that average node a of w_ea dG/drho_e drho_e/dmu_e.  DONE: g is
+// dG/dmu_e already; it takes a pass over the elements but one FP64 instruction per node and element instead
+// of two (96^3, FCC: 45 us in one launch, 28 us in two; below GRAD_PASS elements the launch costs more).
+// OCTANT: eight threads of a warp take the eight images of a variable and add up their sums in order.
+template <bool DONE, bool OCTANT>
+__global__ void k_project_grad(const double* __restrict__ g, const double* __restrict__ dmu,
                                const DesignEntry* __restrict__ tab, const int* __restrict__ cstart, int nclass,
-                               int n1, int n2, int nd0, int nd1, int nd2, int sp, double* __restrict__ gphi) {
-  const long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= (long long)nd0 * nd1 * nd2) return;
-  const int a2 = (int)(a % nd2), a1 = (int)((a / nd2) % nd1), a0 = (int)(a / ((long long)nd1 * nd2));
+                               int n1, int n2, int nd0, int nd1, int nd2, int sp, double* __restrict__ gx) {
+  const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in = t0 < (long long)nd0 * nd1 * nd2;
+  if (!OCTANT && !in) return;
+  int a0, a1, a2;
+  const int m = (int)(t0 & 7);
+  if (OCTANT) {
+    const int h1 = nd1 / 2, h2 = nd2 / 2;
+    const long long v = in ? t0 >> 3 : 0;
+    const int c = (int)(v % h2), b = (int)((v / h2) % h1), a = (int)(v / ((long long)h1 * h2));
+    a0 = (m & 1) ? nd0 - 1 - a : a;
+    a1 = (m & 2) ? nd1 - 1 - b : b;
+    a2 = (m & 4) ? nd2 - 1 - c : c;
+  } else {
+    a2 = (int)(t0 % nd2);
+    a1 = (int)((t0 / nd2) % nd1);
+    a0 = (int)(t0 / ((long long)nd1 * nd2));
+  }
   double s = 0.0;
   for (int p = 0; p < nclass; ++p) {
     const int p0 = p / (sp * sp), p1 = (p / sp) % sp, p2 = p % sp;
+#pragma unroll 4
     for (int q = cstart[p]; q < cstart[p + 1]; ++q) {
       const DesignEntry t = tab[q];
       const int b0 = wrap(a0 - t.d0, nd0), b1 = wrap(a1 - t.d1, nd1), b2 = wrap(a2 - t.d2, nd2);
-      const long long e = ((long long)(sp * b0 + p0) * n1 + (sp * b1 + p1)) * n2 + (sp * b2 + p2);
-      s += t.w * g_rho[e] * dmu[e];
+      const int e = ((sp * b0 + p0) * n1 + (sp * b1 + p1)) * n2 + (sp * b2 + p2);
+      s = fma(t.w, DONE ? g[e] : g[e] * dmu[e], s);
     }
   }
-  gphi[a] = s;
+  if (OCTANT) {
+    double f = 0.0;
+    for (int i = 0; i < 8; ++i) f += __shfl_sync(0xffffffffu, s, i, 8);
+    if (in && m == 0) gx[t0 >> 3] = f;
+  } else {
+    gx[t0] = s;
+  }
 }
+constexpr long long GRAD_PASS = 1 << 18;
 
 void lattice_columns(int lat, double a, double A[9]) {
   // columns a_1, a_2, a_3 (A[r*3+c] = component r of a_c)
@@ -194,18 +243,26 @@ extern "C" int pc_design_create(const pc_params* cell, const pc_design_params* d
   d->nnodes = (long long)nd[0] * nd[1] * nd[2];
   d->nvars = dp->octant ? d->nnodes / 8 : d->nnodes;
   d->nclass = nclass;
-  bool ok = cudaMalloc(&d->table, sizeof(DesignEntry) * tab.size()) == cudaSuccess &&
-            cudaMalloc(&d->class_start, sizeof(int) * (nclass + 1)) == cudaSuccess &&
-            cudaMalloc(&d->phi, sizeof(double) * d->nnodes) == cudaSuccess &&
-            cudaMalloc(&d->gphi, sizeof(double) * d->nnodes) == cudaSuccess &&
-            cudaMalloc(&d->dmu, sizeof(double) * d->ne) == cudaSuccess;
-  if (!ok) {
+  // [exp2t | table | class_start] as staged on the host, then dmu and gmu
+  const size_t ts = sizeof(DesignEntry) * tab.size(), cs = sizeof(int) * (nclass + 1);
+  const size_t head = (64 * sizeof(double) + ts + cs + 255) / 256 * 256;
+  const size_t field = (sizeof(double) * d->ne + 255) / 256 * 256;
+  unsigned char* base = nullptr;
+  if (cudaMalloc(&base, head + (d->ne < GRAD_PASS ? 1 : 2) * field) != cudaSuccess) {
     cudaGetLastError();
     pc_design_destroy(d);
     return PC_ENOMEM;
   }
-  if (cudaMemcpy(d->table, tab.data(), sizeof(DesignEntry) * tab.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(d->class_start, cstart.data(), sizeof(int) * (nclass + 1), cudaMemcpyHostToDevice) != cudaSuccess ||
+  d->exp2t = (double*)base;
+  d->table = (DesignEntry*)(base + 64 * sizeof(double));
+  d->class_start = (int*)(base + 64 * sizeof(double) + ts);
+  d->dmu = (double*)(base + head);
+  if (d->ne >= GRAD_PASS) d->gmu = (double*)(base + head + field);
+  std::vector<unsigned char> stage(head, 0);
+  for (int j = 0; j < 64; ++j) ((double*)stage.data())[j] = std::exp2(j / 64.0);
+  memcpy(stage.data() + 64 * sizeof(double), tab.data(), ts);
+  memcpy(stage.data() + 64 * sizeof(double) + ts, cstart.data(), cs);
+  if (cudaMemcpy(base, stage.data(), head, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(d->dmu, 0, sizeof(double) * d->ne) != cudaSuccess) {
     pc_design_destroy(d);
     return PC_ECUDA;
@@ -220,14 +277,9 @@ extern "C" int pc_design_project(pc_design* d, const double* x, double beta, dou
   if (!d || !x || !rho || !(beta > 0) || !std::isfinite(beta)) return PC_EINVAL;
   cudaGetLastError();
   cudaStream_t s = (cudaStream_t)stream;
-  const double* phi = x;
-  if (d->octant) {
-    k_octant_expand<<<cdiv(d->nnodes, 256), 256, 0, s>>>(x, d->nd[0], d->nd[1], d->nd[2], d->phi);
-    PC_LAUNCH_CHECK();
-    phi = d->phi;
-  }
-  k_project<<<cdiv(d->ne, 256), 256, 0, s>>>(phi, d->table, d->class_start, d->n[0], d->n[1], d->n[2], d->nd[0],
-                                             d->nd[1], d->nd[2], d->spacing, beta, rho, d->dmu);
+  k_project<<<cdiv(d->ne, 256), 256, 0, s>>>(x, d->table, d->class_start, d->n[0], d->n[1], d->n[2], d->nd[0],
+                                             d->nd[1], d->nd[2], d->spacing, d->octant, beta, std::exp(-beta),
+                                             beta < 690.0, d->exp2t, rho, d->dmu);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
@@ -236,23 +288,22 @@ extern "C" int pc_design_backprop(pc_design* d, const double* g_rho, double* g_x
   if (!d || !g_rho || !g_x) return PC_EINVAL;
   cudaGetLastError();
   cudaStream_t s = (cudaStream_t)stream;
-  double* gphi = d->octant ? d->gphi : g_x;
-  k_project_grad<<<cdiv(d->nnodes, 256), 256, 0, s>>>(g_rho, d->dmu, d->table, d->class_start, d->nclass, d->n[1],
-                                                       d->n[2], d->nd[0], d->nd[1], d->nd[2], d->spacing, gphi);
-  PC_LAUNCH_CHECK();
-  if (d->octant) {
-    k_octant_fold<<<cdiv(d->nvars, 256), 256, 0, s>>>(gphi, d->nd[0], d->nd[1], d->nd[2], g_x);
+  const double* g = g_rho;
+  if (d->gmu) {
+    k_grad_mu<<<cdiv(d->ne, 256), 256, 0, s>>>(g_rho, d->dmu, d->ne, d->gmu);
     PC_LAUNCH_CHECK();
+    g = d->gmu;
   }
+  auto kernel = d->octant ? (d->gmu ? k_project_grad<true, true> : k_project_grad<false, true>)
+                          : (d->gmu ? k_project_grad<true, false> : k_project_grad<false, false>);
+  kernel<<<cdiv(d->nnodes, 128), 128, 0, s>>>(g, d->dmu, d->table, d->class_start, d->nclass, d->n[1], d->n[2], d->nd[0],
+                                              d->nd[1], d->nd[2], d->spacing, g_x);
+  PC_LAUNCH_CHECK();
   return PC_OK;
 }
 
 extern "C" void pc_design_destroy(pc_design* d) {
   if (!d) return;
-  if (d->table) cudaFree(d->table);
-  if (d->class_start) cudaFree(d->class_start);
-  if (d->phi) cudaFree(d->phi);
-  if (d->gphi) cudaFree(d->gphi);
-  if (d->dmu) cudaFree(d->dmu);
+  if (d->exp2t) cudaFree(d->exp2t);
   delete d;
 }
