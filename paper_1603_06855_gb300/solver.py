@@ -9,6 +9,23 @@ import torch
 from . import binding as B
 
 
+def _stream(device: torch.device) -> int:
+    """Handle of PyTorch's current stream, without the Stream object (2 us of a call's host time)."""
+    if device.type != "cuda":
+        return torch.cuda.current_stream(device).cuda_stream
+    i = device.index
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if i is None else i)
+
+
+def _f64(t: torch.Tensor, device: torch.device) -> torch.Tensor:
+    """t as a contiguous float64 tensor on the device, outside any graph: t itself where it is one already."""
+    if t.dtype is torch.float64 and t.is_cuda and not t.requires_grad and t.is_contiguous():
+        i = device.index
+        if t.get_device() == (torch.cuda.current_device() if i is None else i):
+            return t
+    return t.detach().to(device, torch.float64).contiguous()
+
+
 class BandSolver:
     """One design context: lattice, grid, cutoff, bands, precision and a k-point set."""
 
@@ -31,10 +48,10 @@ class BandSolver:
         return cls(w.lattice, w.n, w.M, w.nbands, w.phase1, w.phase0, w.Q, w.penal, precision, w.a, **kw)
 
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        return _stream(self.device)
 
     def set_design(self, rho: torch.Tensor) -> None:
-        rho = rho.detach().to(self.device, torch.float64).contiguous()
+        rho = _f64(rho, self.device)
         if rho.numel() != self.n[0] * self.n[1] * self.n[2]:
             raise ValueError("density size does not match the grid")
         self._rho = rho  # keeps the buffer alive while kernels read it
@@ -54,7 +71,7 @@ class BandSolver:
             grad = grad_out if grad_out is not None else torch.empty(self.n, dtype=torch.float64, device=self.device)
         wptr = 0
         if weights is not None:
-            weights = weights.to(self.device, torch.float64).contiguous()
+            weights = _f64(weights, self.device)
             wptr = weights.data_ptr()
         B.pc_gap_and_grad(self.ctx, n_lower, mode, wptr, gap.data_ptr(), grad.data_ptr() if grad is not None else 0,
                           self._stream())
@@ -142,10 +159,10 @@ class DesignMap:
         self.nvars = B.pc_design_nvars(self.handle)
 
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        return _stream(self.device)
 
     def project(self, x: torch.Tensor, beta: float, out: torch.Tensor | None = None) -> torch.Tensor:
-        x = x.detach().to(self.device, torch.float64).contiguous()
+        x = _f64(x, self.device)
         if x.numel() != self.nvars:
             raise ValueError("x must hold nvars values")
         if out is None:
@@ -156,7 +173,7 @@ class DesignMap:
 
     def backprop(self, g_rho: torch.Tensor) -> torch.Tensor:
         """d/dx from d/drho, at the x and beta of the last project()."""
-        g_rho = g_rho.detach().to(self.device, torch.float64).contiguous()
+        g_rho = _f64(g_rho, self.device)
         gx = torch.empty(self.nvars, dtype=torch.float64, device=self.device)
         B.pc_design_backprop(self.handle, g_rho.data_ptr(), gx.data_ptr(), self._stream())
         return gx
@@ -206,12 +223,12 @@ class MMA:
         """Moves x (contiguous float64 device tensor of n values) in place, ascending along df."""
         if x.dtype != torch.float64 or not x.is_contiguous() or x.numel() != self.n or x.device != self.device:
             raise ValueError("x must be a contiguous float64 tensor of n values on the solver's device")
-        df = df.detach().to(self.device, torch.float64).contiguous()
+        df = _f64(df, self.device)
         if df.numel() != self.n:
             raise ValueError("gradient size does not match the design")
         B.pc_mma_step(self.n, x.data_ptr(), df.data_ptr(), self.xold1.data_ptr(), self.xold2.data_ptr(),
                       self.low.data_ptr(), self.upp.data_ptr(), self.iteration, self.xmin, self.xmax,
-                      torch.cuda.current_stream(self.device).cuda_stream)
+                      _stream(self.device))
         self.iteration += 1
 
 
@@ -279,12 +296,12 @@ class BatchSolver:
         self.off_om = np.concatenate([[0], np.cumsum([k * b for k, b in zip(self.nk, self.nb)])]).astype(int)
 
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        return _stream(self.device)
 
     def set_designs(self, rhos) -> None:
         """rhos: one density tensor per design (any shape with n0 n1 n2 values) or a packed tensor."""
         if isinstance(rhos, torch.Tensor):
-            packed = rhos.detach().to(self.device, torch.float64).contiguous().view(-1)
+            packed = _f64(rhos, self.device).view(-1)
         else:
             packed = torch.cat([torch.as_tensor(r).to(self.device, torch.float64).reshape(-1) for r in rhos])
         if packed.numel() != self.off_rho[-1]:
