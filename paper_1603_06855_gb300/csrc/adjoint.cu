@@ -210,128 +210,215 @@ int launch_gap(const GapArgs& a, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
+// Phases of the synthesis.  Voxel centroids sit at (2 i + 1) / (2 n), so that voxels i and n - 1 - i have
+// conjugate phases: with s_g = x_g + x_-g and d_g = x_g - x_-g,
+//   sum_g x_g e^{i pi g (2i+1)/n} = x_0 + sum_{g>0} s_g cos + i sum_{g>0} d_g sin,
+// and its conjugate phases give the mirrored voxel from the same two sums: 4 M real multiply-adds for two
+// voxels instead of 8 (2M + 1).  ph: (cos, sin) of pi g (2i+1)/n, [axis][g - 1][i].
+template <typename R>
+__global__ void k_adj_phases(int M, int n0, int n1, int n2, typename cplx_t<R>::type* __restrict__ ph) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = n0 + n1 + n2;
+  if (t >= M * n) return;
+  const int first[4] = {0, M * n0, M * (n0 + n1), M * n};
+  const int ax = t >= first[2] ? 2 : (t >= first[1] ? 1 : 0);
+  const int len = ax == 0 ? n0 : (ax == 1 ? n1 : n2), r = t - first[ax];
+  ph[t] = from_d2<R>(phase_pi_over((long long)(r / len + 1) * (2 * (r % len) + 1), len));
+}
+int launch_adj_phases(int M, const int n[3], bool fp32, void* ph, cudaStream_t s) {
+  const int c = cdiv((long long)M * (n[0] + n[1] + n[2]), 128);
+  if (fp32) k_adj_phases<float><<<c, 128, 0, s>>>(M, n[0], n[1], n[2], (float2*)ph);
+  else k_adj_phases<double><<<c, 128, 0, s>>>(M, n[0], n[1], n[2], (double2*)ph);
+  PC_LAUNCH_CHECK();
+  return PC_OK;
+}
+// The two sums from (x_0, s, d) and the phases: z the voxel, zm its mirror image.
+template <typename R, int M, typename C2 = typename cplx_t<R>::type>
+__device__ __forceinline__ void mirror_pair(C2 x0, const C2 (&s)[M], const C2 (&d)[M], const C2 (&ph)[M], C2& z, C2& zm) {
+  C2 c = x0, t = mk<R>(0, 0);
+#pragma unroll
+  for (int g = 0; g < M; ++g) {
+    c.x += s[g].x * ph[g].x; c.y += s[g].y * ph[g].x;
+    t.x += d[g].x * ph[g].y; t.y += d[g].y * ph[g].y;
+  }
+  z = mk<R>(c.x - t.y, c.y + t.x);
+  zm = mk<R>(c.x + t.y, c.y - t.x);
+}
+
 // Axis-2 and axis-1 synthesis of field f of pair p:
 //   t2[p][f][g1][j][l] = sum_{g2,g3} c[g1][g2][g3] e^{i pi G2 (2j+1)/n1} e^{i pi G3 (2l+1)/n2}
 // f < 3: displacement component f of theta; f >= 3: stress coordinate f-3.  R is the
 // arithmetic of the synthesis (FP64 for the FP64 form, FP32 for the mixed form).
-template <typename R>
-__global__ void k_adj_synth12(AdjointArgs a) {
+// One CTA per field and pair.  Axis 1: a thread keeps the column (g1, ., l) in registers and runs over its
+// share of the mirrored pairs of j, so that a value costs one broadcast load and 2 M multiply-adds.
+// 48^3, M = 3, 720 pairs (836 MB of t2, 0.13 ms): 0.68 ms with
+// a full sum per value and FP64 sincospi per CTA, 0.14 ms.
+template <typename R, int M>
+__global__ __launch_bounds__(256) void k_adj_synth12(AdjointArgs a, int jsplit) {
   typedef typename cplx_t<R>::type C2;
+  constexpr int M2 = 2 * M + 1, N = M2 * M2 * M2;
   extern __shared__ __align__(16) unsigned char smem[];
   const int p = blockIdx.x, f = blockIdx.y;
   if (p >= *a.npairs) return;
-  const int M2 = 2 * a.M + 1, N = a.N, n1 = a.n1, n2 = a.n2;
+  const int n1 = a.n1, n2 = a.n2;
   C2* c = (C2*)smem;                 // N
   C2* t1 = c + N;                    // M2*M2*n2
-  C2* ph3 = t1 + M2 * M2 * n2;       // M2*n2
-  C2* ph2 = ph3 + M2 * n2;           // M2*n1
+  C2* ph3 = t1 + M2 * M2 * n2;       // M*n2
+  C2* ph2 = ph3 + M * n2;            // M*n1
   const int pr = a.pairs[p];
   const int k = pr / a.nb, b = pr % a.nb;
   const long long vec = (long long)k * a.m + b;
   const long long nvec = (long long)a.nk * a.m;
   const double2* src = (f < 3) ? a.theta + (vec * 3 + f) * N : a.sig + ((long long)(f - 3) * nvec + vec) * N;
+  const C2* tab = (const C2*)a.phases;
   for (int q = threadIdx.x; q < N; q += blockDim.x) c[q] = from_d2<R>(src[q]);
-  for (int t = threadIdx.x; t < M2 * n2; t += blockDim.x) {
-    int g = t / n2, l = t % n2;
-    ph3[t] = from_d2<R>(phase_pi_over((long long)(g - a.M) * (2 * l + 1), n2));
-  }
-  for (int t = threadIdx.x; t < M2 * n1; t += blockDim.x) {
-    int g = t / n1, j = t % n1;
-    ph2[t] = from_d2<R>(phase_pi_over((long long)(g - a.M) * (2 * j + 1), n1));
-  }
+  for (int t = threadIdx.x; t < M * n2; t += blockDim.x) ph3[t] = tab[M * (a.n0 + n1) + t];
+  for (int t = threadIdx.x; t < M * n1; t += blockDim.x) ph2[t] = tab[M * a.n0 + t];
   __syncthreads();
-  for (int t = threadIdx.x; t < M2 * M2 * n2; t += blockDim.x) {
-    int g12 = t / n2, l = t % n2;
-    C2 s = mk<R>(0, 0);
-    for (int g3 = 0; g3 < M2; ++g3) cfma(s, c[g12 * M2 + g3], ph3[g3 * n2 + l]);
-    t1[t] = s;
+  const int h2 = (n2 + 1) / 2, h1 = (n1 + 1) / 2;
+  C2 s[M], d[M], ph[M], z, zm;
+  for (int t = threadIdx.x; t < M2 * M2 * h2; t += blockDim.x) {
+    const int g12 = t / h2, l = t % h2;
+    const C2* x = c + g12 * M2 + M;
+#pragma unroll
+    for (int g = 0; g < M; ++g) {
+      s[g] = cadd(x[g + 1], x[-g - 1]);
+      d[g] = mk<R>(x[g + 1].x - x[-g - 1].x, x[g + 1].y - x[-g - 1].y);
+      ph[g] = ph3[g * n2 + l];
+    }
+    mirror_pair<R, M>(x[0], s, d, ph, z, zm);
+    t1[g12 * n2 + l] = z;
+    t1[g12 * n2 + n2 - 1 - l] = zm;
   }
   __syncthreads();
   C2* out = (C2*)a.t2 + ((long long)p * 9 + f) * M2 * n1 * n2;
-  for (long long t = threadIdx.x; t < (long long)M2 * n1 * n2; t += blockDim.x) {
-    int l = (int)(t % n2);
-    int j = (int)((t / n2) % n1);
-    int g1 = (int)(t / ((long long)n1 * n2));
-    C2 s = mk<R>(0, 0);
-    for (int g2 = 0; g2 < M2; ++g2) cfma(s, t1[(g1 * M2 + g2) * n2 + l], ph2[g2 * n1 + j]);
-    out[t] = s;
+  for (int t = threadIdx.x; t < jsplit * M2 * n2; t += blockDim.x) {
+    const int l = t % n2, g1 = (t / n2) % M2, jq = t / (n2 * M2);
+    const C2* x = t1 + (g1 * M2 + M) * n2 + l;
+#pragma unroll
+    for (int g = 0; g < M; ++g) {
+      const C2 u = x[(g + 1) * n2], v = x[-(g + 1) * n2];
+      s[g] = cadd(u, v);
+      d[g] = mk<R>(u.x - v.x, u.y - v.y);
+    }
+    const C2 x0 = x[0];
+    C2* o = out + (long long)g1 * n1 * n2 + l;
+    for (int j = jq; j < h1; j += jsplit) {
+#pragma unroll
+      for (int g = 0; g < M; ++g) ph[g] = ph2[g * n1 + j];
+      mirror_pair<R, M>(x0, s, d, ph, z, zm);
+      o[j * n2] = z;
+      o[(n1 - 1 - j) * n2] = zm;
+    }
   }
 }
 
 // Axis-0 synthesis fused with the weighted reduction over (k, band).  The pairs are cut into
-// chunks along the grid's z; each thread synthesises VPT voxels along axis 0 at one (j, l), so
-// that every loaded axis-1/2 coefficient feeds VPT complex FMAs, and sums its chunk's three
+// chunks along the grid's z; each thread synthesises V mirrored pairs of voxels along axis 0 at one (j, l), so
+// that every loaded axis-1/2 coefficient feeds 2 V voxels, and sums its chunk's three
 // weighted quadratic forms in R (FP32 in the mixed form: about a hundred pairs per chunk).  The
 // chunk sums go to part[chunk][3][ne]; k_adj_finish adds them in FP64 in chunk order.
-constexpr int kAdjReduceThreads = 128;  // at 166 registers (M2 = 9, 4 voxels) three blocks per SM
+// A warp takes 32 columns (j, l) of one group of V pairs; the warps of a CTA take the groups of the same columns
+// and share their coefficients through a ring of kAdjStages pairs in shared memory, filled by asynchronous
+// copies two pairs ahead, so that each comes from L2 once.
+// Bound: instruction issue (48^3, M = 3, 720 pairs: 0.25 ms; 836 MB of t2 at the copy rate 0.13 ms).  A full sum
+// per voxel, FP64 sincospi per thread and loads from L2 where they are used took 1.77 ms, the mirrored sums with
+// tabulated phases 0.83 ms, the ring 0.47 ms.
+constexpr int kAdjReduceWarps = 8;
+constexpr int kAdjStages = 3;
 
-template <typename R, int M2, int VPT>
-__global__ __launch_bounds__(kAdjReduceThreads) void k_adj_reduce(AdjointArgs a, int chunk) {
+template <typename R, int M, int V>
+__global__ __launch_bounds__(32 * kAdjReduceWarps) void k_adj_reduce(AdjointArgs a, int chunk) {
   typedef typename cplx_t<R>::type C2;
-  const int n0 = a.n0, n1 = a.n1, n2 = a.n2;
-  const int nig = (n0 + VPT - 1) / VPT;
-  const int j = blockIdx.y;
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= nig * n2) return;
-  const int ig = v / n2, l = v % n2;
-  C2 ph[VPT][M2];  // compile-time sizes and fully unrolled loops keep these in registers
+  constexpr int M2 = 2 * M + 1, ROWS = 9 * M2;
+  extern __shared__ __align__(16) unsigned char adj_ring[];
+  C2* ring = (C2*)adj_ring;  // [kAdjStages][ROWS][32]
+  const int n0 = a.n0, h0 = (n0 + 1) / 2, lane = threadIdx.x;
+  const long long jl = (long long)a.n1 * a.n2;
+  const long long v = (long long)blockIdx.x * 32 + lane, vc = v < jl ? v : jl - 1;
+  const int ig = blockIdx.y * blockDim.y + threadIdx.y;
+  const C2* tab = (const C2*)a.phases;
+  C2 ph[V][M];  // compile-time sizes and fully unrolled loops keep these in registers
 #pragma unroll
-  for (int s = 0; s < VPT; ++s) {
-    const int i = min(ig * VPT + s, n0 - 1);
+  for (int s = 0; s < V; ++s)
 #pragma unroll
-    for (int g = 0; g < M2; ++g) ph[s][g] = from_d2<R>(phase_pi_over((long long)(g - a.M) * (2 * i + 1), n0));
-  }
+    for (int g = 0; g < M; ++g) ph[s][g] = tab[g * n0 + min(ig * V + s, h0 - 1)];
   const int np = *a.npairs;
   const int p0 = blockIdx.z * chunk, p1 = min(np, p0 + chunk);
-  const long long fstride = (long long)M2 * n1 * n2;
-  const long long gstride = (long long)n1 * n2;
-  const C2* t2 = (const C2*)a.t2;
-  // the compliance part's factors d f1/d chi, d f2/d chi belong to the element: three weighted sums
-  R acc_m[VPT], acc_1[VPT], acc_2[VPT];
+  const C2* t2 = (const C2*)a.t2 + vc;
+  auto fill = [&](int p) {  // one group per call, empty past the end, so that the wait counts are constant
+    if (p < p1) {
+      C2* to = ring + (p - p0) % kAdjStages * ROWS * 32 + lane;
+      const C2* from = t2 + (long long)p * ROWS * jl;
+      for (int r = threadIdx.y; r < ROWS; r += blockDim.y)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(to + r * 32)),
+                     "l"(from + r * jl), "n"((int)sizeof(C2))
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // the compliance part's factors d f1/d chi, d f2/d chi belong to the element: three weighted sums, of
+  // the voxels and of their mirror images
+  R acc_m[2][V], acc_1[2][V], acc_2[2][V];
 #pragma unroll
-  for (int s = 0; s < VPT; ++s) acc_m[s] = acc_1[s] = acc_2[s] = (R)0;
+  for (int s = 0; s < V; ++s)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) acc_m[h][s] = acc_1[h][s] = acc_2[h][s] = (R)0;
+  for (int i = 0; i < kAdjStages - 1; ++i) fill(p0 + i);
   for (int p = p0; p < p1; ++p) {
     const int pr = a.pairs[p];
     const double wd = a.weights[pr];
     const R w = (R)wd, wl = (R)(wd * a.lam[pr] * a.lref);
-    const C2* base = t2 + (long long)p * 9 * fstride + (long long)j * n2 + l;
-    R u2[VPT], sd[VPT], q3[VPT];
-#pragma unroll
-    for (int s = 0; s < VPT; ++s) u2[s] = sd[s] = q3[s] = (R)0;
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAdjStages - 2) : "memory");
+    __syncthreads();  // pair p is there, and every warp is done with pair p - 1, whose slot is filled now
+    fill(p + kAdjStages - 1);
+    const C2* base = ring + (p - p0) % kAdjStages * ROWS * 32 + lane;
+    R q[2][V];
 #pragma unroll
     for (int f = 0; f < 9; ++f) {
-      const C2* srcf = base + f * fstride;
-      C2 x[M2];
+      if (f == 0 || f == 3 || f == 4) {
 #pragma unroll
-      for (int g = 0; g < M2; ++g) x[g] = srcf[g * gstride];
-#pragma unroll
-      for (int s = 0; s < VPT; ++s) {
-        C2 z = mk<R>(0, 0);
-#pragma unroll
-        for (int g = 0; g < M2; ++g) cfma(z, x[g], ph[s][g]);
-        const R q = z.x * z.x + z.y * z.y;
-        if (f < 3) u2[s] += q;
-        else if (f == 3) q3[s] = q;
-        else sd[s] += q;
+        for (int s = 0; s < V; ++s) q[0][s] = q[1][s] = (R)0;
       }
-    }
+      C2 x[M2], sg[M], d[M];
 #pragma unroll
-    for (int s = 0; s < VPT; ++s) {
-      acc_m[s] += wl * u2[s];
-      acc_1[s] += w * q3[s];
-      acc_2[s] += w * sd[s];
+      for (int g = 0; g < M2; ++g) x[g] = base[(f * M2 + g) * 32];
+#pragma unroll
+      for (int g = 0; g < M; ++g) {
+        sg[g] = cadd(x[M + 1 + g], x[M - 1 - g]);
+        d[g] = mk<R>(x[M + 1 + g].x - x[M - 1 - g].x, x[M + 1 + g].y - x[M - 1 - g].y);
+      }
+#pragma unroll
+      for (int s = 0; s < V; ++s) {
+        C2 z, zm;
+        mirror_pair<R, M>(x[M], sg, d, ph[s], z, zm);
+        q[0][s] += z.x * z.x + z.y * z.y;
+        q[1][s] += zm.x * zm.x + zm.y * zm.y;
+      }
+#pragma unroll
+      for (int s = 0; s < V; ++s)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (f == 2) acc_m[h][s] += wl * q[h][s];
+          if (f == 3) acc_1[h][s] += w * q[h][s];
+          if (f == 8) acc_2[h][s] += w * q[h][s];
+        }
     }
   }
-  const long long ne = (long long)n0 * n1 * n2;
-  R* part = (R*)a.part + (long long)blockIdx.z * 3 * ne;
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (v >= jl) return;
+  const long long ne = n0 * jl;
+  R* part = (R*)a.part + (long long)blockIdx.z * 3 * ne + v;
 #pragma unroll
-  for (int s = 0; s < VPT; ++s) {
-    const int i = ig * VPT + s;
-    if (i < n0) {
-      const long long e = ((long long)i * n1 + j) * n2 + l;
-      part[e] = acc_m[s];
-      part[ne + e] = acc_1[s];
-      part[2 * ne + e] = acc_2[s];
+  for (int s = 0; s < V; ++s) {
+    const int i = ig * V + s;
+    if (i >= h0) break;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const long long e = (h ? n0 - 1 - i : i) * jl;
+      part[e] = acc_m[h][s];
+      part[ne + e] = acc_1[h][s];
+      part[2 * ne + e] = acc_2[h][s];
     }
   }
 }
@@ -360,29 +447,34 @@ size_t adjoint_staging_bytes(int M, int n1, int n2, bool fp32) {
   return elems * (fp32 ? sizeof(float2) : sizeof(double2));
 }
 
-// Voxels per thread of the reduction: 4 in FP32 (2 at M2 = 11), 1 in FP64 (register budget of
-// the phase tables).
+// Mirrored pairs per thread of the reduction: 4 in FP32 (2 at M = 5), 1 in FP64 (registers).
 template <typename R>
-constexpr int adj_vpt(int M2) { return sizeof(R) == sizeof(float) ? (M2 <= 9 ? 4 : 2) : 1; }
+constexpr int adj_pairs(int M) { return sizeof(R) == sizeof(float) ? (M <= 4 ? 4 : 2) : 1; }
 
-template <typename R>
-static int launch_adjoint_t(const AdjointArgs& a, cudaStream_t s) {
-  const int M2 = 2 * a.M + 1;
-  if (M2 > 11) return PC_EINVAL;
+template <typename R, int M>
+static int launch_adjoint_m(const AdjointArgs& a, cudaStream_t s) {
+  constexpr int M2 = 2 * M + 1, V = adj_pairs<R>(M);
   const size_t sm = adjoint_staging_bytes(a.M, a.n1, a.n2, sizeof(R) == sizeof(float));
   // Set once per instantiation; a function-local static is initialised exactly once even when
   // k groups on several host threads arrive together.
   static const cudaError_t attr =
-      cudaFuncSetAttribute(k_adj_synth12<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjointStagingMax);
+      cudaFuncSetAttribute(k_adj_synth12<R, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjointStagingMax);
   (void)attr;
   if (sm > kAdjointStagingMax) return PC_EINVAL;
   dim3 g1(a.max_pairs, 9);
-  k_adj_synth12<R><<<g1, 256, sm, s>>>(a);
+  const int jsplit = std::max(1, std::min((a.n1 + 1) / 2, (int)cdiv(768, M2 * a.n2)));
+  k_adj_synth12<R, M><<<g1, 256, sm, s>>>(a, jsplit);
   PC_LAUNCH_CHECK();
-  const int vpt = M2 <= 9 ? adj_vpt<R>(9) : adj_vpt<R>(11);
-  const long long gx = cdiv((long long)cdiv(a.n0, vpt) * a.n2, kAdjReduceThreads);
-  // enough pair chunks for about six blocks per SM; the chunks cover max_pairs, and the ones
-  // past the device's pair count write zeros
+  const int h0 = (a.n0 + 1) / 2;
+  const int nig = (int)cdiv(h0, V), wy = std::min(nig, kAdjReduceWarps);
+  const dim3 block(32, wy);
+  dim3 grid((unsigned)cdiv((long long)a.n1 * a.n2, 32), (unsigned)cdiv(nig, wy));
+  // as many pair chunks as are resident at once, so that no last wave is nearly empty; the chunks cover
+  // max_pairs, and the ones past the device's pair count write zeros
+  constexpr size_t ring = sizeof(typename cplx_t<R>::type) * kAdjStages * 9 * M2 * 32;
+  static const cudaError_t rattr =
+      cudaFuncSetAttribute(k_adj_reduce<R, M, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
+  (void)rattr;
   static const int sms = [] {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
@@ -390,23 +482,33 @@ static int launch_adjoint_t(const AdjointArgs& a, cudaStream_t s) {
     cudaGetLastError();
     return n;
   }();
-  int nchunks = (int)std::min<long long>(kAdjChunksMax, std::max<long long>(1, cdiv(6LL * sms, gx * a.n1)));
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_reduce<R, M, V>, 32 * wy, ring) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
+  }
+  int nchunks = (int)std::min<long long>(kAdjChunksMax, std::max<long long>(1, (long long)per_sm * sms / (grid.x * grid.y)));
   nchunks = std::max(1, std::min(nchunks, a.max_pairs));
   const int chunk = (int)cdiv(a.max_pairs, nchunks);
   nchunks = (int)cdiv(a.max_pairs, chunk);
-  dim3 g2((unsigned)gx, a.n1, nchunks);
-  switch (M2) {
-    case 3: k_adj_reduce<R, 3, adj_vpt<R>(3)><<<g2, kAdjReduceThreads, 0, s>>>(a, chunk); break;
-    case 5: k_adj_reduce<R, 5, adj_vpt<R>(5)><<<g2, kAdjReduceThreads, 0, s>>>(a, chunk); break;
-    case 7: k_adj_reduce<R, 7, adj_vpt<R>(7)><<<g2, kAdjReduceThreads, 0, s>>>(a, chunk); break;
-    case 9: k_adj_reduce<R, 9, adj_vpt<R>(9)><<<g2, kAdjReduceThreads, 0, s>>>(a, chunk); break;
-    default: k_adj_reduce<R, 11, adj_vpt<R>(11)><<<g2, kAdjReduceThreads, 0, s>>>(a, chunk); break;
-  }
+  grid.z = nchunks;
+  k_adj_reduce<R, M, V><<<grid, block, ring, s>>>(a, chunk);
   PC_LAUNCH_CHECK();
   const long long ne = (long long)a.n0 * a.n1 * a.n2;
   k_adj_finish<R><<<(unsigned)cdiv(ne, 256), 256, 0, s>>>(a, nchunks);
   PC_LAUNCH_CHECK();
   return PC_OK;
+}
+template <typename R>
+static int launch_adjoint_t(const AdjointArgs& a, cudaStream_t s) {
+  switch (a.M) {
+    case 1: return launch_adjoint_m<R, 1>(a, s);
+    case 2: return launch_adjoint_m<R, 2>(a, s);
+    case 3: return launch_adjoint_m<R, 3>(a, s);
+    case 4: return launch_adjoint_m<R, 4>(a, s);
+    case 5: return launch_adjoint_m<R, 5>(a, s);
+    default: return PC_EINVAL;
+  }
 }
 
 int launch_adjoint(const AdjointArgs& a, bool fp32, cudaStream_t s) {

@@ -230,10 +230,13 @@ struct AdjointArgs {
   double ve;             // element volume
   const double* dchi;
   void* t2;              // scratch: max_pairs x 9 x M2 x n1 x n2 complex (FP64 or FP32)
+  const void* phases;    // launch_adj_phases
   void* part;            // scratch: kAdjChunksMax x 3 x ne chunk sums (FP64 or FP32)
   double* grad;
 };
 constexpr int kAdjChunksMax = 32;  // pair chunks of the adjoint's reduction
+// Phases of the synthesis for a grid and cutoff: M (n0 + n1 + n2) complex values in the adjoint's precision.
+int launch_adj_phases(int M, const int n[3], bool fp32, void* ph, cudaStream_t s);
 // fp32: synthesis in FP32 (mixed form); the weighted sum is accumulated in FP64 either way.
 int launch_adjoint(const AdjointArgs& a, bool fp32, cudaStream_t s);
 // Dynamic shared memory of the adjoint's field-synthesis kernel: the N coefficients of one

@@ -92,6 +92,7 @@ struct pc_ctx {
   int *pairs = nullptr, *npairs = nullptr;
   double2* adj_t2 = nullptr;
   double* adj_part = nullptr;
+  double2* adj_ph = nullptr;  // phases of the adjoint's synthesis (room for FP64)
   float4* Kf = nullptr;  // FP32 wavevectors of the k-points, [k][N] (mixed form)  // chunk sums of the adjoint's reduction
   TcPlan* tc = nullptr;
   TcPlan* tcg[kMaxGroups] = {};  // workspaces of k groups 1.. (operators shared with tc)
@@ -263,7 +264,7 @@ extern "C" void pc_destroy(pc_ctx* c) {
   free_kset(c);
   dfree(c->fields); dfree(c->dchi); dfree(c->chi); dfree(c->chi_mean); dfree(c->dfc);
   dfree(c->t1); dfree(c->t2s); dfree(c->sfac); dfree(c->T); dfree(c->W); dfree(c->gj);
-  dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops); dfree(c->prec_ref);
+  dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops); dfree(c->prec_ref); dfree(c->adj_ph);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   for (cudaEvent_t e : {c->ev_s0, c->ev_s1, c->ev_g0, c->ev_g1})
@@ -399,6 +400,7 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
   rc |= dalloc(&c->gj, (size_t)setup_gj_scratch(N));
   rc |= dalloc(&c->status, 1);
   rc |= dalloc(&c->small_flops, 1);
+  rc |= dalloc(&c->adj_ph, (size_t)std::max(1, p->M * (p->n[0] + p->n[1] + p->n[2])));
   rc |= dalloc(&c->prec_ref, 3 * (size_t)kMaxGroups);
   if (p->precision == PC_MIXED) {
     rc |= dalloc(&c->Wf, 2 * NN);
@@ -411,6 +413,11 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
       cudaEventCreate(&c->ev_g0) != cudaSuccess || cudaEventCreate(&c->ev_g1) != cudaSuccess ||
       cudaMallocHost((void**)&c->h_count, 3 * kMaxGroups * sizeof(int)) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess) {
+    pc_destroy(c);
+    return PC_ECUDA;
+  }
+  if (launch_adj_phases(p->M, p->n, p->precision == PC_MIXED, c->adj_ph, 0) != PC_OK ||
+      cudaStreamSynchronize(0) != cudaSuccess) {
     pc_destroy(c);
     return PC_ECUDA;
   }
@@ -1194,6 +1201,7 @@ static int gap_and_grad_impl(pc_ctx* c, int n_lower, int mode, double beta, cons
     a.ve = c->ve;
     a.dchi = c->dchi;
     a.t2 = c->adj_t2;
+    a.phases = c->adj_ph;
     a.part = c->adj_part;
     a.grad = grad;
     int sl = ph_begin(c, PH_GRAD, 0.0, s);
