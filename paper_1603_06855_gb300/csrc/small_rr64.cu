@@ -17,11 +17,15 @@
 //
 // Two FP64 matrices (72 x 74 complex) and one FP32 matrix fit in shared memory; L, Q and E pass
 // through global scratch (L2), as do the logged rotations.
+#include <cooperative_groups.h>
 #include "jacobi.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 constexpr int S6_THREADS = 800;  // 25 warps: 4 for the planes, 21 for the 2 x 2 blocks at n = 72
 constexpr int S6_PB = 4;         // panel / row-block width (registers)
+constexpr int S6_CLUSTER = 8;    // CTAs per problem where these are few
 
 // Z = A B (herm: A^H B) for n x n matrices, or its upper triangle, in 2 x 2 tiles, up to two per thread
 // (n <= 72: 1296 tiles), which fill the lanes whatever n is; store(i, j, z) runs after every product is
@@ -75,8 +79,54 @@ __device__ __forceinline__ void tiles(int n, const double2* A, int lda, bool her
   __syncthreads();
 }
 
+// One CTA's share of Z = A B (herm: A^H B) or its upper triangle among CL, one output a thread, so that few
+// outputs still spread over the four FP64 units of every SM; `between` runs after the last read of an operand.
+template <int CL, bool UPPER, typename S, typename F>
+__device__ __forceinline__ void share(int rank, int n, const double2* A, int lda, bool herm, const double2* B, int ldb,
+                                      S between, F store) {
+  const int nt = UPPER ? n * (n + 1) / 2 : n * n, per = (nt + CL - 1) / CL;
+  constexpr int Q = (72 * 72 + CL * S6_THREADS - 1) / (CL * S6_THREADS);
+  const int hi = min(nt, (rank + 1) * per);
+  double2 z[Q];
+  int ti[Q], tj[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    int t = rank * per + threadIdx.x + q * S6_THREADS;
+    z[q] = make_double2(0.0, 0.0);
+    ti[q] = -1;
+    tj[q] = 0;
+    if (t < hi) {
+      int i = 0, j;
+      if (UPPER) {
+        while (t >= n - i) { t -= n - i; ++i; }
+        j = i + t;
+      } else {
+        i = t / n;
+        j = t - i * n;
+      }
+      ti[q] = i;
+      tj[q] = j;
+#pragma unroll 4
+      for (int p = 0; p < n; ++p) {
+        double2 a = herm ? A[p * lda + i] : A[i * lda + p];
+        if (herm) a.y = -a.y;
+        cfma(z[q], a, B[p * ldb + j]);
+      }
+    }
+  }
+  between();
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    if (ti[q] >= 0) store(ti[q], tj[q], z[q]);
+}
+
 }  // namespace
 
+// CL > 1: a cluster of CL CTAs per problem.  CTA 0 does everything but the four n x n products of the FP64
+// stage, which it shares with the others: they wait for its next product, copy what has changed of the
+// operands from its shared memory, and store their part of the result there.  For problems too few to fill
+// the chip (one per k-point): a product is bound by the FP64 unit of the SMs it runs on.
+template <int CL>
 __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA, MatRef<double> GO, int n, int m,
                                                           double drop_tol, const int* __restrict__ klist,
                                                             double* __restrict__ lam_out, double2* __restrict__ coef,
@@ -94,9 +144,9 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
   int* idx = drop + SR_NMAX;                 // SR_NMAX: position -> coordinate (-1: padding)
   int* perm = idx + SR_NMAX;                 // SR_NMAX
   int* low = perm + SR_NMAX;                 // SR_NMAX
-  int* misc = low + SR_NMAX;                 // 8
+  int* misc = low + SR_NMAX;                 // 8: [0] kept, [4..5] largest entry, [6] product, [7] X not orthonormal
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int k = blockIdx.x;                        // problem
+  const int k = blockIdx.x / CL;                   // problem
   const int kp = klist ? klist[k] : k;             // its k-point
   double2* Lg = (double2*)(scratch + k * stride);  // n x n: L
   double2* Qg = Lg + n * n;                        // n x n: Q
@@ -104,6 +154,63 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
   void* logk = Eg + n * n;                         // rotations
   double2* ck = coef + (long long)k * n * m;
   double2* cpk = cpo ? cpo + (long long)k * n * m : nullptr;
+  enum { DONE, GRAM_X, X_M, C_Q, QH_T };
+  // one of the products, by all CTAs of the cluster: f0, b0, b1, flag: CTA 0's F, B0, B1 and misc + 7
+  auto product = [&](int what, int rank, int nn, float2* f0, double2* b0, double2* b1, int* flag, auto between) {
+    if (what == GRAM_X)  // E = X^H X - I (upper triangle, mirrored)
+      share<CL, true>(rank, nn, B1, SR_LD, true, B1, SR_LD, between, [&](int i, int j, double2 g) {
+        if (j == i) g = make_double2(g.x - 1.0, 0.0);
+        Eg[i * n + j] = g;
+        Eg[j * n + i] = cconj(g);
+        f0[i * SR_LD + j] = make_float2((float)g.x, (float)g.y);
+        f0[j * SR_LD + i] = make_float2((float)g.x, (float)-g.y);
+        if (!(fabs(g.x) + fabs(g.y) < 1e-3)) *flag = 1;
+      });
+    else if (what == X_M)  // Q = X M
+      share<CL, false>(rank, nn, B1, SR_LD, false, Eg, n, between, [&](int i, int j, double2 v) {
+        b1[i * SR_LD + j] = v;
+        Qg[i * n + j] = v;
+      });
+    else if (what == C_Q)  // T = C Q
+      share<CL, false>(rank, nn, B0, SR_LD, false, B1, SR_LD, between, [&](int i, int j, double2 v) { b0[i * SR_LD + j] = v; });
+    else  // C' = Q^H T (upper triangle)
+      share<CL, true>(rank, nn, B1, SR_LD, true, B0, SR_LD, between, [&](int i, int j, double2 v) { b0[i * SR_LD + j] = v; });
+  };
+  if constexpr (CL > 1) {
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank();
+    if (rank > 0) {
+      float2* f0 = cl.map_shared_rank(F, 0);
+      double2 *b0 = cl.map_shared_rank(B0, 0), *b1 = cl.map_shared_rank(B1, 0);
+      int* m0 = cl.map_shared_rank(misc, 0);
+      for (;;) {
+        cl.sync();  // the next product is announced and its operands stand
+        const int what = m0[6], nn = m0[0];
+        if (what == DONE) break;
+        for (int i = warp; i < nn; i += W)
+          for (int j = lane; j < nn; j += 32) {
+            const int e = i * SR_LD + j;
+            if (what == GRAM_X || what == C_Q) B1[e] = b1[e];
+            if (what == C_Q || what == QH_T) B0[e] = b0[e];
+          }
+        __syncthreads();
+        product(what, rank, nn, f0, b0, b1, m0 + 7, [&] { cl.sync(); });
+        cl.sync();  // the result stands
+      }
+      cl.sync();  // CTA 0's shared memory has been read
+      return;
+    }
+  }
+  auto run = [&](int what) {  // CTA 0: the product by the whole cluster (misc[0] columns)
+    if constexpr (CL > 1) {
+      cg::cluster_group cl = cg::this_cluster();
+      if (tid == 0) misc[6] = what;
+      cl.sync();
+      if (what == DONE) return;
+      product(what, 0, misc[0], F, B0, B1, misc + 7, [&] { cl.sync(); });
+      cl.sync();
+    }
+  };
   // scaling, symmetrised copies
   for (int i = warp; i < n; i += W)
     for (int c = lane; c < n; c += 32) {
@@ -165,6 +272,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
     }
     for (int j = tid; j < m; j += S6_THREADS) lam_out[(long long)kp * m + j] = GA.at(k, j * n + j).x / GO.at(k, j * n + j).x;
     if (tid == 0) set_status(status, PC_ENOCONV);
+    run(DONE);
   } else {
     const int npad = nk_ + (nk_ & 1), np = npad / 2;
     // the kept coordinates of C, in position order, both triangles
@@ -208,17 +316,23 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
           B1[i * SR_LD + j] = make_double2(v.x, v.y);
         }
       __syncthreads();
-      // E = X^H X - I (upper triangle, mirrored)
-      bool bad = false;
-      tiles<true>(nk_, B1, SR_LD, true, B1, SR_LD, [&](int i, int j, double2 g) {
-        if (j == i) g = make_double2(g.x - 1.0, 0.0);
-        Eg[i * n + j] = g;
-        Eg[j * n + i] = cconj(g);
-        F[i * SR_LD + j] = make_float2((float)g.x, (float)g.y);
-        F[j * SR_LD + i] = make_float2((float)g.x, (float)-g.y);
-        bad |= !(fabs(g.x) + fabs(g.y) < 1e-3);
-      });
-      use_q = !__syncthreads_or(bad);
+      // E = X^H X - I
+      if (tid == 0) misc[7] = 0;
+      if constexpr (CL > 1) {
+        run(GRAM_X);
+        use_q = misc[7] == 0;
+      } else {
+        bool bad = false;
+        tiles<true>(nk_, B1, SR_LD, true, B1, SR_LD, [&](int i, int j, double2 g) {
+          if (j == i) g = make_double2(g.x - 1.0, 0.0);
+          Eg[i * n + j] = g;
+          Eg[j * n + i] = cconj(g);
+          F[i * SR_LD + j] = make_float2((float)g.x, (float)g.y);
+          F[j * SR_LD + i] = make_float2((float)g.x, (float)-g.y);
+          bad |= !(fabs(g.x) + fabs(g.y) < 1e-3);
+        });
+        use_q = !__syncthreads_or(bad);
+      }
       if (use_q) {
         for (int i = warp; i < nk_; i += W)
           for (int j = lane; j < nk_; j += 32) {
@@ -229,14 +343,21 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
           }
         __syncthreads();
         // Q = X M (in place), T = C Q (in place), C' = Q^H T (upper triangle, in place)
-        tiles<false>(nk_, B1, SR_LD, false, Eg, n, [&](int i, int j, double2 v) {
-          B1[i * SR_LD + j] = v;
-          Qg[i * n + j] = v;
-        });
-        tiles<false>(nk_, B0, SR_LD, false, B1, SR_LD, [&](int i, int j, double2 v) { B0[i * SR_LD + j] = v; });
-        tiles<true>(nk_, B1, SR_LD, true, B0, SR_LD, [&](int i, int j, double2 v) { B0[i * SR_LD + j] = v; });
+        if constexpr (CL > 1) {
+          run(X_M);
+          run(C_Q);
+          run(QH_T);
+        } else {
+          tiles<false>(nk_, B1, SR_LD, false, Eg, n, [&](int i, int j, double2 v) {
+            B1[i * SR_LD + j] = v;
+            Qg[i * n + j] = v;
+          });
+          tiles<false>(nk_, B0, SR_LD, false, B1, SR_LD, [&](int i, int j, double2 v) { B0[i * SR_LD + j] = v; });
+          tiles<true>(nk_, B1, SR_LD, true, B0, SR_LD, [&](int i, int j, double2 v) { B0[i * SR_LD + j] = v; });
+        }
       }
     }
+    run(DONE);
     // FP64 sweeps
     for (int i = warp; i < npad; i += W)
       for (int j = i + lane; j < npad; j += 32) {
@@ -281,6 +402,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
     pdir<double, S6_THREADS>(GO, k, n, m, pdir_abs, B0, B1, B1 + n * m, B1 + 2 * n * m, (double2*)F, (double2*)F + m * (m | 1),
                              ev, drop, cpk);
   }
+  if constexpr (CL > 1) cg::this_cluster().sync();  // the others have read this CTA's shared memory
 }
 
 // L, Q and E, and the planes (32 bytes) of the rotations of the most sweeps and of the round after them.
@@ -294,11 +416,37 @@ int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n,
   if (n > SR_NMAX || m > n || m > 24 || n < 1 || stride < small_rr64_scratch(n) || stride % 16) return PC_EINVAL;
   const size_t sm = sizeof(double2) * 2 * (size_t)SR_MAT + sizeof(float2) * SR_MAT + sizeof(Plane<double>) * 72 +
                     sizeof(double) * 2 * SR_NMAX + sizeof(int) * (4 * SR_NMAX + 8);
-  static const cudaError_t attr =  // once, thread-safe (k groups launch from several host threads)
-      cudaFuncSetAttribute(k_small_rr64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  (void)attr;
-  k_small_rr64<<<nk, S6_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
-                                          (unsigned char*)scratch, stride);
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 152;
+    cudaGetLastError();
+    return v;
+  }();
+  static const bool clusters =  // once, thread-safe (k groups launch from several host threads)
+      cudaFuncSetAttribute(k_small_rr64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
+      cudaFuncSetAttribute(k_small_rr64<S6_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess;
+  // A cluster per problem while the chip has an SM for each of its CTAs and there are products to share
+  // (n > m); 4 problems, n = 48, as the iteration calls it: 1.17 ms by one CTA each, 1.0 by clusters (reference solve 44.5 -> 40.1 ms).
+  if (clusters && n > m && (long long)nk * S6_CLUSTER <= sms) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nk * S6_CLUSTER);
+    cfg.blockDim = dim3(S6_THREADS);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = S6_CLUSTER;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, k_small_rr64<S6_CLUSTER>, GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
+                           (unsigned char*)scratch, stride) != cudaSuccess)
+      return PC_ECUDA;
+  } else {
+    k_small_rr64<1><<<nk, S6_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
+                                             (unsigned char*)scratch, stride);
+  }
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
