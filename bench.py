@@ -190,12 +190,12 @@ def run_reference(args):
 # kernel's source file when it was captured: once that file changes, the figure is stale and the
 # bench reports null.
 TRAFFIC = {  # DRAM bytes (read + write) per launch from ncu, single-stream pass of the FCC N = 729 workload
-    "k_tc_gram": {"source": "tall_tc.cu", "sha256": "78378b59f258febe9197fcc58c746a92767b5607aaf550d16906971e3962b04e", "bytes": 1.841e+08},
-    "k_tc_update": {"source": "tall_tc.cu", "sha256": "78378b59f258febe9197fcc58c746a92767b5607aaf550d16906971e3962b04e", "bytes": 2.772e+08},
-    "k_tc_gemm": {"source": "gemm_tc.cu", "sha256": "2c173663d760f16a1c803e148a9ef5a7323bdd3c7c262b5b58d0381bed90268f", "bytes": 3.159e+08},
-    "k_small_rr32": {"source": "small_rr.cu", "sha256": "caf29f36352a8d6c949bef63ca800f9978062abb8d790cd4568ff6464c5b4abb", "bytes": 7.744e+06},
-    "k_oz_gemm": {"source": "oz_gemm.cu", "sha256": "79dba0c8329328bf1c050d62d0a79c5b981615f008545982d8e2c97b98c3e863", "bytes": 2.75e+08},
-    "k_adj_synth12+k_adj_reduce": {"source": "adjoint.cu", "sha256": "997172643ab95aec17220765c988d0909ce1bba69a3b1003d49f11ec7982849f", "bytes": 1.398e+09},
+    "k_tc_gram": {"source": "tall_tc.cu", "sha256": "f4575f835187808ceabad893a22623c563e605714c8c7f79e966ee41d1230ca2", "bytes": 1.758e+08},
+    "k_tc_update": {"source": "tall_tc.cu", "sha256": "f4575f835187808ceabad893a22623c563e605714c8c7f79e966ee41d1230ca2", "bytes": 2.938e+08},
+    "k_tc_gemm": {"source": "gemm_tc.cu", "sha256": "49a21c2ec5a69e219d1425ff16f880f551d94ccff662c01000d4feea19966f47", "bytes": 2.578e+08},
+    "k_small_rr32": {"source": "small_rr.cu", "sha256": "89c478ea2d70331b548d063e7010181ef3d54e291d624f34e4c842a45bed9c6d", "bytes": 2.304e+07},
+    "k_oz_gemm": {"source": "oz_gemm.cu", "sha256": "66f77606c504fd7a37a983a2184decbdb7127e2c386dfdcc241f19010c6439be", "bytes": 3.350e+08},
+    "k_adj_synth12+k_adj_reduce": {"source": "adjoint.cu", "sha256": "fa1f321317bd747f25bba84e7cb49d207e16c593d6017cb200155cacad0aa812", "bytes": 1.397e+09},
 }
 
 

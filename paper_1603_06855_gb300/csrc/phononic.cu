@@ -239,12 +239,15 @@ static void free_kset(pc_ctx* c) {
   if (c->S) cudaFree(c->S); c->S = nullptr;
   void** vs[] = {&c->gpart, &c->GA, &c->GO, &c->Cc, &c->Ct, &c->lam};
   for (auto v : vs) { if (*v) cudaFree(*v); *v = nullptr; }
-  dfree(c->sr_scratch); dfree(c->rnorm); dfree(c->active); dfree(c->open_k); dfree(c->open_v); dfree(c->open_pos); dfree(c->fresh_k); dfree(c->d_count); dfree(c->kdone); dfree(c->kdone_f);
-  dfree(c->stall_best); dfree(c->stall_since);
+  dfree(c->sr_scratch);
+  dfree(c->open_k);  // and with it:
+  c->fresh_k = c->kdone = c->kdone_f = c->stall_since = c->open_v = c->open_pos = c->active = c->actived = nullptr;
+  c->d_count = c->pairs = c->npairs = nullptr;
+  dfree(c->GAd);  // and with it:
+  c->GOd = c->Cd = nullptr;
+  c->rnorm = c->lamd = c->rnormd = c->lam_nd = c->weights = c->stall_best = nullptr;
   dfree(c->Xd); dfree(c->AXd); dfree(c->OXd); dfree(c->Ed); dfree(c->Sd); dfree(c->Th); dfree(c->St);
-  dfree(c->gpartd); dfree(c->GAd); dfree(c->GOd); dfree(c->Cd);
-  dfree(c->lamd); dfree(c->lam_nd); dfree(c->rnormd); dfree(c->actived);
-  dfree(c->weights); dfree(c->pairs); dfree(c->npairs); dfree(c->adj_t2); dfree(c->adj_part); dfree(c->Kf);
+  dfree(c->gpartd); dfree(c->adj_t2); dfree(c->adj_part); dfree(c->Kf);
   for (auto& t : c->tcg)
     if (t) { tc_plan_destroy(t); t = nullptr; }
   if (c->tc) { tc_plan_destroy(c->tc); c->tc = nullptr; }
@@ -264,7 +267,7 @@ extern "C" void pc_destroy(pc_ctx* c) {
   free_kset(c);
   dfree(c->fields); dfree(c->dchi); dfree(c->chi); dfree(c->chi_mean); dfree(c->dfc);
   dfree(c->t1); dfree(c->t2s); dfree(c->sfac); dfree(c->T); dfree(c->W); dfree(c->gj);
-  dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops); dfree(c->prec_ref); dfree(c->adj_ph);
+  dfree(c->Wf); dfree(c->Tf); dfree(c->status); dfree(c->small_flops); dfree(c->adj_ph);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   for (cudaEvent_t e : {c->ev_s0, c->ev_s1, c->ev_g0, c->ev_g1})
@@ -376,10 +379,10 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
     c->pr.shift_scale = (sh && atof(sh) > 0) ? atof(sh) : 0.1;
   }
   {
-    // adjoint per weighted (k, band): 9 fields synthesised along axis 2 (M2^3 n2 complex
-    // multiply-adds), axis 1 (M2^2 n1 n2) and axis 0 inside the voxel reduction (M2 n0 n1 n2)
+    // adjoint per weighted (k, band): 9 fields synthesised along axis 2, axis 1 and axis 0 (inside the voxel
+    // reduction), 4 M real multiply-adds for two mirrored values
     const double m2 = M2, n0 = p->n[0], n1 = p->n[1], n2 = p->n[2];
-    c->grad_flops_per_pair = 8.0 * 9.0 * (m2 * m2 * m2 * n2 + m2 * m2 * n1 * n2 + m2 * n0 * n1 * n2);
+    c->grad_flops_per_pair = 4.0 * p->M * 9.0 * (m2 * m2 * n2 + m2 * n1 * n2 + n0 * n1 * n2);
   }
   c->pr.two_pi_sq_V_over_sA = two_pi * two_pi * c->V / c->sA;
   c->pr.half_lref_V_over_sA = 0.5 * c->lref * c->V / c->sA;
@@ -400,8 +403,10 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
   rc |= dalloc(&c->gj, (size_t)setup_gj_scratch(N));
   rc |= dalloc(&c->status, 1);
   rc |= dalloc(&c->small_flops, 1);
-  rc |= dalloc(&c->adj_ph, (size_t)std::max(1, p->M * (p->n[0] + p->n[1] + p->n[2])));
-  rc |= dalloc(&c->prec_ref, 3 * (size_t)kMaxGroups);
+  // one allocation: the phases, then the reference media
+  const size_t nph = (size_t)p->M * (p->n[0] + p->n[1] + p->n[2]);
+  rc |= dalloc(&c->adj_ph, nph + (3 * (size_t)kMaxGroups + 1) / 2);
+  if (c->adj_ph) c->prec_ref = (double*)(c->adj_ph + nph);
   if (p->precision == PC_MIXED) {
     rc |= dalloc(&c->Wf, 2 * NN);
     rc |= dalloc(&c->Tf, 3 * NN);
@@ -416,8 +421,8 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
     pc_destroy(c);
     return PC_ECUDA;
   }
-  if (launch_adj_phases(p->M, p->n, p->precision == PC_MIXED, c->adj_ph, 0) != PC_OK ||
-      cudaStreamSynchronize(0) != cudaSuccess) {
+  // done before any work of a caller's stream: pc_set_kpoints copies on the same (legacy) stream and waits
+  if (launch_adj_phases(p->M, p->n, p->precision == PC_MIXED, c->adj_ph, 0) != PC_OK) {
     pc_destroy(c);
     return PC_ECUDA;
   }
@@ -458,17 +463,37 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   c->sr_stride = c->prm.precision == PC_MIXED ? std::max(small_rr32_scratch(3 * m), small_rr64_scratch(m))
                                               : small_rr64_scratch(3 * m);
   rc |= dalloc(&c->sr_scratch, (size_t)nk * c->sr_stride);
-  rc |= dalloc(&c->rnorm, nvec);
-  rc |= dalloc(&c->active, nvec);
-  rc |= dalloc(&c->d_count, 3 * (size_t)kMaxGroups);
-  rc |= dalloc(&c->open_k, (size_t)nk);
-  rc |= dalloc(&c->fresh_k, (size_t)nk);
-  rc |= dalloc(&c->open_v, nvec);
-  rc |= dalloc(&c->open_pos, nvec);
-  rc |= dalloc(&c->kdone, (size_t)nk);
-  rc |= dalloc(&c->kdone_f, (size_t)nk);
-  rc |= dalloc(&c->stall_best, (size_t)nk);
-  rc |= dalloc(&c->stall_since, (size_t)nk);
+  // The small arrays in two allocations (25 us each).  [open_k | fresh_k | kdone | kdone_f | stall_since] per k,
+  // [open_v | open_pos | active | actived] per vector, d_count, pairs per (k, band), npairs:
+  const size_t nkb = (size_t)nk * c->nb;
+  rc |= dalloc(&c->open_k, 5 * (size_t)nk + 4 * nvec + 3 * (size_t)kMaxGroups + nkb + 1);
+  if (c->open_k) {
+    c->fresh_k = c->open_k + nk;
+    c->kdone = c->fresh_k + nk;
+    c->kdone_f = c->kdone + nk;
+    c->stall_since = c->kdone_f + nk;
+    c->open_v = c->stall_since + nk;
+    c->open_pos = c->open_v + nvec;
+    c->active = c->open_pos + nvec;
+    c->actived = c->active + nvec;
+    c->d_count = c->actived + nvec;
+    c->pairs = c->d_count + 3 * kMaxGroups;
+    c->npairs = c->pairs + nkb;
+  }
+  // [GAd | GOd | Cd] m x m complex per k, then [rnorm | lamd | rnormd] per vector, [lam_nd | weights] per (k, band),
+  // stall_best per k
+  const size_t nmm = (size_t)nk * m * m;
+  rc |= dalloc(&c->GAd, 3 * nmm + (3 * nvec + 2 * nkb + nk + 1) / 2);
+  if (c->GAd) {
+    c->GOd = c->GAd + nmm;
+    c->Cd = c->GOd + nmm;
+    c->rnorm = (double*)(c->Cd + nmm);
+    c->lamd = c->rnorm + nvec;
+    c->rnormd = c->lamd + nvec;
+    c->lam_nd = c->rnormd + nvec;
+    c->weights = c->lam_nd + nkb;
+    c->stall_best = c->weights + nkb;
+  }
   rc |= dalloc(&c->Xd, nvec * n3);
   rc |= dalloc(&c->AXd, nvec * n3);
   rc |= dalloc(&c->OXd, nvec * n3);
@@ -477,16 +502,6 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   rc |= dalloc(&c->Sd, 6 * nvec * N);
   rc |= dalloc(&c->St, 6 * nvec * N);
   rc |= dalloc(&c->gpartd, 8 * (size_t)nk * m * m);
-  rc |= dalloc(&c->GAd, (size_t)nk * m * m);
-  rc |= dalloc(&c->GOd, (size_t)nk * m * m);
-  rc |= dalloc(&c->Cd, (size_t)nk * m * m);
-  rc |= dalloc(&c->lamd, nvec);
-  rc |= dalloc(&c->lam_nd, (size_t)nk * c->nb);
-  rc |= dalloc(&c->rnormd, nvec);
-  rc |= dalloc(&c->actived, nvec);
-  rc |= dalloc(&c->weights, (size_t)nk * c->nb);
-  rc |= dalloc(&c->pairs, (size_t)nk * c->nb);
-  rc |= dalloc(&c->npairs, 1);
   rc |= dalloc(&c->adj_t2, (size_t)nk * c->nb * 9 * c->M2 * c->prm.n[1] * c->prm.n[2]);
   rc |= dalloc(&c->adj_part, (size_t)kAdjChunksMax * 3 * c->prm.n[0] * c->prm.n[1] * c->prm.n[2]);
   if (rc == PC_OK && c->prm.precision == PC_MIXED) {
@@ -911,7 +926,7 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
       for (int k = 0; k < nk; ++k)
         for (int j = 0; j < nb; ++j) {
           if (h[k * m + j] > mx) { mx = h[k * m + j]; kmx = k; }
-          if (!kd[k] && h[k * m + j] > mxo) { mxo = h[k * m + j]; kmxo = k; }
+          if (kd[k] != 1 && h[k * m + j] > mxo) { mxo = h[k * m + j]; kmxo = k; }
         }
       fprintf(stderr, "[pc] k %d+ it %d unconverged_k %d max_res %.3e at k %d; open k: max_res %.3e at k %d\n", k0,
               it, ks.unconv, mx, kmx + k0, mxo, kmxo < 0 ? -1 : kmxo + k0);

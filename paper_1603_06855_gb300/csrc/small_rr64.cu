@@ -428,6 +428,7 @@ int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n,
       cudaFuncSetAttribute(k_small_rr64<S6_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess;
   // A cluster per problem while the chip has an SM for each of its CTAs and there are products to share
   // (n > m); 4 problems, n = 48, as the iteration calls it: 1.17 ms by one CTA each, 1.0 by clusters (reference solve 44.5 -> 40.1 ms).
+  bool launched = false;
   if (clusters && n > m && (long long)nk * S6_CLUSTER <= sms) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nk * S6_CLUSTER);
@@ -440,13 +441,13 @@ int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n,
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, k_small_rr64<S6_CLUSTER>, GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
-                           (unsigned char*)scratch, stride) != cudaSuccess)
-      return PC_ECUDA;
-  } else {
+    launched = cudaLaunchKernelEx(&cfg, k_small_rr64<S6_CLUSTER>, GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs,
+                                  status, (unsigned char*)scratch, stride) == cudaSuccess;
+    if (!launched) cudaGetLastError();  // no room for a cluster here: one CTA per problem
+  }
+  if (!launched)
     k_small_rr64<1><<<nk, S6_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
                                              (unsigned char*)scratch, stride);
-  }
   PC_LAUNCH_CHECK();
   return PC_OK;
 }
