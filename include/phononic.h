@@ -269,6 +269,7 @@ int pc_design_project(pc_design* d, const double* x_dev, double beta, double* rh
 
 /* g_x_dev (nvars doubles) <- d(objective)/dx from g_rho_dev = d(objective)/d(rho_e) (n0 n1 n2
  * doubles), at the x and beta of the last pc_design_project on this map (stream ordered after it).
+ * Calls with different gradients may overlap, on several streams and threads.
  * Errors: PC_EINVAL (NULL), PC_ECUDA. */
 int pc_design_backprop(pc_design* d, const double* g_rho_dev, double* g_x_dev, void* stream);
 

@@ -15,7 +15,9 @@
 // and every node (backward: gather over the elements e = spacing (a - d) + p of each class).
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 #include "kernels.h"
 
@@ -33,7 +35,11 @@ struct pc_design {
   DesignEntry* table = nullptr;  // entries of class 0, then class 1, ...
   int* class_start = nullptr;    // nclass + 1 offsets into table
   double* dmu = nullptr;         // ne, d rho / d mu of the last projection
-  double* gmu = nullptr;         // ne, dG/dmu (large maps)
+  double* gmu = nullptr;         // ne, dG/dmu (large maps); the members below say whose (gmu_claim)
+  std::mutex gmu_lock;
+  cudaEvent_t gmu_read = nullptr;       // after the last launch that reads gmu
+  unsigned long long gmu_stream = 0;    // and the identity of its stream
+  bool gmu_used = false;
 };
 
 namespace {
@@ -154,6 +160,27 @@ __global__ void k_project_grad(const double* __restrict__ g, const double* __res
 }
 constexpr long long GRAD_PASS = 1 << 18;
 
+// Whether a call on stream s (identity id) may write the map's gmu: the last launch that reads it is done, or ahead
+// on the same stream.  Gradients of one projection (objective and constraint) may be carried back on several
+// streams at once, and a captured call replays whenever its graph is launched: these take the kernel without
+// gmu, which gives the same bits.
+bool gmu_claim(pc_design* d, cudaStream_t s, unsigned long long* id) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  bool ok = cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
+            cudaStreamGetId(s, id) == cudaSuccess;
+  if (ok && d->gmu_used && d->gmu_stream != *id) {
+    // the event is none of any capture's, so the query disturbs none, whatever another thread records
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+    if (ok) {
+      ok = cudaEventQuery(d->gmu_read) == cudaSuccess;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+  }
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 void lattice_columns(int lat, double a, double A[9]) {
   // columns a_1, a_2, a_3 (A[r*3+c] = component r of a_c)
   static const double P[3][3][3] = {{{1, 0, 0}, {0, 1, 0}, {0, 0, 1}},
@@ -257,7 +284,13 @@ extern "C" int pc_design_create(const pc_params* cell, const pc_design_params* d
   d->table = (DesignEntry*)(base + 64 * sizeof(double));
   d->class_start = (int*)(base + 64 * sizeof(double) + ts);
   d->dmu = (double*)(base + head);
-  if (d->ne >= GRAD_PASS) d->gmu = (double*)(base + head + field);
+  if (d->ne >= GRAD_PASS) {
+    if (cudaEventCreateWithFlags(&d->gmu_read, cudaEventDisableTiming) != cudaSuccess) {
+      pc_design_destroy(d);
+      return PC_ECUDA;
+    }
+    d->gmu = (double*)(base + head + field);
+  }
   std::vector<unsigned char> stage(head, 0);
   for (int j = 0; j < 64; ++j) ((double*)stage.data())[j] = std::exp2(j / 64.0);
   memcpy(stage.data() + 64 * sizeof(double), tab.data(), ts);
@@ -289,21 +322,35 @@ extern "C" int pc_design_backprop(pc_design* d, const double* g_rho, double* g_x
   cudaGetLastError();
   cudaStream_t s = (cudaStream_t)stream;
   const double* g = g_rho;
-  if (d->gmu) {
-    k_grad_mu<<<cdiv(d->ne, 256), 256, 0, s>>>(g_rho, d->dmu, d->ne, d->gmu);
-    PC_LAUNCH_CHECK();
-    g = d->gmu;
+  std::unique_lock<std::mutex> lock(d->gmu_lock, std::defer_lock);
+  double* gmu = nullptr;
+  unsigned long long id = 0;
+  if (d->ne >= GRAD_PASS) {
+    lock.lock();
+    if (d->gmu && gmu_claim(d, s, &id)) std::swap(gmu, d->gmu);  // given back once its event is recorded
   }
-  auto kernel = d->octant ? (d->gmu ? k_project_grad<true, true> : k_project_grad<false, true>)
-                          : (d->gmu ? k_project_grad<true, false> : k_project_grad<false, false>);
+  if (gmu) {
+    k_grad_mu<<<cdiv(d->ne, 256), 256, 0, s>>>(g_rho, d->dmu, d->ne, gmu);
+    PC_LAUNCH_CHECK();
+    g = gmu;
+  }
+  auto kernel = d->octant ? (gmu ? k_project_grad<true, true> : k_project_grad<false, true>)
+                          : (gmu ? k_project_grad<true, false> : k_project_grad<false, false>);
   kernel<<<cdiv(d->nnodes, 128), 128, 0, s>>>(g, d->dmu, d->table, d->class_start, d->nclass, d->n[1], d->n[2], d->nd[0],
                                               d->nd[1], d->nd[2], d->spacing, g_x);
   PC_LAUNCH_CHECK();
+  if (gmu) {
+    PC_CUDA_TRY(cudaEventRecord(d->gmu_read, s));
+    d->gmu_stream = id;
+    d->gmu_used = true;
+    d->gmu = gmu;
+  }
   return PC_OK;
 }
 
 extern "C" void pc_design_destroy(pc_design* d) {
   if (!d) return;
   if (d->exp2t) cudaFree(d->exp2t);
+  if (d->gmu_read) cudaEventDestroy(d->gmu_read);
   delete d;
 }
