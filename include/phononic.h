@@ -92,15 +92,17 @@ typedef struct {
   double tol;           /* relative residual target of the block iteration (0: default, 1e-8 FP64, 3e-4 mixed).
                            A gradient through one (k, band) pair (a gap) has a relative error of
                            about that pair's final residual: for a 1e-4 gap gradient in the mixed
-                           form pass tol = 1e-4 (the default suits all-band weighted objectives). */
-  int max_iter;         /* iteration cap (0: default); hitting it sets PC_ENOCONV */
+                           form pass tol = 1e-4 (the default suits all-band weighted objectives).
+                           The iteration aims at half of it: a k-point between the two gets one more
+                           iteration, but counts as converged. */
+  int max_iter;         /* iteration cap (0: default); hitting it above the tolerance sets PC_ENOCONV */
   int law;              /* PC_LAW_COMPLIANCE (0, default) | PC_LAW_YOUNG; density is linear in chi either way */
 } pc_params;
 
 typedef struct {
   int status;              /* first device error code seen (PC_OK if none) */
   int iterations;          /* block iterations of the last pc_bands */
-  int unconverged_k;       /* k-points above tolerance when the iteration stopped */
+  int unconverged_k;       /* k-points above tolerance at the last check before the iteration stopped */
   int nk;                  /* k-points set */
   int N;                   /* plane waves */
   int block;               /* block width m (bands + guard vectors) */

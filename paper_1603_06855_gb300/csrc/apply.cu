@@ -267,13 +267,13 @@ __global__ void k_resnorm(const typename cplx_t<R>::type* __restrict__ AX, const
 __global__ __launch_bounds__(256) void k_open(const int* __restrict__ active, const double* __restrict__ rnorm, double tol,
                                               int nopen, int m, int nb, int* __restrict__ kdone, double* __restrict__ best,
                                               int* __restrict__ since, OpenSet o, int lists) {
-  __shared__ int sums[3][8], base[3];
+  __shared__ int sums[4][8], base[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (tid < 3) base[tid] = 0;
+  if (tid < 4) base[tid] = 0;
   __syncthreads();
   for (int p0 = 0; p0 < nopen; p0 += 256) {
     const int p = p0 + tid;
-    int k = -1, open = 0, fresh = 0, cols = 0;
+    int k = -1, open = 0, fresh = 0, cols = 0, above = 0;
     if (p < nopen) {
       k = lists ? o.klist[p] : p;
       int a = 0;
@@ -301,11 +301,12 @@ __global__ __launch_bounds__(256) void k_open(const int* __restrict__ active, co
       if (done || kdone[k] != 2) kdone[k] = done ? 1 : 0;
       open = done ? 0 : 1;
       fresh = done ? 1 : 0;
+      above = open && worst > tol ? 1 : 0;
       if (done) cols = 0;
     }
-    int v[3] = {open, cols, fresh}, x[3];
+    int v[4] = {open, cols, fresh, above}, x[4];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
+    for (int i = 0; i < 4; ++i) {
       x[i] = v[i];
       for (int d = 1; d < 32; d <<= 1) {
         const int y = __shfl_up_sync(0xffffffffu, x[i], d);
@@ -330,11 +331,11 @@ __global__ __launch_bounds__(256) void k_open(const int* __restrict__ active, co
         }
     }
     __syncthreads();
-    if (tid < 3)
+    if (tid < 4)
       for (int w = 0; w < 8; ++w) base[tid] += sums[tid][w];
     __syncthreads();
   }
-  if (tid < 3) o.count[tid] = base[tid];
+  if (tid < 4) o.count[tid] = base[tid];
 }
 // All k-points open; and the reference medium of the preconditioner, from the mean chi.
 __global__ void k_open_all(int* klist, int nk, PrecRef pr, const double* __restrict__ chi_mean, double* __restrict__ ref) {

@@ -92,7 +92,7 @@ struct PrecRef {  // reference medium from the mean of chi (device scalar)
 };
 // k-points still iterated, kept on the device and counted on the host: klist the open k-points in
 // order, vlist their unconverged vectors (k m + j), fresh the k-points that the last test locked, count
-// {open, unconverged vectors, fresh}.
+// {open, unconverged vectors, fresh, open ones above the tolerance}: an open k-point may have met it.
 struct OpenSet {
   int *klist, *vlist, *fresh, *count;
   int* vpos;  // position of an open k-point's vector in vlist, or -1

@@ -60,7 +60,7 @@ struct pc_ctx {
   cudaEvent_t ev_s0 = nullptr, ev_s1 = nullptr;        // pc_set_design
   cudaEvent_t ev_g0 = nullptr, ev_g1 = nullptr;        // pc_gap_and_grad
   bool have_grad_events = false;
-  int* h_count = nullptr;   // pinned, 3 per k group (OpenSet::count)
+  int* h_count = nullptr;   // pinned, 4 per k group (OpenSet::count)
   // per-design (FP64)
   double *fields = nullptr, *dchi = nullptr, *chi = nullptr, *chi_mean = nullptr, *dfc = nullptr;
   double2 *t1 = nullptr, *t2s = nullptr, *sfac = nullptr, *T = nullptr, *W = nullptr, *gj = nullptr;
@@ -416,7 +416,7 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
       cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess ||
       cudaEventCreate(&c->ev_s0) != cudaSuccess || cudaEventCreate(&c->ev_s1) != cudaSuccess ||
       cudaEventCreate(&c->ev_g0) != cudaSuccess || cudaEventCreate(&c->ev_g1) != cudaSuccess ||
-      cudaMallocHost((void**)&c->h_count, 3 * kMaxGroups * sizeof(int)) != cudaSuccess ||
+      cudaMallocHost((void**)&c->h_count, 4 * kMaxGroups * sizeof(int)) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess) {
     pc_destroy(c);
     return PC_ECUDA;
@@ -466,7 +466,7 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   // The small arrays in two allocations (25 us each).  [open_k | fresh_k | kdone | kdone_f | stall_since] per k,
   // [open_v | open_pos | active | actived] per vector, d_count, pairs per (k, band), npairs:
   const size_t nkb = (size_t)nk * c->nb;
-  rc |= dalloc(&c->open_k, 5 * (size_t)nk + 4 * nvec + 3 * (size_t)kMaxGroups + nkb + 1);
+  rc |= dalloc(&c->open_k, 5 * (size_t)nk + 4 * nvec + 4 * (size_t)kMaxGroups + nkb + 1);
   if (c->open_k) {
     c->fresh_k = c->open_k + nk;
     c->kdone = c->fresh_k + nk;
@@ -477,7 +477,7 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
     c->active = c->open_pos + nvec;
     c->actived = c->active + nvec;
     c->d_count = c->actived + nvec;
-    c->pairs = c->d_count + 3 * kMaxGroups;
+    c->pairs = c->d_count + 4 * kMaxGroups;
     c->npairs = c->pairs + nkb;
   }
   // [GAd | GOd | Cd] m x m complex per k, then [rnorm | lamd | rnormd] per vector, [lam_nd | weights] per (k, band),
@@ -700,7 +700,7 @@ struct KSet {
 };
 
 static OpenSet open_set(const pc_ctx* c, int k0, int group) {
-  return OpenSet{c->open_k + k0, c->open_v + (long long)k0 * c->m, c->fresh_k + k0, c->d_count + 3 * group,
+  return OpenSet{c->open_k + k0, c->open_v + (long long)k0 * c->m, c->fresh_k + k0, c->d_count + 4 * group,
                  c->open_pos + (long long)k0 * c->m};
 }
 
@@ -908,12 +908,13 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
       hasP = false;
     }
     TRY(launch_resnorm<R>(AX, OX, lam, nk, m, nb, n3, c->prm.tol, rnorm, active, kdone, o, nopen, s, sbest, ssince));
-    PC_CUDA_TRY(cudaMemcpyAsync(ks.h_count, o.count, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    PC_CUDA_TRY(cudaMemcpyAsync(ks.h_count, o.count, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
     // While profiling, the stream's idle gap while the host waits for the count and enqueues the
     // next step: from the completion of the copy to the next work the host enqueues.
     const int idle_slot = ph_begin(c, PH_IDLE, 0.0, s);
     PC_CUDA_TRY(cudaStreamSynchronize(s));
-    ks.unconv = nopen = ks.h_count[0];
+    nopen = ks.h_count[0];
+    ks.unconv = ks.h_count[3];  // what the call reports: open k-points may have met the tolerance already
     const int ncol = ks.h_count[1], nfresh = ks.h_count[2];
     if (c->debug) {
       const int nv = nk * m;
@@ -1030,7 +1031,7 @@ static int run_split_iteration(pc_ctx* c, cudaStream_t s) {
     ks[g].s = c->sk[g];
     ks[g].group = g;
     ks[g].open = open_set(c, ks[g].k0, g);
-    ks[g].h_count = c->h_count + 3 * g;
+    ks[g].h_count = c->h_count + 4 * g;
     ks[g].tc = g ? c->tcg[g] : c->tc;
     ks[g].oz = (c->oz_ready && c->oz) ? (g ? c->ozg[g] : c->oz) : nullptr;
     PC_CUDA_TRY(cudaStreamWaitEvent(c->sk[g], c->ev_fork, 0));
