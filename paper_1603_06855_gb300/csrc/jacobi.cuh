@@ -675,6 +675,31 @@ __device__ __forceinline__ void replay(const Plane<R>* __restrict__ logk, int K,
   __syncthreads();
 }
 
+// The factor that makes nearly orthonormal columns X orthonormal in FP64: E = X^H X - I (n x n, row stride lde, and
+// in FP32 in F, stride SR_LD) is replaced by M = I - E/2 + 3/8 E^2, the binomial series of (I + E)^-1/2; E^2 by
+// FP32 products (their rounding stays below 1e-16 for the E let through).  Q = X M has Q^H Q - I = -5/8 E^3 to
+// leading order.  Returns, to all threads, whether that is below FP64's rounding: ||E^3|| <= ||E^2||^1.5, and the row
+// sums of |E^2|, which bound that norm, are held to 1e-10 (6e-16 is left).  Columns from rotations in FP32 have row sums of
+// 2e-12 (n = 24) to 2.2e-11 (n = 72) at most on the reference solves' problems.
+template <int THREADS>
+__device__ __forceinline__ bool orthonormal_factor(const float2* F, double2* E, int lde, int n) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  bool bad = false;
+  for (int i = warp; i < n; i += THREADS / 32) {
+    float row = 0.f;
+    for (int j = lane; j < n; j += 32) {
+      float2 q = make_float2(0.f, 0.f);
+      for (int p = 0; p < n; ++p) cfma(q, F[i * SR_LD + p], F[p * SR_LD + j]);
+      row += fabsf(q.x) + fabsf(q.y);
+      const double2 e = E[i * lde + j];
+      E[i * lde + j] = make_double2((i == j ? 1.0 : 0.0) - 0.5 * e.x + 0.375 * q.x, -0.5 * e.y + 0.375 * q.y);
+    }
+    for (int o = 16; o > 0; o >>= 1) row += __shfl_xor_sync(0xffffffffu, row, o);
+    bad |= !(row <= 1e-10f);  // also NaN
+  }
+  return !__syncthreads_or(bad);
+}
+
 // Conjugate-direction coefficients, inside the CTA that solved the projected problem.  With the
 // Ritz coefficients cX (n x m, cX^H GO cX = I) of the basis S = [X_old, W, P_old], the next
 // conjugate block spans the part of span(X_old) that is GO-orthogonal to the new Ritz block:

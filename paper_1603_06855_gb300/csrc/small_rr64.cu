@@ -5,11 +5,11 @@
 // takes some ten sweeps of 6 n^3 FP64 multiply-adds (and as many for V).  So where the basis holds
 // search directions (n > m) the matrix C = L^-1 GA L^-H is first diagonalised in FP32 (six sweeps at
 // FP32 rates, the replayed rotations give the eigenvectors X of its rounded copy, orthonormal to 1e-6),
-// X is made orthonormal in FP64, Q = X (I - E/2 + 3/8 E^2) with E = X^H X - I (the next term is 1e-18; E^2
-// needs only FP32), and C' = Q^H C Q, diagonal to 1e-7, takes one or two FP64 sweeps; the result is that of
-// the FP64 iteration (same convergence test, same floor).  A problem whose X is not orthonormal to 1e-3
-// (overflow or NaN in FP32) is diagonalised from C itself.  Rayleigh-Ritz of Ritz vectors (n = m) is nearly
-// diagonal already and goes to FP64 directly.
+// X is made orthonormal in FP64, Q = X (I - E/2 + 3/8 E^2) with E = X^H X - I (orthonormal_factor), and
+// C' = Q^H C Q, diagonal to 1e-7, takes one or two FP64 sweeps; Q is orthonormal to FP64's rounding, so the
+// result is that of the FP64 iteration (same convergence test, same floor).  A problem whose X is further off
+// than that series reaches (overflow or NaN in FP32 among them) is diagonalised from C itself.
+// Rayleigh-Ritz of Ritz vectors (n = m) is nearly diagonal already and goes to FP64 directly.
 //
 // With the conjugate directions, per launch of the reference solves' problems (4 to 6): n = 48 5.6 -> 1.5 ms,
 // n = 30 2.4 -> 0.56 ms; n = 72 18 -> 5.6 ms.  What is left: products 0.35, the FP64 sweep 0.33, FP32 stage 0.19,
@@ -144,7 +144,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
   int* idx = drop + SR_NMAX;                 // SR_NMAX: position -> coordinate (-1: padding)
   int* perm = idx + SR_NMAX;                 // SR_NMAX
   int* low = perm + SR_NMAX;                 // SR_NMAX
-  int* misc = low + SR_NMAX;                 // 8: [0] kept, [4..5] largest entry, [6] product, [7] X not orthonormal
+  int* misc = low + SR_NMAX;                 // 8: [0] kept, [4..5] largest entry, [6] product
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int k = blockIdx.x / CL;                   // problem
   const int kp = klist ? klist[k] : k;             // its k-point
@@ -155,8 +155,8 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
   double2* ck = coef + (long long)k * n * m;
   double2* cpk = cpo ? cpo + (long long)k * n * m : nullptr;
   enum { DONE, GRAM_X, X_M, C_Q, QH_T };
-  // one of the products, by all CTAs of the cluster: f0, b0, b1, flag: CTA 0's F, B0, B1 and misc + 7
-  auto product = [&](int what, int rank, int nn, float2* f0, double2* b0, double2* b1, int* flag, auto between) {
+  // one of the products, by all CTAs of the cluster: f0, b0, b1: CTA 0's F, B0, B1
+  auto product = [&](int what, int rank, int nn, float2* f0, double2* b0, double2* b1, auto between) {
     if (what == GRAM_X)  // E = X^H X - I (upper triangle, mirrored)
       share<CL, true>(rank, nn, B1, SR_LD, true, B1, SR_LD, between, [&](int i, int j, double2 g) {
         if (j == i) g = make_double2(g.x - 1.0, 0.0);
@@ -164,7 +164,6 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
         Eg[j * n + i] = cconj(g);
         f0[i * SR_LD + j] = make_float2((float)g.x, (float)g.y);
         f0[j * SR_LD + i] = make_float2((float)g.x, (float)-g.y);
-        if (!(fabs(g.x) + fabs(g.y) < 1e-3)) *flag = 1;
       });
     else if (what == X_M)  // Q = X M
       share<CL, false>(rank, nn, B1, SR_LD, false, Eg, n, between, [&](int i, int j, double2 v) {
@@ -194,7 +193,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
             if (what == C_Q || what == QH_T) B0[e] = b0[e];
           }
         __syncthreads();
-        product(what, rank, nn, f0, b0, b1, m0 + 7, [&] { cl.sync(); });
+        product(what, rank, nn, f0, b0, b1, [&] { cl.sync(); });
         cl.sync();  // the result stands
       }
       cl.sync();  // CTA 0's shared memory has been read
@@ -207,7 +206,7 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
       if (tid == 0) misc[6] = what;
       cl.sync();
       if (what == DONE) return;
-      product(what, 0, misc[0], F, B0, B1, misc + 7, [&] { cl.sync(); });
+      product(what, 0, misc[0], F, B0, B1, [&] { cl.sync(); });
       cl.sync();
     }
   };
@@ -317,31 +316,19 @@ __global__ __launch_bounds__(S6_THREADS, 1) void k_small_rr64(MatRef<double> GA,
         }
       __syncthreads();
       // E = X^H X - I
-      if (tid == 0) misc[7] = 0;
       if constexpr (CL > 1) {
         run(GRAM_X);
-        use_q = misc[7] == 0;
       } else {
-        bool bad = false;
         tiles<true>(nk_, B1, SR_LD, true, B1, SR_LD, [&](int i, int j, double2 g) {
           if (j == i) g = make_double2(g.x - 1.0, 0.0);
           Eg[i * n + j] = g;
           Eg[j * n + i] = cconj(g);
           F[i * SR_LD + j] = make_float2((float)g.x, (float)g.y);
           F[j * SR_LD + i] = make_float2((float)g.x, (float)-g.y);
-          bad |= !(fabs(g.x) + fabs(g.y) < 1e-3);
         });
-        use_q = !__syncthreads_or(bad);
       }
+      use_q = orthonormal_factor<S6_THREADS>(F, Eg, n, nk_);
       if (use_q) {
-        for (int i = warp; i < nk_; i += W)
-          for (int j = lane; j < nk_; j += 32) {
-            float2 q = make_float2(0.f, 0.f);
-            for (int p = 0; p < nk_; ++p) cfma(q, F[i * SR_LD + p], F[p * SR_LD + j]);
-            const double2 e = Eg[i * n + j];
-            Eg[i * n + j] = make_double2((i == j ? 1.0 : 0.0) - 0.5 * e.x + 0.375 * q.x, -0.5 * e.y + 0.375 * q.y);
-          }
-        __syncthreads();
         // Q = X M (in place), T = C Q (in place), C' = Q^H T (upper triangle, in place)
         if constexpr (CL > 1) {
           run(X_M);
