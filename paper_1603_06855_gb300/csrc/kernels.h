@@ -183,12 +183,13 @@ int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s);
 // iteration come from the same CTA (directions at or below pdir_abs dropped); when flops is given, the
 // algorithmic flops of every problem solved are added to it (device counter).  scratch: global scratch of
 // `stride` bytes per problem, at least small_rr32_scratch(n) / small_rr64_scratch(n), a multiple of 16.
+// others: problems that other calls are solving meanwhile (launch_rules.h).
 int launch_small_rr32(const MatRef<float>& GA, const MatRef<float>& GO, int n, int m, int nk, float drop_tol, const int* klist,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
                       void* scratch, long long stride, cudaStream_t s);
 int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n, int m, int nk, double drop_tol, const int* klist,
                       double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
-                      long long stride, cudaStream_t s);
+                      long long stride, long long others, cudaStream_t s);
 long long small_rr32_scratch(int n);
 long long small_rr64_scratch(int n);
 // Cholesky-QR transform of the Gram matrices G (m x m).

@@ -1,0 +1,15 @@
+// Rules that choose between launch forms, in plain C++ (also compiled for the host alone, to be checked).
+#pragma once
+
+// CTAs of a cluster that shares one FP64 projected problem (small_rr64.cu).
+constexpr int kRr64Cluster = 8;
+
+// Whether each of nk FP64 projected problems (n basis columns, m wanted) gets a cluster.  The cluster shares the
+// four products of the FP32 stage's correction (n > m) and its CTAs take a whole SM each, so it pays while
+// there is an SM for every CTA, counting the `others` problems that calls running beside this one solve.
+// Solves of 12 bands at N = 125, 4 k-points each, by clusters or one CTA a problem: one design 37.4 and 41.4 ms, two
+// 41.2 and 43.3, four 52.2 and 53.2 (128 CTAs), eight 79 and 61, sixteen 148 and 110; two of 12 k-points 62 and 57;
+// sixteen of 14 k-points, 6 bands at N = 27, 112 and 43.
+inline bool rr64_uses_clusters(int n, int m, long long nk, long long others, int sms) {
+  return n > m && kRr64Cluster * (nk + others) <= sms;
+}

@@ -774,6 +774,15 @@ static MatRef<R> mats(const void* p, long long nel) {
   return r;
 }
 
+// k-points of the pc_bands calls running in this process (from other threads too): how many projected problems
+// may want an SM at once.  It only chooses between launch forms of the same bits.
+static std::atomic<long long> g_running_k{0};
+struct RunningK {
+  const long long nk;
+  explicit RunningK(int n) : nk(n) { g_running_k += nk; }
+  ~RunningK() { g_running_k -= nk; }
+};
+
 // The projected problems (Rayleigh-Ritz pencil, conjugate-direction coefficients and the
 // Cholesky-QR of the search directions) of the mixed form's block iteration take FP32
 // Gram matrices; they are solved in FP32 (their inputs carry FP32 accuracy, and an FP64
@@ -795,7 +804,7 @@ static int small_rr_any(pc_ctx* c, int k0, int nk, const MatRef<R>& GA, const Ma
                              c->status, c->profiling ? c->small_flops : nullptr, scratch, c->sr_stride, s);
   else
     return launch_small_rr64(GA, GO, n, m, nk, Ops<R>::drop_small, klist, lam, cX, cP, SmallTol<R>::pdir_abs,
-                             c->status, scratch, c->sr_stride, s);
+                             c->status, scratch, c->sr_stride, g_running_k.load() - c->nk, s);
 }
 // The batched block iteration (all k at once).  Per iteration and k:
 //   R = A X - Omega X Lambda,  W = P R on the unconverged columns (P: waves.cuh);
@@ -1094,7 +1103,7 @@ static int fp64_rayleigh_ritz(pc_ctx* c, const KSet& ks) {
   rc = launch_gram<double>(A1, 1, B2, 1, nk, m, n3, 1.0, gpartd, GOd, &gO, s);
   if (rc) return rc;
   rc = launch_small_rr64(gA, gO, m, m, nk, 1e-12, nullptr, lamd, Cd, nullptr, 0.0, c->status,
-                         c->sr_scratch + k0 * c->sr_stride, c->sr_stride, s);
+                         c->sr_scratch + k0 * c->sr_stride, c->sr_stride, 0, s);
   if (rc) return rc;
   // theta = X C; A theta and Omega theta for the residual report
   UpdateArgs<double> u = upd<double>(c, nk, 1, 0, mats<double>(Cd, (long long)m * m), m, m);
@@ -1133,6 +1142,7 @@ extern "C" int pc_bands(pc_ctx* c, double* omega, void* stream) {
   if (!c || !omega) return PC_EINVAL;
   cudaGetLastError();  // launch checks below report only this call's launches
   if (!c->have_design || c->nk == 0) return PC_ESTATE;
+  const RunningK running(c->nk);
   cudaStream_t s = (cudaStream_t)stream;
   PC_CUDA_TRY(cudaEventRecord(c->ev0, s));
   int sl = ph_begin(c, PH_LOOP, 0.0, s);

@@ -1,5 +1,6 @@
 // Projected Rayleigh-Ritz problems in FP64 (the FP64 form's iteration and the final step of both
-// forms): one CTA per k-point, the same steps as the FP32 kernel (small_rr.cu).
+// forms): one CTA per k-point, or a cluster of CTAs where the problems are few (launch_rules.h); the same
+// steps as the FP32 kernel (small_rr.cu).
 //
 // Bound: the FP64 pipe of one SM, two multiply-adds a clock.  A cyclic Jacobi iteration from scratch
 // takes some ten sweeps of 6 n^3 FP64 multiply-adds (and as many for V).  So where the basis holds
@@ -19,13 +20,14 @@
 // through global scratch (L2), as do the logged rotations.
 #include <cooperative_groups.h>
 #include "jacobi.cuh"
+#include "launch_rules.h"
 
 namespace cg = cooperative_groups;
 
 namespace {
 constexpr int S6_THREADS = 800;  // 25 warps: 4 for the planes, 21 for the 2 x 2 blocks at n = 72
 constexpr int S6_PB = 4;         // panel / row-block width (registers)
-constexpr int S6_CLUSTER = 8;    // CTAs per problem where these are few
+constexpr int S6_CLUSTER = kRr64Cluster;  // CTAs per problem where these are few
 
 // Z = A B (herm: A^H B) for n x n matrices, or its upper triangle, in 2 x 2 tiles, up to two per thread
 // (n <= 72: 1296 tiles), which fill the lanes whatever n is; store(i, j, z) runs after every product is
@@ -399,7 +401,7 @@ long long small_rr64_scratch(int n) {
 
 int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n, int m, int nk, double drop_tol, const int* klist,
                       double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
-                      long long stride, cudaStream_t s) {
+                      long long stride, long long others, cudaStream_t s) {
   if (n > SR_NMAX || m > n || m > 24 || n < 1 || stride < small_rr64_scratch(n) || stride % 16) return PC_EINVAL;
   const size_t sm = sizeof(double2) * 2 * (size_t)SR_MAT + sizeof(float2) * SR_MAT + sizeof(Plane<double>) * 72 +
                     sizeof(double) * 2 * SR_NMAX + sizeof(int) * (4 * SR_NMAX + 8);
@@ -413,10 +415,9 @@ int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n,
   static const bool clusters =  // once, thread-safe (k groups launch from several host threads)
       cudaFuncSetAttribute(k_small_rr64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
       cudaFuncSetAttribute(k_small_rr64<S6_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess;
-  // A cluster per problem while the chip has an SM for each of its CTAs and there are products to share
-  // (n > m); 4 problems, n = 48, as the iteration calls it: 1.17 ms by one CTA each, 1.0 by clusters (reference solve 44.5 -> 40.1 ms).
+  // (4 problems, n = 48, as the iteration calls it: 1.17 ms by one CTA each, 1.0 by clusters; the same bits)
   bool launched = false;
-  if (clusters && n > m && (long long)nk * S6_CLUSTER <= sms) {
+  if (clusters && rr64_uses_clusters(n, m, nk, others, sms)) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nk * S6_CLUSTER);
     cfg.blockDim = dim3(S6_THREADS);
