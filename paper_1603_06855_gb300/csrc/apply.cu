@@ -102,7 +102,7 @@ __global__ __launch_bounds__(256) void k_gemm(int Mrows, int K, int lda, long lo
   }
 }
 
-static int sm_count_apply() {
+int device_sms() {
   static const int n = [] {  // queried once; thread-safe static initialisation
     int dev = 0, v = 0;
     cudaGetDevice(&dev);
@@ -123,7 +123,7 @@ int launch_gemms(int Mrows, int K, int lda, long long ldb, long long ldc, const 
     long long tiles = 0;
     for (int g = 0; g < nseg; ++g) tiles += (seg[g].ncols + T - 1) / T;
     tiles *= cdiv(Mrows, T);
-    const long long t = (tiles + sm_count_apply() - 1) / sm_count_apply() * T * T;
+    const long long t = (tiles + device_sms() - 1) / device_sms() * T * T;
     if (best_t < 0 || t < best_t) { best_t = t; best = u; }
   }
   GemmSegs<R> a;

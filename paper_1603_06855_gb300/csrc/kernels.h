@@ -37,6 +37,8 @@ struct SetupArgs {
 long long setup_gj_scratch(int N);
 int launch_setup(const SetupArgs& a, cudaStream_t s);
 
+int device_sms();  // multiprocessors of the device (152 where it cannot be asked)
+
 // Geometry needed on the device to form K_q = T (Q_k + g_q).
 struct Geom {
   double T[9];  // reciprocal basis, row-major: K_i = sum_j T[i*3+j] * (Q_j + g_j)
@@ -144,6 +146,11 @@ template <typename R> struct MatRef {
     for (int t = 1; t < nsplit; ++t) s = cadd(s, q[t * nel]);
     return cscale(s, scale);
   }
+  MatRef from(long long i) const {  // the problems from i on
+    MatRef r = *this;
+    r.p = p + i * nsplit * nel;
+    return r;
+  }
 };
 // Gram products of nk k-points (of klist, or all); problem i of the result is the i-th of them.  part:
 // workspace of at most max_split partial results per problem; G: the reduced result, where the kernel
@@ -182,14 +189,15 @@ int launch_update_tc(const UpdateArgs<float>& u, int* status, cudaStream_t s);
 // index) and their coefficients (n x m).  When cp is given, the conjugate-direction coefficients of the next
 // iteration come from the same CTA (directions at or below pdir_abs dropped); when flops is given, the
 // algorithmic flops of every problem solved are added to it (device counter).  scratch: global scratch of
-// `stride` bytes per problem, at least small_rr32_scratch(n) / small_rr64_scratch(n), a multiple of 16.
+// `stride` bytes, at least small_rr32_scratch(n) / small_rr64_scratch(n) and a multiple of 16, for each of `slots` problems;
+// more problems than that take several launches.
 // others: problems that other calls are solving meanwhile (launch_rules.h).
 int launch_small_rr32(const MatRef<float>& GA, const MatRef<float>& GO, int n, int m, int nk, float drop_tol, const int* klist,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
-                      void* scratch, long long stride, cudaStream_t s);
+                      void* scratch, long long stride, int slots, cudaStream_t s);
 int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n, int m, int nk, double drop_tol, const int* klist,
                       double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
-                      long long stride, long long others, cudaStream_t s);
+                      long long stride, int slots, long long others, cudaStream_t s);
 long long small_rr32_scratch(int n);
 long long small_rr64_scratch(int n);
 // Cholesky-QR transform of the Gram matrices G (m x m).

@@ -13,3 +13,10 @@ constexpr int kRr64Cluster = 8;
 inline bool rr64_uses_clusters(int n, int m, long long nk, long long others, int sms) {
   return n > m && kRr64Cluster * (nk + others) <= sms;
 }
+
+// Projected problems of one launch: larger sets take several launches over the same scratch (0.66 MB a problem in the
+// mixed form, 1.58 MB in FP64, at the widest blocks), which would else be the largest array of a set of many k-points:
+// 103 GB of 239 for 65535 k-points of the FP64 form at N = 27, 3.8 GB now.  Each problem has an SM to itself and a
+// launch ends with its slowest, so sixteen per SM: with four, solves of 700 and 1300 k-points (FP64, 20 bands)
+// were 4 and 5.5 % slower.
+inline int rr_problems_per_launch(long long nk, int sms) { return (int)(nk < 16LL * sms ? nk : 16LL * sms); }

@@ -22,6 +22,7 @@
 #include <vector>
 #include "kernels.h"
 #include "gemm_tc.h"
+#include "launch_rules.h"
 
 
 std::atomic<long long> g_pc_launches{0};
@@ -76,8 +77,8 @@ struct pc_ctx {
   void *E = nullptr, *S = nullptr;  // strain / stress stacks (R precision)
   void *gpart = nullptr, *GA = nullptr, *GO = nullptr, *Cc = nullptr, *Ct = nullptr;
   void* lam = nullptr;           // nk*m (R)
-  unsigned char* sr_scratch = nullptr;  // per k: scratch of the projected problems (small_rr.cu, small_rr64.cu)
-  long long sr_stride = 0;
+  unsigned char* sr_scratch = nullptr;  // scratch of the projected problems in flight (small_rr.cu, small_rr64.cu)
+  long long sr_stride = 0;              // bytes per problem
   double *rnorm = nullptr;
   int *active = nullptr, *kdone = nullptr, *kdone_f = nullptr;
   int *open_k = nullptr, *open_v = nullptr, *open_pos = nullptr, *fresh_k = nullptr, *d_count = nullptr;  // OpenSet, per k group at its k0
@@ -121,6 +122,15 @@ struct pc_ctx {
 static int kgroups(const pc_ctx* c, int nk) {
   if (!c->split || c->prm.precision != PC_MIXED) return 1;
   return std::max(1, std::min(c->groups, nk / kSplitMinK));
+}
+
+// First of the projected problems' scratch slots of group g of `groups` (g = groups: all of them; the set as one group
+// needs no more).
+static long long rr_first(int nk, int groups, int g) {
+  long long first = 0;
+  for (int h = 0; h < g; ++h)
+    first += rr_problems_per_launch((long long)nk * (h + 1) / groups - (long long)nk * h / groups, device_sms());
+  return first;
 }
 
 // Opens a timed phase on stream s (no-op unless profiling); returns the slot index or -1.
@@ -462,7 +472,8 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
   // FP32 problems of up to 3m columns and the FP64 ones of m of the final step, or FP64 ones of up to 3m
   c->sr_stride = c->prm.precision == PC_MIXED ? std::max(small_rr32_scratch(3 * m), small_rr64_scratch(m))
                                               : small_rr64_scratch(3 * m);
-  rc |= dalloc(&c->sr_scratch, (size_t)nk * c->sr_stride);
+  const int groups = kgroups(c, nk);
+  rc |= dalloc(&c->sr_scratch, (size_t)rr_first(nk, groups, groups) * c->sr_stride);
   // The small arrays in two allocations (25 us each).  [open_k | fresh_k | kdone | kdone_f | stall_since] per k,
   // [open_v | open_pos | active | actived] per vector, d_count, pairs per (k, band), npairs:
   const size_t nkb = (size_t)nk * c->nb;
@@ -695,6 +706,8 @@ struct KSet {
   OpenSet open;             // its k-points still iterated (indices from k0), on the device
   int* h_count = nullptr;   // pinned host copy of open.count
   int unconv = 0, iterations = 0, group = 0;
+  unsigned char* rr_scratch = nullptr;  // of its projected problems, rr_slots of them a launch
+  int rr_slots = 0;
   TcPlan* tc = nullptr;     // tensor-core workspaces of this subset
   OzPlan* oz = nullptr;     // sliced products of this subset's final Rayleigh-Ritz step (or NULL)
 };
@@ -795,16 +808,15 @@ template <> struct SmallTol<double> { static constexpr double pdir_abs = 1e-26; 
 template <> struct SmallTol<float> { static constexpr float pdir_abs = 1e-14f; };
 
 template <typename R>
-static int small_rr_any(pc_ctx* c, int k0, int nk, const MatRef<R>& GA, const MatRef<R>& GO, int n, int m,
+static int small_rr_any(pc_ctx* c, const KSet& ks, int nk, const MatRef<R>& GA, const MatRef<R>& GO, int n, int m,
                         const int* klist, R* lam, typename Ops<R>::C2* cX, typename Ops<R>::C2* cP, cudaStream_t s) {
   // the conjugate directions come from the same CTAs
-  unsigned char* scratch = c->sr_scratch + k0 * c->sr_stride;
   if constexpr (std::is_same<R, float>::value)
     return launch_small_rr32(GA, GO, n, m, nk, Ops<R>::drop_small, klist, lam, cX, cP, SmallTol<R>::pdir_abs,
-                             c->status, c->profiling ? c->small_flops : nullptr, scratch, c->sr_stride, s);
+                             c->status, c->profiling ? c->small_flops : nullptr, ks.rr_scratch, c->sr_stride, ks.rr_slots, s);
   else
     return launch_small_rr64(GA, GO, n, m, nk, Ops<R>::drop_small, klist, lam, cX, cP, SmallTol<R>::pdir_abs,
-                             c->status, scratch, c->sr_stride, g_running_k.load() - c->nk, s);
+                             c->status, ks.rr_scratch, c->sr_stride, ks.rr_slots, g_running_k.load() - c->nk, s);
 }
 // The batched block iteration (all k at once).  Per iteration and k:
 //   R = A X - Omega X Lambda,  W = P R on the unconverged columns (P: waves.cuh);
@@ -896,7 +908,7 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
     const int sp = splits(nk, m * m);
     TRY(gram_ph<R>(c, A1, 1, B1, 1, nk, m, n3, (R)1, part, GA, &gA, klist, sp, s));
     TRY(gram_ph<R>(c, A1, 1, B2, 1, nk, m, n3, (R)1, part2, GO, &gO, klist, sp, s));
-    TRY(small_rr_any<R>(c, k0, nk, gA, gO, m, m, klist, lam, Cc, nullptr, s));
+    TRY(small_rr_any<R>(c, ks, nk, gA, gO, m, m, klist, lam, Cc, nullptr, s));
     UpdateArgs<R> u = upd<R>(c, nk, 1, 0, mats<R>(Cc, (long long)m * m), m, m, klist);
     u.in[0][0] = X; u.in[1][0] = AX; u.in[2][0] = OX;
     u.out[0] = Xn; u.out[1] = AXn; u.out[2] = OXn;
@@ -994,7 +1006,7 @@ static int run_block_iteration(pc_ctx* c, KSet& ks) {
     TRY(gram_ph<R>(c, S1, ns, SO, ns, nopen, m, n3, (R)1, part2, GO, &gO, klist, sp, s));
     {
       int sl = ph_begin(c, PH_SMALL, 0.0, s);
-      TRY(small_rr_any<R>(c, k0, nopen, gA, gO, n, m, klist, lam, Cc, Ct, s));
+      TRY(small_rr_any<R>(c, ks, nopen, gA, gO, n, m, klist, lam, Cc, Ct, s));
       ph_end(c, sl, s);
     }
     {
@@ -1041,6 +1053,8 @@ static int run_split_iteration(pc_ctx* c, cudaStream_t s) {
     ks[g].group = g;
     ks[g].open = open_set(c, ks[g].k0, g);
     ks[g].h_count = c->h_count + 4 * g;
+    ks[g].rr_scratch = c->sr_scratch + rr_first(c->nk, ng, g) * c->sr_stride;
+    ks[g].rr_slots = rr_problems_per_launch(ks[g].nk, device_sms());
     ks[g].tc = g ? c->tcg[g] : c->tc;
     ks[g].oz = (c->oz_ready && c->oz) ? (g ? c->ozg[g] : c->oz) : nullptr;
     PC_CUDA_TRY(cudaStreamWaitEvent(c->sk[g], c->ev_fork, 0));
@@ -1103,7 +1117,7 @@ static int fp64_rayleigh_ritz(pc_ctx* c, const KSet& ks) {
   rc = launch_gram<double>(A1, 1, B2, 1, nk, m, n3, 1.0, gpartd, GOd, &gO, s);
   if (rc) return rc;
   rc = launch_small_rr64(gA, gO, m, m, nk, 1e-12, nullptr, lamd, Cd, nullptr, 0.0, c->status,
-                         c->sr_scratch + k0 * c->sr_stride, c->sr_stride, 0, s);
+                         ks.rr_scratch, c->sr_stride, ks.rr_slots, 0, s);
   if (rc) return rc;
   // theta = X C; A theta and Omega theta for the residual report
   UpdateArgs<double> u = upd<double>(c, nk, 1, 0, mats<double>(Cd, (long long)m * m), m, m);
@@ -1162,6 +1176,8 @@ extern "C" int pc_bands(pc_ctx* c, double* omega, void* stream) {
     ks.s = s;
     ks.open = open_set(c, 0, 0);
     ks.h_count = c->h_count;
+    ks.rr_scratch = c->sr_scratch;
+    ks.rr_slots = rr_problems_per_launch(c->nk, device_sms());
     ks.tc = c->tc;
     ks.oz = (c->oz_ready && c->oz) ? c->oz : nullptr;
     rc = (c->prm.precision == PC_FP64) ? run_block_iteration<double>(c, ks) : run_block_iteration<float>(c, ks);

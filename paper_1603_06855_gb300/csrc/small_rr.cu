@@ -35,6 +35,7 @@
 // 60 % of the rounds' shared-memory bytes) and CTA-wide barriers in every column of the reductions.
 // This is the mixed form's version (FP32, four 72 x 74 complex matrices in shared memory);
 // FP64 problems have theirs (small_rr64.cu).
+#include <algorithm>
 #include "jacobi.cuh"
 
 namespace {
@@ -203,15 +204,19 @@ long long small_rr32_scratch(int n) { return 16LL * ((long long)SR_MAX_SWEEPS * 
 
 int launch_small_rr32(const MatRef<float>& GA, const MatRef<float>& GO, int n, int m, int nk, float drop_tol, const int* klist,
                       float* lam_out, float2* coef, float2* cp, float pdir_abs, int* status, double* flops,
-                      void* scratch, long long stride, cudaStream_t s) {
-  if (n > SR_NMAX || m > n || m > 24 || n < 1 || stride < small_rr32_scratch(n) || stride % 16) return PC_EINVAL;
+                      void* scratch, long long stride, int slots, cudaStream_t s) {
+  if (n > SR_NMAX || m > n || m > 24 || n < 1 || slots < 1 || stride < small_rr32_scratch(n) || stride % 16) return PC_EINVAL;
   const size_t sm = sizeof(float2) * 4 * (size_t)SR_MAT + sizeof(Plane<float>) * 72 + sizeof(float) * 2 * SR_NMAX +
                     sizeof(int) * (4 * SR_NMAX + 8);
   static const cudaError_t attr =  // once, thread-safe (k groups launch from several host threads)
       cudaFuncSetAttribute(k_small_rr32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   (void)attr;
-  k_small_rr32<<<nk, SR_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status, flops,
-                                             (unsigned char*)scratch, stride);
-  PC_LAUNCH_CHECK();
+  for (int f = 0; f < nk; f += slots) {
+    const long long o = (long long)f * n * m;
+    k_small_rr32<<<std::min(slots, nk - f), SR_THREADS, sm, s>>>(
+        GA.from(f), GO.from(f), n, m, drop_tol, klist ? klist + f : nullptr, klist ? lam_out : lam_out + (long long)f * m,
+        coef + o, cp ? cp + o : nullptr, pdir_abs, status, flops, (unsigned char*)scratch, stride);
+    PC_LAUNCH_CHECK();
+  }
   return PC_OK;
 }

@@ -18,6 +18,7 @@
 //
 // Two FP64 matrices (72 x 74 complex) and one FP32 matrix fit in shared memory; L, Q and E pass
 // through global scratch (L2), as do the logged rotations.
+#include <algorithm>
 #include <cooperative_groups.h>
 #include "jacobi.cuh"
 #include "launch_rules.h"
@@ -401,41 +402,43 @@ long long small_rr64_scratch(int n) {
 
 int launch_small_rr64(const MatRef<double>& GA, const MatRef<double>& GO, int n, int m, int nk, double drop_tol, const int* klist,
                       double* lam_out, double2* coef, double2* cp, double pdir_abs, int* status, void* scratch,
-                      long long stride, long long others, cudaStream_t s) {
-  if (n > SR_NMAX || m > n || m > 24 || n < 1 || stride < small_rr64_scratch(n) || stride % 16) return PC_EINVAL;
+                      long long stride, int slots, long long others, cudaStream_t s) {
+  if (n > SR_NMAX || m > n || m > 24 || n < 1 || slots < 1 || stride < small_rr64_scratch(n) || stride % 16) return PC_EINVAL;
   const size_t sm = sizeof(double2) * 2 * (size_t)SR_MAT + sizeof(float2) * SR_MAT + sizeof(Plane<double>) * 72 +
                     sizeof(double) * 2 * SR_NMAX + sizeof(int) * (4 * SR_NMAX + 8);
-  static const int sms = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 152;
-    cudaGetLastError();
-    return v;
-  }();
   static const bool clusters =  // once, thread-safe (k groups launch from several host threads)
       cudaFuncSetAttribute(k_small_rr64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess &&
       cudaFuncSetAttribute(k_small_rr64<S6_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess;
   // (4 problems, n = 48, as the iteration calls it: 1.17 ms by one CTA each, 1.0 by clusters; the same bits)
-  bool launched = false;
-  if (clusters && rr64_uses_clusters(n, m, nk, others, sms)) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nk * S6_CLUSTER);
-    cfg.blockDim = dim3(S6_THREADS);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = S6_CLUSTER;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    launched = cudaLaunchKernelEx(&cfg, k_small_rr64<S6_CLUSTER>, GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs,
-                                  status, (unsigned char*)scratch, stride) == cudaSuccess;
-    if (!launched) cudaGetLastError();  // no room for a cluster here: one CTA per problem
+  const bool cluster = clusters && rr64_uses_clusters(n, m, nk, others, device_sms());
+  for (int f = 0; f < nk; f += slots) {
+    const int count = std::min(slots, nk - f);
+    const MatRef<double> ga = GA.from(f), go = GO.from(f);
+    const int* kl = klist ? klist + f : nullptr;
+    double* lam = klist ? lam_out : lam_out + (long long)f * m;
+    const long long o = (long long)f * n * m;
+    double2 *cx = coef + o, *cpf = cp ? cp + o : nullptr;
+    bool launched = false;
+    if (cluster) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(count * S6_CLUSTER);
+      cfg.blockDim = dim3(S6_THREADS);
+      cfg.dynamicSmemBytes = sm;
+      cfg.stream = s;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = S6_CLUSTER;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      launched = cudaLaunchKernelEx(&cfg, k_small_rr64<S6_CLUSTER>, ga, go, n, m, drop_tol, kl, lam, cx, cpf, pdir_abs,
+                                    status, (unsigned char*)scratch, stride) == cudaSuccess;
+      if (!launched) cudaGetLastError();  // no room for a cluster here: one CTA per problem
+    }
+    if (!launched)
+      k_small_rr64<1><<<count, S6_THREADS, sm, s>>>(ga, go, n, m, drop_tol, kl, lam, cx, cpf, pdir_abs, status,
+                                                    (unsigned char*)scratch, stride);
+    PC_LAUNCH_CHECK();
   }
-  if (!launched)
-    k_small_rr64<1><<<nk, S6_THREADS, sm, s>>>(GA, GO, n, m, drop_tol, klist, lam_out, coef, cp, pdir_abs, status,
-                                             (unsigned char*)scratch, stride);
-  PC_LAUNCH_CHECK();
   return PC_OK;
 }

@@ -1,5 +1,5 @@
 """The rules that choose between launch forms, compiled for the host: clusters for the FP64 projected problems only
-while every CTA of every running call has an SM."""
+while every CTA of every running call has an SM, projected problems in launches of bounded size."""
 import ctypes
 import os
 import shutil
@@ -11,6 +11,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1603_06855_gb300", "csrc")
 HARNESS = r"""
 #include "launch_rules.h"
+extern "C" int per_launch(long long nk, int sms) { return rr_problems_per_launch(nk, sms); }
 extern "C" int clusters(int n, int m, long long nk, long long others, int sms) { return rr64_uses_clusters(n, m, nk, others, sms); }
 """
 
@@ -27,6 +28,7 @@ def rules(tmp_path_factory):
                    capture_output=True)
     so = ctypes.CDLL(str(lib))
     so.clusters.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
+    so.per_launch.argtypes = [ctypes.c_longlong, ctypes.c_int]
     return so
 
 
@@ -37,3 +39,10 @@ def test_clusters_alone_and_beside_others(rules):
         assert not rules.clusters(16, 16, 1, 0, sms)  # no products to share
         for others in (0, 4, most - 1, most, 60, 10**6):  # a batch's other designs
             assert rules.clusters(48, 16, 1, others, sms) == (others <= most - 1)
+
+
+def test_projected_problems_per_launch(rules):
+    for nk in (1, 152, 2431, 2432):
+        assert rules.per_launch(nk, 152) == nk
+    for nk in (2433, 65535):
+        assert rules.per_launch(nk, 152) == 2432
