@@ -12,6 +12,7 @@
 // quadratic forms over all (k, band): per chunk of pairs, then over the chunks in FP64.
 #include <algorithm>
 #include "kernels.h"
+#include "launch_rules.h"
 
 // ---------------------------------------------------------------------------
 __global__ void k_omega(const double* __restrict__ lam_m, int nk, int nb, int m, double lref,
@@ -316,7 +317,7 @@ __global__ __launch_bounds__(256) void k_adj_synth12(AdjointArgs a, int jsplit) 
 // Axis-0 synthesis fused with the weighted reduction over (k, band).  The pairs are cut into
 // chunks along the grid's z; each thread synthesises V mirrored pairs of voxels along axis 0 at one (j, l), so
 // that every loaded axis-1/2 coefficient feeds 2 V voxels, and sums its chunk's three
-// weighted quadratic forms in R (FP32 in the mixed form: about a hundred pairs per chunk).  The
+// weighted quadratic forms in R (FP32 in the mixed form: at most 128 pairs, adj_chunks in launch_rules.h).  The
 // chunk sums go to part[chunk][3][ne]; k_adj_finish adds them in FP64 in chunk order.
 // A warp takes 32 columns (j, l) of one group of V pairs; the warps of a CTA take the groups of the same columns
 // and share their coefficients through a ring of kAdjStages pairs in shared memory, filled by asynchronous
@@ -333,6 +334,8 @@ __global__ __launch_bounds__(32 * kAdjReduceWarps) void k_adj_reduce(AdjointArgs
   constexpr int M2 = 2 * M + 1, ROWS = 9 * M2;
   extern __shared__ __align__(16) unsigned char adj_ring[];
   C2* ring = (C2*)adj_ring;  // [kAdjStages][ROWS][32]
+  const int np = *a.npairs;
+  if ((int)blockIdx.z * chunk >= np) return;  // k_adj_finish leaves this chunk out
   const int n0 = a.n0, h0 = (n0 + 1) / 2, lane = threadIdx.x;
   const long long jl = (long long)a.n1 * a.n2;
   const long long v = (long long)blockIdx.x * 32 + lane, vc = v < jl ? v : jl - 1;
@@ -343,7 +346,6 @@ __global__ __launch_bounds__(32 * kAdjReduceWarps) void k_adj_reduce(AdjointArgs
   for (int s = 0; s < V; ++s)
 #pragma unroll
     for (int g = 0; g < M; ++g) ph[s][g] = tab[g * n0 + min(ig * V + s, h0 - 1)];
-  const int np = *a.npairs;
   const int p0 = blockIdx.z * chunk, p1 = min(np, p0 + chunk);
   const C2* t2 = (const C2*)a.t2 + vc;
   auto fill = [&](int p) {  // one group per call, empty past the end, so that the wait counts are constant
@@ -425,11 +427,12 @@ __global__ __launch_bounds__(32 * kAdjReduceWarps) void k_adj_reduce(AdjointArgs
 
 // The chunk sums added in FP64 and combined with the per-element factors.
 template <typename R>
-__global__ void k_adj_finish(AdjointArgs a, int nchunks) {
+__global__ void k_adj_finish(AdjointArgs a, int chunk) {
   const long long ne = (long long)a.n0 * a.n1 * a.n2;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= ne) return;
   const R* part = (const R*)a.part;
+  const int nchunks = (*a.npairs + chunk - 1) / chunk;
   double acc_m = 0.0, acc_1 = 0.0, acc_2 = 0.0;
   for (int c = 0; c < nchunks; ++c) {
     const R* pc = part + (long long)c * 3 * ne;
@@ -469,33 +472,28 @@ static int launch_adjoint_m(const AdjointArgs& a, cudaStream_t s) {
   const int nig = (int)cdiv(h0, V), wy = std::min(nig, kAdjReduceWarps);
   const dim3 block(32, wy);
   dim3 grid((unsigned)cdiv((long long)a.n1 * a.n2, 32), (unsigned)cdiv(nig, wy));
-  // as many pair chunks as are resident at once, so that no last wave is nearly empty; the chunks cover
-  // max_pairs, and the ones past the device's pair count write zeros
+  // as many pair chunks as are resident at once, or a multiple, so that no last wave is nearly empty; the chunks
+  // cover max_pairs, and the ones past the device's pair count are left out
   constexpr size_t ring = sizeof(typename cplx_t<R>::type) * kAdjStages * 9 * M2 * 32;
   static const cudaError_t rattr =
       cudaFuncSetAttribute(k_adj_reduce<R, M, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
   (void)rattr;
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-    cudaGetLastError();
-    return n;
-  }();
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adj_reduce<R, M, V>, 32 * wy, ring) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     per_sm = 1;
   }
-  int nchunks = (int)std::min<long long>(kAdjChunksMax, std::max<long long>(1, (long long)per_sm * sms / (grid.x * grid.y)));
+  int nchunks = (int)std::min<long long>(kAdjChunksMax, std::max<long long>(1, (long long)per_sm * device_sms() / (grid.x * grid.y)));
   nchunks = std::max(1, std::min(nchunks, a.max_pairs));
+  // (the room for kAdjChunksMax FP64 sums a voxel holds twice as many in FP32)
+  if (sizeof(R) == sizeof(float)) nchunks = adj_chunks(a.max_pairs, nchunks, 2 * kAdjChunksMax);
   const int chunk = (int)cdiv(a.max_pairs, nchunks);
   nchunks = (int)cdiv(a.max_pairs, chunk);
   grid.z = nchunks;
   k_adj_reduce<R, M, V><<<grid, block, ring, s>>>(a, chunk);
   PC_LAUNCH_CHECK();
   const long long ne = (long long)a.n0 * a.n1 * a.n2;
-  k_adj_finish<R><<<(unsigned)cdiv(ne, 256), 256, 0, s>>>(a, nchunks);
+  k_adj_finish<R><<<(unsigned)cdiv(ne, 256), 256, 0, s>>>(a, chunk);
   PC_LAUNCH_CHECK();
   return PC_OK;
 }

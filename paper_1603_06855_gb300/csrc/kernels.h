@@ -240,7 +240,7 @@ struct AdjointArgs {
   const double* dchi;
   void* t2;              // scratch: max_pairs x 9 x M2 x n1 x n2 complex (FP64 or FP32)
   const void* phases;    // launch_adj_phases
-  void* part;            // scratch: kAdjChunksMax x 3 x ne chunk sums (FP64 or FP32)
+  void* part;            // scratch: room for kAdjChunksMax x 3 x ne FP64 sums, or twice as many in FP32
   double* grad;
 };
 constexpr int kAdjChunksMax = 32;  // pair chunks of the adjoint's reduction

@@ -20,3 +20,12 @@ inline bool rr64_uses_clusters(int n, int m, long long nk, long long others, int
 // launch ends with its slowest, so sixteen per SM: with four, solves of 700 and 1300 k-points (FP64, 20 bands)
 // were 4 and 5.5 % slower.
 inline int rr_problems_per_launch(long long nk, int sms) { return (int)(nk < 16LL * sms ? nk : 16LL * sms); }
+
+// Chunks of the adjoint's (k, band) pairs, each summed in FP32 before FP64 adds the sums up: the `wave` chunks that the
+// chip holds at once, or a whole multiple, so that a sum runs over at most 128 pairs while there is room for all
+// (`most` sums a voxel; 128 most / 2 pairs and more may take longer ones).  A wave follows the chip and the cell: from some 72^3
+// voxels on it is one chunk, which alone would be one sum over 2000 pairs of a hundred k-points and 20 bands.
+inline int adj_chunks(int pairs, int wave, int most) {
+  const int want = (int)((pairs + 128LL * wave - 1) / (128LL * wave)), room = most / wave;
+  return wave * (want < room ? want : (room > 1 ? room : 1));
+}
