@@ -57,7 +57,7 @@ __device__ __forceinline__ double clamp01(double v) {
 // x = (64 k + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^k 2^(j/64) (1 + r + r^2/2 + ... + r^5/120).
 // The remainder r^6/720 is below 4e-17.  10 FP64 instructions.
 __device__ __forceinline__ double exp_tab(double x, const double* __restrict__ tab) {
-  constexpr double ln2_hi = 6.93147180369123816490e-01;  // ln 2 to 33 bits, and the rest
+  constexpr double ln2_hi = 6.93147180369123816490e-01;  // ln 2 to 33 bits, and the rest (the split of fdlibm)
   constexpr double ln2_lo = 1.90821492927058770002e-10;
   constexpr double shift = 6755399441055744.0;  // 1.5 2^52: rounds to an integer in the low word
   const double t = fma(x, 64.0 / 0.69314718055994530942, shift);

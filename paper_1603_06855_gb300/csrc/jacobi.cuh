@@ -113,7 +113,7 @@ __device__ __forceinline__ Plane<float> make_plane(float app, float aqq, float2 
 }
 
 // The same in FP64.  The hardware's FP64 root and reciprocal approximations carry some 20 bits; one
-// Newton step each gives the angle to about 1e-12, and what that leaves of a_uv goes to the next
+// Newton-Raphson step each gives the angle to about 1e-12, and what that leaves of a_uv goes to the next
 // sweep (the entry is not set to zero).  c = (1 + t^2)^-1/2 is exact to rounding for the tangent used: its
 // binomial series for small t^2 (all but a few rotations here), else the correctly rounded root.
 __device__ __forceinline__ bool plane_rotates(double app, double aqq, double b2, double floor_abs) {

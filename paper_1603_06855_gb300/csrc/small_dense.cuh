@@ -13,7 +13,8 @@ __device__ __forceinline__ double rcp_approx(double x) {
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   return y;
 }
-// 1 / x to rounding for a normal x: two Newton steps on the hardware's 20 bits, four FP64 instructions.
+// 1 / x to an ulp for a normal x > 0 with a normal result: two steps of the Newton-Raphson iteration
+// y <- y + y (1 - x y) from the hardware's approximation of some 20 bits, four FP64 instructions.
 __device__ __forceinline__ double inv_newton(double x) {
   double y = rcp_approx(x);
   y = fma(y, fma(-x, y, 1.0), y);
@@ -21,7 +22,7 @@ __device__ __forceinline__ double inv_newton(double x) {
 }
 // 1 / sqrt(x) to rounding, for the factorisations.
 __device__ __forceinline__ float inv_sqrt(float x) { return 1.f / sqrtf(x); }
-__device__ __forceinline__ double inv_sqrt(double x) {  // two Newton steps: a few FP64 instructions
+__device__ __forceinline__ double inv_sqrt(double x) {  // two Newton-Raphson steps y <- y + y (1 - x y^2) / 2, as above
   double y = rsqrt_approx(x);
   y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
   return fma(0.5 * y, fma(-x * y, y, 1.0), y);
