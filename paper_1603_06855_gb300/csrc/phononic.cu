@@ -803,9 +803,11 @@ struct RunningK {
 // in FP64 on FP64 Grams.
 template <typename R> struct SmallTol;
 template <> struct SmallTol<double> { static constexpr double pdir_abs = 1e-26; };
-// FP32: directions of norm 1e-7 still lead somewhere after the second projection (one or two iterations
-// fewer than with 1e-12 on the design workloads).
-template <> struct SmallTol<float> { static constexpr float pdir_abs = 1e-14f; };
+// FP32: at norms of a few roundings (1e-7) what is left of a direction is rounding, and normalising it puts that into
+// P and, ten million times enlarged, into the carried A P and Omega P: of 16 start blocks on uniform SC cells (N = 125, 21
+// bands, 40 k-points) eight then broke down at 1e-14, with 41 to 50 iterations and frequencies off by up to 2.4e-6;
+// at 1e-12 all take 17 to 19, for 7 % more iterations (and no more time) over a mix of designs.
+template <> struct SmallTol<float> { static constexpr float pdir_abs = 1e-12f; };
 
 template <typename R>
 static int small_rr_any(pc_ctx* c, const KSet& ks, int nk, const MatRef<R>& GA, const MatRef<R>& GO, int n, int m,
