@@ -166,7 +166,13 @@ __global__ void k_toeplitz(const double2* __restrict__ sf, int M, double V, doub
 // Rows already swept (i before the block) and those to come keep A_ij = -A_ji^H between them and
 // A_ij = A_ji^H among themselves, so the upper triangle of 16 x 16 tiles is enough: R_j = -A_j1^H for a
 // swept j, Ai1 = s_i R_i^H with s_i = -1 for a swept i and +1 else, and Ai1 <- ((P R)_i)^H above the block.
-// Two launches a panel: P R, and the update of the tiles, in which one more CTA per matrix inverts the
+// The pivot block enters by the inverse of its Cholesky factor, A11 = L L^H: with Y = L^-1 R the update is
+// Aij <- Aij - s_i Y_i^H Y_j, and P R = L^-H Y, P = L^-H L^-1.  An inverse P itself, formed from the block and
+// multiplied in, stands for a block that differs by eps cond(A11) of its size, which the condition then
+// multiplies once more: T W - 1 of compliance operators of N = 343 and condition 1.7e4 is 8e-12 by the factor,
+// 1e-11 to 1e-9 by P, 6e-11 to 2e-6 by P on the whole matrix in 32 columns, and was 2e-7 to 7e-3 by P of a block
+// whose two triangles had drifted apart by rounding (everything is taken from upper triangles).
+// Two launches a panel: Y and P R, and the update of the tiles, in which one more CTA per matrix factors the
 // next pivot block.  That block is ready early: the update before stored it as of then, and the CTA
 // applies this panel's term itself.  The tiles of the next panel's rows store R for the next step.
 // blockIdx.z or .y selects the matrix.
@@ -179,30 +185,38 @@ constexpr int GJ_B = 16;
 struct GjBufs {
   double2* A;   // 2 x N x N
   double2* R;   // 2 parities x 2 x GJ_B x N: rows of the pivot block
-  double2* PR;  // 2 x GJ_B x N
-  double2* P;   // 2 parities x 2 x GJ_B x GJ_B: inverse pivot blocks
+  double2* Y;   // 2 x GJ_B x N: L^-1 R
+  double2* PR;  // 2 x GJ_B x N: P R, and P in the block's own columns
+  double2* Li;  // 2 parities x 2 x GJ_B x GJ_B: L^-1
   double2* D;   // 2 parities x 2 x GJ_B x GJ_B: diagonal blocks two panels ahead
 };
 
-// Inverse of the Hermitian positive definite block held by 256 threads, one entry each (rows and columns
-// past N: the identity), scalar Gauss-Jordan steps.  Every warp forms the pivot's reciprocal for itself (a
-// broadcast would cost a barrier), so it is kept to a few FP64 instructions.
-__device__ __forceinline__ double2 gj_block_inverse(double2 v, double2 (*S)[GJ_B + 1]) {
+// L^-1 of the Hermitian positive definite block held by 256 threads, one entry each (rows and columns past N: the
+// identity), from its upper triangle: Gaussian elimination of the block, its row operations applied to the identity,
+// whose part below the diagonal takes the place of the lower triangle; then the rows over the roots of the
+// pivots.  Every warp forms the pivot's reciprocal for itself (a broadcast would cost a barrier), so it is kept to a
+// few FP64 instructions.
+__device__ __forceinline__ double2 gj_factor_inverse(double2 v, double2 (*S)[GJ_B + 1]) {
   const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  if (r > c) v = make_double2(0.0, 0.0);
   for (int k = 0; k < GJ_B; ++k) {
     S[r][c] = v;
     __syncthreads();
-    const double ip = inv_newton(S[k][k].x);  // real for a Hermitian block
-    const double2 row = S[k][c], col = cscale(S[r][k], -ip);
-    if (r == k) v = c == k ? make_double2(ip, 0.0) : cscale(row, ip);
-    else if (c == k) v = col;
-    else cfma(v, col, row);
+    const double ip = inv_newton(S[k][k].x);
+    const double2 row = S[k][c], l = cscale(cconj(S[k][r]), -ip);
+    if (r > k) {
+      if (c == k) v = l;
+      else if (c >= r || c < k) cfma(v, l, row);
+    }
     __syncthreads();
   }
-  return v;
+  S[r][c] = v;
+  __syncthreads();
+  const double d = inv_sqrt(S[r][r].x);
+  return r < c ? make_double2(0.0, 0.0) : (r == c ? make_double2(d, 0.0) : cscale(v, d));
 }
 
-// Start: R of panel 0, the inverse of pivot block 0 and the diagonal block of panel 1.
+// Start: R of panel 0, the factor of pivot block 0 and the diagonal block of panel 1.
 __global__ __launch_bounds__(256) void k_gj_start(GjBufs g, int N) {
   __shared__ double2 S[GJ_B][GJ_B + 1];
   const int z = blockIdx.y;
@@ -211,7 +225,7 @@ __global__ __launch_bounds__(256) void k_gj_start(GjBufs g, int N) {
   if (blockIdx.x == 0) {
     double2 v = make_double2(r == c ? 1.0 : 0.0, 0.0);
     if (r < N && c < N) v = A[(long long)r * N + c];
-    g.P[z * GJ_B * GJ_B + threadIdx.x] = gj_block_inverse(v, S);
+    g.Li[z * GJ_B * GJ_B + threadIdx.x] = gj_factor_inverse(v, S);
     const int r1 = GJ_B + r, c1 = GJ_B + c;
     g.D[2 * GJ_B * GJ_B + z * GJ_B * GJ_B + threadIdx.x] =
         (r1 < N && c1 < N) ? A[(long long)r1 * N + c1] : make_double2(r == c ? 1.0 : 0.0, 0.0);
@@ -220,43 +234,54 @@ __global__ __launch_bounds__(256) void k_gj_start(GjBufs g, int N) {
   if (j < N) g.R[((long long)z * GJ_B + r) * N + j] = r < N ? A[(long long)r * N + j] : make_double2(0.0, 0.0);
 }
 
-// P R of one panel.
-__global__ __launch_bounds__(256) void k_gj_panel(GjBufs g, int N, int par) {
-  __shared__ double2 Ps[GJ_B][GJ_B + 1], Rs[GJ_B][GJ_B + 1];
-  const int z = blockIdx.y, r = threadIdx.x >> 4, c = threadIdx.x & 15, j = blockIdx.x * GJ_B + c;
+// Y and P R of panel p; in the pivot block's own columns P.
+__global__ __launch_bounds__(256) void k_gj_panel(GjBufs g, int N, int p) {
+  __shared__ double2 Ls[GJ_B][GJ_B + 1], Rs[GJ_B][GJ_B + 1], Ys[GJ_B][GJ_B + 1];
+  const int z = blockIdx.y, par = p & 1, r = threadIdx.x >> 4, c = threadIdx.x & 15, j = blockIdx.x * GJ_B + c;
   const long long o = ((long long)z * GJ_B + r) * N + j;
-  Ps[r][c] = g.P[(2 * par + z) * GJ_B * GJ_B + threadIdx.x];
+  Ls[r][c] = g.Li[(2 * par + z) * GJ_B * GJ_B + threadIdx.x];
   Rs[r][c] = j < N ? g.R[(long long)par * 2 * GJ_B * N + o] : make_double2(0.0, 0.0);
   __syncthreads();
-  double2 acc = make_double2(0.0, 0.0);
+  double2 y = make_double2(0.0, 0.0);
+  if ((int)blockIdx.x == p) {
+    y = Ls[r][c];
+  } else {
 #pragma unroll
-  for (int l = 0; l < GJ_B; ++l) cfma(acc, Ps[r][l], Rs[l][c]);
-  if (j < N) g.PR[o] = acc;
+    for (int l = 0; l < GJ_B; ++l) cfma(y, Ls[r][l], Rs[l][c]);
+  }
+  Ys[r][c] = y;
+  __syncthreads();
+  double2 pr = make_double2(0.0, 0.0);
+#pragma unroll
+  for (int l = 0; l < GJ_B; ++l) cfmac(pr, Ls[l][r], Ys[l][c]);
+  if (j < N) {
+    g.Y[o] = y;
+    g.PR[o] = pr;
+  }
 }
 
 // One panel step: the upper tiles (blockIdx.x - 1 numbers them by rows), and in blockIdx.x = 0 the next
-// pivot block's inverse.
+// pivot block's factor.
 __global__ __launch_bounds__(256) void k_gj_update(GjBufs g, int N, int p, int nt) {
-  __shared__ double2 X[GJ_B][GJ_B + 1], Y[GJ_B][GJ_B + 1];
+  __shared__ double2 X[GJ_B][GJ_B + 1], Z[GJ_B][GJ_B + 1];
   const int z = blockIdx.y, par = p & 1, r = threadIdx.x >> 4, c = threadIdx.x & 15;
   double2* A = g.A + (long long)z * N * N;
-  const double2* R = g.R + (long long)(2 * par + z) * GJ_B * N;
+  const double2* Y = g.Y + (long long)z * GJ_B * N;
   double2* Rn = g.R + (long long)(2 * (par ^ 1) + z) * GJ_B * N;
   const double2* PR = g.PR + (long long)z * GJ_B * N;
   const double2 zero = make_double2(0.0, 0.0);
   if (blockIdx.x == 0) {
     if (p + 1 >= nt) return;
     const int j = (p + 1) * GJ_B + c;
-    X[r][c] = j < N ? R[(long long)r * N + j] : zero;
-    Y[r][c] = j < N ? PR[(long long)r * N + j] : zero;
+    X[r][c] = j < N ? Y[(long long)r * N + j] : zero;
     double2 v = g.D[(2 * (par ^ 1) + z) * GJ_B * GJ_B + threadIdx.x];
     __syncthreads();
     double2 acc = zero;
 #pragma unroll
-    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Y[l][c]);
+    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], X[l][c]);
     v = csub(v, acc);
     __syncthreads();
-    g.P[(2 * (par ^ 1) + z) * GJ_B * GJ_B + threadIdx.x] = gj_block_inverse(v, X);
+    g.Li[(2 * (par ^ 1) + z) * GJ_B * GJ_B + threadIdx.x] = gj_factor_inverse(v, X);
     return;
   }
   // tile (I, J), I <= J, number t = I nt - I (I - 1) / 2 + J - I
@@ -270,8 +295,7 @@ __global__ __launch_bounds__(256) void k_gj_update(GjBufs g, int N, int p, int n
   const bool in = i < N && j < N;
   double2 v = zero;
   if (I == p) {
-    if (J == p) v = g.P[(2 * par + z) * GJ_B * GJ_B + threadIdx.x];
-    else if (j < N) v = PR[(long long)r * N + j];
+    if (j < N) v = PR[(long long)r * N + j];
   } else if (J == p) {  // above the block: transposed through shared memory
     const int ii = I * GJ_B + c;
     X[r][c] = ii < N ? PR[(long long)r * N + ii] : zero;
@@ -279,13 +303,13 @@ __global__ __launch_bounds__(256) void k_gj_update(GjBufs g, int N, int p, int n
     v = cconj(X[c][r]);
   } else {
     const int ii = I * GJ_B + c;
-    X[r][c] = ii < N ? R[(long long)r * N + ii] : zero;
-    Y[r][c] = j < N ? PR[(long long)r * N + j] : zero;
+    X[r][c] = ii < N ? Y[(long long)r * N + ii] : zero;
+    Z[r][c] = j < N ? Y[(long long)r * N + j] : zero;
     if (in) v = A[(long long)i * N + j];
     __syncthreads();
     double2 acc = zero;
 #pragma unroll
-    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Y[l][c]);
+    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Z[l][c]);
     v = I < p ? cadd(v, acc) : csub(v, acc);
   }
   if (in) A[(long long)i * N + j] = v;
@@ -351,13 +375,14 @@ int launch_setup(const SetupArgs& a, cudaStream_t s) {
   GjBufs g;
   g.A = a.W;
   g.R = a.gj;
-  g.PR = g.R + 4LL * GJ_B * N;
-  g.P = g.PR + 2LL * GJ_B * N;
-  g.D = g.P + 4LL * GJ_B * GJ_B;
+  g.Y = g.R + 4LL * GJ_B * N;
+  g.PR = g.Y + 2LL * GJ_B * N;
+  g.Li = g.PR + 2LL * GJ_B * N;
+  g.D = g.Li + 4LL * GJ_B * GJ_B;
   k_gj_start<<<dim3(nt, 2), 256, 0, s>>>(g, N);
   PC_LAUNCH_CHECK();
   for (int p = 0; p < nt; ++p) {
-    k_gj_panel<<<dim3(nt, 2), 256, 0, s>>>(g, N, p & 1);
+    k_gj_panel<<<dim3(nt, 2), 256, 0, s>>>(g, N, p);
     PC_LAUNCH_CHECK();
     k_gj_update<<<dim3(1 + nt * (nt + 1) / 2, 2), 256, 0, s>>>(g, N, p, nt);
     PC_LAUNCH_CHECK();
@@ -368,4 +393,4 @@ int launch_setup(const SetupArgs& a, cudaStream_t s) {
 }
 
 // double2 elements of SetupArgs::gj for N plane waves.
-long long setup_gj_scratch(int N) { return 6LL * GJ_B * N + 8LL * GJ_B * GJ_B; }
+long long setup_gj_scratch(int N) { return 8LL * GJ_B * N + 8LL * GJ_B * GJ_B; }
