@@ -72,6 +72,31 @@ def test_traffic_entries_name_existing_sources_and_go_stale_with_them(tmp_path, 
     assert bench.traffic_per_launch("k_tc_gram") is None
 
 
+def test_traffic_entries_go_stale_with_their_headers(tmp_path, monkeypatch):
+    """A kernel whose device code lives in headers too: a changed byte there turns the entry into null."""
+    csrc = os.path.join(ROOT, "paper_1603_06855_gb300", "csrc")
+    src = tmp_path / "paper_1603_06855_gb300" / "csrc"
+    src.mkdir(parents=True)
+    for kernel, headers in (("k_small_rr32", ["jacobi.cuh", "small_dense.cuh"]), ("k_tc_gemm", ["waves.cuh"])):
+        entry = dict(bench.TRAFFIC[kernel])
+        assert entry["headers"] == headers
+        text = open(os.path.join(csrc, entry["source"]), "rb").read()
+        (src / entry["source"]).write_bytes(text)
+        entry["sha256"] = hashlib.sha256(text).hexdigest()
+        data = [open(os.path.join(csrc, h), "rb").read() for h in headers]
+        entry["headers_sha256"] = hashlib.sha256(b"".join(data)).hexdigest()
+        monkeypatch.setitem(bench.TRAFFIC, kernel, entry)
+        monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+        assert bench.traffic_per_launch(kernel) is None  # no headers there
+        for h, d in zip(headers, data):
+            (src / h).write_bytes(d)
+        assert bench.traffic_per_launch(kernel) == entry["bytes"]
+        for h, d in zip(headers, data):
+            (src / h).write_bytes(d + b" ")
+            assert bench.traffic_per_launch(kernel) is None
+            (src / h).write_bytes(d)
+
+
 def _run_reference_arm(env_extra):
     import json
     import subprocess
