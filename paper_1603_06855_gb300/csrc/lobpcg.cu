@@ -162,7 +162,7 @@ static int launch_gram64(const BlockList<double>& A, int na, const BlockList<dou
   const int nx = cdiv(nel, 608);
   const int threads = cdiv(cdiv(nel, nx), 32) * 32;
   int split = 1;
-  while (split < max_split && (long long)nx * split * nk < 4 * 152) ++split;
+  while (split < max_split && (long long)nx * split * nk < 4LL * device_sms()) ++split;
   const int chunk = cdiv(cdiv(n3, split), GRAM64_ROWS) * GRAM64_ROWS;
   const size_t sm = sizeof(double2) * GRAM64_ROWS * ((size_t)((na * m) | 1) + ((nbk * m) | 1));
   k_gram64<<<dim3(nx, split, nk), threads, sm, s>>>(A, na, B, nbk, m, n3, chunk, klist, part);
