@@ -53,7 +53,10 @@ extern "C" {
                                 ratio linear in chi, each element the isotropic material they give */
 
 /* Arithmetic of the eigensolver. */
-#define PC_FP64   0  /* every step in FP64 on CUDA cores */
+#define PC_FP64   0  /* FP64 on CUDA cores: operators, blocks, sums and results.  The iteration's projected
+                        problems are first rotated in FP32; that basis is made orthonormal to FP64's
+                        rounding and the problem is then diagonalised in it in FP64 (or from the start, where
+                        the FP32 stage is not good enough) */
 #define PC_MIXED  1  /* split-BF16 tensor-core operator, FP32 block iteration,
                         FP64 Rayleigh-Ritz and stresses at the end */
 
@@ -135,7 +138,8 @@ typedef struct {
                               (32/3) n^3 + s n_k (n_k - 1) 12 (n_k + n) */
   long long grad_pairs;    /* weighted (k, band) pairs of the last pc_gap_and_grad / pc_gap_ks_and_grad */
   double grad_flops_per_pair; /* algorithmic flops of the adjoint per weighted pair:
-                              72 ((2M+1)^3 n2 + (2M+1)^2 n1 n2 + (2M+1) n0 n1 n2) */
+                              36 M ((2M+1)^2 n2 + (2M+1) n1 n2 + n0 n1 n2): sums over mirrored pairs, 4 M
+                              real multiply-adds for the values at two mirrored voxels */
   double ms_host_idle;     /* stream idle time while the host reads the convergence count of each block
                               iteration and enqueues the next one (profiling; summed over the k groups) */
   int rr_sliced;           /* 1 when the Rayleigh-Ritz operator products run as exact 6-bit slice products on

@@ -248,9 +248,9 @@ constexpr int kAdjChunksMax = 32;  // pair chunks of the adjoint's reduction
 int launch_adj_phases(int M, const int n[3], bool fp32, void* ph, cudaStream_t s);
 // fp32: synthesis in FP32 (mixed form); the weighted sum is accumulated in FP64 either way.
 int launch_adjoint(const AdjointArgs& a, bool fp32, cudaStream_t s);
-// Dynamic shared memory of the adjoint's field-synthesis kernel: the N coefficients of one
-// eigenvector component plus the (2M+1)^2 n2 and (2M+1)(n1 + n2) phase tables, complex values
-// of the form's precision.  Grids and cutoffs above kAdjointStagingMax are refused.
+// Dynamic shared memory allowed for the adjoint's field-synthesis kernel: the N coefficients of one
+// eigenvector component, (2M+1)^2 n2 sums along axis 2 and (2M+1)(n1 + n2) phases, of which it stages
+// M (n1 + n2); complex values of the form's precision.  Grids and cutoffs above kAdjointStagingMax are refused.
 size_t adjoint_staging_bytes(int M, int n1, int n2, bool fp32);
 constexpr size_t kAdjointStagingMax = 200 * 1024;
 

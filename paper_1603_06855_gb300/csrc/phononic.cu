@@ -92,9 +92,9 @@ struct pc_ctx {
   double *weights = nullptr;
   int *pairs = nullptr, *npairs = nullptr;
   double2* adj_t2 = nullptr;
-  double* adj_part = nullptr;
+  double* adj_part = nullptr;  // chunk sums of the adjoint's reduction
   double2* adj_ph = nullptr;  // phases of the adjoint's synthesis (room for FP64)
-  float4* Kf = nullptr;  // FP32 wavevectors of the k-points, [k][N] (mixed form)  // chunk sums of the adjoint's reduction
+  float4* Kf = nullptr;  // FP32 wavevectors of the k-points, [k][N] (mixed form)
   TcPlan* tc = nullptr;
   TcPlan* tcg[kMaxGroups] = {};  // workspaces of k groups 1.. (operators shared with tc)
   OzPlan* oz = nullptr;          // sliced FP64-accurate operators of the final Rayleigh-Ritz step (mixed form)
@@ -519,7 +519,7 @@ extern "C" int pc_set_kpoints(pc_ctx* c, const double* q, int nk) {
     c->tc = tc_plan_create(N, (int)nvec, c->status);
     c->tc_ready = false;
     if (!c->tc) rc = PC_ENOMEM;
-    // second k half, run concurrently on its own stream (see pc_bands)
+    // the other k groups, run concurrently on streams of their own (run_split_iteration)
     const int ng = kgroups(c, nk);
     for (int g = 1; g < ng && c->tc; ++g) {
       const int gk = (int)(((long long)nk * (g + 1)) / ng - ((long long)nk * g) / ng);
@@ -596,17 +596,13 @@ extern "C" int pc_set_design(pc_ctx* c, const double* rho, void* stream) {
 // ---------------------------------------------------------------------------
 template <typename R> struct Ops;
 // drop_small: pivot below which a unit-scaled Gram column counts as dependent.
-// rel_drop: a new direction whose Omega-norm^2 after projection is below this fraction of
-// its norm^2 before carries mostly rounding noise and is dropped.
 template <> struct Ops<double> {
   typedef double2 C2;
   static constexpr double drop_small = 1e-12;
-  static constexpr double rel_drop = 1e-10;
 };
 template <> struct Ops<float> {
   typedef float2 C2;
   static constexpr float drop_small = 1e-5f;
-  static constexpr float rel_drop = 1e-4f;
 };
 
 // A x and Omega x for nvec (selected) vectors with the per-k geometry Q (vector v belongs to k = v / m).
