@@ -96,7 +96,7 @@ typedef struct {
                            A gradient through one (k, band) pair (a gap) has a relative error of
                            about that pair's final residual: for a 1e-4 gap gradient in the mixed
                            form pass tol = 1e-4 (the default suits all-band weighted objectives).
-                           The iteration aims at half of it: a k-point between the two gets one more
+                           The iteration aims at 0.4 of it: a k-point between the two gets one more
                            iteration, but counts as converged. */
   int max_iter;         /* iteration cap (0: default); hitting it above the tolerance sets PC_ENOCONV */
   int law;              /* PC_LAW_COMPLIANCE (0, default) | PC_LAW_YOUNG; density is linear in chi either way */

@@ -1,6 +1,6 @@
-"""The iteration cap at the edge of the residual target.  The block iteration aims at half the tolerance and gives a
-k-point that has met the tolerance one more iteration to get there, but the tolerance is what a call promises: where the
-last check before the cap finds the residual between half the tolerance and the tolerance, the call has converged
+"""The iteration cap at the edge of the residual target.  The block iteration aims below the tolerance and gives a
+k-point that has met it one more iteration to get there, but the tolerance is what a call promises: where the
+last check before the cap finds the residual a little below the tolerance, the call has converged
 (PC_OK, no k-point counted as unconverged), and one check earlier, above the tolerance, it has not.  The residual of
 every check is read from the library's debug output; tolerances an eighth of a decade apart, of which the
 residuals' steps (a factor of two to four an iteration) leave a quarter or more in that window."""
