@@ -180,7 +180,8 @@ __global__ void k_toeplitz(const double2* __restrict__ sf, int M, double V, doub
 // Bound: FP64 multiply-adds, 4 N^3 per matrix for the half (N = 729, two matrices: 2.5 ms); 16 columns a
 // panel keep the next pivot's chain (16 dependent steps on one SM, some 20 us) beside the update (30 us a
 // panel at N = 343, 72 at 729, 200 at 1331).  Both matrices, against the whole matrix with 32 columns a panel,
-// three to four launches and two events between streams: N = 343 2.7 -> 0.8 ms, 729 7.6 -> 3.6, 1331 33 -> 18.
+// three to four launches and two events between streams: N = 343 2.7 -> 0.85 ms, 729 7.6 -> 3.7, 1331 33 -> 18.7
+// (0.05, 0.1 and 0.7 ms of it for the factor instead of the inverse).
 constexpr int GJ_B = 16;
 struct GjBufs {
   double2* A;   // 2 x N x N

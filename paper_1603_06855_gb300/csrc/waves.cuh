@@ -62,8 +62,8 @@ __device__ __forceinline__ void strain6_t(R k0, R k1, R k2, const C2* __restrict
 // (up to s) a left inverse of B, and B0 T B0^T inverts A but for the part of the stress that the reference
 // medium cannot tell from an incompatible strain.  For a homogeneous cell P = R0, which is what the
 // iteration used alone before; on strong contrasts R0 leaves the condition of the contrast, P about its
-// square root: the block iterations fall 2 to 2.5 times (level set, FCC N = 729: 113 -> 71; spheres,
-// N = 343: 98-221 -> 39-68; random fields 14-32 -> 11-15) for one more product of two thirds of the operator's.
+// square root: the block iterations fall 1.5 to 3 times (level sets, FCC N = 729: 113 -> 54-82; spheres,
+// N = 343: 98-221 -> 37-69; random fields 14-32 -> 11-17) for one more product of two thirds of the operator's.
 // R0 is diagonal in the plane waves: (a I + b K K^T)^-1 = (I - b/(a + b|K|^2) K K^T) / a with
 // a = mu |K|^2 + s, b = lambda + mu.
 template <typename R>
