@@ -370,7 +370,7 @@ __global__ __launch_bounds__(32 * kAdjReduceWarps) void k_adj_reduce(AdjointArgs
   for (int p = p0; p < p1; ++p) {
     const int pr = a.pairs[p];
     const double wd = a.weights[pr];
-    const R w = (R)wd, wl = (R)(wd * a.lam[pr] * a.lref);
+    const R w = (R)(wd * a.w_scale), wl = (R)(wd * a.lam[pr] * a.lref);
     asm volatile("cp.async.wait_group %0;" ::"n"(kAdjStages - 2) : "memory");
     __syncthreads();  // pair p is there, and every warp is done with pair p - 1, whose slot is filled now
     fill(p + kAdjStages - 1);
@@ -440,7 +440,7 @@ __global__ void k_adj_finish(AdjointArgs a, int chunk) {
     acc_1 += (double)pc[ne + e];
     acc_2 += (double)pc[2 * ne + e];
   }
-  const double acc = -a.d_rho * acc_m - a.two_pi_V_sq * (a.dfc[e] * acc_1 + a.dfc[ne + e] * acc_2);
+  const double acc = -a.d_rho * acc_m - a.two_pi_V_sq * (a.w_inv * (a.dfc[e] * acc_1 + a.dfc[ne + e] * acc_2));
   a.grad[e] = acc * a.inv_sO * a.ve * a.dchi[e];
 }
 

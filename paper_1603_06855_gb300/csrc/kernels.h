@@ -235,7 +235,8 @@ struct AdjointArgs {
   double inv_sO;         // |theta_phys|^2 = |X'|^2 / sO
   double d_rho;
   const double* dfc;     // 2 x ne: d f1 / d chi and d f2 / d chi per element
-  double two_pi_V_sq;    // (2 pi V)^2
+  double two_pi_V_sq;    // (2 pi V)^2 over the square of the stresses' scale
+  double w_scale, w_inv; // power of two that the weights are multiplied by, and its inverse
   double ve;             // element volume
   const double* dchi;
   void* t2;              // scratch: max_pairs x 9 x M2 x n1 x n2 complex (FP64 or FP32)

@@ -70,6 +70,7 @@ struct pc_ctx {
   double* prec_ref = nullptr;           // preconditioner reference medium, 3 values per k group
   int* status = nullptr;
   double* small_flops = nullptr;  // device: algorithmic flops of the FP32 projected problems while profiling
+  double sig_scale = 1, w_scale = 1;  // powers of two: the final step's stresses and the adjoint's weights in FP32's range
   double grad_flops_per_pair = 0;  // algorithmic flops of the adjoint per weighted (k, band)
   // per k-set
   double* Q = nullptr;
@@ -355,6 +356,18 @@ extern "C" int pc_create(const pc_params* p, pc_ctx** out) {
   c->sO = c->V * p->phase1.rho;
   c->sA = c->lref * c->sO;
   c->cA = two_pi * two_pi * c->V * c->V / c->sA;
+  {
+    // The stress coefficients sigma of a normalised eigenvector satisfy (2 pi V)^2 V f |sigma|^2 / sO = lambda (f a
+    // compliance modulus), and the gradient sums w |sigma|^2 with w = dG/dlambda.  In SI sigma goes as a^-4 and its
+    // square leaves FP32 for cells of a millimetre; scaled to |sigma|^2 = lambda / lref, and w by lref, both
+    // factors are nondimensional.  Exact, being powers of two.
+    const double f = (1.0 + p->phase1.nu) / p->phase1.E;
+    const double v = two_pi * c->V * std::sqrt(f * c->V / c->sO) / std::sqrt(c->lref);
+    if (std::isnormal(v) && std::isnormal(c->lref)) {
+      c->sig_scale = std::ldexp(1.0, std::ilogb(v));
+      c->w_scale = std::ldexp(1.0, std::ilogb(c->lref));
+    }
+  }
   memcpy(c->geom.T, c->Tm, sizeof(c->Tm));
   c->geom.M = p->M;
   c->geom.N = N;
@@ -580,8 +593,8 @@ extern "C" int pc_set_design(pc_ctx* c, const double* rho, void* stream) {
       c->tc_ready = true;
     }
     c->oz_ready = false;
-    if (c->oz) {  // the final step's operators: W in SI (the epilogue scales), T_rho / sO
-      rc = oz_prepare_operators(c->oz, c->W, c->T, 1.0, 1.0 / c->sO, s);
+    if (c->oz) {  // the final step's operators: W in SI but for its power of two (the epilogue scales), T_rho / sO
+      rc = oz_prepare_operators(c->oz, c->W, c->T, c->sig_scale, 1.0 / c->sO, s);
       if (rc) return rc;
       c->oz_ready = true;
     }
@@ -607,7 +620,8 @@ template <> struct Ops<float> {
 
 // A x and Omega x for nvec (selected) vectors with the per-k geometry Q (vector v belongs to k = v / m).
 static int apply_fp64(pc_ctx* c, const double2* X, double2* AX, double2* OX, int nvec, int m, const double* Q,
-                      double epi, double alpha_omega, double2* E, double2* S, cudaStream_t s, int phase = -1, VecSel sel = {}) {
+                      double epi, double alpha_omega, double2* E, double2* S, cudaStream_t s, int phase = -1, VecSel sel = {},
+                      double alpha_stress = 1.0) {
   const int N = c->N;
   const long long NN = (long long)N * N;
   const double f = 8.0 * (double)N * (double)N;  // algorithmic flops per complex column
@@ -615,7 +629,7 @@ static int apply_fp64(pc_ctx* c, const double2* X, double2* AX, double2* OX, int
   if (rc) return rc;
   const long long o = (long long)nvec * N;
   const GemmSeg<double> seg[3] = {
-      {c->W, E, S, nvec, 1.0}, {c->W + NN, E + o, S + o, 5 * nvec, 1.0}, {c->T, X, OX, 3 * nvec, alpha_omega, sel}};
+      {c->W, E, S, nvec, alpha_stress}, {c->W + NN, E + o, S + o, 5 * nvec, alpha_stress}, {c->T, X, OX, 3 * nvec, alpha_omega, sel}};
   const int slot = phase >= 0 ? ph_begin(c, phase, f * 9.0 * nvec, s) : -1;
   rc = launch_gemms<double>(N, N, N, N, N, seg, 3, s);
   ph_end(c, slot, s);
@@ -1103,10 +1117,11 @@ static int fp64_rayleigh_ritz(pc_ctx* c, const KSet& ks) {
   double* lamd = c->lamd + vo;
   int rc;
   const double2* X = c->Xd + vo * n3;
+  const double epi = c->cA / c->sig_scale;
   if (ks.oz)
-    rc = apply_sliced(c, ks.oz, X, AXd, OXd, (int)nvec, m, c->Q + 3 * k0, c->cA, Ed, Sd, s);
+    rc = apply_sliced(c, ks.oz, X, AXd, OXd, (int)nvec, m, c->Q + 3 * k0, epi, Ed, Sd, s);
   else
-    rc = apply_fp64(c, X, AXd, OXd, (int)nvec, m, c->Q + 3 * k0, c->cA, 1.0 / c->sO, Ed, Sd, s, PH_RR_GEMM);
+    rc = apply_fp64(c, X, AXd, OXd, (int)nvec, m, c->Q + 3 * k0, epi, 1.0 / c->sO, Ed, Sd, s, PH_RR_GEMM, {}, c->sig_scale);
   if (rc) return rc;
   BlockList<double> A1 = {{X, nullptr, nullptr}}, B1 = {{AXd, nullptr, nullptr}}, B2 = {{OXd, nullptr, nullptr}};
   MatRef<double> gA, gO;
@@ -1237,7 +1252,10 @@ static int gap_and_grad_impl(pc_ctx* c, int n_lower, int mode, double beta, cons
     a.inv_sO = 1.0 / c->sO;
     a.d_rho = c->mc.rho1 - c->mc.rho0;
     a.dfc = c->dfc;
-    a.two_pi_V_sq = (2.0 * M_PI * c->V) * (2.0 * M_PI * c->V);
+    a.w_scale = c->w_scale;
+    a.w_inv = 1.0 / c->w_scale;
+    const double tv = 2.0 * M_PI * c->V / c->sig_scale;
+    a.two_pi_V_sq = tv * tv;
     a.ve = c->ve;
     a.dchi = c->dchi;
     a.t2 = c->adj_t2;
