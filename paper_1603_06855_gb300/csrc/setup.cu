@@ -172,22 +172,21 @@ __global__ void k_toeplitz(const double2* __restrict__ sf, int M, double V, doub
 // multiplies once more: T W - 1 of compliance operators of N = 343 and condition 1.7e4 is 8e-12 by the factor,
 // 1e-11 to 1e-9 by P, 6e-11 to 2e-6 by P on the whole matrix in 32 columns, and was 2e-7 to 7e-3 by P of a block
 // whose two triangles had drifted apart by rounding (everything is taken from upper triangles).
-// Two launches a panel: Y and P R, and the update of the tiles, in which one more CTA per matrix factors the
-// next pivot block.  That block is ready early: the update before stored it as of then, and the CTA
+// Two launches a panel: Y, and the update of the tiles (one 16^3 product each, the pivot's rows and columns
+// among them), in which one more CTA per matrix factors the next pivot block.  That block is ready early: the update before stored it as of then, and the CTA
 // applies this panel's term itself.  The tiles of the next panel's rows store R for the next step.
 // blockIdx.z or .y selects the matrix.
 //
 // Bound: FP64 multiply-adds, 4 N^3 per matrix for the half (N = 729, two matrices: 2.5 ms); 16 columns a
 // panel keep the next pivot's chain (16 dependent steps on one SM, some 20 us) beside the update (30 us a
 // panel at N = 343, 72 at 729, 200 at 1331).  Both matrices, against the whole matrix with 32 columns a panel,
-// three to four launches and two events between streams: N = 343 2.7 -> 0.85 ms, 729 7.6 -> 3.7, 1331 33 -> 18.7
-// (0.05, 0.1 and 0.7 ms of it for the factor instead of the inverse).
+// three to four launches and two events between streams: N = 343 2.7 -> 0.75 ms, 729 7.6 -> 3.6, 1331 33 -> 18.3.
+// P R in the panel launch instead of the pivot's tiles, which would else only copy it: 0.12, 0.2 and 0.4 ms more.
 constexpr int GJ_B = 16;
 struct GjBufs {
   double2* A;   // 2 x N x N
   double2* R;   // 2 parities x 2 x GJ_B x N: rows of the pivot block
   double2* Y;   // 2 x GJ_B x N: L^-1 R
-  double2* PR;  // 2 x GJ_B x N: P R, and P in the block's own columns
   double2* Li;  // 2 parities x 2 x GJ_B x GJ_B: L^-1
   double2* D;   // 2 parities x 2 x GJ_B x GJ_B: diagonal blocks two panels ahead
 };
@@ -235,30 +234,18 @@ __global__ __launch_bounds__(256) void k_gj_start(GjBufs g, int N) {
   if (j < N) g.R[((long long)z * GJ_B + r) * N + j] = r < N ? A[(long long)r * N + j] : make_double2(0.0, 0.0);
 }
 
-// Y and P R of panel p; in the pivot block's own columns P.
-__global__ __launch_bounds__(256) void k_gj_panel(GjBufs g, int N, int p) {
-  __shared__ double2 Ls[GJ_B][GJ_B + 1], Rs[GJ_B][GJ_B + 1], Ys[GJ_B][GJ_B + 1];
-  const int z = blockIdx.y, par = p & 1, r = threadIdx.x >> 4, c = threadIdx.x & 15, j = blockIdx.x * GJ_B + c;
+// Y of one panel (L^-1 is lower triangular; a warp holds rows r and r | 1).
+__global__ __launch_bounds__(256) void k_gj_panel(GjBufs g, int N, int par) {
+  __shared__ double2 Ls[GJ_B][GJ_B + 1], Rs[GJ_B][GJ_B + 1];
+  const int z = blockIdx.y, r = threadIdx.x >> 4, c = threadIdx.x & 15, j = blockIdx.x * GJ_B + c;
   const long long o = ((long long)z * GJ_B + r) * N + j;
   Ls[r][c] = g.Li[(2 * par + z) * GJ_B * GJ_B + threadIdx.x];
   Rs[r][c] = j < N ? g.R[(long long)par * 2 * GJ_B * N + o] : make_double2(0.0, 0.0);
   __syncthreads();
   double2 y = make_double2(0.0, 0.0);
-  if ((int)blockIdx.x == p) {
-    y = Ls[r][c];
-  } else {
-#pragma unroll
-    for (int l = 0; l < GJ_B; ++l) cfma(y, Ls[r][l], Rs[l][c]);
-  }
-  Ys[r][c] = y;
-  __syncthreads();
-  double2 pr = make_double2(0.0, 0.0);
-#pragma unroll
-  for (int l = 0; l < GJ_B; ++l) cfmac(pr, Ls[l][r], Ys[l][c]);
-  if (j < N) {
-    g.Y[o] = y;
-    g.PR[o] = pr;
-  }
+#pragma unroll 2
+  for (int l = 0; l <= (r | 1); ++l) cfma(y, Ls[r][l], Rs[l][c]);
+  if (j < N) g.Y[o] = y;
 }
 
 // One panel step: the upper tiles (blockIdx.x - 1 numbers them by rows), and in blockIdx.x = 0 the next
@@ -269,7 +256,7 @@ __global__ __launch_bounds__(256) void k_gj_update(GjBufs g, int N, int p, int n
   double2* A = g.A + (long long)z * N * N;
   const double2* Y = g.Y + (long long)z * GJ_B * N;
   double2* Rn = g.R + (long long)(2 * (par ^ 1) + z) * GJ_B * N;
-  const double2* PR = g.PR + (long long)z * GJ_B * N;
+  const double2* Li = g.Li + (2 * par + z) * GJ_B * GJ_B;
   const double2 zero = make_double2(0.0, 0.0);
   if (blockIdx.x == 0) {
     if (p + 1 >= nt) return;
@@ -294,34 +281,24 @@ __global__ __launch_bounds__(256) void k_gj_update(GjBufs g, int N, int p, int n
   const int J = I + t - (I * nt - I * (I - 1) / 2);
   const int i = I * GJ_B + r, j = J * GJ_B + c;
   const bool in = i < N && j < N;
-  double2 v = zero;
-  if (I == p) {
-    if (j < N) v = PR[(long long)r * N + j];
-  } else if (J == p) {  // above the block: transposed through shared memory
-    const int ii = I * GJ_B + c;
-    X[r][c] = ii < N ? PR[(long long)r * N + ii] : zero;
-    __syncthreads();
-    v = cconj(X[c][r]);
-  } else {
-    const int ii = I * GJ_B + c;
-    X[r][c] = ii < N ? Y[(long long)r * N + ii] : zero;
-    Z[r][c] = j < N ? Y[(long long)r * N + j] : zero;
-    if (in) v = A[(long long)i * N + j];
-    __syncthreads();
-    double2 acc = zero;
+  const int ii = I * GJ_B + c;
+  // Y_i^H Y_j, with L^-1 in the block's own place: L^-H Y = P R in its rows, Y^H L^-1 = (P R)^H above it, P on it
+  X[r][c] = I == p ? Li[threadIdx.x] : (ii < N ? Y[(long long)r * N + ii] : zero);
+  Z[r][c] = J == p ? Li[threadIdx.x] : (j < N ? Y[(long long)r * N + j] : zero);
+  double2 v = in && I != p && J != p ? A[(long long)i * N + j] : zero;
+  __syncthreads();
+  double2 acc = zero;
 #pragma unroll
-    for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Z[l][c]);
-    v = I < p ? cadd(v, acc) : csub(v, acc);
-  }
+  for (int l = 0; l < GJ_B; ++l) cfmac(acc, X[l][r], Z[l][c]);
+  v = I <= p ? cadd(v, acc) : csub(v, acc);
   if (in) A[(long long)i * N + j] = v;
   const int n1 = p + 1;
   if (I == n1) {
     if (j < N) Rn[(long long)r * N + j] = i < N ? v : zero;
-  } else if (J == n1) {  // R of the swept columns: -A_i1^H, written by rows
+  } else if (J == n1) {  // R of the swept columns: -A_i1^H, written by rows (c: row of the tile, r: column of the panel)
     __syncthreads();
     X[r][c] = in ? v : zero;
     __syncthreads();
-    const int ii = I * GJ_B + c;  // c: row of the tile, r: column within the panel
     if (ii < N) Rn[(long long)r * N + ii] = make_double2(-X[c][r].x, X[c][r].y);
   }
   if (I == p + 2 && J == I)
@@ -377,13 +354,12 @@ int launch_setup(const SetupArgs& a, cudaStream_t s) {
   g.A = a.W;
   g.R = a.gj;
   g.Y = g.R + 4LL * GJ_B * N;
-  g.PR = g.Y + 2LL * GJ_B * N;
-  g.Li = g.PR + 2LL * GJ_B * N;
+  g.Li = g.Y + 2LL * GJ_B * N;
   g.D = g.Li + 4LL * GJ_B * GJ_B;
   k_gj_start<<<dim3(nt, 2), 256, 0, s>>>(g, N);
   PC_LAUNCH_CHECK();
   for (int p = 0; p < nt; ++p) {
-    k_gj_panel<<<dim3(nt, 2), 256, 0, s>>>(g, N, p);
+    k_gj_panel<<<dim3(nt, 2), 256, 0, s>>>(g, N, p & 1);
     PC_LAUNCH_CHECK();
     k_gj_update<<<dim3(1 + nt * (nt + 1) / 2, 2), 256, 0, s>>>(g, N, p, nt);
     PC_LAUNCH_CHECK();
@@ -394,4 +370,4 @@ int launch_setup(const SetupArgs& a, cudaStream_t s) {
 }
 
 // double2 elements of SetupArgs::gj for N plane waves.
-long long setup_gj_scratch(int N) { return 8LL * GJ_B * N + 8LL * GJ_B * GJ_B; }
+long long setup_gj_scratch(int N) { return 6LL * GJ_B * N + 8LL * GJ_B * GJ_B; }
