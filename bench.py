@@ -197,7 +197,7 @@ TRAFFIC = {  # DRAM bytes (read + write) per launch from ncu, single-stream pass
     "k_small_rr32": {"source": "small_rr.cu", "sha256": "8a5461725f7aedf5a91600d021b281fa92e055602ed0ed3f716c293ffb9cc6de", "headers": ["jacobi.cuh", "small_dense.cuh"],
                      "headers_sha256": "0a49ad42df642bd3184ef0e41102548862217cb8d03189bca23d4fc3d0cd1083", "bytes": 2.300e+07},
     "k_oz_gemm": {"source": "oz_gemm.cu", "sha256": "66f77606c504fd7a37a983a2184decbdb7127e2c386dfdcc241f19010c6439be", "bytes": 3.399e+08},
-    "k_adj_synth12+k_adj_reduce": {"source": "adjoint.cu", "sha256": "8bd4f79f0b3a264d8df2f69ce64eca81b3ec3cd1046089a9637214fb0394a900", "bytes": 1.399e+09},
+    "k_adj_synth12+k_adj_reduce": {"source": "adjoint.cu", "sha256": "2a7898a92ce728c1681e3334e297726333fe3c37ba7513ac42c9f9751790c9f6", "bytes": 1.399e+09},
 }
 
 
