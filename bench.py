@@ -193,7 +193,7 @@ TRAFFIC = {  # DRAM bytes (read + write) per launch from ncu, single-stream pass
     "k_tc_gram": {"source": "tall_tc.cu", "sha256": "f4575f835187808ceabad893a22623c563e605714c8c7f79e966ee41d1230ca2", "bytes": 1.816e+08},
     "k_tc_update": {"source": "tall_tc.cu", "sha256": "f4575f835187808ceabad893a22623c563e605714c8c7f79e966ee41d1230ca2", "bytes": 2.964e+08},
     "k_tc_gemm": {"source": "gemm_tc.cu", "sha256": "49a21c2ec5a69e219d1425ff16f880f551d94ccff662c01000d4feea19966f47", "headers": ["waves.cuh"],
-                  "headers_sha256": "620c31bf4098218e1f0f58d39fa871f3637484f4699bf92b6dab82f3d05f3293", "bytes": 2.584e+08},
+                  "headers_sha256": "fd1433382ba05e1e78de6e9fa72163126da509e6e34591424bdb1b9144206fdb", "bytes": 2.582e+08},
     "k_small_rr32": {"source": "small_rr.cu", "sha256": "8a5461725f7aedf5a91600d021b281fa92e055602ed0ed3f716c293ffb9cc6de", "headers": ["jacobi.cuh", "small_dense.cuh"],
                      "headers_sha256": "0a49ad42df642bd3184ef0e41102548862217cb8d03189bca23d4fc3d0cd1083", "bytes": 2.300e+07},
     "k_oz_gemm": {"source": "oz_gemm.cu", "sha256": "66f77606c504fd7a37a983a2184decbdb7127e2c386dfdcc241f19010c6439be", "bytes": 3.399e+08},
